@@ -209,50 +209,58 @@ __device__ __forceinline__ uint32_t pack_e4m3x2(float lo, float hi) {
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return (uint32_t)r;
 }
-// four floats -> four E2M1 codes in the low 16 bits (x0 in bits 3:0)
-__device__ __forceinline__ uint32_t pack_e2m1x4(float x0, float x1, float x2, float x3) {
+// four floats -> four E4M3 codes, eight floats -> eight E2M1 codes (the first in the low bits): one assembly block each, so
+// that the narrow results are merged by the conversions themselves and not by separate shifts and permutes
+__device__ __forceinline__ uint32_t pack_e4m3x4(const float *x) {
   uint32_t r;
-  asm("{ .reg .b8 a, b; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
-      "mov.b32 %0, {a, b, 0, 0}; }"
+  asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
       : "=r"(r)
-      : "f"(x0), "f"(x1), "f"(x2), "f"(x3));
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]));
   return r;
 }
-__device__ __forceinline__ float decode_e4m3(uint32_t c) {
-  const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
-  return __half2float(*reinterpret_cast<const __half *>(&h));
+__device__ __forceinline__ uint32_t pack_e2m1x8(const float *x) {
+  uint32_t r;
+  asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
+      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
+      : "=r"(r)
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]));
+  return r;
+}
+// two E4M3 codes -> two floats
+__device__ __forceinline__ void decode_e4m3x2(uint32_t codes, float &lo, float &hi) {
+  asm("{ .reg .b32 t; .reg .b16 a, b; cvt.rn.f16x2.e4m3x2 t, %2; mov.b32 {a, b}, t; cvt.f32.f16 %0, a; cvt.f32.f16 %1, b; }"
+      : "=f"(lo), "=f"(hi)
+      : "h"((uint16_t)codes));
 }
 
 // bounded wait that also gives up as soon as another thread of the CTA has flagged a failure
 // (the flag then holds 1 + the shared-memory offset of the barrier that was never completed, for diagnosis)
 //
-// Waiting warps share their scheduler with the warps doing the softmax arithmetic.  A plain mbarrier.try_wait blocks
-// in hardware for a while before it reports failure, so the retry loop issues few instructions (the variant with an
-// explicit time hint is expanded into a polling loop with nanosleep and clock reads: more instructions, same run
-// time).  The bound is on elapsed clock cycles, checked once per 16 tries.
-constexpr long long kWaitLimitCycles = 400000000ll;  // about 0.2 s
-__device__ __forceinline__ bool wait_slow(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                          long long limit = kWaitLimitCycles) {
-  const long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int k = 0; k < 16; ++k)
-      if (tc::mbar_try_wait(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (clock64() - t0 > limit) break;
-  }
-  atomicCAS(const_cast<int *>(abort_flag), 0, 1 + (int)(tc::smem_u32(bar) & 0xffff));
-  return false;
+// A plain mbarrier.try_wait blocks in hardware for a while (about 4 us here) before it reports failure, so the retry loop
+// issues next to nothing.  The bound is on elapsed clock cycles.  Barriers are named by their shared-memory address, and
+// the loop is kept short: every wait is a copy of it, and the hot code of all roles shares a 32 KB instruction cache.
+constexpr uint32_t kWaitLimitCycles = 400000000u;  // about 0.2 s
+__device__ __forceinline__ uint32_t clock32() {
+  uint32_t t;
+  asm volatile("mov.u32 %0, %%clock;" : "=r"(t));
+  return t;
 }
-__device__ __forceinline__ bool wait_or_abort(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
-                                              long long limit = kWaitLimitCycles) {
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, int *abort_flag,
+                                              uint32_t limit = kWaitLimitCycles) {
   if (tc::mbar_try_wait(bar, parity)) return true;
-  return wait_slow(bar, parity, abort_flag, limit);
+  const uint32_t t0 = clock32();
+  for (;;) {
+    if (tc::mbar_try_wait(bar, parity)) return true;
+    if (*(volatile int *)abort_flag) return false;
+    if (clock32() - t0 > limit) break;
+  }
+  atomicCAS(abort_flag, 0, 1 + (int)(bar & 0xffffu));
+  return false;
 }
 
 // One arrival per warp: every lane's earlier writes are ordered before the elected lane's arrive by the warp barrier.
 // (A per-thread arrive is a shared-memory atomic per thread; hundreds of them per step dominate the step time.)
-__device__ __forceinline__ void warp_arrive(uint64_t *bar) {
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) tc::mbar_arrive(bar);
 }
@@ -330,7 +338,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
   const StreamInfo st0 = load_stream(p, bh, a0), st1 = load_stream(p, bh, a1);
 
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + sm.bars);
-  auto bar = [&](int s, int which) -> uint64_t * { return bars + s * B_COUNT + which; };
+  const uint32_t bars0 = tc::smem_u32(bars);
+  auto bar = [&](int s, int which) -> uint32_t { return bars0 + (uint32_t)(s * B_COUNT + which) * 8u; };
   float *s_factor = reinterpret_cast<float *>(smem + sm.factor);      // [s][set][64]
   uint32_t *s_chg = reinterpret_cast<uint32_t *>(smem + sm.chg);      // [s][set][2]
   uint2 *s_hx = reinterpret_cast<uint2 *>(smem + sm.hx);              // [s][set][64]
@@ -370,7 +379,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = s_tmem_base;
-  volatile int *abortp = &s_abort;
+  int *abortp = &s_abort;
 
   // =========================================================================================== softmax warps
   if (warp < kSoftmaxWarps) {
@@ -460,12 +469,12 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
       if (i > 0) {
         uint2 hv = ld_shared_volatile_v2(prev_hx);
         for (uint32_t spin = 0; hv.y != (uint32_t)(i - 1); ++spin) {
-          if ((spin & 1023u) == 1023u && (*abortp || spin > (1u << 24))) break;
+          if ((spin & 1023u) == 1023u && (*(volatile int *)abortp || spin > (1u << 24))) break;
           hv = ld_shared_volatile_v2(prev_hx);
         }
         const bool got = hv.y == (uint32_t)(i - 1);
         if (!__all_sync(0xffffffffu, got)) {
-          atomicCAS(const_cast<int *>(abortp), 0, 1 + (int)(tc::smem_u32(bar(s, B_CORROK)) & 0xffff));
+          atomicCAS(abortp, 0, 1 + (int)(bar(s, B_CORROK) & 0xffffu));
           break;
         }
         h_prev = __uint_as_float(hv.x);
@@ -511,7 +520,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
             unf2(fma2(f2(v[c * 16 + 4 * j + 2], v[c * 16 + 4 * j + 3]), coef2, bias2), t2, t3);
             const float w0 = ex2(t0), w1 = ex2(t1), w2 = ex2(t2), w3 = ex2(t3);
             sum2 = add2(add2(sum2, f2(w0, w1)), f2(w2, w3));
-            w4[j] = pack_e4m3x2(w0, w1) | (pack_e4m3x2(w2, w3) << 16);
+            const float w[4] = {w0, w1, w2, w3};
+            w4[j] = pack_e4m3x4(w);
           }
           *reinterpret_cast<uint4 *>(prow + c * 1024) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
         }
@@ -545,8 +555,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
             uint32_t w4[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              w4[j] = pack_e4m3x2(v[c * 16 + 4 * j], v[c * 16 + 4 * j + 1]) |
-                      (pack_e4m3x2(v[c * 16 + 4 * j + 2], v[c * 16 + 4 * j + 3]) << 16);
+              w4[j] = pack_e4m3x4(v + c * 16 + 4 * j);
             *reinterpret_cast<uint4 *>(prow + c * 1024) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
           }
           ell += kEtaP8 * (s0 + s1);  // the denominator sums the amplified fp32 weights; eta restores the unit
@@ -556,21 +565,25 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
         // sigma = E4M3(448 * max w); scaled weight u = w * 2688 / sigma = 2^(x - m + log2(2688) - log2(sigma)).
         // The four scale chains run first (interleaved), then the exponentials in batches of 32 that are all issued
         // before any is consumed.
-        uint32_t sfword = 0;
+        // A group whose scale code is 0 takes the smallest scale for u: its codes do not matter, the product multiplies
+        // them by the stored scale 0, and the denominator gets w = u * sigma / 2688 either way.
         float bb[4], sl[4];
-        bool live[4];
+        uint32_t sfw[2];
 #pragma unroll
-        for (int gi = 0; gi < 4; ++gi) {
-          const float gw = ex2(fmaf(gm[gi], coef, -m_new));
-          const uint32_t sc = pack_e4m3x2(__fmul_rn(448.0f, gw), 0.f) & 0xffu;
-          sfword |= sc << (8 * gi);
-          // E4M3 code -> fp32: for normal codes the bit pattern is a shift and a re-bias; the 7 subnormal codes
-          // and zero (weights below 2^-15 of the row maximum) take the general conversion
-          const float sigma = sc >= 8u ? __uint_as_float((sc << 20) + 0x3C000000u) : decode_e4m3(sc);
-          live[gi] = sc != 0u;
-          bb[gi] = (live[gi] ? 11.392317422778762f - lg2(sigma) : 0.f) - m_new;  // log2(2688) = 11.3923...
-          sl[gi] = live[gi] ? sigma * (1.0f / 2688.0f) : 1.0f;
+        for (int h = 0; h < 2; ++h) {
+          const float g0 = __fmul_rn(448.0f, ex2(fmaf(gm[2 * h], coef, -m_new)));
+          const float g1 = __fmul_rn(448.0f, ex2(fmaf(gm[2 * h + 1], coef, -m_new)));
+          sfw[h] = pack_e4m3x2(g0, g1);
+          float s0, s1;
+          decode_e4m3x2(sfw[h], s0, s1);
+          s0 = fmaxf(s0, 0.001953125f);
+          s1 = fmaxf(s1, 0.001953125f);
+          bb[2 * h] = (11.392317422778762f - lg2(s0)) - m_new;  // log2(2688) = 11.3923...
+          bb[2 * h + 1] = (11.392317422778762f - lg2(s1)) - m_new;
+          sl[2 * h] = s0 * (1.0f / 2688.0f);
+          sl[2 * h + 1] = s1 * (1.0f / 2688.0f);
         }
+        const uint32_t sfword = __byte_perm(sfw[0], sfw[1], 0x5410);
         *reinterpret_cast<uint32_t *>(smem + sm.sfp[s][g] + (r & 31) * 16 + (r >> 5) * 4) = sfword;
         {
           // the scores of the row become the exponent arguments, then the scaled weights, in place
@@ -592,10 +605,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
               float s0, s1;
               unf2(add2(add2(sa, sb), add2(sc2, sd)), s0, s1);
               ell = fmaf(s0 + s1, sl[gp * 2 + h], ell);
-              const uint32_t c0 = pack_e2m1x4(x[0], x[1], x[2], x[3]) | (pack_e2m1x4(x[4], x[5], x[6], x[7]) << 16);
-              const uint32_t c1 = pack_e2m1x4(x[8], x[9], x[10], x[11]) | (pack_e2m1x4(x[12], x[13], x[14], x[15]) << 16);
-              cw[h * 2 + 0] = live[gp * 2 + h] ? c0 : 0u;
-              cw[h * 2 + 1] = live[gp * 2 + h] ? c1 : 0u;
+              cw[h * 2 + 0] = pack_e2m1x8(x);
+              cw[h * 2 + 1] = pack_e2m1x8(x + 8);
             }
             *reinterpret_cast<uint4 *>(prow + gp * 1024) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
           }
@@ -876,7 +887,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     if (S.a >= 0) {
       const unsigned long long qmask = table_mask(p, S.a);
       uint16_t *stage = reinterpret_cast<uint16_t *>(smem + sm.kst[s][0]);  // [64][D] bf16 over the K ring
-      bool ok = S.L > 0 && !*abortp;
+      bool ok = S.L > 0 && !*(volatile int *)abortp;
       if (ok) ok = wait_or_abort(bar(s, B_ELL), 0, abortp);
       if (ok) ok = wait_or_abort(bar(s, B_PVDONE + ((S.L - 1) & kMask)), ((S.L - 1) >> kShift) & 1, abortp);
       const int ltid = tid - (kSoftmaxWarps + 4 * s) * 32;  // thread index inside the stream's correction group
@@ -946,13 +957,12 @@ __global__ void bounded_wait_probe_kernel(int *status, long long limit) {
   __shared__ uint64_t never;
   __shared__ int s_abort;
   if (threadIdx.x == 0) {
-    tc::mbar_init(&never, 1);
+    tc::mbar_init(tc::smem_u32(&never), 1);
     tc::fence_barrier_init();
     s_abort = 0;
   }
   __syncthreads();
-  volatile int *abortp = &s_abort;
-  const bool ok = wait_or_abort(&never, 0, abortp, limit);
+  const bool ok = wait_or_abort(tc::smem_u32(&never), 0, &s_abort, (uint32_t)limit);
   __syncthreads();
   if (threadIdx.x == 0 && (!ok || s_abort)) {
     atomicExch(status, kDevTimeout);

@@ -27,7 +27,7 @@ __global__ void __launch_bounds__(kPeakThreads, 1) mma_peak_kernel(int n, int it
     tc::tmem_relinquish();
   }
   if (tid == 32) {
-    tc::mbar_init(&s_bar, 1);
+    tc::mbar_init(tc::smem_u32(&s_bar), 1);
     tc::fence_barrier_init();
     s_fail = 0;
   }
@@ -71,9 +71,9 @@ __global__ void __launch_bounds__(kPeakThreads, 1) mma_peak_kernel(int n, int it
       }
       __syncwarp();
     }
-    if (tc::elect_one()) tc::mma_commit(&s_bar);
+    if (tc::elect_one()) tc::mma_commit(tc::smem_u32(&s_bar));
     __syncwarp();
-    if (!tc::mbar_wait(&s_bar, 0)) s_fail = 1;  // bounded
+    if (!tc::mbar_wait(tc::smem_u32(&s_bar), 0)) s_fail = 1;  // bounded
     const long long t1 = clock64();
     if (blockIdx.x == 0 && (tid & 31) == 0) {
       out[0] = t1 - t0;
