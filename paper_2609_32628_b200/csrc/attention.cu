@@ -193,6 +193,24 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// eight accumulator columns of one channel times the columns' factors (and the channel's change of unit)
+__device__ __forceinline__ void scale8(uint32_t (&o)[8], const float *fac, float lane_factor) {
+  const float4 f0 = *reinterpret_cast<const float4 *>(fac), f1 = *reinterpret_cast<const float4 *>(fac + 4);
+  const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+  const uint64_t l2 = f2(lane_factor, lane_factor);
+#pragma unroll
+  for (int j = 0; j < 8; j += 2) {
+    float a, b;
+    unf2(mul2(f2(__uint_as_float(o[j]), __uint_as_float(o[j + 1])), mul2(f2(f[j], f[j + 1]), l2)), a, b);
+    o[j] = __float_as_uint(a);
+    o[j + 1] = __float_as_uint(b);
+  }
+}
 // maximum of 16 values in 8 instructions
 __device__ __forceinline__ float max16(const float *x) {
   const float m0 = max3(x[0], x[1], x[2]), m1 = max3(x[3], x[4], x[5]), m2 = max3(x[6], x[7], x[8]);
@@ -870,12 +888,10 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
         tc::tmem_ld8(tmem + lane_addr + col_o(s) + c0 * 8, o0);
         if (c1 >= 0) tc::tmem_ld8(tmem + lane_addr + col_o(s) + c1 * 8, o1);
         tc::wait_ld();
-#pragma unroll
-        for (int j = 0; j < 8; ++j) o0[j] = __float_as_uint(__uint_as_float(o0[j]) * (fac[c0 * 8 + j] * lane_factor));
+scale8(o0, fac + c0 * 8, lane_factor);
         tc::tmem_st8(tmem + lane_addr + col_o(s) + c0 * 8, o0);
         if (c1 >= 0) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) o1[j] = __float_as_uint(__uint_as_float(o1[j]) * (fac[c1 * 8 + j] * lane_factor));
+          scale8(o1, fac + c1 * 8, lane_factor);
           tc::tmem_st8(tmem + lane_addr + col_o(s) + c1 * 8, o1);
         }
       }
