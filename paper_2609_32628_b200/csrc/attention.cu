@@ -54,18 +54,14 @@ namespace da2 {
 
 namespace {
 
-// Softmax warp sets: set k takes the steps i = k (mod SETS), one thread per 64-key row, four warps (one per TMEM lane
-// quarter) per set.  Plans without a 16-bit tier run four sets; a 16-bit tier needs 8 KB per P image and 16 KB ring
-// stages, which leaves shared memory for two.
-constexpr int kMaxSets = 4;
-template <int SETS> struct Roles {
-  static constexpr int kSoftmaxWarps = 4 * SETS, kCorrWarps = 8;  // four correction warps per stream
-  static constexpr int kMmaWarp0 = kSoftmaxWarps + kCorrWarps;    // Q K^T issue for stream 0, 1
-  static constexpr int kPvWarp0 = kMmaWarp0 + 2;                  // V^T P^T issue for stream 0, 1
-  static constexpr int kLoadWarp0 = kPvWarp0 + 2;                 // K loaders for stream 0, 1, then V loaders
-  static constexpr int NT = (kLoadWarp0 + 4) * 32;                // 1024 (four sets) or 768 (two): whole warpgroups
-  static constexpr int kShift = SETS == 4 ? 2 : 1, kMask = SETS - 1;
-};
+// Softmax warp sets: set k takes the steps i = k (mod 4), one thread per 64-key row, four warps (one per TMEM lane
+// quarter) per set.
+constexpr int kSets = 4, kShift = 2, kMask = kSets - 1;
+constexpr int kSoftmaxWarps = 4 * kSets, kCorrWarps = 8;  // four correction warps per stream
+constexpr int kMmaWarp0 = kSoftmaxWarps + kCorrWarps;     // Q K^T issue for stream 0, 1
+constexpr int kPvWarp0 = kMmaWarp0 + 2;                   // V^T P^T issue for stream 0, 1
+constexpr int kLoadWarp0 = kPvWarp0 + 2;                  // K loaders for stream 0, 1, then V loaders
+constexpr int NT = (kLoadWarp0 + 4) * 32;                 // 1024
 constexpr uint32_t kTmemCols = 512;
 // TMEM column map
 __host__ __device__ constexpr uint32_t col_s(int s, int buf) { return (uint32_t)(s * 2 + buf) * 64u; }
@@ -83,81 +79,99 @@ constexpr float kOffsetP8 = 8.807f;      // base-2 exponent offset (about log2 4
 // barrier indices inside one stream's group
 // (a parity wait can only tell the latest completion from the one before, so every barrier is laid out such that no
 // waiter can fall two completions behind: buffers indexed by step parity get one barrier per buffer)
-enum { B_FULLK = 0, B_FULLV = 4, B_KFREE = 10, B_VFREE = 14, B_SREADY = 20, B_SFREE = 24, B_PREADY = 26, B_CORROK = 30, B_PVDONE = 34, B_ELL = 38, B_Q = 39, B_COUNT = 40 };
-constexpr int kMaxK = 4, kMaxV = 6, kInfoRing = 8;
+constexpr int kMaxK = 6, kMaxV = 8, kInfoRing = 16;
+constexpr int kStepBars = 8;  // barriers for the steps of a stream between softmax and product (kSets of them unless SEGMENTED)
+enum {
+  B_FULLK = 0, B_KFREE = B_FULLK + kMaxK, B_FULLV = B_KFREE + kMaxK, B_VFREE = B_FULLV + kMaxV, B_SREADY = B_VFREE + kMaxV,
+  B_SFREE = B_SREADY + kSets, B_PREADY = B_SFREE + 2, B_CORROK = B_PREADY + kStepBars, B_PVDONE = B_CORROK + kStepBars,
+  B_ELL = B_PVDONE + kStepBars, B_Q = B_ELL + 1, B_COUNT = B_Q + 1
+};
 
+// Shared memory.  The operand rings and the P slots hold blocks of one size (the largest of the plan's tiers) and the Q
+// records of all tiers are resident, if that leaves rings of at least 2 K and 3 V blocks.  Otherwise (a 16-bit tier at
+// head_dim 128: 16 KB blocks, 8 KB P images) the layout is SEGMENTED: every segment cuts the same bytes into blocks of its
+// own tier, so that only the 16-bit segment has shallow rings, and a stream has one Q buffer, reloaded at the segment
+// boundary.  The price is a drain of the rings at each boundary (about 1.5 us a row).
 struct SmemMap {
-  uint32_t q[2][3];   // Q record per stream and tier
-  uint32_t kst[2][kMaxK];  // K ring per stream (K image + its scale atoms)
-  uint32_t vst[2][kMaxV];  // V ring per stream (V^T image + its scale atom)
-  int nk, nv;                   // ring depths
-  uint32_t kbytes[3], vbytes[3];
-  uint32_t p[2][kMaxSets];   // P operand images per stream, one per softmax set (64 x 64 x <= 2 bytes)
-  uint32_t sfp[2][kMaxSets]; // P scale atoms (512 B)
-  uint32_t factor;    // float [2 streams][sets][64]
+  uint32_t q[2][3];               // Q record per stream and tier (SEGMENTED: the same buffer for every tier)
+  uint32_t kring[2], vring[2];    // per stream: K blocks (K image + scale atoms), V blocks (V^T image + scale atom)
+  uint32_t kbytes[3], vbytes[3];  // bytes to copy per block
+  uint32_t kstage[3], vstage[3];  // bytes per ring entry
+  int nk[3], nv[3];               // ring entries
+  uint32_t p[2];                  // P operand images per stream
+  uint32_t pbytes[3];             // bytes of a P slot (there are four, or SEGMENTED 8, 4, 2)
+  uint32_t sfp[2];    // P scale atoms (512 B), one per step barrier
+  uint32_t factor;    // float [2 streams][kStepBars][64]
   uint32_t hx;        // {float h, int step} [2][sets][64]: running maximum after a step, handed from thread to thread
   uint32_t href;      // float [2][sets][64]: reference of each set's partial denominator
   uint32_t ell;       // float [2][sets][64]
   uint32_t info;      // per stream, ring of kInfoRing steps: {u64 mask, float dk8, pad}
   uint32_t bars;      // uint64 [2][B_COUNT]
-  uint32_t kstage, vstage;  // bytes per ring stage
-  uint32_t pbytes;          // bytes of one P image (the kSets images of a stream are contiguous)
-  uint32_t chg;             // uint32 [2 streams][sets][2]: ballots of the queries whose maximum moved this step
+  uint32_t chg;       // uint32 [2 streams][kStepBars][2]: ballots of the queries whose maximum moved this step
   uint32_t total;
-  bool fits;                // the layout fits the 227 KB a block may use
+  bool fits;          // the layout fits the 227 KB a block may use
 };
 
-__host__ SmemMap make_smem_map(const Params &p, int kSets) {
+__host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   SmemMap m;
   uint32_t cur = 0;
-  auto take = [&](uint32_t bytes) { uint32_t o = cur; cur = (cur + bytes + 127u) / 128u * 128u; return o; };
-  // stream 1's Q descriptors start 1 KB before its images: stream 0's records precede them, so that is valid memory
-  for (int s = 0; s < 2; ++s)
-    for (int t = 0; t < 3; ++t) m.q[s][t] = p.tier_active[t] ? take(p.qrec_bytes[t]) : 0;
-  uint32_t kstage = 0, vstage = 0;
+  auto r128 = [](uint32_t b) { return (b + 127u) / 128u * 128u; };
+  auto take = [&](uint32_t bytes) { uint32_t o = cur; cur = r128(cur + bytes); return o; };
+  uint32_t qmax = 0, kmax = 0, vmax = 0, pmax = 0;
   for (int t = 0; t < 3; ++t) {
     m.kbytes[t] = p.qrec_bytes[t];                     // the K part of a record is laid out like a Q record
     m.vbytes[t] = p.kvrec_bytes[t] - p.qrec_bytes[t];
-    if (p.tier_active[t]) { kstage = max(kstage, m.kbytes[t]); vstage = max(vstage, m.vbytes[t]); }
+    if (!p.tier_active[t]) continue;
+    qmax = max(qmax, p.qrec_bytes[t]);
+    kmax = max(kmax, r128(m.kbytes[t]));
+    vmax = max(vmax, r128(m.vbytes[t]));
+    pmax = 2048u << t;
   }
-  kstage = (kstage + 127u) / 128u * 128u;
-  vstage = (vstage + 127u) / 128u * 128u;
-  const uint32_t q_end = cur;
-  const uint32_t pbytes = p.tier_active[2] ? 8192u : (p.tier_active[1] ? 4096u : 2048u);
-  // ring depths: as deep as shared memory allows (the K ring also serves as the 16 KB output staging tile)
-  auto r128 = [](uint32_t b) { return (b + 127u) / 128u * 128u; };
-  const uint32_t fixed = 2 * kSets * (pbytes + 512) + 3 * r128(2 * kSets * 64 * 4) + r128(2 * kSets * 2 * 4) +
-                         r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 16) + r128(2 * B_COUNT * 8);
-  const uint32_t budget = q_end + fixed < 232448u ? 232448u - q_end - fixed : 0u;
+  // stream 1's Q descriptors start 1 KB before its images: stream 0's records precede them, so that is valid memory
+  for (int s = 0; s < 2; ++s) {
+    const uint32_t one = segmented ? take(qmax) : 0;
+    for (int t = 0; t < 3; ++t) m.q[s][t] = segmented ? one : (p.tier_active[t] ? take(p.qrec_bytes[t]) : 0);
+  }
+  const uint32_t pregion = segmented ? 16384u : kSets * pmax;  // per stream
+  const uint32_t fixed = 2 * (pregion + kStepBars * 512) + r128(2 * kStepBars * 64 * 4) + 2 * r128(2 * kSets * 64 * 4) +
+                         r128(2 * kStepBars * 2 * 4) + r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 16) + r128(2 * B_COUNT * 8);
+  constexpr uint32_t kLimit = 232448u - 128u;  // less the static shared variables
+  const uint32_t left = cur + fixed < kLimit ? (kLimit - cur - fixed) / 256u * 128u : 0u;  // ring bytes per stream
   // a K block is consumed as soon as a score buffer is free (two per stream), a V block only after the weights of
   // its step are written: the V ring is the deep one
-  const int cand[7][2] = {{3, 6}, {3, 5}, {3, 4}, {2, 4}, {2, 3}, {2, 2}, {2, 2}};
-  m.nk = 2; m.nv = 2; m.fits = false;
-  for (int c = 0; c < 7; ++c) {
-    if (2u * (cand[c][0] * kstage + cand[c][1] * vstage) <= budget) {
-      m.nk = cand[c][0]; m.nv = cand[c][1]; m.fits = true;
-      break;
+  uint32_t kring = 2 * kmax, vring = 2 * vmax;
+  m.fits = kring + vring <= left;
+  if (segmented) {
+    if (m.fits) vring = left - kring;
+  } else {
+    const int cand[5][2] = {{3, 6}, {3, 5}, {3, 4}, {2, 4}, {2, 3}};
+    m.fits = false;
+    for (int c = 0; c < 5 && !m.fits; ++c) {
+      kring = cand[c][0] * kmax; vring = cand[c][1] * vmax;
+      m.fits = kring + vring <= left;
     }
+    kring = max(kring, 16384u);  // the K ring also serves as the 16 KB output staging tile
   }
-  while ((uint32_t)m.nk * kstage < 16384u) kstage += 128u;
-  m.kstage = kstage; m.vstage = vstage;
-  for (int s = 0; s < 2; ++s) {
-    for (int g = 0; g < kMaxK; ++g) m.kst[s][g] = g < m.nk ? take(kstage) : 0;
+  for (int t = 0; t < 3; ++t) {
+    m.kstage[t] = segmented ? r128(m.kbytes[t]) : kmax;
+    m.vstage[t] = segmented ? r128(m.vbytes[t]) : vmax;
+    m.pbytes[t] = segmented ? 2048u << t : pmax;
+    m.nk[t] = m.kstage[t] ? min(kMaxK, (int)(kring / m.kstage[t])) : 1;
+    m.nv[t] = m.vstage[t] ? min(kMaxV, (int)(vring / m.vstage[t])) : 1;
   }
-  for (int s = 0; s < 2; ++s)
-    for (int g = 0; g < kMaxV; ++g) m.vst[s][g] = g < m.nv ? take(vstage) : 0;
-  m.pbytes = pbytes;
-  for (int s = 0; s < 2; ++s) for (int g = 0; g < kSets; ++g) m.p[s][g] = take(pbytes);
-  for (int s = 0; s < 2; ++s) for (int g = 0; g < kSets; ++g) m.sfp[s][g] = take(512);
-  m.factor = take(2 * kSets * 64 * 4);
-  m.chg = take(2 * kSets * 2 * 4);
+  for (int s = 0; s < 2; ++s) m.kring[s] = take(kring);
+  for (int s = 0; s < 2; ++s) m.vring[s] = take(vring);
+  for (int s = 0; s < 2; ++s) m.p[s] = take(pregion);
+  for (int s = 0; s < 2; ++s) m.sfp[s] = take(kStepBars * 512);
+  m.factor = take(2 * kStepBars * 64 * 4);
+  m.chg = take(2 * kStepBars * 2 * 4);
   m.hx = take(2 * kSets * 64 * 8);
   m.href = take(2 * kSets * 64 * 4);
   m.ell = take(2 * kSets * 64 * 4);
   m.info = take(2 * kInfoRing * 16);
   m.bars = take(2 * B_COUNT * 8);
   m.total = cur;
-  if (cur > 232448u) m.fits = false;
+  if (cur > kLimit) m.fits = false;
   return m;
 }
 
@@ -332,11 +346,9 @@ __device__ __forceinline__ StreamInfo load_stream(const Params &p, int bh, int a
 // otherwise they are blocks 2p and 2p+1 (per-row budgets: every row has the same length, the order is the identity).
 // FP4: the plan has an NVFP4 tier.  Without one the exponentiate phase keeps the per-pair interleaved form, which is
 // the faster one for the 8-bit and bf16 bodies alone (the compiler's schedule of the unrolled softmax body decides).
-template <int D, bool ORDERED, bool FP4, int SETS>
-__global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p, SmemMap sm, __nv_bfloat16 *__restrict__ out) {
-  constexpr int kSets = SETS, NT = Roles<SETS>::NT, kSoftmaxWarps = Roles<SETS>::kSoftmaxWarps;
-  constexpr int kMmaWarp0 = Roles<SETS>::kMmaWarp0, kPvWarp0 = Roles<SETS>::kPvWarp0, kLoadWarp0 = Roles<SETS>::kLoadWarp0;
-  constexpr int kShift = Roles<SETS>::kShift, kMask = Roles<SETS>::kMask;
+template <int D, bool ORDERED, bool FP4, bool SEGMENTED>
+__global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, __nv_bfloat16 *__restrict__ out) {
+  constexpr int kStepShift = SEGMENTED ? 3 : kShift, kStepMask = (1 << kStepShift) - 1;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint32_t s_tmem_base;
   __shared__ int s_abort;
@@ -373,8 +385,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
   if (tid == 32) {
     for (int s = 0; s < 2; ++s) {
       for (int g = 0; g < 2; ++g) tc::mbar_init(bar(s, B_SFREE + g), 2);
-      for (int g = 0; g < kSets; ++g) {
-        tc::mbar_init(bar(s, B_SREADY + g), 1);
+      for (int g = 0; g < kSets; ++g) tc::mbar_init(bar(s, B_SREADY + g), 1);
+      for (int g = 0; g < kStepBars; ++g) {
         tc::mbar_init(bar(s, B_PREADY + g), 2);  // the two softmax warps of the step (P written)
         tc::mbar_init(bar(s, B_PVDONE + g), 1);
         tc::mbar_init(bar(s, B_CORROK + g), 4);  // the stream's four correction warps (accumulator rescaled)
@@ -401,7 +413,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
 
   // =========================================================================================== softmax warps
   if (warp < kSoftmaxWarps) {
-    reg_inc<(SETS == 4 ? 88 : 128)>();
+    reg_inc<88>();
     // The warps w, w+4, w+8, ... share a scheduler and own the same 32 query rows; they take the steps of their sets
     // in turn, one thread per full 64-key row: while one exponentiates and packs its step (special-function bound),
     // the others fetch, mask and reduce later ones.  The only hand-off between them is the running maximum.
@@ -413,16 +425,21 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     const float dq8s = (S.a >= 0 && S.a < R && p.tier_active[1]) ? p.dq8[(size_t)bh * R + S.a] * p.scale * kLog2e : 0.f;
     const float c16 = p.scale * kLog2e;
     float h_own = -INFINITY, ell = 0.f;  // log2-domain maximum after this warp's last step; its partial denominator
-    const int g = set;                   // P buffer, barriers and hand-off slot of this set
     uint2 *my_hx = s_hx + (s * kSets + set) * 64 + r;                // running maximum after my steps, tagged with the step
     const uint32_t prev_hx = tc::smem_u32(s_hx + (s * kSets + ((set + kSets - 1) % kSets)) * 64 + r);
-    uint8_t *prow = smem + sm.p[s][g] + r * 16;
+    uint8_t *const p_row0 = smem + sm.p[s] + r * 16;
+    uint8_t *const sf_row0 = smem + sm.sfp[s] + (r & 31) * 16 + (r >> 5) * 4;
 
     for (int i = set; i < S.L; i += kSets) {
       const int tier = S.tier(i);
-      const uint32_t kp = (uint32_t)(i >> kShift) & 1u;  // completion parity of this set's k-th step
+      const int g = SEGMENTED ? i & kStepMask : set;  // barriers, factors, ballots, scale atom
+      // the step's P slot, and the product that last used it (SEGMENTED: at the start of a segment, the last product of the
+      // segment before, whose slots were cut differently)
+      const int seg0 = tier == 0 ? 0 : (tier == 1 ? S.n4 : S.n48), pm = SEGMENTED ? 7 >> tier : kMask;
+      uint8_t *prow = p_row0 + (SEGMENTED ? ((i - seg0) & pm) << (11 + tier) : set * sm.pbytes[0]);
+      const int busy = SEGMENTED && i - seg0 <= pm ? seg0 - 1 : i - 1 - pm;
       const uint32_t s_col = tmem + lane_addr + col_s(s, i & 1);
-      if (!wait_or_abort(bar(s, B_SREADY + g), kp, abortp)) break;
+      if (!wait_or_abort(bar(s, B_SREADY + set), (i >> kShift) & 1, abortp)) break;
       tc::fence_after_sync();
       // the step's mask and key scale (written before its K block was requested) are read while the scores load
       const uint8_t *info = s_info + (s * kInfoRing + (i & (kInfoRing - 1))) * 16;
@@ -479,8 +496,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
 #pragma unroll
       for (int q = 0; q < 4; ++q) gm[q] = max16(v + q * 16);
       const float pmax = fmaxf(max3(gm[0], gm[1], gm[2]), gm[3]) * coef;  // log2 domain
-      // PV(i-4) done: this set's P buffer is free and the correction warps are past step i-4
-      if (i >= kSets && !wait_or_abort(bar(s, B_PVDONE + g), (kp ^ 1u), abortp)) break;
+      // the step's P slot, factors and ballots are free
+      if (busy >= 0 && !wait_or_abort(bar(s, B_PVDONE + (busy & kStepMask)), (busy >> kStepShift) & 1, abortp)) break;
       // running maximum after step i-1: the thread that owns this row in the previous set leaves it, tagged with its
       // step, in shared memory (one 8-byte store, one 8-byte load: no barrier on this chain)
       float h_prev = -INFINITY;
@@ -499,9 +516,9 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
       }
       const float m_new = fmaxf(h_prev, pmax);
       *my_hx = make_uint2(__float_as_uint(m_new), (uint32_t)i);
-      s_factor[(s * kSets + g) * 64 + r] = ex2(h_prev - m_new);  // 0 on the first block (h_prev = -inf)
+      s_factor[(s * kStepBars + g) * 64 + r] = ex2(h_prev - m_new);  // 0 on the first block (h_prev = -inf)
       const uint32_t moved = __ballot_sync(0xffffffffu, m_new != h_prev);
-      if (lane == 0) s_chg[(s * kSets + g) * 2 + (warp & 1)] = moved;
+      if (lane == 0) s_chg[(s * kStepBars + g) * 2 + (warp & 1)] = moved;
       ell *= ex2(h_own - m_new);
       h_own = m_new;
 
@@ -602,7 +619,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
           sl[2 * h + 1] = s1 * (1.0f / 2688.0f);
         }
         const uint32_t sfword = __byte_perm(sfw[0], sfw[1], 0x5410);
-        *reinterpret_cast<uint32_t *>(smem + sm.sfp[s][g] + (r & 31) * 16 + (r >> 5) * 4) = sfword;
+        *reinterpret_cast<uint32_t *>(sf_row0 + g * 512) = sfword;
         {
           // the scores of the row become the exponent arguments, then the scaled weights, in place
 #pragma unroll
@@ -656,16 +673,19 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
     if (S.L > 0) {
-      if (!is_v && tc::elect_one()) {
+      // Q records: of every segment at once, or (SEGMENTED) of the segment that starts, into the stream's one buffer
+      auto load_q = [&](int first, int last) {
+        if (is_v || !tc::elect_one()) return;
         const int nn[3] = {S.n4, S.n48 - S.n4, S.L - S.n48};
         uint32_t bytes = 0;
-        for (int t = 0; t < 3; ++t) if (nn[t] > 0) bytes += p.qrec_bytes[t];
+        for (int t = first; t <= last; ++t) if (nn[t] > 0) bytes += p.qrec_bytes[t];
         tc::mbar_arrive_expect_tx(bar(s, B_Q), bytes);
-        for (int t = 0; t < 3; ++t)
+        for (int t = first; t <= last; ++t)
           if (nn[t] > 0)
-            tc::bulk_g2s(smem + sm.q[s][t], p.qrec[t] + ((size_t)bh * rec_blocks(p, t) + S.a) * p.qrec_bytes[t], p.qrec_bytes[t],
+            tc::bulk_g2s(tc::smem_u32(smem + sm.q[s][t]), p.qrec[t] + ((size_t)bh * rec_blocks(p, t) + S.a) * p.qrec_bytes[t], p.qrec_bytes[t],
                          bar(s, B_Q));
-      }
+      };
+      if (!SEGMENTED) load_q(0, 2);
       __syncwarp();
       const size_t head_blocks = (size_t)bh * R;
       auto list_id = [&](int idx) -> int {
@@ -685,15 +705,16 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
       int nxt_b = list_id(lane), nn_b = list_id(32 + lane);
       float cur_dk = 0.f, nxt_dk = key_scale(lane, nxt_b);
       unsigned long long cur_rec = 0, cur_mask = 0;
+      const uint32_t dst = tc::smem_u32(smem) + (is_v ? sm.vring[s] : sm.kring[s]);
+      const int b_full = is_v ? B_FULLV : B_FULLK, b_free = is_v ? B_VFREE : B_KFREE;
       const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1],
                      nb2 = is_v ? sm.vbytes[2] : sm.kbytes[2];
-      uint8_t *dst = smem + (is_v ? sm.vst[s][0] : sm.kst[s][0]);
-      const uint32_t stage = is_v ? sm.vstage : sm.kstage;
-      const int depth = is_v ? sm.nv : sm.nk;
-      const int b_full = is_v ? B_FULLV : B_FULLK, b_free = is_v ? B_VFREE : B_KFREE;
-      int kk = 0;         // ring slot
-      uint32_t kpar = 1;  // parity of the consumption that frees the slot (first pass: nothing to wait for)
-      bool kwrapped = false;
+      uint32_t stage = is_v ? sm.vstage[0] : sm.kstage[0];  // bytes per ring entry
+      int depth = is_v ? sm.nv[0] : sm.nk[0];               // ring entries
+      int kk = 0;                                           // ring entry
+      uint32_t used = 0, par = 0;     // per ring entry: used so far, parity of its last use
+      uint32_t kpar = 1;              // (not SEGMENTED: parity of the consumption that frees the entry, ring gone round)
+      bool kwrapped = false, ok = true;
       for (int i = -1; i < S.L; ++i) {
         const int src = i & 31;
         if (i >= 0) {
@@ -704,14 +725,33 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
         const float dk = __shfl_sync(0xffffffffu, cur_dk, src);
         const uint8_t *rec = reinterpret_cast<const uint8_t *>(((unsigned long long)rhi << 32) | rlo);
         const uint32_t nb = i < S.n4 ? nb0 : (i < S.n48 ? nb1 : nb2);
-        if (kwrapped && !wait_or_abort(bar(s, b_free + kk), kpar, abortp)) break;
+        if (SEGMENTED) {
+          if (i == 0 || i == S.n4 || i == S.n48) {  // the ring is cut anew once every block of the segment before is consumed
+            const int t = S.tier(i);
+            for (int k = 0; ok && k < (is_v ? kMaxV : kMaxK); ++k)
+              if ((used >> k) & 1u) ok = wait_or_abort(bar(s, b_free + k), (par >> k) & 1u, abortp);
+            if (!ok) break;
+            stage = is_v ? sm.vstage[t] : sm.kstage[t];
+            depth = is_v ? sm.nv[t] : sm.nk[t];
+            kk = 0;
+            load_q(t, t);
+            __syncwarp();
+          }
+          if ((used >> kk) & 1u) {
+            if (!(ok = wait_or_abort(bar(s, b_free + kk), (par >> kk) & 1u, abortp))) break;
+            par ^= 1u << kk;
+          }
+          used |= 1u << kk;
+        } else if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) {
+          break;
+        }
         if (tc::elect_one()) {
           // the step's mask and key scale enter the info ring before the data the softmax waits for is requested
           if (!is_v)
             *reinterpret_cast<uint4 *>(s_info + (s * kInfoRing + (i & (kInfoRing - 1))) * 16) =
                 make_uint4(mlo, mhi, __float_as_uint(dk), 0u);
           tc::mbar_arrive_expect_tx(bar(s, b_full + kk), nb);
-          tc::bulk_g2s(dst + kk * stage, rec, nb, bar(s, b_full + kk));
+          tc::bulk_g2s(dst + (uint32_t)kk * stage, rec, nb, bar(s, b_full + kk));
         }
         __syncwarp();
         if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
@@ -726,6 +766,14 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
           nn_b = list_id(i + 65 + lane);
         }
       }
+      if (!ok || *(volatile int *)abortp) {  // after a give-up: this warp's own copies land before the block may exit (bounded)
+        if (!SEGMENTED) {  // entries before kk were used in this round of the ring, the others in the round before
+          used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
+          par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
+        }
+        for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
+          if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
+      }
     }
   }
   // =========================================================================================== MMA warps
@@ -738,30 +786,41 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     S.n4 = __shfl_sync(0xffffffffu, S.n4, 0);
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
-    if (S.L > 0 && wait_or_abort(bar(s, B_Q), 0, abortp)) {
+    if (S.L > 0 && (SEGMENTED || wait_or_abort(bar(s, B_Q), 0, abortp))) {
       // operand descriptors, built once; inside the loop only the 16-byte-unit start address (low bits) moves
       const uint64_t qd0 = tc::smem_desc(tc::smem_u32(smem + sm.q[s][0]) - (s ? 1024u : 0u), 1024, 128);
       const uint64_t qd1 = tc::smem_desc(tc::smem_u32(smem + sm.q[s][1]) - (s ? 1024u : 0u), 1024, 128);
       const uint64_t qd2 = tc::smem_desc(tc::smem_u32(smem + sm.q[s][2]) - (s ? 1024u : 0u), 1024, 128);
-      const uint64_t kd0 = tc::smem_desc(tc::smem_u32(smem + sm.kst[s][0]), 1024, 128);
-      const uint64_t ksf0 = tc::smem_desc(tc::smem_u32(smem + sm.kst[s][0]) + kSlots * D / 2, 128, 128);
-      const uint32_t kstep = sm.kstage >> 4;
+      const uint64_t kd0 = tc::smem_desc(tc::smem_u32(smem + sm.kring[s]), 1024, 128);
+      const uint64_t ksf0 = tc::smem_desc(tc::smem_u32(smem + sm.kring[s]) + kSlots * D / 2, 128, 128);
       const uint32_t t_sfq = tmem + col_sfq(s), t_sfk = tmem + col_sfk(s);
-      if (S.n4 > 0) {  // Q scale factors go to TMEM once; the record carries them for rows 0..63 and again for rows
-                       // 64..127, so the same atom serves either stream
-        if (tc::elect_one()) {
+      int kk = 0, nk = sm.nk[0];
+      uint32_t kpar = 0, kstep = sm.kstage[0] >> 4;  // parity of the next use (SEGMENTED: a bit per ring entry); ring stride
+      uint32_t qseg = 0;                             // segments so far
+      auto q_scales = [&]() {  // Q scale factors go to TMEM once; the record carries them for rows 0..63 and again for rows
+        if (tc::elect_one()) { // 64..127, so the same atom serves either stream
 #pragma unroll
           for (int k = 0; k < D / 64; ++k)
             tc::tmem_cp_sf(t_sfq + 4 * k, tc::smem_desc(tc::smem_u32(smem + sm.q[s][0]) + kSlots * D / 2 + k * kSfAtomBytes,
                                                          128, 128));
         }
-      }
-      int kk = 0;
-      uint32_t kpar = 0;
+        __syncwarp();
+      };
+      if (!SEGMENTED && S.n4 > 0) q_scales();
       // the score tiles are double buffered, so Q K^T runs up to two steps ahead of the softmax
       for (int j = 0; j < S.L; ++j) {
         const int g = j & 1;
-        if (!wait_or_abort(bar(s, B_FULLK + kk), kpar, abortp)) break;
+        if (SEGMENTED && (j == 0 || j == S.n4 || j == S.n48)) {
+          const int t = S.tier(j);
+          kstep = sm.kstage[t] >> 4;
+          nk = sm.nk[t];
+          kk = 0;
+          if (!wait_or_abort(bar(s, B_Q), qseg & 1u, abortp)) break;
+          ++qseg;
+          if (j < S.n4) q_scales();
+        }
+        if (!wait_or_abort(bar(s, B_FULLK + kk), SEGMENTED ? (kpar >> kk) & 1u : kpar, abortp)) break;
+        if (SEGMENTED) kpar ^= 1u << kk;
         if (!wait_or_abort(bar(s, B_SFREE + g), ((j >> 1) & 1) ^ 1, abortp)) break;
         tc::fence_after_sync();
         const uint64_t kd = kd0 + (uint64_t)(kk * kstep);
@@ -785,7 +844,7 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
           tc::mma_commit(bar(s, B_KFREE + kk));
         }
         __syncwarp();
-        if (++kk == sm.nk) { kk = 0; kpar ^= 1u; }
+        if (++kk == nk) { kk = 0; if (!SEGMENTED) kpar ^= 1u; }
       }
     }
   }
@@ -797,24 +856,32 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
     if (S.L > 0) {
-      const uint64_t vd0 = tc::smem_desc(tc::smem_u32(smem + sm.vst[s][0]), D * 16, 128);
-      const uint64_t vsf0 = tc::smem_desc(tc::smem_u32(smem + sm.vst[s][0]) + D * kSlots / 2, 128, 128);
-      const uint64_t pd0 = tc::smem_desc(tc::smem_u32(smem + sm.p[s][0]), 1024, 128);
-      const uint64_t sfpd0 = tc::smem_desc(tc::smem_u32(smem + sm.sfp[s][0]), 128, 128);
-      const uint32_t pstep = sm.pbytes >> 4;
-      const uint32_t vstep = sm.vstage >> 4;
+      const uint64_t vd0 = tc::smem_desc(tc::smem_u32(smem + sm.vring[s]), D * 16, 128);
+      const uint64_t vsf0 = tc::smem_desc(tc::smem_u32(smem + sm.vring[s]) + D * kSlots / 2, 128, 128);
+      const uint64_t pd0 = tc::smem_desc(tc::smem_u32(smem + sm.p[s]), 1024, 128);
+      const uint64_t sfpd0 = tc::smem_desc(tc::smem_u32(smem + sm.sfp[s]), 128, 128);
       const uint32_t t_sfv = tmem + col_sfv(s), t_sfp = tmem + col_sfp(s), t_o = tmem + col_o(s);
-      int vv = 0;
-      uint32_t vpar = 0;
+      int vv = 0, nv = sm.nv[0], pp = 0, pm = 0;  // V ring entry and depth; SEGMENTED: P slot and number of slots - 1
+      uint32_t vpar = 0;                          // parity of the next use (SEGMENTED: a bit per ring entry)
+      uint32_t vstep = sm.vstage[0] >> 4, pstep = sm.pbytes[0] >> 4;
       for (int j = 0; j < S.L; ++j) {
         // ---- O^T += V(j)^T P(j)^T, once P(j) is written and the accumulator is rescaled for step j
-        const int g = j & kMask;
-        if (!wait_or_abort(bar(s, B_FULLV + vv), vpar, abortp)) break;
+        const int g = j & kStepMask;
+        if (SEGMENTED && (j == 0 || j == S.n4 || j == S.n48)) {
+          const int t = S.tier(j);
+          vstep = sm.vstage[t] >> 4;
+          nv = sm.nv[t];
+          pstep = sm.pbytes[t] >> 4;
+          pm = 7 >> t;
+          vv = 0; pp = 0;
+        }
+        if (!wait_or_abort(bar(s, B_FULLV + vv), SEGMENTED ? (vpar >> vv) & 1u : vpar, abortp)) break;
+        if (SEGMENTED) vpar ^= 1u << vv;
         // P(j) is written and the stream's correction warps have rescaled the accumulator where step j asked for it
-        if (!wait_or_abort(bar(s, B_CORROK + g), (j >> kShift) & 1, abortp)) break;
+        if (!wait_or_abort(bar(s, B_CORROK + g), (j >> kStepShift) & 1, abortp)) break;
         tc::fence_after_sync();
         const uint64_t vd = vd0 + (uint64_t)(vv * vstep);
-        const uint64_t pdg = pd0 + (uint64_t)(g * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
+        const uint64_t pdg = pd0 + (uint64_t)((SEGMENTED ? pp : g) * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
         const uint32_t acc = j > 0;
         if (tc::elect_one()) {
           if (j >= S.n48) {
@@ -834,7 +901,8 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
           tc::mma_commit(bar(s, B_VFREE + vv));
         }
         __syncwarp();
-        if (++vv == sm.nv) { vv = 0; vpar ^= 1u; }
+        if (++vv == nv) { vv = 0; if (!SEGMENTED) vpar ^= 1u; }
+        if (SEGMENTED) pp = (pp + 1) & pm;
       }
     }
   }
@@ -854,10 +922,10 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
     // step's "maximum moved" ballots and, only if one is set or the segment changes, wait for product i-1 and rescale
     // their lane quarter of the accumulator; then they let product i go.  Most steps move no maximum.
     for (int i = 0; i < S.L; ++i) {
-      const int g = i & kMask;
-      if (!wait_or_abort(bar(s, B_PREADY + g), (i >> kShift) & 1, abortp)) break;
+      const int g = i & kStepMask;
+      if (!wait_or_abort(bar(s, B_PREADY + g), (i >> kStepShift) & 1, abortp)) break;
       const bool tier_switch = (i == S.n4) || (i == S.n48);
-      const uint2 moved = ld_shared_volatile_v2(tc::smem_u32(s_chg + (s * kSets + g) * 2));
+      const uint2 moved = ld_shared_volatile_v2(tc::smem_u32(s_chg + (s * kStepBars + g) * 2));
       if (i == 0 || ((moved.x | moved.y) == 0u && !tier_switch)) {
         if (lane == 0) tc::mbar_arrive(bar(s, B_CORROK + g));
         continue;
@@ -869,14 +937,14 @@ __global__ void __launch_bounds__(Roles<SETS>::NT, 1) attention_kernel(Params p,
         const float un = unit_of(tier), up = unit_of(S.tier(i - 1));
         lane_factor = un > 0.f ? __fdiv_rn(up, un) : 0.f;
       }
-      const float *fac = s_factor + (s * kSets + g) * 64;
+      const float *fac = s_factor + (s * kStepBars + g) * 64;
       // column groups (eight queries each) with a moved maximum; all of them when the segment changes.  Two groups
       // are in flight at a time: their loads are issued together, so a rescale costs one TMEM round trip per pair.
       uint32_t todo = 0;
 #pragma unroll
       for (int c = 0; c < 8; ++c)
         if (tier_switch || (((c < 4 ? moved.x : moved.y) >> ((c & 3) * 8)) & 0xffu) != 0u) todo |= 1u << c;
-      if (!wait_or_abort(bar(s, B_PVDONE + ((i - 1) & kMask)), ((i - 1) >> kShift) & 1, abortp)) break;
+      if (!wait_or_abort(bar(s, B_PVDONE + ((i - 1) & kStepMask)), ((i - 1) >> kStepShift) & 1, abortp)) break;
       tc::fence_after_sync();
 #pragma unroll 1
       while (todo) {
@@ -902,12 +970,12 @@ scale8(o0, fac + c0 * 8, lane_factor);
     // ---------------------------------------------------------- epilogue: O = U / l, back to raster order
     if (S.a >= 0) {
       const unsigned long long qmask = table_mask(p, S.a);
-      uint16_t *stage = reinterpret_cast<uint16_t *>(smem + sm.kst[s][0]);  // [64][D] bf16 over the K ring
+      uint16_t *stage = reinterpret_cast<uint16_t *>(smem + sm.kring[s]);  // [64][D] bf16 over the K ring
       bool ok = S.L > 0 && !*(volatile int *)abortp;
       if (ok) ok = wait_or_abort(bar(s, B_ELL), 0, abortp);
-      if (ok) ok = wait_or_abort(bar(s, B_PVDONE + ((S.L - 1) & kMask)), ((S.L - 1) >> kShift) & 1, abortp);
+      if (ok) ok = wait_or_abort(bar(s, B_PVDONE + ((S.L - 1) & kStepMask)), ((S.L - 1) >> kStepShift) & 1, abortp);
       const int ltid = tid - (kSoftmaxWarps + 4 * s) * 32;  // thread index inside the stream's correction group
-      float *s_inv = s_factor + (s * kSets) * 64;            // 1 / l per query (the factors are no longer needed)
+      float *s_inv = s_factor + (s * kStepBars) * 64;            // 1 / l per query (the factors are no longer needed)
       if (ok && ltid < 64) {
         // the sets of a row kept partial denominators relative to their own last maximum
         float hf = -INFINITY, l = 0.f;
@@ -994,35 +1062,30 @@ cudaError_t launch_bounded_wait_probe(int *status, long long limit_cycles, cudaS
 }
 
 cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t st, int *launches) {
-  // four softmax sets when their P images leave room for rings of at least 2 K and 3 V stages, else two
-  SmemMap sm = make_smem_map(p, 4);
-  int sets = 4;
-  if (!sm.fits || sm.nv < 3) {
-    sm = make_smem_map(p, 2);
-    sets = 2;
-  }
+  SmemMap sm = make_smem_map(p, false);
+  const bool segmented = !sm.fits;
+  if (segmented) sm = make_smem_map(p, true);
   if (!sm.fits) return cudaErrorInvalidConfiguration;
   cudaError_t e;
   const int grid = p.BH * ((p.Rt + 1) / 2);
-  auto launch = [&](auto kernel, int nt) -> cudaError_t {
+  auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm.total);
     if (err != cudaSuccess) return err;
-    kernel<<<grid, nt, sm.total, st>>>(p, sm, out);
+    kernel<<<grid, NT, sm.total, st>>>(p, sm, out);
     return cudaSuccess;
   };
   const bool ordered = p.rank_scope != 0, fp4 = p.tier_active[0] != 0;
   auto pick = [&](auto dtag, auto stag) -> cudaError_t {
-    constexpr int D = decltype(dtag)::value, S = decltype(stag)::value;
-    constexpr int nt = Roles<S>::NT;
-    return ordered ? (fp4 ? launch(attention_kernel<D, true, true, S>, nt) : launch(attention_kernel<D, true, false, S>, nt))
-                   : (fp4 ? launch(attention_kernel<D, false, true, S>, nt) : launch(attention_kernel<D, false, false, S>, nt));
+    constexpr int D = decltype(dtag)::value;
+    constexpr bool S = decltype(stag)::value;
+    return ordered ? (fp4 ? launch(attention_kernel<D, true, true, S>) : launch(attention_kernel<D, true, false, S>))
+                   : (fp4 ? launch(attention_kernel<D, false, true, S>) : launch(attention_kernel<D, false, false, S>));
   };
   using I64 = std::integral_constant<int, 64>;
   using I128 = std::integral_constant<int, 128>;
-  using S2 = std::integral_constant<int, 2>;
-  using S4 = std::integral_constant<int, 4>;
-  if (p.d == 128) e = sets == 4 ? pick(I128{}, S4{}) : pick(I128{}, S2{});
-  else e = sets == 4 ? pick(I64{}, S4{}) : pick(I64{}, S2{});
+  if (p.d == 128) e = segmented ? pick(I128{}, std::true_type{}) : pick(I128{}, std::false_type{});
+  else if (!segmented) e = pick(I64{}, std::false_type{});
+  else e = cudaErrorInvalidConfiguration;  // (head_dim 64 always fits)
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();
