@@ -107,6 +107,7 @@ struct SmemMap {
   uint32_t ell;       // float [2][sets][64]
   uint32_t info;      // per stream, ring of kInfoRing steps: {u64 mask, float dk8, pad}
   uint32_t bars;      // uint64 [2][B_COUNT]
+  uint32_t tok;       // int [2 streams][64]: token of each query slot, -1 at padding
   uint32_t chg;       // uint32 [2 streams][kStepBars][2]: ballots of the queries whose maximum moved this step
   uint32_t total;
   bool fits;          // the layout fits the 227 KB a block may use
@@ -134,7 +135,8 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   }
   const uint32_t pregion = segmented ? 16384u : kSets * pmax;  // per stream
   const uint32_t fixed = 2 * (pregion + kStepBars * 512) + r128(2 * kStepBars * 64 * 4) + 2 * r128(2 * kSets * 64 * 4) +
-                         r128(2 * kStepBars * 2 * 4) + r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 16) + r128(2 * B_COUNT * 8);
+                         r128(2 * kStepBars * 2 * 4) + r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 16) + r128(2 * 64 * 4) +
+                         r128(2 * B_COUNT * 8);
   constexpr uint32_t kLimit = 232448u - 128u;  // less the static shared variables
   const uint32_t left = cur + fixed < kLimit ? (kLimit - cur - fixed) / 256u * 128u : 0u;  // ring bytes per stream
   // a K block is consumed as soon as a score buffer is free (two per stream), a V block only after the weights of
@@ -150,7 +152,6 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
       kring = cand[c][0] * kmax; vring = cand[c][1] * vmax;
       m.fits = kring + vring <= left;
     }
-    kring = max(kring, 16384u);  // the K ring also serves as the 16 KB output staging tile
   }
   for (int t = 0; t < 3; ++t) {
     m.kstage[t] = segmented ? r128(m.kbytes[t]) : kmax;
@@ -169,6 +170,7 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   m.href = take(2 * kSets * 64 * 4);
   m.ell = take(2 * kSets * 64 * 4);
   m.info = take(2 * kInfoRing * 16);
+  m.tok = take(2 * 64 * 4);
   m.bars = take(2 * B_COUNT * 8);
   m.total = cur;
   if (cur > kLimit) m.fits = false;
@@ -329,13 +331,18 @@ struct StreamInfo {
   __device__ __forceinline__ int tier(int i) const { return i < n4 ? 0 : (i < n48 ? 1 : 2); }
 };
 
-__device__ __forceinline__ StreamInfo load_stream(const Params &p, int bh, int a) {
+// Per-row budgets (ROW scope) give every video row the same bounds and a fixed place in the id array, so that nothing has to
+// be read before the ids; in HEAD scope (ORDERED) the bounds are the counts that came with the list.
+template <bool ORDERED> __device__ __forceinline__ StreamInfo load_stream(const Params &p, int bh, int a) {
   StreamInfo st;
   st.a = a < p.Rt ? a : -1;
   st.n4 = st.n48 = st.L = 0;
   st.ids = nullptr;
   if (a < p.Rt) {
-    const int4 c = *reinterpret_cast<const int4 *>(p.counts + ((size_t)bh * p.Rt + a) * 4);
+    int4 c;
+    if (ORDERED) c = *reinterpret_cast<const int4 *>(p.counts + ((size_t)bh * p.Rt + a) * 4);
+    else if (a < p.R) c = make_int4((int)p.quota[0], (int)p.quota[1], (int)p.quota[2] + p.Rp, a * p.row_stride);
+    else c = make_int4(0, 0, p.Rt, p.R * p.row_stride + (a - p.R) * ((p.Rt + 7) / 8 * 8));  // a prefix row keeps every block
     st.n4 = c.x; st.n48 = c.x + c.y; st.L = c.x + c.y + c.z;
     st.ids = p.ids + (size_t)bh * p.ids_per_head + c.w;
   }
@@ -365,7 +372,21 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     a0 = ord[0];
     a1 = ord[1];
   }
-  const StreamInfo st0 = load_stream(p, bh, a0), st1 = load_stream(p, bh, a1);
+  const StreamInfo st0 = load_stream<ORDERED>(p, bh, a0), st1 = load_stream<ORDERED>(p, bh, a1);
+  // the loaders' first ids, and the correction warps' table of query tokens, are on their way while the block is set up
+  const int pre_s = warp >= kLoadWarp0 ? (warp - kLoadWarp0) & 1 : (warp - kSoftmaxWarps) >> 2;
+  const int pre_a = pre_s ? st1.a : st0.a;
+  int pre0 = 0, pre1 = 0;
+  if (warp >= kLoadWarp0) {
+    const uint16_t *ids = pre_s ? st1.ids : st0.ids;
+    const int L = pre_s ? st1.L : st0.L;
+    if (lane < L) pre0 = ids[lane];
+    if (32 + lane < L) pre1 = ids[32 + lane];
+  } else if (warp >= kSoftmaxWarps && warp < kMmaWarp0 && (warp & 3) < 2 && pre_a >= 0) {
+    const int j = (warp & 1) * 32 + lane;
+    reinterpret_cast<int *>(smem + sm.tok)[pre_s * 64 + j] =
+        (table_mask(p, pre_a) >> j) & 1ull ? (int)table_token(p, pre_a, j) : -1;
+  }
 
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + sm.bars);
   const uint32_t bars0 = tc::smem_u32(bars);
@@ -382,28 +403,15 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     tc::tmem_alloc(&s_tmem_base, kTmemCols);
     tc::tmem_relinquish();
   }
-  if (tid == 32) {
-    for (int s = 0; s < 2; ++s) {
-      for (int g = 0; g < 2; ++g) tc::mbar_init(bar(s, B_SFREE + g), 2);
-      for (int g = 0; g < kSets; ++g) tc::mbar_init(bar(s, B_SREADY + g), 1);
-      for (int g = 0; g < kStepBars; ++g) {
-        tc::mbar_init(bar(s, B_PREADY + g), 2);  // the two softmax warps of the step (P written)
-        tc::mbar_init(bar(s, B_PVDONE + g), 1);
-        tc::mbar_init(bar(s, B_CORROK + g), 4);  // the stream's four correction warps (accumulator rescaled)
-      }
-      for (int g = 0; g < kMaxK; ++g) {
-        tc::mbar_init(bar(s, B_FULLK + g), 1);
-        tc::mbar_init(bar(s, B_KFREE + g), 1);
-      }
-      for (int g = 0; g < kMaxV; ++g) {
-        tc::mbar_init(bar(s, B_FULLV + g), 1);
-        tc::mbar_init(bar(s, B_VFREE + g), 1);
-      }
-      tc::mbar_init(bar(s, B_ELL), 2 * kSets);
-      tc::mbar_init(bar(s, B_Q), 1);
+  if (warp == 1) {
+    // arrivals per barrier: 1 (a commit or a copy), but two softmax warps per step (scores in registers, weights written),
+    // four correction warps (accumulator rescaled), and two warps of each set for the denominators
+    for (int k = lane; k < 2 * B_COUNT; k += 32) {
+      const int b = k % B_COUNT;
+      tc::mbar_init(bars0 + (uint32_t)k * 8u, (b >= B_SFREE && b < B_CORROK) ? 2 : ((b >= B_CORROK && b < B_PVDONE) ? 4 : (b == B_ELL ? 2 * kSets : 1)));
     }
     tc::fence_barrier_init();
-    s_abort = 0;
+    if (lane == 0) s_abort = 0;
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -688,11 +696,11 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       if (!SEGMENTED) load_q(0, 2);
       __syncwarp();
       const size_t head_blocks = (size_t)bh * R;
-      auto list_id = [&](int idx) -> int {
-        int b = idx < S.L ? (int)S.ids[idx] : 0;
+      auto checked = [&](int b) -> int {
         if (b >= Rt) { atomicExch(p.status, kDevBadList); b = 0; }
         return b;
       };
+      auto list_id = [&](int idx) -> int { return checked(idx < S.L ? (int)S.ids[idx] : 0); };
       auto key_scale = [&](int idx, int b) -> float {
         return (!is_v && idx < S.L && S.tier(idx) == 1) ? p.dk8[head_blocks + b] : 0.f;
       };
@@ -702,7 +710,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
                                                     (is_v ? sm.kbytes[t] : 0u));
       };
       // batch -1 is empty: the loop's refill at "src == 31" then also serves the first batch
-      int nxt_b = list_id(lane), nn_b = list_id(32 + lane);
+      int nxt_b = checked(pre0), nn_b = checked(pre1);
       float cur_dk = 0.f, nxt_dk = key_scale(lane, nxt_b);
       unsigned long long cur_rec = 0, cur_mask = 0;
       const uint32_t dst = tc::smem_u32(smem) + (is_v ? sm.vring[s] : sm.kring[s]);
@@ -969,55 +977,50 @@ scale8(o0, fac + c0 * 8, lane_factor);
     }
     // ---------------------------------------------------------- epilogue: O = U / l, back to raster order
     if (S.a >= 0) {
-      const unsigned long long qmask = table_mask(p, S.a);
-      uint16_t *stage = reinterpret_cast<uint16_t *>(smem + sm.kring[s]);  // [64][D] bf16 over the K ring
       bool ok = S.L > 0 && !*(volatile int *)abortp;
       if (ok) ok = wait_or_abort(bar(s, B_ELL), 0, abortp);
       if (ok) ok = wait_or_abort(bar(s, B_PVDONE + ((S.L - 1) & kStepMask)), ((S.L - 1) >> kStepShift) & 1, abortp);
       const int ltid = tid - (kSoftmaxWarps + 4 * s) * 32;  // thread index inside the stream's correction group
-      float *s_inv = s_factor + (s * kStepBars) * 64;            // 1 / l per query (the factors are no longer needed)
-      if (ok && ltid < 64) {
-        // the sets of a row kept partial denominators relative to their own last maximum
-        float hf = -INFINITY, l = 0.f;
-#pragma unroll 1
-        for (int k = 0; k < kSets; ++k) hf = fmaxf(hf, s_href[(s * kSets + k) * 64 + ltid]);
-#pragma unroll 1
-        for (int k = 0; k < kSets; ++k) {  // a set without a step has ell = 0 and reference -inf
-          const float lk = s_ell[(s * kSets + k) * 64 + ltid];
-          if (lk > 0.f) l += lk * ex2(s_href[(s * kSets + k) * 64 + ltid] - hf);
+      float *s_inv = s_factor + (s * kStepBars) * 64;        // 1 / l per query (the factors are no longer needed)
+      const int *s_tok = reinterpret_cast<const int *>(smem + sm.tok) + s * 64;
+      if (ltid < 64) {
+        // the sets of a row kept partial denominators relative to their own last maximum (a set without a step has ell = 0
+        // and reference -inf); rows without a retained key return zero (App. C.1)
+        float l = 0.f;
+        if (ok) {
+          float hf = -INFINITY;
+#pragma unroll
+          for (int k = 0; k < kSets; ++k) hf = fmaxf(hf, s_href[(s * kSets + k) * 64 + ltid]);
+#pragma unroll
+          for (int k = 0; k < kSets; ++k) {
+            const float lk = s_ell[(s * kSets + k) * 64 + ltid];
+            if (lk > 0.f) l += lk * ex2(s_href[(s * kSets + k) * 64 + ltid] - hf);
+          }
         }
         s_inv[ltid] = l > 0.f ? __fdiv_rn(1.0f, l) : 0.f;
       }
       if (s == 0) asm volatile("bar.sync 1, 128;" ::: "memory"); else asm volatile("bar.sync 2, 128;" ::: "memory");
-      if (ok) {
+      if ((ok || S.L == 0) && cw * 32 < D) {
         tc::fence_after_sync();
-        const float unit = ch < D ? unit_of(S.tier(S.L - 1)) : 0.f;
+        const float unit = ok ? unit_of(S.tier(S.L - 1)) : 0.f;
+        uint32_t *out_ch = reinterpret_cast<uint32_t *>(out_head + (ch & ~1));
 #pragma unroll 1
-        for (int c = 0; c < 8; ++c) {
-          uint32_t o[8];
-          tc::tmem_ld8(tmem + lane_addr + col_o(s) + c * 8, o);
+        for (int c = 0; c < 4; ++c) {
+          uint32_t o[16];
+          tc::tmem_ld16(tmem + lane_addr + col_o(s) + c * 16, o);
           tc::wait_ld();
-          if (ch < D) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int qr = c * 8 + j;
-              const float inv = s_inv[qr];
-              const float val = inv > 0.f ? __uint_as_float(o[j]) * unit * inv : 0.f;
-              stage[qr * D + ch] = __bfloat16_as_ushort(__float2bfloat16_rn(val));
-            }
+          for (int j = 0; j < 16; j += 2) {
+            // lanes 2x and 2x+1 hold neighbouring channels: after one exchange the even lane writes both of query j, the odd
+            // lane both of query j + 1 (64 contiguous bytes per query and warp, no staging tile, no barrier)
+            const float2 inv = *reinterpret_cast<const float2 *>(s_inv + c * 16 + j);
+            const float x = inv.x > 0.f ? __uint_as_float(o[j]) * unit * inv.x : 0.f;
+            const float y = inv.y > 0.f ? __uint_as_float(o[j + 1]) * unit * inv.y : 0.f;
+            const float got = __shfl_xor_sync(0xffffffffu, (lane & 1) ? x : y, 1);
+            const uint32_t word = (lane & 1) ? pack_bf16x2(got, y) : pack_bf16x2(x, got);
+            const int tok = s_tok[c * 16 + j + (lane & 1)];
+            if (tok >= 0) out_ch[(size_t)tok * (D / 2)] = word;
           }
-        }
-      } else if (S.L == 0) {  // rows without a retained key return zero (App. C.1)
-        for (int idx = ltid; idx < kSlots * (D / 8); idx += 128) reinterpret_cast<uint4 *>(stage)[idx] = make_uint4(0, 0, 0, 0);
-      }
-      if (s == 0) asm volatile("bar.sync 1, 128;" ::: "memory"); else asm volatile("bar.sync 2, 128;" ::: "memory");
-      if (ok || S.L == 0) {
-#pragma unroll 1
-        for (int idx = ltid; idx < kSlots * (D / 8); idx += 128) {
-          const int j = idx / (D / 8), c8 = idx % (D / 8);
-          if ((qmask >> j) & 1ull)
-            *reinterpret_cast<uint4 *>(out_head + (size_t)table_token(p, S.a, j) * D + c8 * 8) =
-                *reinterpret_cast<const uint4 *>(stage + j * D + c8 * 8);
         }
       }
     }
