@@ -79,7 +79,7 @@ constexpr float kOffsetP8 = 8.807f;      // base-2 exponent offset (about log2 4
 // barrier indices inside one stream's group
 // (a parity wait can only tell the latest completion from the one before, so every barrier is laid out such that no
 // waiter can fall two completions behind: buffers indexed by step parity get one barrier per buffer)
-constexpr int kMaxK = 6, kMaxV = 8, kInfoRing = 16;
+constexpr int kMaxK = 6, kMaxV = 8, kInfoRing = 16;  // (steps between a K request and its scores: at most nk + 2)
 constexpr int kStepBars = 8;  // barriers for the steps of a stream between softmax and product (kSets of them unless SEGMENTED)
 enum {
   B_FULLK = 0, B_KFREE = B_FULLK + kMaxK, B_FULLV = B_KFREE + kMaxK, B_VFREE = B_FULLV + kMaxV, B_SREADY = B_VFREE + kMaxV,
@@ -105,7 +105,8 @@ struct SmemMap {
   uint32_t hx;        // {float h, int step} [2][sets][64]: running maximum after a step, handed from thread to thread
   uint32_t href;      // float [2][sets][64]: reference of each set's partial denominator
   uint32_t ell;       // float [2][sets][64]
-  uint32_t info;      // per stream, ring of kInfoRing steps: {u64 mask, float dk8, pad}
+  uint32_t info;      // per stream, ring of kInfoRing steps: {float key scale, uint32 "has padding keys"}
+  uint32_t lim;       // beside it, float [64] per step: +inf, -inf at padding keys (written where there are any)
   uint32_t bars;      // uint64 [2][B_COUNT]
   uint32_t tok;       // int [2 streams][64]: token of each query slot, -1 at padding
   uint32_t chg;       // uint32 [2 streams][kStepBars][2]: ballots of the queries whose maximum moved this step
@@ -135,7 +136,7 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   }
   const uint32_t pregion = segmented ? 16384u : kSets * pmax;  // per stream
   const uint32_t fixed = 2 * (pregion + kStepBars * 512) + r128(2 * kStepBars * 64 * 4) + 2 * r128(2 * kSets * 64 * 4) +
-                         r128(2 * kStepBars * 2 * 4) + r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 16) + r128(2 * 64 * 4) +
+                         r128(2 * kStepBars * 2 * 4) + r128(2 * kSets * 64 * 8) + r128(2 * kInfoRing * 8) + 2 * kInfoRing * 256 + r128(2 * 64 * 4) +
                          r128(2 * B_COUNT * 8);
   constexpr uint32_t kLimit = 232448u - 128u;  // less the static shared variables
   const uint32_t left = cur + fixed < kLimit ? (kLimit - cur - fixed) / 256u * 128u : 0u;  // ring bytes per stream
@@ -169,7 +170,8 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   m.hx = take(2 * kSets * 64 * 8);
   m.href = take(2 * kSets * 64 * 4);
   m.ell = take(2 * kSets * 64 * 4);
-  m.info = take(2 * kInfoRing * 16);
+  m.info = take(2 * kInfoRing * 8);
+  m.lim = take(2 * kInfoRing * 256);
   m.tok = take(2 * 64 * 4);
   m.bars = take(2 * B_COUNT * 8);
   m.total = cur;
@@ -353,8 +355,9 @@ template <bool ORDERED> __device__ __forceinline__ StreamInfo load_stream(const 
 // otherwise they are blocks 2p and 2p+1 (per-row budgets: every row has the same length, the order is the identity).
 // FP4: the plan has an NVFP4 tier.  Without one the exponentiate phase keeps the per-pair interleaved form, which is
 // the faster one for the 8-bit and bf16 bodies alone (the compiler's schedule of the unrolled softmax body decides).
-template <int D, bool ORDERED, bool FP4, bool SEGMENTED>
+template <int D, bool ORDERED, bool FP4, bool B16>
 __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, __nv_bfloat16 *__restrict__ out) {
+  constexpr bool SEGMENTED = B16 && D == 128;
   constexpr int kStepShift = SEGMENTED ? 3 : kShift, kStepMask = (1 << kStepShift) - 1;
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint32_t s_tmem_base;
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   uint2 *s_hx = reinterpret_cast<uint2 *>(smem + sm.hx);              // [s][set][64]
   float *s_href = reinterpret_cast<float *>(smem + sm.href);          // [s][set][64]
   float *s_ell = reinterpret_cast<float *>(smem + sm.ell);            // [s][set][64]
-  uint8_t *s_info = smem + sm.info;                                   // [s][kInfoRing] 16 bytes
+  uint2 *s_info = reinterpret_cast<uint2 *>(smem + sm.info);          // [s][kInfoRing]
 
   for (int k_ = tid; k_ < 2 * kSets * 64; k_ += NT) s_hx[k_] = make_uint2(0u, 0xffffffffu);  // no step has this tag
   if (warp == 0) {
@@ -406,6 +409,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   if (warp == 1) {
     // arrivals per barrier: 1 (a commit or a copy), but two softmax warps per step (scores in registers, weights written),
     // four correction warps (accumulator rescaled), and two warps of each set for the denominators
+#pragma unroll 1
     for (int k = lane; k < 2 * B_COUNT; k += 32) {
       const int b = k % B_COUNT;
       tc::mbar_init(bars0 + (uint32_t)k * 8u, (b >= B_SFREE && b < B_CORROK) ? 2 : ((b >= B_CORROK && b < B_PVDONE) ? 4 : (b == B_ELL ? 2 * kSets : 1)));
@@ -450,11 +454,11 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       if (!wait_or_abort(bar(s, B_SREADY + set), (i >> kShift) & 1, abortp)) break;
       tc::fence_after_sync();
       // the step's mask and key scale (written before its K block was requested) are read while the scores load
-      const uint8_t *info = s_info + (s * kInfoRing + (i & (kInfoRing - 1))) * 16;
-      const uint2 kmask = *reinterpret_cast<const uint2 *>(info);
+      const uint2 info = s_info[s * kInfoRing + (i & (kInfoRing - 1))];
+      const bool padded = info.y != 0u;
       float coef;
-      if (tier == 2) coef = c16;
-      else if (tier == 1) coef = dq8s * *reinterpret_cast<const float *>(info + 8);
+      if (B16 && tier == 2) coef = c16;
+      else if (tier == 1) coef = dq8s * __uint_as_float(info.x);
       else coef = gqk;
       float v[64];
       {
@@ -485,18 +489,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       }
       tc::fence_before_sync();
       warp_arrive(bar(s, B_SFREE + (i & 1)));
-      if ((kmask.x & kmask.y) != 0xffffffffu) {  // padding keys take no part
-        if (kmask.x == 0xffffffffu && kmask.y == 0x7fffffffu) {
-          v[63] = -INFINITY;  // a region of 63 tokens (the balanced partition's common case): one padding slot
-        } else if (kmask.x == 0xffffffffu) {
+      if (padded) {  // padding keys take no part: the loader left -inf for them and +inf for the others
+        const float4 *lim = reinterpret_cast<const float4 *>(smem + sm.lim + (s * kInfoRing + (i & (kInfoRing - 1))) * 256);
 #pragma unroll
-          for (int c = 0; c < 32; ++c) v[32 + c] = ((kmask.y >> c) & 1u) ? v[32 + c] : -INFINITY;
-        } else {  // ragged edge tile
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            v[c] = ((kmask.x >> c) & 1u) ? v[c] : -INFINITY;
-            v[32 + c] = ((kmask.y >> c) & 1u) ? v[32 + c] : -INFINITY;
-          }
+        for (int c = 0; c < 64; c += 4) {
+          const float4 x = lim[c >> 2];
+          v[c] = fminf(v[c], x.x); v[c + 1] = fminf(v[c + 1], x.y); v[c + 2] = fminf(v[c + 2], x.z); v[c + 3] = fminf(v[c + 3], x.w);
         }
       }
       // maxima of the four 16-key groups (pairwise trees), then of the row
@@ -531,7 +529,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       h_own = m_new;
 
       const uint64_t coef2 = f2(coef, coef);
-      if (!FP4 && tier == 2) {
+      if (!FP4 && B16 && tier == 2) {
         const uint64_t bias2 = f2(-m_new, -m_new);
         uint64_t sum2 = 0;
 #pragma unroll
@@ -574,7 +572,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       } else if (tier != 0) {
         // the scores of the row become the exponent arguments, then the weights, in place: all 64 exponentials are
         // issued before any is consumed (the 8-bit path carries the 2^8.807 offset in the exponent)
-        const float b = tier == 1 ? kOffsetP8 - m_new : -m_new;
+        const float b = !B16 || tier == 1 ? kOffsetP8 - m_new : -m_new;
         const uint64_t bias2 = f2(b, b);
 #pragma unroll
         for (int j = 0; j < 32; ++j) unf2(fma2(f2(v[2 * j], v[2 * j + 1]), coef2, bias2), v[2 * j], v[2 * j + 1]);
@@ -585,7 +583,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         for (int j = 0; j < 32; j += 2) sum2 = add2(sum2, add2(f2(v[2 * j], v[2 * j + 1]), f2(v[2 * j + 2], v[2 * j + 3])));
         float s0, s1;
         unf2(sum2, s0, s1);
-        if (tier == 2) {
+        if (B16 && tier == 2) {
 #pragma unroll
           for (int c = 0; c < 8; ++c)
             *reinterpret_cast<uint4 *>(prow + c * 1024) =
@@ -713,6 +711,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       int nxt_b = checked(pre0), nn_b = checked(pre1);
       float cur_dk = 0.f, nxt_dk = key_scale(lane, nxt_b);
       unsigned long long cur_rec = 0, cur_mask = 0;
+      uint32_t padded_lanes = 0;
       const uint32_t dst = tc::smem_u32(smem) + (is_v ? sm.vring[s] : sm.kring[s]);
       const int b_full = is_v ? B_FULLV : B_FULLK, b_free = is_v ? B_VFREE : B_KFREE;
       const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1],
@@ -728,9 +727,6 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         if (i >= 0) {
         const uint32_t rlo = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src);
         const uint32_t rhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src);
-        const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src);
-        const uint32_t mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src);
-        const float dk = __shfl_sync(0xffffffffu, cur_dk, src);
         const uint8_t *rec = reinterpret_cast<const uint8_t *>(((unsigned long long)rhi << 32) | rlo);
         const uint32_t nb = i < S.n4 ? nb0 : (i < S.n48 ? nb1 : nb2);
         if (SEGMENTED) {
@@ -753,11 +749,21 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         } else if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) {
           break;
         }
+        if (!is_v) {
+          // the step's mask and key scale are written before the data the softmax waits for is requested
+          const int e = s * kInfoRing + (i & (kInfoRing - 1));
+          const bool padded = (padded_lanes >> src) & 1u;
+          if (padded) {
+            const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src);
+            const uint32_t mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src);
+            float *lim = reinterpret_cast<float *>(smem + sm.lim) + e * 64;
+            lim[lane] = (mlo >> lane) & 1u ? INFINITY : -INFINITY;
+            lim[32 + lane] = (mhi >> lane) & 1u ? INFINITY : -INFINITY;
+          }
+          if (lane == src) s_info[e] = make_uint2(__float_as_uint(cur_dk), padded);
+          __syncwarp();
+        }
         if (tc::elect_one()) {
-          // the step's mask and key scale enter the info ring before the data the softmax waits for is requested
-          if (!is_v)
-            *reinterpret_cast<uint4 *>(s_info + (s * kInfoRing + (i & (kInfoRing - 1))) * 16) =
-                make_uint4(mlo, mhi, __float_as_uint(dk), 0u);
           tc::mbar_arrive_expect_tx(bar(s, b_full + kk), nb);
           tc::bulk_g2s(dst + (uint32_t)kk * stage, rec, nb, bar(s, b_full + kk));
         }
@@ -768,7 +774,8 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           const int b = nxt_b;
           cur_dk = nxt_dk;
           cur_rec = record(i + 1 + lane, b);
-          cur_mask = table_mask(p, b);
+          cur_mask = is_v ? ~0ull : table_mask(p, b);
+          padded_lanes = __ballot_sync(0xffffffffu, cur_mask != ~0ull);
           nxt_b = nn_b;
           nxt_dk = key_scale(i + 33 + lane, nxt_b);
           nn_b = list_id(i + 65 + lane);
@@ -779,6 +786,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
           par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
         }
+#pragma unroll 1
         for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
           if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
       }
@@ -834,10 +842,10 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         const uint64_t kd = kd0 + (uint64_t)(kk * kstep);
         const uint32_t d_s = tmem + col_s(s, g);
         if (tc::elect_one()) {
-          if (j >= S.n48) {
+          if (B16 && j >= S.n48) {
 #pragma unroll
             for (int ks = 0; ks < D / 16; ++ks) tc::mma_f16(d_s, qd2 + ks * 128, kd + ks * 128, tc::idesc_bf16(64), ks > 0);
-          } else if (j >= S.n4) {
+          } else if (!FP4 || j >= S.n4) {
 #pragma unroll
             for (int ks = 0; ks < D / 32; ++ks) tc::mma_i8(d_s, qd1 + ks * 128, kd + ks * 128, tc::idesc_i8(64), ks > 0);
           } else {
@@ -892,11 +900,11 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         const uint64_t pdg = pd0 + (uint64_t)((SEGMENTED ? pp : g) * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
         const uint32_t acc = j > 0;
         if (tc::elect_one()) {
-          if (j >= S.n48) {
+          if (B16 && j >= S.n48) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               tc::mma_f16(t_o, vd + ks * (2 * D), pdg + ks * 128, tc::idesc_bf16(64), acc | (ks > 0));
-          } else if (j >= S.n4) {
+          } else if (!FP4 || j >= S.n4) {
 #pragma unroll
             for (int ks = 0; ks < 2; ++ks)
               tc::mma_f8f6f4(t_o, vd + ks * (2 * D), pdg + ks * 128, tc::idesc_e4m3(64), acc | (ks > 0));
@@ -1065,9 +1073,8 @@ cudaError_t launch_bounded_wait_probe(int *status, long long limit_cycles, cudaS
 }
 
 cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t st, int *launches) {
-  SmemMap sm = make_smem_map(p, false);
-  const bool segmented = !sm.fits;
-  if (segmented) sm = make_smem_map(p, true);
+  const bool b16 = p.tier_active[2] != 0;
+  const SmemMap sm = make_smem_map(p, b16 && p.d == 128);
   if (!sm.fits) return cudaErrorInvalidConfiguration;
   cudaError_t e;
   const int grid = p.BH * ((p.Rt + 1) / 2);
@@ -1086,9 +1093,8 @@ cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t s
   };
   using I64 = std::integral_constant<int, 64>;
   using I128 = std::integral_constant<int, 128>;
-  if (p.d == 128) e = segmented ? pick(I128{}, std::true_type{}) : pick(I128{}, std::false_type{});
-  else if (!segmented) e = pick(I64{}, std::false_type{});
-  else e = cudaErrorInvalidConfiguration;  // (head_dim 64 always fits)
+  if (p.d == 128) e = b16 ? pick(I128{}, std::true_type{}) : pick(I128{}, std::false_type{});
+  else e = b16 ? pick(I64{}, std::true_type{}) : pick(I64{}, std::false_type{});
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();
