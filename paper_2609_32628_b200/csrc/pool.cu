@@ -1,9 +1,12 @@
 // Kernel 1: spatial-tile reorder + 2D average / max pooling of Q and K into per-block draft tokens
 // (Eq. "v2-descriptors"; padding of ragged edge tiles excluded, App. C.1), plus the statistics the quantisers
-// need before they can run: per-head max|Q|, max|K|, max|V| and per-(head, channel) max|V| (App. C.3).
+// need before they can run: per-head max|Q|, max|K|, max|V| and per-(head, channel) max|V| (App. C.3), and the scales
+// derived from them.
 //
-// One CTA per (block, head).  A block is an 8 x 8 tile of one frame: each of its 8 tile rows is 8 consecutive
-// tokens, i.e. 8*d*2 contiguous bytes in the raster tensor, so 16-byte loads of a tile row are fully coalesced.
+// A block is an 8 x 8 tile of one frame (or a run of 64 tokens).  A warp walks tokens of one block and every lane owns
+// D / 32 channels of it, so a token row is one coalesced load and sums and maxima stay in registers from the first token
+// to the last: no shuffles and no shared memory per block.  SPLIT warps share a block (1 where there are enough blocks to
+// fill the GPU, up to 8 for the smallest calls, whose time is the latency of one block); only their results are combined.
 // HBM-bound: reads Q, K, V once (3*N*d*2 bytes per head), writes 4*R*d*4 bytes.
 //
 // Sums are carried in fp64: a sum of at most 64 bf16 values is exact there, so the fp32 descriptor equals the
@@ -14,132 +17,172 @@ namespace da2 {
 
 namespace {
 
+constexpr int kPoolWarps = 8;
+
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+// magnitudes of bf16 pairs order like 16-bit integers
+__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a, uint32_t b) {
+  return __vimax3_u16x2(m, a & 0x7fff7fffu, b & 0x7fff7fffu);
+}
+__device__ __forceinline__ float abs_max_of(uint32_t m) { return fmaxf(bf16lo(m), bf16hi(m)); }
 
-template <int D>
-__global__ void __launch_bounds__(256) pool_kernel(Params p, const __nv_bfloat16 *__restrict__ q,
-                                                   const __nv_bfloat16 *__restrict__ k,
-                                                   const __nv_bfloat16 *__restrict__ v) {
-  constexpr int CPR = D / 8;          // 16-byte chunks per token row
-  constexpr int TP = 256 / CPR;       // token rows per pass
-  constexpr int PASSES = kSlots / TP;
-  const int a = blockIdx.x, bh = blockIdx.y;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cidx = tid % CPR, tsub = tid / CPR;
-  const unsigned long long mask = block_valid_mask(p, a);
-  const int n_valid = __popcll(mask);
-  const size_t head_off = (size_t)bh * p.Ntot * D;
-
-  double sq[8], sk[8];
-  float mq[8], mk[8], av[8];
-  float aq = 0.f, ak = 0.f;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) { sq[i] = 0.0; sk[i] = 0.0; mq[i] = -INFINITY; mk[i] = -INFINITY; av[i] = 0.f; }
-
-  // all loads of the thread are issued before the first is used (a padding slot reads slot 0's row and is ignored)
-  uint4 xq[PASSES], xk[PASSES], xv[PASSES];
-#pragma unroll
-  for (int ps = 0; ps < PASSES; ++ps) {
-    const int j = ps * TP + tsub;
-    const int js = ((mask >> j) & 1ull) ? j : 0;
-    const size_t off = head_off + (size_t)slot_token(p, a, js) * D + cidx * 8;
-    xq[ps] = *reinterpret_cast<const uint4 *>(q + off);
-    xk[ps] = *reinterpret_cast<const uint4 *>(k + off);
-    xv[ps] = *reinterpret_cast<const uint4 *>(v + off);
+template <int W> struct Row { uint32_t w[W]; };  // one token's channels of a lane
+template <int W> __device__ __forceinline__ Row<W> load_row(const uint16_t *p) {
+  Row<W> r;
+  if (W == 2) {
+    const uint2 x = __ldg(reinterpret_cast<const uint2 *>(p));
+    r.w[0] = x.x; r.w[W - 1] = x.y;
+  } else {
+    r.w[0] = __ldg(reinterpret_cast<const uint32_t *>(p));
   }
+  return r;
+}
+
+template <int D, int SPLIT>
+__global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const uint16_t *__restrict__ q, const uint16_t *__restrict__ k,
+                                                               const uint16_t *__restrict__ v) {
+  constexpr int W = D / 64;                  // words (channel pairs) per lane
+  constexpr int BLOCKS = kPoolWarps / SPLIT;  // blocks per CTA
+  constexpr int TOK = kSlots / SPLIT;        // tokens per warp
+  constexpr int BATCH = 8;                   // tokens whose loads are in flight together
+  const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int a = blockIdx.x * BLOCKS + warp / SPLIT, part = warp % SPLIT;
+  const bool live = a < p.R;
+
+  double sq[2 * W], sk[2 * W];
+  uint32_t mq[W], mk[W], av[W], aq = 0, ak = 0;
 #pragma unroll
-  for (int ps = 0; ps < PASSES; ++ps) {
-    const int j = ps * TP + tsub;
-    if ((mask >> j) & 1ull) {
-      const uint32_t wq[4] = {xq[ps].x, xq[ps].y, xq[ps].z, xq[ps].w}, wk[4] = {xk[ps].x, xk[ps].y, xk[ps].z, xk[ps].w},
-                     wv[4] = {xv[ps].x, xv[ps].y, xv[ps].z, xv[ps].w};
+  for (int i = 0; i < W; ++i) {
+    sq[2 * i] = sq[2 * i + 1] = sk[2 * i] = sk[2 * i + 1] = 0.0;
+    mq[i] = mk[i] = 0xff80ff80u;  // -inf
+    av[i] = 0;
+  }
+  int n_valid = 0;
+  if (live) {
+    const unsigned long long mask = block_valid_mask(p, a);
+    n_valid = __popcll(mask);
+    const size_t base = (size_t)bh * p.Ntot * D + lane * (2 * W);
+    // the tokens of a warp: lane l keeps the index of slot part * TOK + l (+ 32), -1 at padding
+    int tok[(TOK + 31) / 32];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        float f0 = bf16lo(wq[i]), f1 = bf16hi(wq[i]);
-        sq[2 * i] += (double)f0; sq[2 * i + 1] += (double)f1;
-        mq[2 * i] = fmaxf(mq[2 * i], f0); mq[2 * i + 1] = fmaxf(mq[2 * i + 1], f1);
-        aq = fmaxf(aq, fmaxf(fabsf(f0), fabsf(f1)));
-        f0 = bf16lo(wk[i]); f1 = bf16hi(wk[i]);
-        sk[2 * i] += (double)f0; sk[2 * i + 1] += (double)f1;
-        mk[2 * i] = fmaxf(mk[2 * i], f0); mk[2 * i + 1] = fmaxf(mk[2 * i + 1], f1);
-        ak = fmaxf(ak, fmaxf(fabsf(f0), fabsf(f1)));
-        f0 = fabsf(bf16lo(wv[i])); f1 = fabsf(bf16hi(wv[i]));
-        av[2 * i] = fmaxf(av[2 * i], f0); av[2 * i + 1] = fmaxf(av[2 * i + 1], f1);
+    for (int i = 0; i < (TOK + 31) / 32; ++i) {
+      const int j = part * TOK + i * 32 + lane;
+      tok[i] = i * 32 + lane < TOK && ((mask >> (j & 63)) & 1ull) ? (int)slot_token(p, a, j) : -1;
+    }
+#pragma unroll 1
+    for (int j0 = 0; j0 < TOK; j0 += BATCH) {
+      Row<W> xq[BATCH], xk[BATCH], xv[BATCH];
+      int t[BATCH];
+#pragma unroll
+      for (int i = 0; i < BATCH; ++i) {
+        const int src = TOK > 32 && j0 >= 32 ? tok[(TOK + 31) / 32 - 1] : tok[0];
+        t[i] = __shfl_sync(0xffffffffu, src, (j0 + i) & 31);
+        const size_t off = base + (size_t)max(t[i], 0) * D;
+        xq[i] = load_row<W>(q + off);
+        xk[i] = load_row<W>(k + off);
+        xv[i] = load_row<W>(v + off);
+      }
+#pragma unroll
+      for (int i = 0; i < BATCH; ++i) {
+        if (t[i] < 0) continue;  // (uniform) padding takes no part
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+          sq[2 * c] += (double)bf16lo(xq[i].w[c]); sq[2 * c + 1] += (double)bf16hi(xq[i].w[c]);
+          sk[2 * c] += (double)bf16lo(xk[i].w[c]); sk[2 * c + 1] += (double)bf16hi(xk[i].w[c]);
+          mq[c] = max_bf16x2(mq[c], xq[i].w[c]);
+          mk[c] = max_bf16x2(mk[c], xk[i].w[c]);
+          av[c] = max_abs2(av[c], xv[i].w[c], 0u);
+        }
+        aq = max_abs2(aq, xq[i].w[0], xq[i].w[W - 1]);
+        ak = max_abs2(ak, xk[i].w[0], xk[i].w[W - 1]);
       }
     }
   }
-  // combine the token rows that share a warp (lanes cidx, cidx+CPR, ...)
+
+  __shared__ uint32_t s_av[kPoolWarps][D / 2];
+  __shared__ uint32_t s_a[2][kPoolWarps];
+  __shared__ int s_last;
+  if (SPLIT > 1) {  // the warps of a block hand their sums and maxima to its first warp
+    __shared__ double s_sum[2][kPoolWarps][D];
+    __shared__ uint32_t s_max[2][kPoolWarps][D / 2];
 #pragma unroll
-  for (int off = 16; off >= CPR; off >>= 1) {
+    for (int c = 0; c < W; ++c) {
+      s_sum[0][warp][lane * 2 * W + 2 * c] = sq[2 * c]; s_sum[0][warp][lane * 2 * W + 2 * c + 1] = sq[2 * c + 1];
+      s_sum[1][warp][lane * 2 * W + 2 * c] = sk[2 * c]; s_sum[1][warp][lane * 2 * W + 2 * c + 1] = sk[2 * c + 1];
+      s_max[0][warp][lane * W + c] = mq[c];
+      s_max[1][warp][lane * W + c] = mk[c];
+    }
+    __syncthreads();
+    if (part == 0) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      sq[i] += __shfl_xor_sync(0xffffffffu, sq[i], off);
-      sk[i] += __shfl_xor_sync(0xffffffffu, sk[i], off);
-      mq[i] = fmaxf(mq[i], __shfl_xor_sync(0xffffffffu, mq[i], off));
-      mk[i] = fmaxf(mk[i], __shfl_xor_sync(0xffffffffu, mk[i], off));
-      av[i] = fmaxf(av[i], __shfl_xor_sync(0xffffffffu, av[i], off));
+      for (int w = 1; w < SPLIT; ++w)
+#pragma unroll
+        for (int c = 0; c < W; ++c) {
+          sq[2 * c] += s_sum[0][warp + w][lane * 2 * W + 2 * c]; sq[2 * c + 1] += s_sum[0][warp + w][lane * 2 * W + 2 * c + 1];
+          sk[2 * c] += s_sum[1][warp + w][lane * 2 * W + 2 * c]; sk[2 * c + 1] += s_sum[1][warp + w][lane * 2 * W + 2 * c + 1];
+          mq[c] = max_bf16x2(mq[c], s_max[0][warp + w][lane * W + c]);
+          mk[c] = max_bf16x2(mk[c], s_max[1][warp + w][lane * W + c]);
+        }
     }
   }
-  __shared__ double s_sum[2][8][D];
-  __shared__ float s_max[3][8][D];
-  __shared__ float s_amax[2][8];
-  if (lane < CPR) {
+  if (live && part == 0) {
+    const size_t o = ((size_t)bh * p.R + a) * D + lane * 2 * W;
+    const double n = (double)n_valid;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      s_sum[0][warp][cidx * 8 + i] = sq[i];
-      s_sum[1][warp][cidx * 8 + i] = sk[i];
-      s_max[0][warp][cidx * 8 + i] = mq[i];
-      s_max[1][warp][cidx * 8 + i] = mk[i];
-      s_max[2][warp][cidx * 8 + i] = av[i];
+    for (int c = 0; c < W; ++c) {
+      *reinterpret_cast<float2 *>(p.desc[0] + o + 2 * c) = make_float2((float)(sq[2 * c] / n), (float)(sq[2 * c + 1] / n));
+      *reinterpret_cast<float2 *>(p.desc[1] + o + 2 * c) = make_float2(bf16lo(mq[c]), bf16hi(mq[c]));
+      *reinterpret_cast<float2 *>(p.desc[2] + o + 2 * c) = make_float2((float)(sk[2 * c] / n), (float)(sk[2 * c + 1] / n));
+      *reinterpret_cast<float2 *>(p.desc[3] + o + 2 * c) = make_float2(bf16lo(mk[c]), bf16hi(mk[c]));
     }
   }
+  // statistics of the head: combined over the CTA first, then one atomic per channel (non-negative floats order like
+  // their bit patterns)
+#pragma unroll
+  for (int c = 0; c < W; ++c) s_av[warp][lane * W + c] = av[c];
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
-    aq = fmaxf(aq, __shfl_xor_sync(0xffffffffu, aq, off));
-    ak = fmaxf(ak, __shfl_xor_sync(0xffffffffu, ak, off));
+    aq = __vmaxu2(aq, __shfl_xor_sync(0xffffffffu, aq, off));
+    ak = __vmaxu2(ak, __shfl_xor_sync(0xffffffffu, ak, off));
   }
-  if (lane == 0) { s_amax[0][warp] = aq; s_amax[1][warp] = ak; }
+  if (lane == 0) { s_a[0][warp] = aq; s_a[1][warp] = ak; }
   __syncthreads();
-  if (tid < D) {
-    double tq = 0.0, tk = 0.0;
-    float xq = -INFINITY, xk = -INFINITY, xv = 0.f;
+  if (tid < D / 2) {
+    uint32_t m = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      tq += s_sum[0][w][tid]; tk += s_sum[1][w][tid];
-      xq = fmaxf(xq, s_max[0][w][tid]); xk = fmaxf(xk, s_max[1][w][tid]); xv = fmaxf(xv, s_max[2][w][tid]);
-    }
-    const size_t o = ((size_t)bh * p.R + a) * D + tid;
-    p.desc[0][o] = (float)(tq / (double)n_valid);
-    p.desc[1][o] = xq;
-    p.desc[2][o] = (float)(tk / (double)n_valid);
-    p.desc[3][o] = xk;
-    // non-negative floats order like their bit patterns
-    atomicMax(&p.vmax[(size_t)bh * D + tid], __float_as_uint(xv));
+    for (int w = 0; w < kPoolWarps; ++w) m = __vmaxu2(m, s_av[w][tid]);
+    atomicMax(&p.vmax[(size_t)bh * D + 2 * tid], m << 16);
+    atomicMax(&p.vmax[(size_t)bh * D + 2 * tid + 1], m & 0xffff0000u);
     // head maximum of |V| from the channel maxima: reduce within the warp first
-    float hv = xv;
+    float hv = abs_max_of(m);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) hv = fmaxf(hv, __shfl_xor_sync(0xffffffffu, hv, off));
     if (lane == 0) atomicMax(&p.amax[bh * 4 + 2], __float_as_uint(hv));
-  }
-  if (tid == 0) {
-    float tq = 0.f, tk = 0.f;
+  } else if (tid >= 128 && tid < 130) {
+    uint32_t m = 0;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) { tq = fmaxf(tq, s_amax[0][w]); tk = fmaxf(tk, s_amax[1][w]); }
-    atomicMax(&p.amax[bh * 4 + 0], __float_as_uint(tq));
-    atomicMax(&p.amax[bh * 4 + 1], __float_as_uint(tk));
+    for (int w = 0; w < kPoolWarps; ++w) m = __vmaxu2(m, s_a[tid - 128][w]);
+    atomicMax(&p.amax[bh * 4 + tid - 128], __float_as_uint(abs_max_of(m)));
   }
-}
-
-// Derived scales (App. C.3): NVFP4 per-tensor scale g_X = amax_X / 2688 (1 for an all-zero head), and the E4M3
-// per-channel value scale delta_c = max_v |V_vc| / 2.25 (0 marks an all-zero channel).
-__global__ void finalize_stats_kernel(Params p) {
-  const int bh = blockIdx.x;
-  for (int i = threadIdx.x; i < p.d; i += blockDim.x)
-    p.dv8[(size_t)bh * p.d + i] = __fdiv_rn(__uint_as_float(p.vmax[(size_t)bh * p.d + i]), 2.25f);
-  if (threadIdx.x < 3) {
-    const float am = __uint_as_float(p.amax[bh * 4 + threadIdx.x]);
-    p.gscale[bh * 4 + threadIdx.x] = am > 0.f ? __fdiv_rn(am, 2688.0f) : 1.0f;
+  // the last CTA of the head derives the scales (App. C.3): NVFP4 per-tensor scale g_X = amax_X / 2688 (1 for an all-zero
+  // head), and the E4M3 per-channel value scale delta_c = max_v |V_vc| / 2.25 (0 marks an all-zero channel)
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&p.amax[bh * 4 + 3], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (tid < D)
+    p.dv8[(size_t)bh * D + tid] = __fdiv_rn(__uint_as_float(__ldcg(&p.vmax[(size_t)bh * D + tid])), 2.25f);
+  if (tid < 3) {
+    const float am = __uint_as_float(__ldcg(&p.amax[bh * 4 + tid]));
+    p.gscale[bh * 4 + tid] = am > 0.f ? __fdiv_rn(am, 2688.0f) : 1.0f;
   }
 }
 
@@ -147,13 +190,16 @@ __global__ void finalize_stats_kernel(Params p) {
 
 cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                         cudaStream_t st, int *launches) {
-  dim3 grid(p.R, p.BH);
-  if (p.d == 128) pool_kernel<128><<<grid, 256, 0, st>>>(p, q, k, v);
-  else pool_kernel<64><<<grid, 256, 0, st>>>(p, q, k, v);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  finalize_stats_kernel<<<p.BH, 128, 0, st>>>(p);
-  *launches += 2;
+  // warps per block: one where the blocks alone give every SM about 16 warps, else up to all eight
+  const long long blocks = (long long)p.R * p.BH;
+  const int split = blocks >= 148 * 16 ? 1 : (blocks >= 148 * 4 ? 4 : 8);
+  const dim3 grid((p.R * split + kPoolWarps - 1) / kPoolWarps, p.BH);
+  const uint16_t *q16 = reinterpret_cast<const uint16_t *>(q), *k16 = reinterpret_cast<const uint16_t *>(k),
+                 *v16 = reinterpret_cast<const uint16_t *>(v);
+  auto launch = [&](auto kernel) { kernel<<<grid, kPoolWarps * 32, 0, st>>>(p, q16, k16, v16); };
+  if (p.d == 128) split == 1 ? launch(pool_kernel<128, 1>) : (split == 4 ? launch(pool_kernel<128, 4>) : launch(pool_kernel<128, 8>));
+  else split == 1 ? launch(pool_kernel<64, 1>) : (split == 4 ? launch(pool_kernel<64, 4>) : launch(pool_kernel<64, 8>));
+  *launches += 1;
   return cudaGetLastError();
 }
 

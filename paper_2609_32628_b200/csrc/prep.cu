@@ -7,7 +7,11 @@
 //   NVFP4 Q/K : E2M1 with one E4M3 scale per 16 channels; V: per 16 key slots of a channel; per-head scale g_X
 //   BF16      : the stored values, reordered only
 // Every fp32 operation below is a single correctly rounded operation in the order the format definition gives, so
-// codes and scales are reproducible bit for bit.  HBM-bound: reads 3*64*d*2 bytes per block, writes the records.
+// codes and scales are reproducible bit for bit.  Reads 3*64*d*2 bytes per block, writes the records.
+// HBM would allow it in half the time it takes: what bounds it is the integer and conversion work per element.  So every
+// thread takes its 32 channels of a row (Q, K) or 16 slots of two channels (V) out of shared memory once and makes the
+// codes of all formats from those registers, in packed pairs where an instruction for pairs exists, and the block needs
+// three barriers in all.
 #include <cuda_fp8.h>
 
 #include "da2_internal.cuh"
@@ -18,8 +22,6 @@ namespace {
 
 constexpr int NT = 256;
 
-__device__ __forceinline__ float bf16_to_f32(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
-
 // round half away from zero for |x| < 2^23: adding the largest float below one half (with the sign of x) and truncating
 // gives the same integer as roundf for every x in that range (the sum can only round up to the next integer when x
 // is at least one half above the integer below it)
@@ -28,36 +30,87 @@ __device__ __forceinline__ int round_half_away(float x) { return __float2int_rz(
 __device__ __forceinline__ uint32_t cast_e4m3(float x) {
   return (uint32_t)__nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
 }
-
-// two floats -> two E2M1 codes, `lo` in bits 3:0 and `hi` in bits 7:4 (round to nearest even, saturating)
-__device__ __forceinline__ uint32_t cast_e2m1x2(float lo, float hi) {
-  uint16_t r;
-  asm("{ .reg .b8 t; cvt.rn.satfinite.e2m1x2.f32 t, %2, %1; mov.b16 %0, {t, 0}; }" : "=h"(r) : "f"(lo), "f"(hi));
-  return (uint32_t)r;
-}
-
 __device__ __forceinline__ float decode_e4m3(uint32_t c) {
   const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
   return __half2float(*reinterpret_cast<const __half *>(&h));
 }
+// four ints -> four int8 codes; four floats -> four E4M3 codes; eight floats -> eight E2M1 codes (round to nearest even,
+// saturating; the first in the low bits)
+__device__ __forceinline__ uint32_t pack_s8x4(int c0, int c1, int c2, int c3) {
+  uint32_t r;
+  asm("{ .reg .b32 t; cvt.pack.sat.s8.s32.b32 t, %4, %3, 0; cvt.pack.sat.s8.s32.b32 %0, %2, %1, t; }"
+      : "=r"(r)
+      : "r"(c0), "r"(c1), "r"(c2), "r"(c3));
+  return r;
+}
+__device__ __forceinline__ uint32_t pack_e4m3x4(const float *x) {
+  uint32_t r;
+  asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
+      : "=r"(r)
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]));
+  return r;
+}
+__device__ __forceinline__ uint32_t pack_e2m1x8(const float *x) {
+  uint32_t r;
+  asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
+      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
+      : "=r"(r)
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]));
+  return r;
+}
+// packed pairs of fp32
+__device__ __forceinline__ uint64_t f2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// magnitudes of bf16 pairs order like 16-bit integers
+__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a, uint32_t b) {
+  return __vimax3_u16x2(m, a & 0x7fff7fffu, b & 0x7fff7fffu);
+}
+__device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // Correctly rounded x / d for many x and one positive divisor d, without a division per element: with r = RN(1/d),
-// q0 = RN(x r), e = x - q0 d (exact in one fused multiply-add) and q = RN(q0 + e r) is the correctly rounded quotient
+// q0 = RN(x r), e = q0 d - x (exact in one fused multiply-add) and q = RN(q0 - e r) is the correctly rounded quotient
 // (Markstein's division theorem).  Checked exhaustively on the device against the IEEE division for every bf16 x
-// with |x| >= 2^-100 and millions of divisors in [2^-60, 2^60], significands of all ones included: the only
-// difference is the sign of a zero quotient, which the sign copy restores (d > 0).  For |x| < 2^-100 the residual can
+// with |x| >= 2^-100 and millions of divisors in [2^-60, 2^60], significands of all ones included.  The callers hand in
+// y = -x, so that all three steps are plain multiply-adds on pairs and a zero quotient keeps the sign of x: q0 = y (-r) is
+// a zero of the sign of x, e = +0, and q = (+0)(-r) + q0 = q0.  For |x| < 2^-100 the residual can
 // underflow; the quotient is then below 2^-40 in magnitude either way and every format here encodes it as a signed
 // zero.  Divisors outside [2^-60, 2^60] (or not finite) keep the plain division.  da2_selfcheck_quantiser_arithmetic
 // repeats the check with these very functions.
 struct Divider {
   float d, r;
   bool fast;
-  __device__ __forceinline__ float quick(float x) const {
-    const float q0 = __fmul_rn(x, r);
-    const float e = __fmaf_rn(-q0, d, x);
-    return copysignf(__fmaf_rn(e, r, q0), x);
+  __device__ __forceinline__ void quick2(float y0, float y1, float &q0, float &q1) const {  // -y0 / d, -y1 / d
+    const uint64_t y = f2(y0, y1), nr = f2(-r, -r);
+    const uint64_t q = mul2(y, nr);
+    const uint64_t e = fma2(q, f2(d, d), y);
+    const uint64_t z = fma2(e, nr, q);
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(q0), "=f"(q1) : "l"(z));
   }
   __device__ __forceinline__ float exact(float x) const { return __fdiv_rn(x, d); }
+  // the quotients of N bf16 pairs given as words with both signs flipped
+  template <int N> __device__ __forceinline__ void quotients(const uint32_t (&nw)[N], float (&x)[2 * N]) const {
+    if (fast) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) quick2(bf16lo(nw[i]), bf16hi(nw[i]), x[2 * i], x[2 * i + 1]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; ++i) { x[2 * i] = exact(-bf16lo(nw[i])); x[2 * i + 1] = exact(-bf16hi(nw[i])); }
+    }
+  }
 };
 __device__ __forceinline__ Divider make_divider(float d) {
   Divider v;
@@ -67,23 +120,17 @@ __device__ __forceinline__ Divider make_divider(float d) {
   return v;
 }
 
-// NVFP4 group of 16 values (Eq. "v2-nvfp4-quantization"): returns the E4M3 scale code, writes 8 bytes of codes
-__device__ __forceinline__ uint32_t nvfp4_group(const float (&x)[16], float g, uint32_t (&packed)[2]) {
-  float gmax = 0.f;
-#pragma unroll
-  for (int i = 0; i < 16; ++i) gmax = fmaxf(gmax, fabsf(x[i]));
-  const uint32_t sc = cast_e4m3(__fdiv_rn(gmax, __fmul_rn(6.0f, g)));
+// NVFP4 group of 16 values (Eq. "v2-nvfp4-quantization") given as sign-flipped bf16 words and their largest magnitude:
+// returns the E4M3 scale code, writes 8 bytes of codes
+__device__ __forceinline__ uint32_t nvfp4_group(const uint32_t (&nw)[8], float gmax, float g6, float g, uint32_t &lo, uint32_t &hi) {
+  const uint32_t sc = cast_e4m3(__fdiv_rn(gmax, g6));
   const float sigma = decode_e4m3(sc);
-  packed[0] = 0; packed[1] = 0;
+  lo = 0; hi = 0;
   if (sigma == 0.f) return sc;  // a group whose encoded scale is zero is encoded as zero
-  const Divider dv = make_divider(__fmul_rn(g, sigma));
-  if (dv.fast) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) packed[i >> 2] |= cast_e2m1x2(dv.quick(x[2 * i]), dv.quick(x[2 * i + 1])) << (8 * (i & 3));
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) packed[i >> 2] |= cast_e2m1x2(dv.exact(x[2 * i]), dv.exact(x[2 * i + 1])) << (8 * (i & 3));
-  }
+  float x[16];
+  make_divider(__fmul_rn(g, sigma)).quotients(nw, x);
+  lo = pack_e2m1x8(x);
+  hi = pack_e2m1x8(x + 8);
   return sc;
 }
 
@@ -91,18 +138,19 @@ __device__ __forceinline__ uint32_t nvfp4_group(const float (&x)[16], float g, u
 // call whose quantiser statistics are already known reads Q, K, V from HBM exactly once (Sec. 3.3, "Fused
 // quantization and reordering").
 template <int D, bool POOL>
-__global__ void __launch_bounds__(NT) prep_kernel(Params p, const __nv_bfloat16 *__restrict__ q,
+__global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat16 *__restrict__ q,
                                                   const __nv_bfloat16 *__restrict__ k,
                                                   const __nv_bfloat16 *__restrict__ v) {
   extern __shared__ __align__(16) uint8_t smem[];
-  uint16_t *tq = reinterpret_cast<uint16_t *>(smem);   // [64][D]
-  // rows are padded by 16 bytes: threads that read the same channels of consecutive slots then fall on different banks
-  constexpr int LD = D + 8;
-  uint16_t *tk = tq + kSlots * LD;
-  uint16_t *tv = tk + kSlots * LD;
-  uint8_t *sf_img = reinterpret_cast<uint8_t *>(tv + kSlots * LD);  // up to 3 atoms (Q or K: D/64, V: 1)
-  __shared__ float s_red[2][NT / 32];
-  __shared__ float s_delta[2];
+  // Q, K: rows padded by 16 bytes, so that threads that read the same channels of consecutive slots fall on different
+  // banks.  V: the 64-byte halves of a 128-byte line are swapped in every other group of 16 rows, so that the two groups a
+  // warp reads at a time fall on different banks.
+  constexpr int LD = D + 8, ROW = LD * 2;
+  uint8_t *tq = smem, *tk = tq + kSlots * ROW, *tv = tk + kSlots * ROW;
+  uint8_t *sf_img = tv + kSlots * D * 2;  // scale atoms: Q and K D/64 each, V one
+  constexpr int NATOM = D / 64;
+  uint8_t *sf_v = sf_img + 2 * NATOM * kSfAtomBytes;
+  __shared__ uint32_t s_red[2][NT / 32];
 
   const int a = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned long long mask = block_valid_mask(p, a);
@@ -110,6 +158,7 @@ __global__ void __launch_bounds__(NT) prep_kernel(Params p, const __nv_bfloat16 
   const size_t blk = (size_t)bh * p.R + a;        // record index in the quantised tiers (video blocks only)
   const size_t blk16 = (size_t)bh * p.Rt + a;     // record index in the 16-bit tier (video and prefix blocks)
   const bool video = a < p.R;                      // prefix blocks only ever run in the 16-bit tier (App. C.1)
+  const bool t4 = p.tier_active[0] && video, t8 = p.tier_active[1] && video, t16 = p.tier_active[2];
   // the regions of the first frame also leave the frame's region table for the attention kernel
   if (bh == 0 && a < p.R_f) {
     if (tid < kSlots) p.region_cell[a * kSlots + tid] = (int)(slot_token(p, a, tid) - p.P);
@@ -117,41 +166,41 @@ __global__ void __launch_bounds__(NT) prep_kernel(Params p, const __nv_bfloat16 
   }
 
   // stage the three tiles, padding slots as zeros; track max|Q|, max|K| of the block
-  float aq = 0.f, ak = 0.f;
-  constexpr int CPR = D / 8;
-  for (int idx = tid; idx < kSlots * CPR; idx += NT) {
-    const int j = idx / CPR, c8 = idx % CPR;
-    uint4 xq = make_uint4(0, 0, 0, 0), xk = xq, xv = xq;
-    if ((mask >> j) & 1ull) {
-      const size_t off = head_off + (size_t)slot_token(p, a, j) * D + c8 * 8;
-      xq = *reinterpret_cast<const uint4 *>(q + off);
-      xk = *reinterpret_cast<const uint4 *>(k + off);
-      xv = *reinterpret_cast<const uint4 *>(v + off);
+  {
+    constexpr int CPR = D / 8, PASSES = kSlots * CPR / NT;
+    const int c8 = tid % CPR;
+    uint4 xq[PASSES], xk[PASSES], xv[PASSES];
+#pragma unroll
+    for (int i = 0; i < PASSES; ++i) {
+      const int j = (tid + i * NT) / CPR;
+      xq[i] = xk[i] = xv[i] = make_uint4(0, 0, 0, 0);
+      if ((mask >> j) & 1ull) {
+        const size_t off = head_off + (size_t)slot_token(p, a, j) * D + c8 * 8;
+        xq[i] = __ldg(reinterpret_cast<const uint4 *>(q + off));
+        xk[i] = __ldg(reinterpret_cast<const uint4 *>(k + off));
+        xv[i] = __ldg(reinterpret_cast<const uint4 *>(v + off));
+      }
     }
-    *reinterpret_cast<uint4 *>(tq + j * LD + c8 * 8) = xq;
-    *reinterpret_cast<uint4 *>(tk + j * LD + c8 * 8) = xk;
-    *reinterpret_cast<uint4 *>(tv + j * LD + c8 * 8) = xv;
-    const uint32_t wq[4] = {xq.x, xq.y, xq.z, xq.w}, wk[4] = {xk.x, xk.y, xk.z, xk.w};
+    uint32_t aq = 0, ak = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      aq = fmaxf(aq, fmaxf(fabsf(__uint_as_float(wq[i] << 16)), fabsf(__uint_as_float(wq[i] & 0xffff0000u))));
-      ak = fmaxf(ak, fmaxf(fabsf(__uint_as_float(wk[i] << 16)), fabsf(__uint_as_float(wk[i] & 0xffff0000u))));
+    for (int i = 0; i < PASSES; ++i) {
+      const int j = (tid + i * NT) / CPR;
+      *reinterpret_cast<uint4 *>(tq + j * ROW + c8 * 16) = xq[i];
+      *reinterpret_cast<uint4 *>(tk + j * ROW + c8 * 16) = xk[i];
+      *reinterpret_cast<uint4 *>(tv + j * (D * 2) + (c8 ^ (((j >> 4) & 1) << 2)) * 16) = xv[i];
+      aq = max_abs2(max_abs2(aq, xq[i].x, xq[i].y), xq[i].z, xq[i].w);
+      ak = max_abs2(max_abs2(ak, xk[i].x, xk[i].y), xk[i].z, xk[i].w);
     }
-  }
+    if (t8) {
 #pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    aq = fmaxf(aq, __shfl_xor_sync(0xffffffffu, aq, o));
-    ak = fmaxf(ak, __shfl_xor_sync(0xffffffffu, ak, o));
-  }
-  if (lane == 0) { s_red[0][warp] = aq; s_red[1][warp] = ak; }
-  __syncthreads();
-  if (tid < 2) {
-    float m = 0.f;
-#pragma unroll
-    for (int w = 0; w < NT / 32; ++w) m = fmaxf(m, s_red[tid][w]);
-    const float delta = __fadd_rn(__fdiv_rn(m, 127.0f), 1e-7f);
-    s_delta[tid] = delta;
-    if (p.tier_active[1] && video) (tid == 0 ? p.dq8 : p.dk8)[blk] = delta;
+      for (int o = 16; o >= 1; o >>= 1) {
+        aq = __vmaxu2(aq, __shfl_xor_sync(0xffffffffu, aq, o));
+        ak = __vmaxu2(ak, __shfl_xor_sync(0xffffffffu, ak, o));
+      }
+      if (lane == 0) { s_red[0][warp] = aq; s_red[1][warp] = ak; }
+    }
+    // head_dim 64 leaves the atom of V half empty (channels 64..127)
+    if (D == 64 && tid < kSfAtomBytes / 16) *reinterpret_cast<uint4 *>(sf_v + tid * 16) = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
 
@@ -160,13 +209,13 @@ __global__ void __launch_bounds__(NT) prep_kernel(Params p, const __nv_bfloat16 
     // 64 bf16 values is exact in fp64, so the mean is correctly rounded whatever the order.
     const int n_valid = __popcll(mask);
     for (int idx = tid; idx < 2 * D; idx += NT) {
-      const uint16_t *src = (idx < D ? tq : tk) + (idx % D);
+      const uint8_t *src = (idx < D ? tq : tk) + (idx % D) * 2;
       double sum = 0.0;
       float mx = -INFINITY;
 #pragma unroll 8
       for (int j = 0; j < kSlots; ++j) {
         if ((mask >> j) & 1ull) {
-          const float x = bf16_to_f32(src[j * LD]);
+          const float x = bf16lo(*reinterpret_cast<const uint16_t *>(src + j * ROW));
           sum += (double)x;
           mx = fmaxf(mx, x);
         }
@@ -177,139 +226,149 @@ __global__ void __launch_bounds__(NT) prep_kernel(Params p, const __nv_bfloat16 
     }
   }
 
-  // ------------------------------------------------------------------ tier 2: BF16, reorder only
-  if (p.tier_active[2]) {
-    uint8_t *qr = p.qrec[2] + blk16 * p.qrec_bytes[2];
-    uint8_t *kr = p.kvrec[2] + blk16 * p.kvrec_bytes[2];
-    uint8_t *vr = kr + kSlots * D * 2;
-    for (int idx = tid; idx < kSlots * D / 8; idx += NT) {  // chunk (kc, r): channels kc*8.. of slot r
-      const int kc = idx / kSlots, r = idx % kSlots;
-      *reinterpret_cast<uint4 *>(qr + (size_t)idx * 16) = *reinterpret_cast<const uint4 *>(tq + r * LD + kc * 8);
-      *reinterpret_cast<uint4 *>(kr + (size_t)idx * 16) = *reinterpret_cast<const uint4 *>(tk + r * LD + kc * 8);
+  // ------------------------------------------------------------------ Q and K: 32 channels of one slot per thread
+#pragma unroll 1
+  for (int u = tid; u < 2 * kSlots * (D / 32); u += NT) {
+    const int which = u / (kSlots * (D / 32)), r = u % kSlots, kc = (u / kSlots) % (D / 32);  // 0: Q, 1: K (warp-uniform)
+    uint32_t w[16];
+    const uint8_t *src = (which ? tk : tq) + r * ROW + kc * 64;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(w + 4 * i) = *reinterpret_cast<const uint4 *>(src + 16 * i);
+    if (t16) {  // chunk (c, r): channels c*8.. of slot r
+      uint8_t *dst = (which ? p.kvrec[2] + blk16 * p.kvrec_bytes[2] : p.qrec[2] + blk16 * p.qrec_bytes[2]) + (kc * 4 * kSlots + r) * 16;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) *reinterpret_cast<uint4 *>(dst + i * kSlots * 16) = *reinterpret_cast<const uint4 *>(w + 4 * i);
     }
-    for (int idx = tid; idx < D * kSlots / 8; idx += NT) {  // chunk (kc, c): slots kc*8.. of channel c
-      const int kc = idx / D, c = idx % D;
-      uint32_t w[4];
+    if (!t8 && !t4) continue;
+    uint32_t nw[2][8];  // signs flipped (see Divider)
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        w[i] = (uint32_t)tv[(kc * 8 + 2 * i) * LD + c] | ((uint32_t)tv[(kc * 8 + 2 * i + 1) * LD + c] << 16);
-      *reinterpret_cast<uint4 *>(vr + (size_t)idx * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-  }
-
-  // ------------------------------------------------------------------ tier 1: INT8 Q/K, E4M3 V
-  if (p.tier_active[1] && video) {
-    uint8_t *qr = p.qrec[1] + blk * p.qrec_bytes[1];
-    uint8_t *kr = p.kvrec[1] + blk * p.kvrec_bytes[1];
-    uint8_t *vr = kr + kSlots * D;
-    const Divider dq = make_divider(s_delta[0]), dk = make_divider(s_delta[1]);  // delta >= 1e-7: always in the quick range
-    for (int idx = tid; idx < kSlots * D / 16; idx += NT) {  // chunk (kc, r): channels kc*16.. of slot r
-      const int kc = idx / kSlots, r = idx % kSlots;
-      uint32_t wq[4] = {0, 0, 0, 0}, wk[4] = {0, 0, 0, 0};
-      uint32_t xq[8], xk[8];  // 16 bf16 values each, two per word
-      *reinterpret_cast<uint4 *>(xq) = *reinterpret_cast<const uint4 *>(tq + r * LD + kc * 16);
-      *reinterpret_cast<uint4 *>(xq + 4) = *reinterpret_cast<const uint4 *>(tq + r * LD + kc * 16 + 8);
-      *reinterpret_cast<uint4 *>(xk) = *reinterpret_cast<const uint4 *>(tk + r * LD + kc * 16);
-      *reinterpret_cast<uint4 *>(xk + 4) = *reinterpret_cast<const uint4 *>(tk + r * LD + kc * 16 + 8);
+    for (int i = 0; i < 16; ++i) nw[i >> 3][i & 7] = w[i] ^ 0x80008000u;
+    if (t8) {  // chunk (c, r): channels c*16.. of slot r
+      uint32_t m = 0;
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const float fq = __uint_as_float((i & 1) ? (xq[i >> 1] & 0xffff0000u) : (xq[i >> 1] << 16));
-        const float fk = __uint_as_float((i & 1) ? (xk[i >> 1] & 0xffff0000u) : (xk[i >> 1] << 16));
-        const int cq = round_half_away(dq.fast ? dq.quick(fq) : dq.exact(fq));
-        const int ck = round_half_away(dk.fast ? dk.quick(fk) : dk.exact(fk));
-        wq[i >> 2] |= (uint32_t)(cq & 0xff) << (8 * (i & 3));
-        wk[i >> 2] |= (uint32_t)(ck & 0xff) << (8 * (i & 3));
-      }
-      *reinterpret_cast<uint4 *>(qr + (size_t)idx * 16) = make_uint4(wq[0], wq[1], wq[2], wq[3]);
-      *reinterpret_cast<uint4 *>(kr + (size_t)idx * 16) = make_uint4(wk[0], wk[1], wk[2], wk[3]);
-    }
-    for (int idx = tid; idx < D * kSlots / 16; idx += NT) {  // chunk (kc, c): slots kc*16.. of channel c
-      const int kc = idx / D, c = idx % D;
-      const float dv = p.dv8[(size_t)bh * D + c];
-      uint32_t w[4] = {0, 0, 0, 0};
-      if (dv > 0.f) {
-        const Divider div = make_divider(dv);
-        const uint32_t m16 = (uint32_t)(mask >> (kc * 16)) & 0xffffu;
-        if (div.fast) {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const uint32_t code = cast_e4m3(div.quick(bf16_to_f32(tv[(kc * 16 + i) * LD + c])));
-            w[i >> 2] |= ((m16 >> i) & 1u) ? code << (8 * (i & 3)) : 0u;
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const uint32_t code = cast_e4m3(div.exact(bf16_to_f32(tv[(kc * 16 + i) * LD + c])));
-            w[i >> 2] |= ((m16 >> i) & 1u) ? code << (8 * (i & 3)) : 0u;
-          }
-        }
-      }
-      *reinterpret_cast<uint4 *>(vr + (size_t)idx * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-  }
-
-  // ------------------------------------------------------------------ tier 0: NVFP4
-  if (p.tier_active[0] && video) {
-    const float gq = p.gscale[bh * 4 + 0], gk = p.gscale[bh * 4 + 1], gv = p.gscale[bh * 4 + 2];
-    constexpr int QK_IMG = kSlots * D / 2, NATOM = D / 64;
-    uint8_t *qr = p.qrec[0] + blk * p.qrec_bytes[0];
-    uint8_t *kr = p.kvrec[0] + blk * p.kvrec_bytes[0];
-    uint8_t *vr = kr + QK_IMG + NATOM * kSfAtomBytes;
-    for (int which = 0; which < 2; ++which) {  // 0: Q, 1: K
-      const uint16_t *src = which ? tk : tq;
-      uint8_t *dst = which ? kr : qr;
-      const float g = which ? gk : gq;
-      __syncthreads();
-      for (int i = tid; i < NATOM * kSfAtomBytes / 4; i += NT) reinterpret_cast<uint32_t *>(sf_img)[i] = 0;
-      __syncthreads();
-      for (int idx = tid; idx < kSlots * D / 32; idx += NT) {  // chunk (kc, r): channels kc*32.. of slot r
-        const int kc = idx / kSlots, r = idx % kSlots;
-        uint32_t w[4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float x[16];
-          uint32_t pk[2];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) x[i] = bf16_to_f32(src[r * LD + kc * 32 + h * 16 + i]);
-          const uint32_t sc = nvfp4_group(x, g, pk);
-          w[2 * h] = pk[0]; w[2 * h + 1] = pk[1];
-          const int grp = kc * 2 + h;  // 16-channel group index; 4 groups per atom
-          // rows 0..63 and, duplicated, rows 64..127: the attention kernel places a block's queries in either half
-          uint8_t *sfp = sf_img + (grp >> 2) * kSfAtomBytes + (r & 31) * 16 + (r >> 5) * 4 + (grp & 3);
-          sfp[0] = (uint8_t)sc;
-          sfp[8] = (uint8_t)sc;
-        }
-        *reinterpret_cast<uint4 *>(dst + (size_t)idx * 16) = make_uint4(w[0], w[1], w[2], w[3]);
-      }
-      __syncthreads();
-      for (int i = tid; i < NATOM * kSfAtomBytes / 16; i += NT)
-        *reinterpret_cast<uint4 *>(dst + QK_IMG + (size_t)i * 16) = reinterpret_cast<const uint4 *>(sf_img)[i];
-    }
-    __syncthreads();
-    for (int i = tid; i < kSfAtomBytes / 4; i += NT) reinterpret_cast<uint32_t *>(sf_img)[i] = 0;
-    __syncthreads();
-    for (int idx = tid; idx < D * kSlots / 32; idx += NT) {  // chunk (kc, c): slots kc*32.. of channel c
-      const int kc = idx / D, c = idx % D;
-      uint32_t w[4];
+      for (int i = 0; i < NT / 32; ++i) m = __vmaxu2(m, s_red[which][i]);
+      const float delta = __fadd_rn(__fdiv_rn(fmaxf(bf16lo(m), bf16hi(m)), 127.0f), 1e-7f);
+      if (r == 0 && kc == 0) (which ? p.dk8 : p.dq8)[blk] = delta;
+      const Divider dv = make_divider(delta);  // delta >= 1e-7: always in the quick range (unless it is not finite)
+      uint8_t *dst = (which ? p.kvrec[1] + blk * p.kvrec_bytes[1] : p.qrec[1] + blk * p.qrec_bytes[1]) + (kc * 2 * kSlots + r) * 16;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float x[16];
-        uint32_t pk[2];
+        dv.quotients(nw[h], x);
+        uint32_t c[4];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) x[i] = bf16_to_f32(tv[(kc * 32 + h * 16 + i) * LD + c]);
-        const uint32_t sc = nvfp4_group(x, gv, pk);
-        w[2 * h] = pk[0]; w[2 * h + 1] = pk[1];
-        sf_img[(c & 31) * 16 + (c >> 5) * 4 + (kc * 2 + h)] = (uint8_t)sc;
+        for (int i = 0; i < 4; ++i)
+          c[i] = pack_s8x4(round_half_away(x[4 * i]), round_half_away(x[4 * i + 1]), round_half_away(x[4 * i + 2]), round_half_away(x[4 * i + 3]));
+        *reinterpret_cast<uint4 *>(dst + h * kSlots * 16) = make_uint4(c[0], c[1], c[2], c[3]);
       }
-      *reinterpret_cast<uint4 *>(vr + (size_t)idx * 16) = make_uint4(w[0], w[1], w[2], w[3]);
     }
+    if (t4) {  // chunk (kc, r): channels kc*32.. of slot r
+      const float g = p.gscale[bh * 4 + which], g6 = __fmul_rn(6.0f, g);
+      uint32_t c[4], sc[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t m = max_abs2(max_abs2(0u, nw[h][0], nw[h][1]), nw[h][2], nw[h][3]);
+        m = max_abs2(max_abs2(m, nw[h][4], nw[h][5]), nw[h][6], nw[h][7]);
+        sc[h] = nvfp4_group(nw[h], fmaxf(bf16lo(m), bf16hi(m)), g6, g, c[2 * h], c[2 * h + 1]);
+      }
+      uint8_t *dst = which ? p.kvrec[0] + blk * p.kvrec_bytes[0] : p.qrec[0] + blk * p.qrec_bytes[0];
+      *reinterpret_cast<uint4 *>(dst + (kc * kSlots + r) * 16) = make_uint4(c[0], c[1], c[2], c[3]);
+      // rows 0..63 and, duplicated, rows 64..127: the attention kernel places a block's queries in either half
+      uint8_t *sfp = sf_img + (which * NATOM + (kc >> 1)) * kSfAtomBytes + (r & 31) * 16 + (r >> 5) * 4 + (kc & 1) * 2;
+      const uint16_t two = (uint16_t)(sc[0] | (sc[1] << 8));
+      *reinterpret_cast<uint16_t *>(sfp) = two;
+      *reinterpret_cast<uint16_t *>(sfp + 8) = two;
+    }
+  }
+
+  // ------------------------------------------------------------------ V: 16 slots of two channels per thread
+  // Lanes 2x and 2x + 1 hold neighbouring groups of 16 slots of the same channels; before a store they exchange halves, so
+  // that lane parity stands for the channel and a warp writes 512 contiguous bytes.
+  if (tid < 2 * D) {
+    const int h = lane & 1, pair = (warp % (D / 32)) * 16 + (lane >> 1), gh = warp / (D / 32), g = gh * 2 + h;
+    uint32_t w[16];  // slot g*16 + i: channels 2 * pair (low half) and 2 * pair + 1
+    const uint8_t *src = tv + g * 16 * (D * 2) + ((pair >> 2) ^ (h << 2)) * 16 + (pair & 3) * 4;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = *reinterpret_cast<const uint32_t *>(src + i * (D * 2));
+    uint32_t nw[2][8], m = 0;  // per channel, slots in pairs, signs flipped
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      m = max_abs2(m, w[2 * i], w[2 * i + 1]);
+      nw[0][i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410) ^ 0x80008000u;
+      nw[1][i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632) ^ 0x80008000u;
+    }
+    // Hands over the channel the other lane stores; mine[e]: this lane's 16 bytes of channel e.  Afterwards out[0] / out[1]
+    // are the 16 bytes of slot groups gh*2 / gh*2 + 1 of channel 2 * pair + h.
+    auto exchange = [&](const uint4 (&mine)[2], uint4 (&both)[2]) {
+      const uint4 give = h ? mine[0] : mine[1], own = h ? mine[1] : mine[0];
+      uint4 got;
+      got.x = __shfl_xor_sync(0xffffffffu, give.x, 1); got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
+      got.z = __shfl_xor_sync(0xffffffffu, give.z, 1); got.w = __shfl_xor_sync(0xffffffffu, give.w, 1);
+      both[0] = h ? got : own;
+      both[1] = h ? own : got;
+    };
+    const int ch = 2 * pair + h;
+    if (t16) {  // chunk (c, ch): slots c*8.. of channel ch
+      uint8_t *dst = p.kvrec[2] + blk16 * p.kvrec_bytes[2] + kSlots * D * 2;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint4 mine[2], both[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          mine[e] = make_uint4(nw[e][half * 4] ^ 0x80008000u, nw[e][half * 4 + 1] ^ 0x80008000u, nw[e][half * 4 + 2] ^ 0x80008000u,
+                               nw[e][half * 4 + 3] ^ 0x80008000u);
+        exchange(mine, both);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) *reinterpret_cast<uint4 *>(dst + (((gh * 2 + e) * 2 + half) * D + ch) * 16) = both[e];
+      }
+    }
+    if (t8) {  // chunk (c, ch): slots c*16.. of channel ch (padding slots hold +0: code 0)
+      const float2 dv = *reinterpret_cast<const float2 *>(p.dv8 + (size_t)bh * D + 2 * pair);
+      uint4 mine[2], both[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float d = e ? dv.y : dv.x;
+        mine[e] = make_uint4(0, 0, 0, 0);
+        if (d > 0.f) {  // an all-zero channel is encoded as zero
+          float x[16];
+          make_divider(d).quotients(nw[e], x);
+          mine[e] = make_uint4(pack_e4m3x4(x), pack_e4m3x4(x + 4), pack_e4m3x4(x + 8), pack_e4m3x4(x + 12));
+        }
+      }
+      exchange(mine, both);
+      uint8_t *dst = p.kvrec[1] + blk * p.kvrec_bytes[1] + kSlots * D + (gh * 2 * D + ch) * 16;
+      *reinterpret_cast<uint4 *>(dst) = both[0];
+      *reinterpret_cast<uint4 *>(dst + D * 16) = both[1];
+    }
+    if (t4) {  // chunk (gh, ch): slots gh*32.. of channel ch
+      const float gv = p.gscale[bh * 4 + 2], g6 = __fmul_rn(6.0f, gv);
+      uint2 mine[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int c = 2 * pair + e;
+        sf_v[(c & 31) * 16 + (c >> 5) * 4 + g] = (uint8_t)nvfp4_group(nw[e], e ? bf16hi(m) : bf16lo(m), g6, gv, mine[e].x, mine[e].y);
+      }
+      const uint2 give = h ? mine[0] : mine[1], own = h ? mine[1] : mine[0];
+      uint2 got;
+      got.x = __shfl_xor_sync(0xffffffffu, give.x, 1); got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
+      *reinterpret_cast<uint4 *>(p.kvrec[0] + blk * p.kvrec_bytes[0] + kSlots * D / 2 + NATOM * kSfAtomBytes + (gh * D + ch) * 16) =
+          h ? make_uint4(got.x, got.y, own.x, own.y) : make_uint4(own.x, own.y, got.x, got.y);
+    }
+  }
+  if (t4) {  // the scale atoms: Q, K (behind their images), V (behind its image)
     __syncthreads();
-    for (int i = tid; i < kSfAtomBytes / 16; i += NT)
-      *reinterpret_cast<uint4 *>(vr + D * kSlots / 2 + (size_t)i * 16) = reinterpret_cast<const uint4 *>(sf_img)[i];
+    constexpr int QK_IMG = kSlots * D / 2, ATOM16 = kSfAtomBytes / 16;
+    for (int i = tid; i < (2 * NATOM + 1) * ATOM16; i += NT) {
+      uint8_t *dst;
+      if (i < NATOM * ATOM16) dst = p.qrec[0] + blk * p.qrec_bytes[0] + QK_IMG + i * 16;
+      else if (i < 2 * NATOM * ATOM16) dst = p.kvrec[0] + blk * p.kvrec_bytes[0] + QK_IMG + (i - NATOM * ATOM16) * 16;
+      else dst = p.kvrec[0] + blk * p.kvrec_bytes[0] + QK_IMG + NATOM * kSfAtomBytes + D * kSlots / 2 + (i - 2 * NATOM * ATOM16) * 16;
+      *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(sf_img + i * 16);
+    }
   }
 }
 
-// Self-check of Divider::quick and round_half_away against the IEEE division and roundf (see da2.h).
+// Self-check of Divider::quick2 and round_half_away against the IEEE division and roundf (see da2.h).
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
   x ^= x >> 16; x *= 0x7feb352dU; x ^= x >> 15; x *= 0x846ca68bU; x ^= x >> 16;
   return x;
@@ -327,7 +386,9 @@ __global__ void selfcheck_quotient_kernel(int n_divisors, int all_ones, uint32_t
     if (!(fabsf(x) <= 3.0e38f) || (x != 0.f && fabsf(x) < 7.9e-31f)) continue;  // finite, zero or at least 2^-100
     const float ref = div.exact(x);
     if (!(fabsf(ref) < 3.0e38f) || (ref != 0.f && fabsf(ref) < 1e-30f)) continue;  // quotient in the normal range
-    if (__float_as_uint(div.quick(x)) != __float_as_uint(ref)) ++bad;
+    float q0, q1;
+    div.quick2(-x, x, q0, q1);
+    if (__float_as_uint(q0) != __float_as_uint(ref) || __float_as_uint(q1) != (__float_as_uint(ref) ^ 0x80000000u)) ++bad;
   }
   if (bad) atomicAdd(bad_out, bad);
 }
@@ -355,7 +416,7 @@ cudaError_t launch_quantiser_selfcheck(int mode, int n_divisors, uint32_t seed, 
 cudaError_t launch_prep(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                         cudaStream_t st, int *launches, bool pool) {
   dim3 grid(p.Rt, p.BH);
-  const size_t smem = 3 * (size_t)kSlots * (p.d + 8) * 2 + 3 * kSfAtomBytes;
+  const size_t smem = (size_t)kSlots * (2 * (p.d + 8) + p.d) * 2 + (2 * (p.d / 64) + 1) * kSfAtomBytes;
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
