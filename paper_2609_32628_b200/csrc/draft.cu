@@ -8,65 +8,88 @@
 // scores by 1e-4.  It is a small GEMM: 4*R*R*d flops per head, against 4*64*64*d flops per retained block pair in
 // the attention kernel.
 // The plain fp64 pipe sustains about half of what the fp64 tensor-core path does on this part, so the products run as
-// mma.sync m8n8k4 (fp64 in, fp64 accumulate): 128 x 64 output tile per CTA, 32 x 32 per warp (4 x 4 fragments), K
-// panels of 16 channels in shared memory.  The descriptors are widened to fp64 once, when a panel is staged.
+// mma.sync m8n8k4 (fp64 in, fp64 accumulate): 64 x 64 output tile per CTA of four warps, 32 x 32 per warp (4 x 4
+// fragments).  Both operand tiles are requested at once, as fp32 and for all channels (64 KB at d = 128), by asynchronous
+// copies in groups of 32 channels: the first products start when the first group is there, and with three CTAs an SM the
+// loads of one hide behind the products of the others.  Fragments are widened to fp64 as they are read (8 conversions for
+// 16 products of 15 cycles each).  64 x 64 tiles instead of 128 x 64 give small maps (a few hundred blocks, a few heads)
+// enough CTAs to fill the GPU evenly.
 #include "da2_internal.cuh"
 
 namespace da2 {
 
 namespace {
 
-constexpr int TM = 128, TN = 64, TK = 16;
-constexpr int LDA = TM + 4, LDB = TN + 4;  // row strides = 4 mod 16 doubles: the 16 lanes of a half warp hit 16 bank pairs
+constexpr int TILE = 64, TK = 32, kChunk = 128;  // channels per copy group, channels staged at a time
 
 __device__ __forceinline__ void dmma(double (&c)[2], double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
                : "+d"(c[0]), "+d"(c[1])
                : "d"(a), "d"(b));
 }
+__device__ __forceinline__ void copy16(uint32_t dst, const float *src, bool valid) {  // zeros where not valid
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+template <int N> __device__ __forceinline__ void copies_left() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-__global__ void __launch_bounds__(256) draft_logits_kernel(Params p) {
+__global__ void __launch_bounds__(128) draft_logits_kernel(Params p) {
+  extern __shared__ __align__(16) float dsm[];
+  const int d = p.d, ld = min(d, kChunk) + 4;  // row stride = 4 mod 32 words: the 8 rows x 4 channels of a fragment hit 32 banks
+  float *As = dsm, *Bs = dsm + TILE * ld;  // [block][channel]
   const int which = blockIdx.z & 1, bh = blockIdx.z >> 1;
-  const float *__restrict__ Qd = p.desc[which] + (size_t)bh * p.R * p.d;       // Qavg or Qmax
-  const float *__restrict__ Kd = p.desc[2 + which] + (size_t)bh * p.R * p.d;   // Kavg or Kmax
+  const float *__restrict__ Qd = p.desc[which] + (size_t)bh * p.R * d;       // Qavg or Qmax
+  const float *__restrict__ Kd = p.desc[2 + which] + (size_t)bh * p.R * d;   // Kavg or Kmax
   float *__restrict__ out = p.logits[which] + (size_t)bh * p.R * p.R;
-  const int a0 = blockIdx.y * TM, b0 = blockIdx.x * TN;
-  __shared__ __align__(16) double As[TK][LDA];  // [channel][query block]
-  __shared__ __align__(16) double Bs[TK][LDB];  // [channel][key block]
+  const int a0 = blockIdx.y * TILE, b0 = blockIdx.x * TILE;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = (warp & 3) * 32, wn = (warp >> 2) * 32;  // warp tile origin inside the CTA tile
+  const uint32_t as = (uint32_t)__cvta_generic_to_shared(As), bs = (uint32_t)__cvta_generic_to_shared(Bs);
+
+  const int wm = (warp & 1) * 32, wn = (warp >> 1) * 32;  // warp tile origin inside the CTA tile
   const int fr = lane >> 2, fc = lane & 3;                // fragment row (or column of B) and channel inside a k4 step
+  const bool live = a0 + wm < p.R && b0 + wn < p.R;
   double acc[4][4][2];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
-
-  // loader mapping: 64 rows x 16 channels = 256 float4 quarters -> one float4 per thread per 64 rows
-  const int lr = tid >> 2, lc = (tid & 3) * 4;
-  for (int c0 = 0; c0 < p.d; c0 += TK) {
-    float4 xa0 = make_float4(0.f, 0.f, 0.f, 0.f), xa1 = xa0, xb = xa0;
-    if (a0 + lr < p.R) xa0 = *reinterpret_cast<const float4 *>(Qd + (size_t)(a0 + lr) * p.d + c0 + lc);
-    if (a0 + 64 + lr < p.R) xa1 = *reinterpret_cast<const float4 *>(Qd + (size_t)(a0 + 64 + lr) * p.d + c0 + lc);
-    if (b0 + lr < p.R) xb = *reinterpret_cast<const float4 *>(Kd + (size_t)(b0 + lr) * p.d + c0 + lc);
-    __syncthreads();
-    As[lc + 0][lr] = xa0.x; As[lc + 1][lr] = xa0.y; As[lc + 2][lr] = xa0.z; As[lc + 3][lr] = xa0.w;
-    As[lc + 0][64 + lr] = xa1.x; As[lc + 1][64 + lr] = xa1.y; As[lc + 2][64 + lr] = xa1.z; As[lc + 3][64 + lr] = xa1.w;
-    Bs[lc + 0][lr] = xb.x; Bs[lc + 1][lr] = xb.y; Bs[lc + 2][lr] = xb.z; Bs[lc + 3][lr] = xb.w;
-    __syncthreads();
+  // 64 rows x 8 quarters of four channels per operand and group: 4 + 4 copies per thread
+  const int lc = (tid & 7) * 4, lr = tid >> 3;
+  for (int base = 0; base < d; base += kChunk) {
+    const int n = min(kChunk, d - base), groups = (n + TK - 1) / TK;
+    if (base > 0) __syncthreads();
+    for (int g = 0; g < groups; ++g) {
+      const int c = g * TK + lc;
+      if (c < n) {
 #pragma unroll
-    for (int k4 = 0; k4 < TK; k4 += 4) {
-      double af[4], bf[4];
+        for (int i = 0; i < TILE; i += 16) {
+          const int a = a0 + lr + i, b = b0 + lr + i;
+          copy16(as + ((lr + i) * ld + c) * 4, Qd + (size_t)min(a, p.R - 1) * d + base + c, a < p.R);
+          copy16(bs + ((lr + i) * ld + c) * 4, Kd + (size_t)min(b, p.R - 1) * d + base + c, b < p.R);
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int g = 0; g < groups; ++g) {
+      const int left = groups - 1 - g;
+      if (left >= 3) copies_left<3>(); else if (left == 2) copies_left<2>(); else if (left == 1) copies_left<1>(); else copies_left<0>();
+      __syncthreads();
+      if (!live) continue;
+      const int c1 = min(n, (g + 1) * TK);
+#pragma unroll 2
+      for (int c = g * TK; c < c1; c += 4) {
+        double af[4], bf[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) af[i] = As[k4 + fc][wm + i * 8 + fr];
+        for (int i = 0; i < 4; ++i) af[i] = (double)As[(wm + i * 8 + fr) * ld + c + fc];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bf[j] = Bs[k4 + fc][wn + j * 8 + fr];
+        for (int j = 0; j < 4; ++j) bf[j] = (double)Bs[(wn + j * 8 + fr) * ld + c + fc];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) dmma(acc[i][j], af[i], bf[j]);
+          for (int j = 0; j < 4; ++j) dmma(acc[i][j], af[i], bf[j]);
+      }
     }
   }
+  if (!live) return;
   // accumulator fragment: row = lane / 4, columns 2 * (lane % 4) and + 1
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -84,8 +107,13 @@ __global__ void __launch_bounds__(256) draft_logits_kernel(Params p) {
 }  // namespace
 
 cudaError_t launch_draft(const Params &p, cudaStream_t st, int *launches) {
-  dim3 grid((p.R + TN - 1) / TN, (p.R + TM - 1) / TM, p.BH * 2);
-  draft_logits_kernel<<<grid, 256, 0, st>>>(p);
+  const dim3 grid((p.R + TILE - 1) / TILE, (p.R + TILE - 1) / TILE, p.BH * 2);
+  const int smem = 2 * TILE * ((p.d < kChunk ? p.d : kChunk) + 4) * (int)sizeof(float);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+  }
+  draft_logits_kernel<<<grid, 128, smem, st>>>(p);
   *launches += 1;
   return cudaGetLastError();
 }

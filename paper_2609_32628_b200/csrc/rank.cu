@@ -9,7 +9,8 @@
 // non-negative, so bit patterns order like values) finds the boundary score and how many entries equal to it are
 // still admitted; equal entries are admitted in index order through a prefix count.
 //
-// ROW scope: one CTA per (row, head) does everything.  HEAD scope (Alg. 1 as printed, one ranking over all R*R
+// ROW scope: one warp per (row, head) does everything while the row fits its registers (rank_warp_kernel), else one CTA.
+// HEAD scope (Alg. 1 as printed, one ranking over all R*R
 // pairs of a head): the same steps split into small kernels with per-head histograms in the workspace.
 #include "da2_internal.cuh"
 
@@ -18,6 +19,7 @@ namespace da2 {
 namespace {
 
 constexpr int NT = 256;
+constexpr int kRowWarps = 4;  // rows per CTA where a warp takes a row
 
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
@@ -158,7 +160,142 @@ __device__ __forceinline__ int tier_of(uint32_t key, const Boundary *bd, const i
   return -1;
 }
 
-// ---------------------------------------------------------------------------------------------- ROW scope
+// ------------------------------------------------------------------------------ one warp per row, row in registers
+// Lane l holds entries 32 e + l, e < E.  The boundary scores are found by bisection on the bit patterns between the row's
+// smallest and largest score; a step costs two instructions per register and one warp reduction, and a step whose count
+// hits the quota exactly ends the search (about log2(R) + 2 steps; only ties need all of them).  No barrier and no shared
+// memory: the CTA version spends 32 barriers a row, and its 12 histogram passes three times the instructions
+// (R = 1260, two boundaries).
+struct Cut { int value, take; };  // admitted: keys above value, and the first `take` keys equal to it
+
+template <int E> __device__ __forceinline__ int count_at_least(const int (&key)[E], int t) {
+  int n = 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) n += key[e] >= t;
+  return (int)__reduce_add_sync(0xffffffffu, (unsigned)n);
+}
+
+// RANK: ranking and lists (ROW scope); otherwise the draft map rows only
+template <int E, bool RANK>
+__global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
+  const int lane = threadIdx.x & 31, a = blockIdx.x * kRowWarps + (threadIdx.x >> 5), bh = blockIdx.y, R = p.R;
+  if (a >= R) return;
+  const size_t row = ((size_t)bh * R + a) * R;
+  const float *l0 = p.logits[0] + row, *l1 = p.logits[1] + row;
+  float x0[E], x1[E];
+  float m0 = -INFINITY, m1 = -INFINITY;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = e * 32 + lane;
+    x0[e] = i < R ? l0[i] : -INFINITY;
+    x1[e] = i < R ? l1[i] : -INFINITY;
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) { m0 = fmaxf(m0, x0[e]); m1 = fmaxf(m1, x1[e]); }
+  m0 = warp_max(m0);
+  m1 = warp_max(m1);
+  float z0 = 0.f, z1 = 0.f;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    x0[e] = expf(x0[e] - m0);
+    x1[e] = expf(x1[e] - m1);
+    z0 += x0[e];
+    z1 += x1[e];
+  }
+  const float c0 = __fdiv_rn(1.0f - p.lambda, warp_sum(z0)), c1 = __fdiv_rn(p.lambda, warp_sum(z1));
+  float *mp = p.map + row;
+  int key[E];  // scores are non-negative: their bit patterns order like integers; -1 beyond the row
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = e * 32 + lane;
+    const float s = fmaf(x0[e], c0, x1[e] * c1);
+    key[e] = i < R ? __float_as_int(s) : -1;
+    if (i < R) mp[i] = s;
+  }
+  if (!RANK) return;
+
+  int kmin = 0x7fffffff, kmax = -1;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    kmax = max(kmax, key[e]);
+    kmin = min(kmin, key[e] < 0 ? 0x7fffffff : key[e]);
+  }
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  Cut cut[3];  // cumulative: 16-bit, 16 + 8, 16 + 8 + 4
+  int cum = 0, top = kmax + 1, above = 0;  // keys >= top: `above` of them, fewer than any boundary still to come
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    const int c = cum + (int)p.quota[2 - t];
+    if (c <= 0) { cut[t].value = 0x7fffffff; cut[t].take = 0; }
+    else if (c >= R) { cut[t].value = -1; cut[t].take = 0; }
+    else if (t > 0 && c == cum) cut[t] = cut[t - 1];
+    else {
+      int lo = kmin, hi = top, n_hi = above;  // count(>= lo) >= c > count(>= hi)
+      cut[t].take = -1;
+#pragma unroll 1
+      while (hi - lo > 1) {
+        const int mid = lo + ((hi - lo) >> 1);
+        const int n = count_at_least(key, mid);
+        if (n == c) { cut[t].value = mid - 1; cut[t].take = 0; top = mid; above = n; break; }
+        if (n > c) lo = mid; else { hi = mid; n_hi = n; }
+      }
+      if (cut[t].take < 0) {  // entries tie at the boundary: the lower indices among them
+        cut[t].value = lo;
+        cut[t].take = c - n_hi;
+        top = hi;
+        above = n_hi;
+      }
+    }
+    cum = c;
+  }
+
+  uint16_t *ids = p.ids + (size_t)bh * p.ids_per_head + (size_t)a * p.row_stride;
+  const unsigned below = (1u << lane) - 1u;
+  const int k4 = (int)p.quota[0], k8 = (int)p.quota[1], k16 = (int)p.quota[2];
+  int pos4 = 0, pos8 = k4, pos16 = k4 + k8;
+  int eq0 = 0, eq1 = 0, eq2 = 0;  // keys equal to each boundary so far
+  const bool ties = cut[0].take > 0 || cut[1].take > 0 || cut[2].take > 0;
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    bool in16 = key[e] > cut[0].value, in8 = key[e] > cut[1].value, in4 = key[e] > cut[2].value;
+    if (ties) {
+      const unsigned q0 = __ballot_sync(0xffffffffu, key[e] == cut[0].value), q1 = __ballot_sync(0xffffffffu, key[e] == cut[1].value),
+                     q2 = __ballot_sync(0xffffffffu, key[e] == cut[2].value);
+      in16 |= ((q0 >> lane) & 1u) && eq0 + __popc(q0 & below) < cut[0].take;
+      in8 |= ((q1 >> lane) & 1u) && eq1 + __popc(q1 & below) < cut[1].take;
+      in4 |= ((q2 >> lane) & 1u) && eq2 + __popc(q2 & below) < cut[2].take;
+      eq0 += __popc(q0); eq1 += __popc(q1); eq2 += __popc(q2);
+    }
+    const unsigned b16 = __ballot_sync(0xffffffffu, in16), b8 = __ballot_sync(0xffffffffu, in8) & ~b16,
+                   b4 = __ballot_sync(0xffffffffu, in4) & ~(b16 | b8);
+    const unsigned mine = ((b16 >> lane) & 1u) ? b16 : (((b8 >> lane) & 1u) ? b8 : b4);
+    const int base = ((b16 >> lane) & 1u) ? pos16 : (((b8 >> lane) & 1u) ? pos8 : pos4);
+    if ((mine >> lane) & 1u) ids[base + __popc(mine & below)] = (uint16_t)(e * 32 + lane);
+    pos16 += __popc(b16); pos8 += __popc(b8); pos4 += __popc(b4);
+  }
+  // prefix interactions lie outside the budget: every video row keeps all prefix blocks, in the 16-bit segment
+  for (int j = lane; j < p.Rp; j += 32) ids[k4 + k8 + k16 + j] = (uint16_t)(R + j);
+  if (lane == 0)
+    *reinterpret_cast<int4 *>(p.counts + ((size_t)bh * p.Rt + a) * 4) = make_int4(k4, k8, k16 + p.Rp, a * p.row_stride);
+}
+
+// registers per lane that hold a row of R entries, 0 where they would be too many
+template <bool RANK> bool launch_rank_warp(const Params &p, cudaStream_t st) {
+  const dim3 grid((p.R + kRowWarps - 1) / kRowWarps, p.BH);
+  auto go = [&](auto kernel) { kernel<<<grid, kRowWarps * 32, 0, st>>>(p); return true; };
+  const int e = (p.R + 31) / 32;
+  if (e <= 2) return go(rank_warp_kernel<2, RANK>);
+  if (e <= 5) return go(rank_warp_kernel<5, RANK>);
+  if (e <= 10) return go(rank_warp_kernel<10, RANK>);
+  if (e <= 19) return go(rank_warp_kernel<19, RANK>);
+  if (e <= 28) return go(rank_warp_kernel<28, RANK>);
+  if (e <= 40) return go(rank_warp_kernel<40, RANK>);
+  if (e <= 64) return go(rank_warp_kernel<64, RANK>);
+  return false;
+}
+
+// ---------------------------------------------------------------------------------------------- ROW scope, long rows
 __global__ void __launch_bounds__(NT) rank_row_kernel(Params p) {
   extern __shared__ uint32_t dyn[];
   uint32_t *keys = dyn;  // [R]
@@ -416,6 +553,10 @@ __global__ void __launch_bounds__(NT) head_emit_kernel(Params p, int mode) {
 // Draft map rows only (softmax of both logit branches and their mixture into p.map); used by callers that want
 // the map without the ranking.
 cudaError_t launch_map_rows(const Params &p, cudaStream_t st, int *launches) {
+  if (launch_rank_warp<false>(p, st)) {
+    *launches += 1;
+    return cudaGetLastError();
+  }
   dim3 grid(p.R, p.BH);
   const size_t smem = (size_t)p.R * sizeof(uint32_t);
   if (smem > 48 * 1024) {
@@ -432,6 +573,10 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
   const size_t smem = (size_t)p.R * sizeof(uint32_t);
   cudaError_t e;
   if (p.rank_scope == DA2_RANK_ROW) {
+    if (launch_rank_warp<true>(p, st)) {
+      *launches += 1;
+      return cudaGetLastError();
+    }
     if (smem > 48 * 1024) {
       e = cudaFuncSetAttribute(rank_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
@@ -440,15 +585,14 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
     *launches += 1;
     return cudaGetLastError();
   }
+  e = launch_map_rows(p, st, launches);
+  if (e != cudaSuccess) return e;
   if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(head_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(head_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  head_map_kernel<<<grid, NT, smem, st>>>(p);
   head_init_kernel<<<p.BH, NT, 0, st>>>(p);
-  *launches += 2;
+  *launches += 1;
   for (int shift = 24; shift >= 0; shift -= 8) {
     head_hist_kernel<<<grid, NT, 0, st>>>(p, shift);
     head_pick_kernel<<<p.BH, 96, 0, st>>>(p, shift);
