@@ -80,7 +80,8 @@ constexpr float kOffsetP8 = 8.807f;      // base-2 exponent offset (about log2 4
 // (a parity wait can only tell the latest completion from the one before, so every barrier is laid out such that no
 // waiter can fall two completions behind: buffers indexed by step parity get one barrier per buffer)
 constexpr int kMaxK = 6, kMaxV = 8, kInfoRing = 16;  // (steps between a K request and its scores: at most nk + 2)
-constexpr int kStepBars = 8;  // barriers for the steps of a stream between softmax and product (kSets of them unless SEGMENTED)
+// barriers, factors, ballots and scale atoms of the steps between softmax and product (kSets of them unless SEGMENTED)
+constexpr int kStepBars = 8;
 enum {
   B_FULLK = 0, B_KFREE = B_FULLK + kMaxK, B_FULLV = B_KFREE + kMaxK, B_VFREE = B_FULLV + kMaxV, B_SREADY = B_VFREE + kMaxV,
   B_SFREE = B_SREADY + kSets, B_PREADY = B_SFREE + 2, B_CORROK = B_PREADY + kStepBars, B_PVDONE = B_CORROK + kStepBars,
@@ -99,7 +100,7 @@ struct SmemMap {
   uint32_t kstage[3], vstage[3];  // bytes per ring entry
   int nk[3], nv[3];               // ring entries
   uint32_t p[2];                  // P operand images per stream
-  uint32_t pbytes[3];             // bytes of a P slot (there are four, or SEGMENTED 8, 4, 2)
+  uint32_t pbytes[3];             // bytes of a P slot (there are four, or SEGMENTED 4, 4, 2)
   uint32_t sfp[2];    // P scale atoms (512 B), one per step barrier
   uint32_t factor;    // float [2 streams][kStepBars][64]
   uint32_t hx;        // {float h, int step} [2][sets][64]: running maximum after a step, handed from thread to thread
@@ -445,10 +446,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     for (int i = set; i < S.L; i += kSets) {
       const int tier = S.tier(i);
       const int g = SEGMENTED ? i & kStepMask : set;  // barriers, factors, ballots, scale atom
-      // the step's P slot, and the product that last used it (SEGMENTED: at the start of a segment, the last product of the
-      // segment before, whose slots were cut differently)
-      const int seg0 = tier == 0 ? 0 : (tier == 1 ? S.n4 : S.n48), pm = SEGMENTED ? 7 >> tier : kMask;
-      uint8_t *prow = p_row0 + (SEGMENTED ? ((i - seg0) & pm) << (11 + tier) : set * sm.pbytes[0]);
+      // the step's P slot, and the product that last used it: step i - 4, or i - 2 in the 16-bit segment of a SEGMENTED plan,
+      // where the first steps of every segment also wait for the last product of the segment before, whose slots were cut
+      // differently.  (A parity wait for product b must find the barrier's previous use, b - kStepBars, complete: the set's
+      // step before, i - 4, has waited for product i - 8 at least, and b - 8 <= i - 9.)
+      const int seg0 = tier == 0 ? 0 : (tier == 1 ? S.n4 : S.n48), pm = SEGMENTED && tier == 2 ? 1 : kMask;
+      uint8_t *prow = p_row0 + (SEGMENTED ? (set & pm) << (11 + tier) : set * sm.pbytes[0]);
       const int busy = SEGMENTED && i - seg0 <= pm ? seg0 - 1 : i - 1 - pm;
       const uint32_t s_col = tmem + lane_addr + col_s(s, i & 1);
       if (!wait_or_abort(bar(s, B_SREADY + set), (i >> kShift) & 1, abortp)) break;
@@ -877,7 +880,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const uint64_t pd0 = tc::smem_desc(tc::smem_u32(smem + sm.p[s]), 1024, 128);
       const uint64_t sfpd0 = tc::smem_desc(tc::smem_u32(smem + sm.sfp[s]), 128, 128);
       const uint32_t t_sfv = tmem + col_sfv(s), t_sfp = tmem + col_sfp(s), t_o = tmem + col_o(s);
-      int vv = 0, nv = sm.nv[0], pp = 0, pm = 0;  // V ring entry and depth; SEGMENTED: P slot and number of slots - 1
+      int vv = 0, nv = sm.nv[0], pm = kMask;  // V ring entry and depth; number of P slots - 1
       uint32_t vpar = 0;                          // parity of the next use (SEGMENTED: a bit per ring entry)
       uint32_t vstep = sm.vstage[0] >> 4, pstep = sm.pbytes[0] >> 4;
       for (int j = 0; j < S.L; ++j) {
@@ -888,8 +891,8 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           vstep = sm.vstage[t] >> 4;
           nv = sm.nv[t];
           pstep = sm.pbytes[t] >> 4;
-          pm = 7 >> t;
-          vv = 0; pp = 0;
+          pm = t == 2 ? 1 : kMask;
+          vv = 0;
         }
         if (!wait_or_abort(bar(s, B_FULLV + vv), SEGMENTED ? (vpar >> vv) & 1u : vpar, abortp)) break;
         if (SEGMENTED) vpar ^= 1u << vv;
@@ -897,7 +900,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         if (!wait_or_abort(bar(s, B_CORROK + g), (j >> kStepShift) & 1, abortp)) break;
         tc::fence_after_sync();
         const uint64_t vd = vd0 + (uint64_t)(vv * vstep);
-        const uint64_t pdg = pd0 + (uint64_t)((SEGMENTED ? pp : g) * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
+        const uint64_t pdg = pd0 + (uint64_t)((g & pm) * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
         const uint32_t acc = j > 0;
         if (tc::elect_one()) {
           if (B16 && j >= S.n48) {
@@ -918,7 +921,6 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         }
         __syncwarp();
         if (++vv == nv) { vv = 0; if (!SEGMENTED) vpar ^= 1u; }
-        if (SEGMENTED) pp = (pp + 1) & pm;
       }
     }
   }

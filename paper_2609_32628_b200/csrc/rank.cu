@@ -175,6 +175,34 @@ template <int E> __device__ __forceinline__ int count_at_least(const int (&key)[
   return (int)__reduce_add_sync(0xffffffffu, (unsigned)n);
 }
 
+// Sum of a row, in the order of the CTA version (256 threads, entry i with thread i mod 256), so that the scores, and with
+// them the ties among scores that round to the same bits, do not depend on which version ranks a row.
+template <int E> __device__ __forceinline__ float row_sum(const float (&x)[E]) {
+  float r = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w >= E) break;
+    float v = 0.f;
+#pragma unroll
+    for (int e = w; e < E; e += 8) v += x[e];
+    r += warp_sum(v);
+  }
+  return r;
+}
+
+// x / z, correctly rounded, for 0 <= x <= 1 <= z: reciprocal and two corrections by the exact residual (Markstein's theorem:
+// the first brings the quotient within one unit in the last place, the second rounds it) where nothing can underflow, else
+// the division itself
+struct Quotient {
+  float z, r;
+  __device__ __forceinline__ float of(float x) const {
+    if (x < 7.8886091e-31f) return __fdiv_rn(x, z);  // 2^-100
+    float q = __fmul_rn(x, r);
+    q = __fmaf_rn(__fmaf_rn(-q, z, x), r, q);
+    return __fmaf_rn(__fmaf_rn(-q, z, x), r, q);
+  }
+};
+
 // RANK: ranking and lists (ROW scope); otherwise the draft map rows only
 template <int E, bool RANK>
 __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
@@ -194,21 +222,20 @@ __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
   for (int e = 0; e < E; ++e) { m0 = fmaxf(m0, x0[e]); m1 = fmaxf(m1, x1[e]); }
   m0 = warp_max(m0);
   m1 = warp_max(m1);
-  float z0 = 0.f, z1 = 0.f;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     x0[e] = expf(x0[e] - m0);
     x1[e] = expf(x1[e] - m1);
-    z0 += x0[e];
-    z1 += x1[e];
   }
-  const float c0 = __fdiv_rn(1.0f - p.lambda, warp_sum(z0)), c1 = __fdiv_rn(p.lambda, warp_sum(z1));
+  const float z0 = row_sum(x0), z1 = row_sum(x1);
+  const Quotient d0 = {z0, __frcp_rn(z0)}, d1 = {z1, __frcp_rn(z1)};
+  const float w0 = 1.0f - p.lambda, w1 = p.lambda;
   float *mp = p.map + row;
   int key[E];  // scores are non-negative: their bit patterns order like integers; -1 beyond the row
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int i = e * 32 + lane;
-    const float s = fmaf(x0[e], c0, x1[e] * c1);
+    const float s = w0 * d0.of(x0[e]) + w1 * d1.of(x1[e]);
     key[e] = i < R ? __float_as_int(s) : -1;
     if (i < R) mp[i] = s;
   }

@@ -1,0 +1,64 @@
+"""Sizes at which a kernel's split of the work changes: row lengths around the register budgets of the ranking, blocks per
+head around the pooling splits, lists whose segments are shorter or longer than the rings and slots they run through.
+
+Bars as in test_gpu_parity.py (its checks are used): descriptors, codes, scales and lists exact, outputs within the bf16
+tolerance of the oracle.
+"""
+import numpy as np
+import pytest
+import torch
+
+import da2_inputs
+import paper_2609_32628_b200 as da2
+from helpers import oracle_all, run_gpu
+from test_gpu_parity import _check_attention, _check_prepare
+
+pytestmark = pytest.mark.gpu
+W = da2_inputs.Workload
+
+
+# R = T * tiles on either side of 64, 160, 320, 608, 896, 1280 and 2048 entries per row (2, 5, 10, 19, 28, 40 and 64 per
+# lane; longer rows are ranked by a whole thread block), and the smallest rows there are
+@pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (1, 9, 8), (4, 32, 32), (13, 8, 40), (32, 8, 40), (23, 8, 56), (107, 8, 24),
+                                     (29, 24, 56), (23, 24, 104), (61, 24, 56), (128, 32, 32), (683, 8, 24)])
+def test_row_lengths(T, Hg, Wg):
+    w = W("rows", 1, 1, 64, T, Hg, Wg, 0.0, 0.10, 0.20, seed=31)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v)
+    ref = oracle_all(w, q, k, v)
+    bad = _check_prepare(w, plan, ws, ref)
+    R = plan.info.R
+    sel = [(0, a) for a in sorted({0, R // 2, R - 1})]
+    if sum(int(x) for x in plan.info.quota):
+        _check_attention(w, out, ref, sel, bad)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("f16,f8,f4", [(0.15, 0.25, 0.30), (0.15, 0.25, 0.0), (0.15, 0.0, 0.30), (0.02, 0.03, 0.30),
+                                       (0.30, 0.02, 0.02), (0.4, 0.0, 0.0)])
+def test_segments_of_three_tiers(d, f16, f8, f4):
+    """Many heads at once (the order in which warps meet varies), segments of 1 to 23 blocks: bit-identical over repeated
+    runs, and equal to the oracle on sampled blocks."""
+    w = W("segments", 1, 21, d, 5, 23, 40, f16, f8, f4, seed=32, k_outlier_channels=(3, 35), k_outlier_gain=5.0)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v)
+    again = torch.empty_like(out)
+    for _ in range(4):
+        again.fill_(float("nan"))
+        da2.da2_attention_fwd(plan, q, k, v, ws, again)
+        assert torch.equal(out, again)
+    heads = [0, 20]
+    ref = oracle_all(w, q, k, v, heads=heads)
+    bad = _check_prepare(w, plan, ws, ref, heads=heads)
+    sel = [(h, int(a)) for h in range(2) for a in np.random.default_rng(3).choice(plan.info.R, 10, replace=False)]
+    _check_attention(w, out, ref, sel, bad, heads=heads)
+
+
+@pytest.mark.parametrize("H", [1, 8, 30])
+def test_pooling_splits(H):
+    """80 blocks a head: eight, four and one warp per block."""
+    w = W("pool", 1, H, 128, 5, 27, 30, 0.1, 0.2, 0.2, seed=33)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, _ = run_gpu(w, q, k, v)
+    heads = sorted({0, H - 1})
+    _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
