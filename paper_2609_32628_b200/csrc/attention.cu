@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   const int R = p.R, Rt = p.Rt, pairs = (Rt + 1) / 2;
   const int bh = blockIdx.x / pairs, pr = blockIdx.x % pairs;
   __nv_bfloat16 *out_head = out + (size_t)bh * p.Ntot * D;
+  grid_wait();
   // the two query blocks of this CTA: equally long rows of the head (scheduling order written with the lists)
   int a0 = 2 * pr, a1 = 2 * pr + 1;
   if (ORDERED) {
@@ -1083,8 +1084,7 @@ cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t s
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm.total);
     if (err != cudaSuccess) return err;
-    kernel<<<grid, NT, sm.total, st>>>(p, sm, out);
-    return cudaSuccess;
+    return launch_chained(kernel, grid, NT, sm.total, st, p, sm, out);
   };
   const bool ordered = p.rank_scope != 0, fp4 = p.tier_active[0] != 0;
   auto pick = [&](auto dtag, auto stag) -> cudaError_t {

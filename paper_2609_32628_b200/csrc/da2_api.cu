@@ -160,6 +160,8 @@ constexpr int kScaleChunk = 256;
 struct ScaleChunk { float v[kScaleChunk]; };
 __global__ void set_gscale_kernel(float *gscale, int which, int first, int n, ScaleChunk c) {
   const int i = threadIdx.x;
+  da2::grid_trigger();
+  da2::grid_wait();
   if (i < n) gscale[(size_t)(first + i) * 4 + which] = c.v[i];
 }
 
@@ -318,19 +320,20 @@ da2_status_t prepare_impl(const da2_plan_t *plan, const void *q, const void *k, 
       ScaleChunk c;
       const int n = p.BH - first < kScaleChunk ? p.BH - first : kScaleChunk;
       std::memcpy(c.v, plan->g_host[i] + first, sizeof(float) * (size_t)n);
-      set_gscale_kernel<<<1, kScaleChunk, 0, st>>>(p.gscale, i, first, n, c);
-      if (cudaGetLastError() != cudaSuccess) return DA2_ERR_CUDA;
+      if (da2::launch_chained(set_gscale_kernel, dim3(1), kScaleChunk, 0, st, p.gscale, i, first, n, c) != cudaSuccess)
+        return DA2_ERR_CUDA;
       launches += 1;
     }
   }
+  // operands beside the draft logits, which they do not depend on; then the ranking
+  if (select && da2::launch_draft(p, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
+  if (da2::launch_prep(p, qb, kb, vb, st, &launches, /*pool=*/false, /*beside_draft=*/select) != cudaSuccess) return DA2_ERR_CUDA;
   if (select) {
-    if (da2::launch_draft(p, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
     if (da2::launch_rank(p, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
     if (da2::launch_prefix_rows(p, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
     // rows of unequal length (HEAD scope) are paired by length; with per-row budgets the order is the identity
     if (plan->info.rank_scope != 0 && da2::launch_order(p, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   }
-  if (da2::launch_prep(p, qb, kb, vb, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   t_last_launches = launches;
   return DA2_OK;
 }

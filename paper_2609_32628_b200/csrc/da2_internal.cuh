@@ -106,6 +106,29 @@ __host__ __device__ inline long long slot_token(const Params &p, int a, int j) {
 // operand records per head and tier: the 16-bit tier also holds the prefix blocks
 __host__ __device__ inline int rec_blocks(const Params &p, int tier) { return tier == 2 ? p.Rt : p.R; }
 
+// Programmatic dependent launch: a kernel of the chain may be scheduled as soon as every block of the kernel before it has
+// called grid_trigger() (all of them do so at their start), so that launch latency and set-up overlap that kernel's last
+// blocks; grid_wait() then waits until the kernel before has completed and its writes are visible.  Every block of every
+// kernel calls grid_wait() once, before it ends, so a kernel's completion implies that of all kernels before it.
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... KArgs, class... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+#endif
+
 // kernel launchers (each returns the cudaError_t of its launch)
 cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                         cudaStream_t st, int *launches);
@@ -115,7 +138,7 @@ cudaError_t launch_map_rows(const Params &p, cudaStream_t st, int *launches);
 cudaError_t launch_order(const Params &p, cudaStream_t st, int *launches);
 cudaError_t launch_prefix_rows(const Params &p, cudaStream_t st, int *launches);
 cudaError_t launch_prep(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
-                        cudaStream_t st, int *launches, bool pool = false);
+                        cudaStream_t st, int *launches, bool pool = false, bool beside_draft = false);
 cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t st, int *launches);
 cudaError_t launch_bounded_wait_probe(int *status, long long limit_cycles, cudaStream_t st);
 cudaError_t launch_quantiser_selfcheck(int mode, int n_divisors, uint32_t seed, unsigned long long *out, cudaStream_t st);

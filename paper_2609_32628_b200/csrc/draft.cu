@@ -52,6 +52,8 @@ __global__ void __launch_bounds__(128) draft_logits_kernel(Params p) {
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
+  grid_wait();
+  grid_trigger();  // only now: what runs beside this kernel may rely on the kernels before it
   // 64 rows x 8 quarters of four channels per operand and group: 4 + 4 copies per thread
   const int lc = (tid & 7) * 4, lr = tid >> 3;
   for (int base = 0; base < d; base += kChunk) {
@@ -113,7 +115,8 @@ cudaError_t launch_draft(const Params &p, cudaStream_t st, int *launches) {
     const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  draft_logits_kernel<<<grid, 128, smem, st>>>(p);
+  const cudaError_t e = launch_chained(draft_logits_kernel, grid, 128, smem, st, p);
+  if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();
 }

@@ -54,6 +54,8 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
   const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int a = blockIdx.x * BLOCKS + warp / SPLIT, part = warp % SPLIT;
   const bool live = a < p.R;
+  grid_trigger();
+  grid_wait();
 
   double sq[2 * W], sk[2 * W];
   uint32_t mq[W], mk[W], av[W], aq = 0, ak = 0;
@@ -196,9 +198,11 @@ cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bflo
   const dim3 grid((p.R * split + kPoolWarps - 1) / kPoolWarps, p.BH);
   const uint16_t *q16 = reinterpret_cast<const uint16_t *>(q), *k16 = reinterpret_cast<const uint16_t *>(k),
                  *v16 = reinterpret_cast<const uint16_t *>(v);
-  auto launch = [&](auto kernel) { kernel<<<grid, kPoolWarps * 32, 0, st>>>(p, q16, k16, v16); };
-  if (p.d == 128) split == 1 ? launch(pool_kernel<128, 1>) : (split == 4 ? launch(pool_kernel<128, 4>) : launch(pool_kernel<128, 8>));
-  else split == 1 ? launch(pool_kernel<64, 1>) : (split == 4 ? launch(pool_kernel<64, 4>) : launch(pool_kernel<64, 8>));
+  auto launch = [&](auto kernel) { return launch_chained(kernel, grid, kPoolWarps * 32, 0, st, p, q16, k16, v16); };
+  cudaError_t e;
+  if (p.d == 128) e = split == 1 ? launch(pool_kernel<128, 1>) : (split == 4 ? launch(pool_kernel<128, 4>) : launch(pool_kernel<128, 8>));
+  else e = split == 1 ? launch(pool_kernel<64, 1>) : (split == 4 ? launch(pool_kernel<64, 4>) : launch(pool_kernel<64, 8>));
+  if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();
 }

@@ -140,8 +140,12 @@ __device__ __forceinline__ uint32_t nvfp4_group(const uint32_t (&nw)[8], float g
 template <int D, bool POOL>
 __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat16 *__restrict__ q,
                                                   const __nv_bfloat16 *__restrict__ k,
-                                                  const __nv_bfloat16 *__restrict__ v) {
+                                                  const __nv_bfloat16 *__restrict__ v, bool beside_draft) {
   extern __shared__ __align__(16) uint8_t smem[];
+  // beside_draft: the kernel before is the draft-logits kernel, which this one does not depend on; its blocks have waited
+  // for the pooling kernel before they let this kernel start.  So the two overlap, and the wait comes at the end.
+  grid_trigger();
+  if (!beside_draft) grid_wait();
   // Q, K: rows padded by 16 bytes, so that threads that read the same channels of consecutive slots fall on different
   // banks.  V: the 64-byte halves of a 128-byte line are swapped in every other group of 16 rows, so that the two groups a
   // warp reads at a time fall on different banks.
@@ -263,7 +267,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       }
     }
     if (t4) {  // chunk (kc, r): channels kc*32.. of slot r
-      const float g = p.gscale[bh * 4 + which], g6 = __fmul_rn(6.0f, g);
+      const float g = __ldcg(&p.gscale[bh * 4 + which]), g6 = __fmul_rn(6.0f, g);
       uint32_t c[4], sc[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -323,7 +327,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       }
     }
     if (t8) {  // chunk (c, ch): slots c*16.. of channel ch (padding slots hold +0: code 0)
-      const float2 dv = *reinterpret_cast<const float2 *>(p.dv8 + (size_t)bh * D + 2 * pair);
+      const float2 dv = __ldcg(reinterpret_cast<const float2 *>(p.dv8 + (size_t)bh * D + 2 * pair));
       uint4 mine[2], both[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -341,7 +345,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       *reinterpret_cast<uint4 *>(dst + D * 16) = both[1];
     }
     if (t4) {  // chunk (gh, ch): slots gh*32.. of channel ch
-      const float gv = p.gscale[bh * 4 + 2], g6 = __fmul_rn(6.0f, gv);
+      const float gv = __ldcg(&p.gscale[bh * 4 + 2]), g6 = __fmul_rn(6.0f, gv);
       uint2 mine[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -366,6 +370,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(sf_img + i * 16);
     }
   }
+  if (beside_draft) grid_wait();
 }
 
 // Self-check of Divider::quick2 and round_half_away against the IEEE division and roundf (see da2.h).
@@ -414,14 +419,13 @@ cudaError_t launch_quantiser_selfcheck(int mode, int n_divisors, uint32_t seed, 
 }
 
 cudaError_t launch_prep(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
-                        cudaStream_t st, int *launches, bool pool) {
+                        cudaStream_t st, int *launches, bool pool, bool beside_draft) {
   dim3 grid(p.Rt, p.BH);
   const size_t smem = (size_t)kSlots * (2 * (p.d + 8) + p.d) * 2 + (2 * (p.d / 64) + 1) * kSfAtomBytes;
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<grid, NT, smem, st>>>(p, q, k, v);
-    return cudaGetLastError();
+    return launch_chained(kernel, grid, NT, smem, st, p, q, k, v, beside_draft);
   };
   cudaError_t e;
   if (p.d == 128) e = pool ? launch(prep_kernel<128, true>) : launch(prep_kernel<128, false>);

@@ -5,13 +5,13 @@
 // Output per query-block row: key-block ids grouped in execution order NVFP4 | INT8 | BF16 (Sec. 3.3 "Phased
 // execution"), ascending inside a group, plus the three counts and the row's offset in its head's id array.
 //
-// Exact top-k without sorting: for each tier boundary a 4-pass radix select on the fp32 bit patterns (scores are
-// non-negative, so bit patterns order like values) finds the boundary score and how many entries equal to it are
-// still admitted; equal entries are admitted in index order through a prefix count.
+// Exact top-k without sorting: for each tier boundary a search on the fp32 bit patterns (scores are non-negative, so bit
+// patterns order like values) finds the boundary score and how many entries equal to it are still admitted; equal
+// entries are admitted in index order through a prefix count.
 //
 // ROW scope: one warp per (row, head) does everything while the row fits its registers (rank_warp_kernel), else one CTA.
-// HEAD scope (Alg. 1 as printed, one ranking over all R*R
-// pairs of a head): the same steps split into small kernels with per-head histograms in the workspace.
+// HEAD scope (Alg. 1 as printed, one ranking over all R*R pairs of a head): small kernels with per-head histograms in the
+// workspace.
 #include "da2_internal.cuh"
 
 namespace da2 {
@@ -67,7 +67,7 @@ __device__ void draft_map_row(const Params &p, int bh, int a, uint32_t *keys, fl
   z1 = block_sum(z1, red);
   const float w0 = 1.0f - p.lambda, w1 = p.lambda;
   for (int i = threadIdx.x; i < p.R; i += NT) {
-    const float s = w0 * __fdiv_rn(expf(l0[i] - m0), z0) + w1 * __fdiv_rn(expf(l1[i] - m1), z1);
+    const float s = __fmaf_rn(w0, __fdiv_rn(expf(l0[i] - m0), z0), __fmul_rn(w1, __fdiv_rn(expf(l1[i] - m1), z1)));
     keys[i] = __float_as_uint(s);
     mp[i] = s;
   }
@@ -207,6 +207,8 @@ struct Quotient {
 template <int E, bool RANK>
 __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
   const int lane = threadIdx.x & 31, a = blockIdx.x * kRowWarps + (threadIdx.x >> 5), bh = blockIdx.y, R = p.R;
+  grid_trigger();
+  grid_wait();
   if (a >= R) return;
   const size_t row = ((size_t)bh * R + a) * R;
   const float *l0 = p.logits[0] + row, *l1 = p.logits[1] + row;
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int i = e * 32 + lane;
-    const float s = w0 * d0.of(x0[e]) + w1 * d1.of(x1[e]);
+    const float s = __fmaf_rn(w0, d0.of(x0[e]), __fmul_rn(w1, d1.of(x1[e])));
     key[e] = i < R ? __float_as_int(s) : -1;
     if (i < R) mp[i] = s;
   }
@@ -310,7 +312,14 @@ __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
 // registers per lane that hold a row of R entries, 0 where they would be too many
 template <bool RANK> bool launch_rank_warp(const Params &p, cudaStream_t st) {
   const dim3 grid((p.R + kRowWarps - 1) / kRowWarps, p.BH);
-  auto go = [&](auto kernel) { kernel<<<grid, kRowWarps * 32, 0, st>>>(p); return true; };
+  // Chained to the kernel before only where the rows are few: there it hides the launch (2 us of 33 for the smallest call);
+  // waiting blocks of a large grid hold registers the kernel before still wants (1.8 us of 27 for two heads of 588 rows).
+  const bool chained = (long long)p.R * p.BH <= 512;
+  auto go = [&](auto kernel) {
+    if (chained) launch_chained(kernel, grid, kRowWarps * 32, 0, st, p);
+    else kernel<<<grid, kRowWarps * 32, 0, st>>>(p);
+    return true;
+  };
   const int e = (p.R + 31) / 32;
   if (e <= 2) return go(rank_warp_kernel<2, RANK>);
   if (e <= 5) return go(rank_warp_kernel<5, RANK>);
@@ -333,6 +342,8 @@ __global__ void __launch_bounds__(NT) rank_row_kernel(Params p) {
   __shared__ Boundary bd[3];
   const int a = blockIdx.x, bh = blockIdx.y, R = p.R;
 
+  grid_trigger();
+  grid_wait();
   draft_map_row(p, bh, a, keys, red);
 
   // cumulative boundaries: 16-bit, 16+8, 16+8+4
@@ -397,6 +408,8 @@ __global__ void __launch_bounds__(NT) rank_row_kernel(Params p) {
 // Prefix query rows are not sparse (App. C.1): their list is every block of the head, video and prefix, 16-bit.
 __global__ void __launch_bounds__(NT) prefix_rows_kernel(Params p) {
   const int j = blockIdx.x, bh = blockIdx.y, a = p.R + j;
+  grid_trigger();
+  grid_wait();
   const int pstride = (p.Rt + 7) / 8 * 8;
   const int off = p.R * p.row_stride + j * pstride;
   uint16_t *ids = p.ids + (size_t)bh * p.ids_per_head + off;
@@ -407,172 +420,222 @@ __global__ void __launch_bounds__(NT) prefix_rows_kernel(Params p) {
   }
 }
 
+__global__ void __launch_bounds__(NT) head_map_kernel(Params p) {
+  extern __shared__ uint32_t dyn[];
+  __shared__ float red[NT / 32];
+  grid_trigger();
+  grid_wait();
+  draft_map_row(p, blockIdx.y, blockIdx.x, dyn, red);
+}
+
 // --------------------------------------------------------------------------------------------- HEAD scope
-// select scratch per head (uint32): [0..11]  (prefix, mask, need, pad) x 3 boundaries
-//                                   [16..16+768) histograms 3 x 256
-//                                   [1024..1024+3R) per-row equal counts -> exclusive prefixes
-//                                   [1024+3R..1024+7R) per-row tier counts (3) + row total -> offsets
+// Three radix passes (11, 10 and 10 bits of the 31 that a non-negative score has) narrow the three boundary scores of a
+// head; the first digit spreads the scores over 8 bins an octave, after it only the entries in a boundary's bin count at
+// all.  A CTA counts a share of the head's R*R scores in shared memory, and the last CTA of the head picks the bins.  Then
+// a warp per row counts, one CTA per head turns counts into offsets, and a warp per row writes its list.
+//
+// select scratch per head (uint32): [0..11]  (value or prefix, take or need, mode, pad) x 3 boundaries   [12] ticket
+//                                   [16..16+2048) histogram of pass 0; [16..16+3072) 3 x 1024 of passes 1 and 2
+//                                   [4096..4096+3R) per row and boundary: equal scores -> equal scores in earlier rows
+//                                   [4096+3R..4096+6R) higher scores
+constexpr int kBins0 = 2048, kBins = 1024;
 __device__ __forceinline__ uint32_t *sel_base(const Params &p, int bh) {
   return p.select + (size_t)bh * (4096 + 8 * (size_t)p.R);
 }
 
-__global__ void __launch_bounds__(NT) head_map_kernel(Params p) {
-  extern __shared__ uint32_t dyn[];
-  __shared__ float red[NT / 32];
-  draft_map_row(p, blockIdx.y, blockIdx.x, dyn, red);
-}
-
-__global__ void head_init_kernel(Params p) {
+__global__ void __launch_bounds__(NT) head_init_kernel(Params p) {
+  grid_trigger();
+  grid_wait();
   uint32_t *s = sel_base(p, blockIdx.x);
   const long long M = (long long)p.R * p.R;
   if (threadIdx.x < 3) {
     long long cum = 0;
     for (int t = 0; t <= (int)threadIdx.x; ++t) cum += p.quota[2 - t];
     uint32_t *b = s + threadIdx.x * 4;
-    // b[3]: 0 = select normally, 1 = nothing admitted, 2 = everything admitted
-    b[0] = 0; b[1] = 0; b[2] = (uint32_t)cum; b[3] = cum <= 0 ? 1u : (cum >= M ? 2u : 0u);
+    // mode: 0 = select normally, 1 = nothing admitted, 2 = everything admitted
+    const uint32_t mode = cum <= 0 ? 1u : (cum >= M ? 2u : 0u);
+    b[0] = mode == 1 ? 0xffffffffu : 0u;
+    b[1] = mode == 1 ? 0u : (mode == 2 ? 0xffffffffu : (uint32_t)cum);
+    b[2] = mode;
   }
-  for (int i = threadIdx.x; i < 768; i += blockDim.x) s[16 + i] = 0;
+  if (threadIdx.x == 12) s[12] = 0;
+  for (int i = threadIdx.x; i < 3 * kBins; i += NT) s[16 + i] = 0;
 }
 
-__global__ void __launch_bounds__(NT) head_hist_kernel(Params p, int shift) {
-  __shared__ uint32_t h[3][256];
-  const int a = blockIdx.x, bh = blockIdx.y;
-  uint32_t *s = sel_base(p, bh);
-  for (int i = threadIdx.x; i < 768; i += NT) (&h[0][0])[i] = 0;
-  __syncthreads();
-  const uint32_t pf[3] = {s[0], s[4], s[8]}, mk[3] = {s[1], s[5], s[9]};
-  const uint32_t *keys = reinterpret_cast<const uint32_t *>(p.map + ((size_t)bh * p.R + a) * p.R);
-  for (int i = threadIdx.x; i < p.R; i += NT) {
-    const uint32_t key = keys[i];
+// The bin that holds the need-th largest of a histogram's candidates (N bins, one warp): out[0] = bin, out[1] = need minus
+// the count above the bin.
+template <int N> __device__ void pick_bin_of(const uint32_t *hist, uint32_t need, uint32_t *out) {
+  const int lane = threadIdx.x & 31;
+  constexpr int PER = N / 32;
+  uint32_t local = 0;
+#pragma unroll 8
+  for (int i = 0; i < PER; ++i) local += __ldcg(&hist[N - 1 - (lane * PER + i)]);
+  uint32_t incl = local;
 #pragma unroll
-    for (int t = 0; t < 3; ++t)
-      if ((key & mk[t]) == pf[t]) atomicAdd(&h[t][(key >> shift) & 255u], 1u);
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
   }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 768; i += NT) {
-    const uint32_t c = (&h[0][0])[i];
-    if (c) atomicAdd(&s[16 + i], c);
+  uint32_t above = incl - local;  // candidates in higher bins than this lane's
+  if (above < need && need <= incl) {
+    for (int i = 0; i < PER; ++i) {
+      const uint32_t c = __ldcg(&hist[N - 1 - (lane * PER + i)]);
+      if (need <= above + c) { out[0] = N - 1 - (lane * PER + i); out[1] = need - above; break; }
+      above += c;
+    }
   }
 }
 
-__global__ void head_pick_kernel(Params p, int shift) {
+template <int PASS>
+__global__ void __launch_bounds__(NT) head_hist_kernel(Params p) {
+  constexpr int BINS = PASS == 0 ? kBins0 : 3 * kBins, SHIFT = PASS == 0 ? 20 : (PASS == 1 ? 10 : 0);
+  __shared__ uint32_t h[BINS];
   __shared__ uint32_t out[3][2];
-  uint32_t *s = sel_base(p, blockIdx.x);
-  const int t = threadIdx.x >> 5;  // 3 warps, one per boundary
-  if (t < 3) {
-    if (s[t * 4 + 3] == 0) pick_bin(s + 16 + t * 256, s[t * 4 + 2], out[t]);
-  }
-  __syncthreads();
-  if (threadIdx.x < 3 && s[threadIdx.x * 4 + 3] == 0) {
-    uint32_t *b = s + threadIdx.x * 4;
-    b[0] |= out[threadIdx.x][0] << shift;
-    b[1] |= 255u << shift;
-    b[2] = out[threadIdx.x][1];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 768; i += blockDim.x) s[16 + i] = 0;
-}
-
-__device__ __forceinline__ void load_boundaries(const uint32_t *s, int R, Boundary *bd) {
-  for (int t = 0; t < 3; ++t) {
-    const uint32_t mode = s[t * 4 + 3];
-    if (mode == 1) { bd[t].value = 0xffffffffu; bd[t].take = 0; }
-    else if (mode == 2) { bd[t].value = 0u; bd[t].take = 0xffffffffu; }
-    else { bd[t].value = s[t * 4]; bd[t].take = s[t * 4 + 2]; }
-  }
-  (void)R;
-}
-
-// per-row counts of entries equal to each boundary score
-__global__ void __launch_bounds__(NT) head_eqcount_kernel(Params p) {
-  __shared__ int scratch[3 * NT + 8];
-  const int a = blockIdx.x, bh = blockIdx.y;
+  __shared__ bool s_last;
+  const int bh = blockIdx.y, tid = threadIdx.x;
   uint32_t *s = sel_base(p, bh);
-  Boundary bd[3];
-  load_boundaries(s, p.R, bd);
-  const uint32_t *keys = reinterpret_cast<const uint32_t *>(p.map + ((size_t)bh * p.R + a) * p.R);
-  int eq[3] = {0, 0, 0}, tot[3];
-  for (int i = threadIdx.x; i < p.R; i += NT) {
+  for (int i = tid; i < BINS; i += NT) h[i] = 0;
+  grid_trigger();
+  grid_wait();
+  __syncthreads();
+  const size_t M = (size_t)p.R * p.R, share = (M + gridDim.x - 1) / gridDim.x;
+  const size_t lo = min(M, share * blockIdx.x), hi = min(M, lo + share);
+  const uint32_t *keys = reinterpret_cast<const uint32_t *>(p.map) + (size_t)bh * M;
+  const uint32_t pf[3] = {s[0] >> (SHIFT + 10), s[4] >> (SHIFT + 10), s[8] >> (SHIFT + 10)};
+  const bool on[3] = {s[2] == 0u, s[6] == 0u, s[10] == 0u};
+#pragma unroll 4
+  for (size_t i = lo + tid; i < hi; i += NT) {
+    const uint32_t key = __ldg(&keys[i]);
+    if (PASS == 0) {
+      atomicAdd(&h[key >> 20], 1u);
+    } else {
+#pragma unroll
+      for (int t = 0; t < 3; ++t)
+        if (on[t] && (key >> (SHIFT + 10)) == pf[t]) atomicAdd(&h[t * kBins + ((key >> SHIFT) & (kBins - 1))], 1u);
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < BINS; i += NT)
+    if (h[i]) atomicAdd(&s[16 + i], h[i]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = atomicAdd(&s[12], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int t = tid >> 5;  // 3 warps, one per boundary
+  if (t < 3 && s[t * 4 + 2] == 0u) {
+    if (PASS == 0) pick_bin_of<kBins0>(s + 16, s[t * 4 + 1], out[t]);
+    else pick_bin_of<kBins>(s + 16 + t * kBins, s[t * 4 + 1], out[t]);
+  }
+  __syncthreads();
+  if (tid < 3 && s[tid * 4 + 2] == 0u) {
+    s[tid * 4] |= out[tid][0] << SHIFT;
+    s[tid * 4 + 1] = out[tid][1];
+  }
+  if (tid == 12) s[12] = 0;
+  if (PASS < 2)
+    for (int i = tid; i < 3 * kBins; i += NT) s[16 + i] = 0;
+}
+
+// one warp per row: entries equal to, and above, each boundary score
+__global__ void __launch_bounds__(kRowWarps * 32) head_count_kernel(Params p) {
+  const int lane = threadIdx.x & 31, a = blockIdx.x * kRowWarps + (threadIdx.x >> 5), bh = blockIdx.y, R = p.R;
+  grid_trigger();
+  grid_wait();
+  if (a >= R) return;
+  uint32_t *s = sel_base(p, bh);
+  const uint32_t v[3] = {s[0], s[4], s[8]};
+  const uint32_t *keys = reinterpret_cast<const uint32_t *>(p.map + ((size_t)bh * R + a) * R);
+  int eq[3] = {0, 0, 0}, gt[3] = {0, 0, 0};
+#pragma unroll 4
+  for (int i = lane; i < R; i += 32) {
     const uint32_t key = keys[i];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) eq[t] += key == bd[t].value;
+    for (int t = 0; t < 3; ++t) { eq[t] += key == v[t]; gt[t] += key > v[t]; }
   }
-  block_scan<3>(eq, tot, scratch);
-  if (threadIdx.x < 3) s[1024 + threadIdx.x * p.R + a] = (uint32_t)tot[threadIdx.x];
-}
-
-// exclusive prefix over rows of `narr` arrays of length R stored back to back at s[base...]; totals dropped
-__global__ void __launch_bounds__(NT) head_rowscan_kernel(Params p, int base_words, int narr) {
-  __shared__ int scratch[1 * NT + 8];
-  uint32_t *s = sel_base(p, blockIdx.x) + base_words;
-  const int per = (p.R + NT - 1) / NT;
-  for (int arr = 0; arr < narr; ++arr) {
-    uint32_t *x = s + (size_t)arr * p.R;
-    const int lo = min(p.R, (int)threadIdx.x * per), hi = min(p.R, lo + per);
-    int v[1] = {0}, tot[1];
-    for (int i = lo; i < hi; ++i) v[0] += (int)x[i];
-    block_scan<1>(v, tot, scratch);
-    int run = v[0];
-    for (int i = lo; i < hi; ++i) { const int c = (int)x[i]; x[i] = (uint32_t)run; run += c; }
-    __syncthreads();
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    const unsigned e = __reduce_add_sync(0xffffffffu, (unsigned)eq[t]), g = __reduce_add_sync(0xffffffffu, (unsigned)gt[t]);
+    if (lane == 0) { s[4096 + t * R + a] = e; s[4096 + (3 + t) * R + a] = g; }
   }
 }
 
-// mode 0: count the row's entries per tier; mode 1: emit ids at the row's offset
-__global__ void __launch_bounds__(NT) head_emit_kernel(Params p, int mode) {
-  extern __shared__ uint32_t dyn[];
-  uint32_t *keys = dyn;
+// of `eq` entries equal to a boundary score, after `before` of them in earlier rows, those among the first `take`
+__device__ __forceinline__ int admitted(uint32_t take, int before, int eq) {
+  return take > (uint32_t)before ? (int)min(take - (uint32_t)before, (uint32_t)eq) : 0;
+}
+
+// one CTA per head: counts of a row per tier, its offset, and the equal scores in earlier rows
+__global__ void __launch_bounds__(NT) head_offsets_kernel(Params p) {
   __shared__ int scratch[3 * NT + 8];
-  const int a = blockIdx.x, bh = blockIdx.y, R = p.R;
-  uint32_t *s = sel_base(p, bh);
-  Boundary bd[3];
-  load_boundaries(s, R, bd);
-  const uint32_t *gk = reinterpret_cast<const uint32_t *>(p.map + ((size_t)bh * R + a) * R);
-  for (int i = threadIdx.x; i < R; i += NT) keys[i] = gk[i];
-  __syncthreads();
-  const int per = (R + NT - 1) / NT;
-  const int lo = min(R, (int)threadIdx.x * per), hi = min(R, lo + per);
+  const int bh = blockIdx.x, R = p.R;
+  grid_trigger();
+  grid_wait();
+  uint32_t *s = sel_base(p, bh), *eqs = s + 4096, *gts = s + 4096 + 3 * R;
+  const uint32_t take[3] = {s[1], s[5], s[9]};
+  const int per = (R + NT - 1) / NT, lo = min(R, (int)threadIdx.x * per), hi = min(R, lo + per);
   int eq[3] = {0, 0, 0}, tot[3];
-  for (int i = lo; i < hi; ++i) {
+  for (int a = lo; a < hi; ++a)
 #pragma unroll
-    for (int t = 0; t < 3; ++t) eq[t] += keys[i] == bd[t].value;
-  }
+    for (int t = 0; t < 3; ++t) eq[t] += (int)eqs[t * R + a];
   block_scan<3>(eq, tot, scratch);
+  int run[3] = {eq[0], eq[1], eq[2]}, len[1] = {0}, total[1];
+  for (int a = lo; a < hi; ++a) {
+    int c[3];
 #pragma unroll
-  for (int t = 0; t < 3; ++t) eq[t] += (int)s[1024 + t * R + a];  // equal entries in earlier rows of the head
-  int cnt[3] = {0, 0, 0};
-  {
-    int er[3] = {eq[0], eq[1], eq[2]};
-    for (int i = lo; i < hi; ++i) {
-      const int tr = tier_of(keys[i], bd, er);
-      if (tr >= 0) ++cnt[tr];
-#pragma unroll
-      for (int t = 0; t < 3; ++t) er[t] += keys[i] == bd[t].value;
+    for (int t = 0; t < 3; ++t) {
+      const int e = (int)eqs[t * R + a];
+      c[t] = (int)gts[t * R + a] + admitted(take[t], run[t], e);
+      eqs[t * R + a] = (uint32_t)run[t];
+      run[t] += e;
     }
+    len[0] += c[2];
+    *reinterpret_cast<int4 *>(p.counts + ((size_t)bh * R + a) * 4) = make_int4(c[2] - c[1], c[1] - c[0], c[0], 0);
   }
-  int pos[3] = {cnt[0], cnt[1], cnt[2]};
-  block_scan<3>(pos, tot, scratch);
-  uint32_t *rowtot = s + 1024 + 3 * R;  // [R] totals -> offsets after the row scan
-  if (mode == 0) {
-    if (threadIdx.x == 0) {
-      int *c = p.counts + ((size_t)bh * R + a) * 4;
-      c[0] = tot[0]; c[1] = tot[1]; c[2] = tot[2];
-      rowtot[a] = (uint32_t)(tot[0] + tot[1] + tot[2]);
-    }
-    return;
+  block_scan<1>(len, total, scratch);
+  int off = len[0];
+  for (int a = lo; a < hi; ++a) {
+    int *c = p.counts + ((size_t)bh * R + a) * 4;
+    c[3] = off;
+    off += c[0] + c[1] + c[2];
   }
-  const uint32_t off = rowtot[a];
-  uint16_t *ids = p.ids + (size_t)bh * p.ids_per_head + off;
-  const int base[3] = {0, tot[0], tot[0] + tot[1]};
-  int er[3] = {eq[0], eq[1], eq[2]};
-  for (int i = lo; i < hi; ++i) {
-    const int tr = tier_of(keys[i], bd, er);
-    if (tr >= 0) { ids[base[tr] + pos[tr]] = (uint16_t)i; ++pos[tr]; }
+}
+
+// one warp per row: the row's list
+__global__ void __launch_bounds__(kRowWarps * 32) head_emit_kernel(Params p) {
+  const int lane = threadIdx.x & 31, a = blockIdx.x * kRowWarps + (threadIdx.x >> 5), bh = blockIdx.y, R = p.R;
+  grid_trigger();
+  grid_wait();
+  if (a >= R) return;
+  const uint32_t *s = sel_base(p, bh);
+  const uint32_t v[3] = {s[0], s[4], s[8]}, take[3] = {s[1], s[5], s[9]};
+  int before[3];
 #pragma unroll
-    for (int t = 0; t < 3; ++t) er[t] += keys[i] == bd[t].value;
+  for (int t = 0; t < 3; ++t) before[t] = (int)s[4096 + t * R + a];
+  const int4 c = *reinterpret_cast<const int4 *>(p.counts + ((size_t)bh * R + a) * 4);
+  uint16_t *ids = p.ids + (size_t)bh * p.ids_per_head + c.w;
+  int pos4 = 0, pos8 = c.x, pos16 = c.x + c.y;
+  const uint32_t *keys = reinterpret_cast<const uint32_t *>(p.map + ((size_t)bh * R + a) * R);
+  const unsigned below = (1u << lane) - 1u;
+#pragma unroll 4
+  for (int i0 = 0; i0 < R; i0 += 32) {
+    const int i = i0 + lane;
+    const uint32_t key = i < R ? keys[i] : 0u;
+    bool in[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const unsigned q = __ballot_sync(0xffffffffu, i < R && key == v[t]);
+      in[t] = i < R && (key > v[t] || (((q >> lane) & 1u) && (uint32_t)(before[t] + __popc(q & below)) < take[t]));
+      before[t] += __popc(q);
+    }
+    const unsigned b16 = __ballot_sync(0xffffffffu, in[0]), b8 = __ballot_sync(0xffffffffu, in[1]) & ~b16,
+                   b4 = __ballot_sync(0xffffffffu, in[2]) & ~(b16 | b8);
+    const unsigned mine = ((b16 >> lane) & 1u) ? b16 : (((b8 >> lane) & 1u) ? b8 : b4);
+    const int base = ((b16 >> lane) & 1u) ? pos16 : (((b8 >> lane) & 1u) ? pos8 : pos4);
+    if ((mine >> lane) & 1u) ids[base + __popc(mine & below)] = (uint16_t)i;
+    pos16 += __popc(b16); pos8 += __popc(b8); pos4 += __popc(b4);
   }
-  if (threadIdx.x == 0) p.counts[((size_t)bh * R + a) * 4 + 3] = (int)off;
 }
 
 }  // namespace
@@ -590,7 +653,7 @@ cudaError_t launch_map_rows(const Params &p, cudaStream_t st, int *launches) {
     cudaError_t e = cudaFuncSetAttribute(head_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  head_map_kernel<<<grid, NT, smem, st>>>(p);
+  launch_chained(head_map_kernel, grid, NT, smem, st, p);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -608,29 +671,23 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
       e = cudaFuncSetAttribute(rank_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    rank_row_kernel<<<grid, NT, smem, st>>>(p);
+    launch_chained(rank_row_kernel, grid, NT, smem, st, p);
     *launches += 1;
     return cudaGetLastError();
   }
   e = launch_map_rows(p, st, launches);
   if (e != cudaSuccess) return e;
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(head_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  head_init_kernel<<<p.BH, NT, 0, st>>>(p);
-  *launches += 1;
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    head_hist_kernel<<<grid, NT, 0, st>>>(p, shift);
-    head_pick_kernel<<<p.BH, 96, 0, st>>>(p, shift);
-    *launches += 2;
-  }
-  head_eqcount_kernel<<<grid, NT, 0, st>>>(p);
-  head_rowscan_kernel<<<p.BH, NT, 0, st>>>(p, 1024, 3);
-  head_emit_kernel<<<grid, NT, smem, st>>>(p, 0);
-  head_rowscan_kernel<<<p.BH, NT, 0, st>>>(p, 1024 + 3 * p.R, 1);
-  head_emit_kernel<<<grid, NT, smem, st>>>(p, 1);
-  *launches += 5;
+  // about eight CTAs an SM share the scores of all heads; a share is at least one pass of the CTA's threads
+  const long long M = (long long)p.R * p.R, most = (M + 4 * NT - 1) / (4 * NT), fair = (148 * 8 + p.BH - 1) / p.BH;
+  const dim3 shares((unsigned)(most < fair ? most : fair), p.BH), rows((p.R + kRowWarps - 1) / kRowWarps, p.BH);
+  launch_chained(head_init_kernel, p.BH, NT, 0, st, p);
+  launch_chained(head_hist_kernel<0>, shares, NT, 0, st, p);
+  launch_chained(head_hist_kernel<1>, shares, NT, 0, st, p);
+  launch_chained(head_hist_kernel<2>, shares, NT, 0, st, p);
+  launch_chained(head_count_kernel, rows, kRowWarps * 32, 0, st, p);
+  launch_chained(head_offsets_kernel, p.BH, NT, 0, st, p);
+  launch_chained(head_emit_kernel, rows, kRowWarps * 32, 0, st, p);
+  *launches += 7;
   return cudaGetLastError();
 }
 
@@ -640,27 +697,37 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
 namespace {
 __global__ void __launch_bounds__(256) order_rows_kernel(Params p) {
   extern __shared__ int s_len[];
-  const int bh = blockIdx.x, R = p.R, Rp = 2 * ((R + 1) / 2);
-  const int *cnt = p.counts + (size_t)bh * R * 4;
-  for (int a = threadIdx.x; a < R; a += blockDim.x) s_len[a] = cnt[a * 4] + cnt[a * 4 + 1] + cnt[a * 4 + 2];
+  const int bh = blockIdx.y, R = p.R, Rp = 2 * ((R + 1) / 2);
+  grid_trigger();
+  grid_wait();
+  const int4 *cnt = reinterpret_cast<const int4 *>(p.counts + (size_t)bh * R * 4);
+  for (int a = threadIdx.x; a < R; a += 256) {
+    const int4 c = cnt[a];
+    s_len[a] = c.x + c.y + c.z;
+  }
   __syncthreads();
   uint16_t *ord = p.order + (size_t)bh * Rp;
-  if (threadIdx.x == 0 && Rp > R) ord[R] = 0xFFFFu;
-  for (int a = threadIdx.x; a < R; a += blockDim.x) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && Rp > R) ord[R] = 0xFFFFu;
+  // eight threads per row, each against an eighth of the others
+  const int a = blockIdx.x * 32 + (threadIdx.x >> 3), part = threadIdx.x & 7;
+  int pos = 0;
+  if (a < R) {
     const int la = s_len[a];
-    int pos = 0;
-    for (int b = 0; b < R; ++b) {
+#pragma unroll 4
+    for (int b = part; b < R; b += 8) {
       const int lb = s_len[b];
       pos += (lb > la) || (lb == la && b < a);
     }
-    ord[pos] = (uint16_t)a;
   }
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) pos += __shfl_xor_sync(0xffffffffu, pos, o);
+  if (a < R && part == 0) ord[pos] = (uint16_t)a;
 }
 }  // namespace
 
 cudaError_t launch_prefix_rows(const Params &p, cudaStream_t st, int *launches) {
   if (p.Rp == 0) return cudaSuccess;
-  prefix_rows_kernel<<<dim3(p.Rp, p.BH), NT, 0, st>>>(p);
+  launch_chained(prefix_rows_kernel, dim3(p.Rp, p.BH), NT, 0, st, p);
   *launches += 1;
   return cudaGetLastError();
 }
@@ -671,7 +738,7 @@ cudaError_t launch_order(const Params &p, cudaStream_t st, int *launches) {
     cudaError_t e = cudaFuncSetAttribute(order_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  order_rows_kernel<<<p.BH, 256, smem, st>>>(p);
+  launch_chained(order_rows_kernel, dim3((p.R + 31) / 32, p.BH), 256, smem, st, p);
   *launches += 1;
   return cudaGetLastError();
 }

@@ -62,3 +62,32 @@ def test_pooling_splits(H):
     plan, ws, _ = run_gpu(w, q, k, v)
     heads = sorted({0, H - 1})
     _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
+
+
+@pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (3, 9, 20), (13, 8, 40), (23, 24, 56), (683, 8, 24)])
+@pytest.mark.parametrize("f16,f8,f4", [(0.1, 0.2, 0.3), (0.0, 0.1, 0.2)])
+def test_head_scope_sizes(T, Hg, Wg, f16, f8, f4):
+    if T == 683 and f16:
+        pytest.skip("one budget is enough for the longest rows")
+    w = W("head", 1, 2, 64, T, Hg, Wg, f16, f8, f4, seed=34)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v, rank_scope=1)
+    ref = oracle_all(w, q, k, v, rank_scope=1)
+    bad = _check_prepare(w, plan, ws, ref)
+    R = plan.info.R
+    _check_attention(w, out, ref, [(h, a) for h in range(2) for a in sorted({0, R // 2, R - 1})], bad)
+
+
+@pytest.mark.parametrize("rank_scope", [0, 1])
+@pytest.mark.parametrize("T,Hg,Wg", [(2, 16, 16), (9, 24, 40), (2, 24, 352)])
+def test_ties_go_to_the_lower_index(T, Hg, Wg, rank_scope):
+    """Constant Q and K: every score of the map is the same, so every boundary is a tie (the bisection of a row and the
+    radix passes of a head run to their last bit)."""
+    w = W("ties", 1, 2, 64, T, Hg, Wg, 0.1, 0.2, 0.3, seed=35)
+    _, _, v = da2_inputs.make_qkv(w, "cuda")
+    q = torch.ones_like(v)
+    k = torch.ones_like(v)
+    plan, ws, out = run_gpu(w, q, k, v, rank_scope=rank_scope)
+    ref = oracle_all(w, q, k, v, rank_scope=rank_scope)
+    assert _check_prepare(w, plan, ws, ref) == []
+    _check_attention(w, out, ref, [(1, 0), (1, plan.info.R - 1)], [])
