@@ -472,16 +472,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         tc::tmem_ld16(s_col + 32, a2);
         tc::tmem_ld16(s_col + 48, a3);
         tc::wait_ld();
-        // int32 accumulators become floats exactly through a magic-number add and subtract (|S| < 2^22): two
-        // full-rate operations instead of a conversion on the special-function unit
+        // int32 accumulators (exact as floats: |S| < 2^22)
         if (tier == 1) {
-          const uint64_t moff = f2(-12582912.0f, -12582912.0f);
 #pragma unroll
-          for (int c = 0; c < 16; c += 2) {
-            unf2(add2(f2(__uint_as_float(a0[c] + 0x4B400000u), __uint_as_float(a0[c + 1] + 0x4B400000u)), moff), v[c], v[c + 1]);
-            unf2(add2(f2(__uint_as_float(a1[c] + 0x4B400000u), __uint_as_float(a1[c + 1] + 0x4B400000u)), moff), v[16 + c], v[17 + c]);
-            unf2(add2(f2(__uint_as_float(a2[c] + 0x4B400000u), __uint_as_float(a2[c + 1] + 0x4B400000u)), moff), v[32 + c], v[33 + c]);
-            unf2(add2(f2(__uint_as_float(a3[c] + 0x4B400000u), __uint_as_float(a3[c + 1] + 0x4B400000u)), moff), v[48 + c], v[49 + c]);
+          for (int c = 0; c < 16; ++c) {
+            v[c] = (float)(int)a0[c]; v[16 + c] = (float)(int)a1[c];
+            v[32 + c] = (float)(int)a2[c]; v[48 + c] = (float)(int)a3[c];
           }
         } else {
 #pragma unroll
