@@ -62,6 +62,7 @@ constexpr int kMmaWarp0 = kSoftmaxWarps + kCorrWarps;     // Q K^T issue for str
 constexpr int kPvWarp0 = kMmaWarp0 + 2;                   // V^T P^T issue for stream 0, 1
 constexpr int kLoadWarp0 = kPvWarp0 + 2;                  // K loaders for stream 0, 1, then V loaders
 constexpr int NT = (kLoadWarp0 + 4) * 32;                 // 1024
+constexpr int kSms = 148;
 constexpr uint32_t kTmemCols = 512;
 // TMEM column map
 __host__ __device__ constexpr uint32_t col_s(int s, int buf) { return (uint32_t)(s * 2 + buf) * 64u; }
@@ -112,11 +113,15 @@ struct SmemMap {
   uint32_t tok;       // int [2 streams][64]: token of each query slot, -1 at padding
   uint32_t chg;       // uint32 [2 streams][kStepBars][2]: ballots of the queries whose maximum moved this step
   uint32_t total;
+  int single;         // one query block per CTA: stream 1 has none
   bool fits;          // the layout fits the 227 KB a block may use
 };
 
 __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   SmemMap m;
+  // Where the query blocks of all heads are no more than the SMs, each gets a CTA of its own: the call lasts as long as one
+  // list, and a stream that has the SM to itself walks its list faster.
+  m.single = (long long)p.BH * p.Rt <= kSms;
   uint32_t cur = 0;
   auto r128 = [](uint32_t b) { return (b + 127u) / 128u * 128u; };
   auto take = [&](uint32_t bytes) { uint32_t o = cur; cur = r128(cur + bytes); return o; };
@@ -366,16 +371,16 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
-  const int R = p.R, Rt = p.Rt, pairs = (Rt + 1) / 2;
+  const int R = p.R, Rt = p.Rt, pairs = sm.single ? Rt : (Rt + 1) / 2;
   const int bh = blockIdx.x / pairs, pr = blockIdx.x % pairs;
   __nv_bfloat16 *out_head = out + (size_t)bh * p.Ntot * D;
   grid_wait();
   // the two query blocks of this CTA: equally long rows of the head (scheduling order written with the lists)
-  int a0 = 2 * pr, a1 = 2 * pr + 1;
+  int a0 = sm.single ? pr : 2 * pr, a1 = sm.single ? p.Rt : 2 * pr + 1;
   if (ORDERED) {
-    const uint16_t *ord = p.order + ((size_t)bh * pairs + pr) * 2;
-    a0 = ord[0];
-    a1 = ord[1];
+    const uint16_t *ord = p.order + (size_t)bh * ((Rt + 1) / 2) * 2;
+    a0 = ord[a0];
+    if (!sm.single) a1 = ord[a1];
   }
   const StreamInfo st0 = load_stream<ORDERED>(p, bh, a0), st1 = load_stream<ORDERED>(p, bh, a1);
   // the loaders' first ids, and the correction warps' table of query tokens, are on their way while the block is set up
@@ -955,10 +960,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const float *fac = s_factor + (s * kStepBars + g) * 64;
       // column groups (eight queries each) with a moved maximum; all of them when the segment changes.  Two groups
       // are in flight at a time: their loads are issued together, so a rescale costs one TMEM round trip per pair.
-      uint32_t todo = 0;
-#pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (tier_switch || (((c < 4 ? moved.x : moved.y) >> ((c & 3) * 8)) & 0xffu) != 0u) todo |= 1u << c;
+      uint32_t todo = 0xffu;
+      if (!tier_switch) {  // a bit per byte that is not zero: into the byte's top bit, then four of them gathered by a product
+        const uint32_t nx = (((moved.x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | moved.x) & 0x80808080u;
+        const uint32_t ny = (((moved.y & 0x7f7f7f7fu) + 0x7f7f7f7fu) | moved.y) & 0x80808080u;
+        todo = ((nx >> 7) * 0x10204080u >> 28) | (((ny >> 7) * 0x10204080u >> 28) << 4);
+      }
       if (!wait_or_abort(bar(s, B_PVDONE + ((i - 1) & kStepMask)), ((i - 1) >> kStepShift) & 1, abortp)) break;
       tc::fence_after_sync();
 #pragma unroll 1
@@ -971,7 +978,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         tc::tmem_ld8(tmem + lane_addr + col_o(s) + c0 * 8, o0);
         if (c1 >= 0) tc::tmem_ld8(tmem + lane_addr + col_o(s) + c1 * 8, o1);
         tc::wait_ld();
-scale8(o0, fac + c0 * 8, lane_factor);
+        scale8(o0, fac + c0 * 8, lane_factor);
         tc::tmem_st8(tmem + lane_addr + col_o(s) + c0 * 8, o0);
         if (c1 >= 0) {
           scale8(o1, fac + c1 * 8, lane_factor);
@@ -1076,7 +1083,7 @@ cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t s
   const SmemMap sm = make_smem_map(p, b16 && p.d == 128);
   if (!sm.fits) return cudaErrorInvalidConfiguration;
   cudaError_t e;
-  const int grid = p.BH * ((p.Rt + 1) / 2);
+  const int grid = p.BH * (sm.single ? p.Rt : (p.Rt + 1) / 2);
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm.total);
     if (err != cudaSuccess) return err;
