@@ -122,16 +122,21 @@ struct SmemMap {
   uint32_t tok;       // int [2 streams][64]: token of each query slot, -1 at padding
   uint32_t chg;       // uint32 [2 streams][kStepBars][2]: ballots of the queries whose maximum moved this step
   uint32_t total;
-  int single;         // one query block per CTA: stream 1 has none
+  int pair_ctas;      // CTAs with two query blocks; the CTAs after them have one each,
+  int first_single;   // from this one on (head * Rt + block): stream 1 has none
   bool fits;          // the layout fits the 227 KB a block may use
 };
 
 __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   SmemMap m;
-  // Where the query blocks of all heads are no more than the SMs, each gets a CTA of its own: the call lasts as long as one
-  // list, and a stream that has the SM to itself walks its list faster (1,024 tokens x 4 heads: 16.0 -> 14.0 us).  Above
-  // that line two blocks per CTA need fewer waves of CTAs.
-  m.single = (long long)p.BH * p.Rt <= kSms;
+  // Two query blocks per CTA, but one in the last wave of CTAs if its blocks are no more than the SMs: the wave lasts as long
+  // as one list, and a stream that has the SM to itself walks its list faster (calls of one such wave: 144 blocks of 144
+  // 4- and 8-bit entries 59.9 -> 52.6 us, the smallest call's 32 blocks 13.3 -> 12.5 us).
+  const int pairs = (p.Rt + 1) / 2, total = p.BH * pairs;
+  auto block_of = [&](int cta) { return cta / pairs * p.Rt + cta % pairs * 2; };
+  m.pair_ctas = total - total % kSms;
+  if (p.BH * p.Rt - block_of(m.pair_ctas) > kSms) m.pair_ctas = total;
+  m.first_single = block_of(m.pair_ctas);
   uint32_t cur = 0;
   auto r128 = [](uint32_t b) { return (b + 127u) / 128u * 128u; };
   auto take = [&](uint32_t bytes) { uint32_t o = cur; cur = r128(cur + bytes); return o; };
@@ -381,31 +386,35 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // warp-uniform by construction
-  const int R = p.R, Rt = p.Rt, pairs = sm.single ? Rt : (Rt + 1) / 2;
-  const int bh = blockIdx.x / pairs, pr = blockIdx.x % pairs;
+  const int R = p.R, Rt = p.Rt;
+  const bool single = (int)blockIdx.x >= sm.pair_ctas;
+  int bh, pr;
+  if (single) {
+    const int idx = (int)blockIdx.x + (sm.first_single - sm.pair_ctas);
+    bh = idx / Rt; pr = idx % Rt;
+  } else {
+    const int pairs = (Rt + 1) / 2;
+    bh = blockIdx.x / pairs; pr = blockIdx.x % pairs;
+  }
   __nv_bfloat16 *out_head = out + (size_t)bh * p.Ntot * D;
   grid_wait();
-  // the two query blocks of this CTA: equally long rows of the head (scheduling order written with the lists)
-  int a0 = sm.single ? pr : 2 * pr, a1 = sm.single ? p.Rt : 2 * pr + 1;
+  // this warp's stream and its query block: block 2 pr or 2 pr + 1, or that entry of the scheduling order (equally long rows
+  // of the head)
+  const int stream = warp < kSoftmaxWarps ? (warp & 3) >> 1 : (warp < kMmaWarp0 ? (warp - kSoftmaxWarps) >> 2 : warp & 1);
+  int a = single ? (stream ? Rt : pr) : 2 * pr + stream;
   if (ORDERED) {
-    const uint16_t *ord = p.order + (size_t)bh * ((Rt + 1) / 2) * 2;
-    a0 = ord[a0];
-    if (!sm.single) a1 = ord[a1];
+    if (a < Rt) a = p.order[(size_t)bh * ((Rt + 1) / 2) * 2 + a];
   }
-  const StreamInfo st0 = load_stream<ORDERED>(p, bh, a0), st1 = load_stream<ORDERED>(p, bh, a1);
+  StreamInfo S = load_stream<ORDERED>(p, bh, a);
   // the loaders' first ids, and the correction warps' table of query tokens, are on their way while the block is set up
-  const int pre_s = warp >= kLoadWarp0 ? (warp - kLoadWarp0) & 1 : (warp - kSoftmaxWarps) >> 2;
-  const int pre_a = pre_s ? st1.a : st0.a;
   int pre0 = 0, pre1 = 0;
   if (warp >= kLoadWarp0) {
-    const uint16_t *ids = pre_s ? st1.ids : st0.ids;
-    const int L = pre_s ? st1.L : st0.L;
-    if (lane < L) pre0 = ids[lane];
-    if (32 + lane < L) pre1 = ids[32 + lane];
-  } else if (warp >= kSoftmaxWarps && warp < kMmaWarp0 && (warp & 3) < 2 && pre_a >= 0) {
+    if (lane < S.L) pre0 = S.ids[lane];
+    if (32 + lane < S.L) pre1 = S.ids[32 + lane];
+  } else if (warp >= kSoftmaxWarps && warp < kMmaWarp0 && (warp & 3) < 2 && S.a >= 0) {
     const int j = (warp & 1) * 32 + lane;
-    reinterpret_cast<int *>(smem + sm.tok)[pre_s * 64 + j] =
-        (table_mask(p, pre_a) >> j) & 1ull ? (int)table_token(p, pre_a, j) : -1;
+    reinterpret_cast<int *>(smem + sm.tok)[stream * 64 + j] =
+        (table_mask(p, S.a) >> j) & 1ull ? (int)table_token(p, S.a, j) : -1;
   }
 
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + sm.bars);
@@ -446,19 +455,25 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     // The warps w, w+4, w+8, ... share a scheduler and own the same 32 query rows; they take the steps of their sets
     // in turn, one thread per full 64-key row: while one exponentiates and packs its step (special-function bound),
     // the others fetch, mask and reduce later ones.  The only hand-off between them is the running maximum.
-    const int s = (warp & 3) >> 1, set = warp >> 2;
+    // (`stream` again, from the warp directly or not: the compiler's schedule of the step decides, as for FP4 above)
+    const int s = FP4 ? stream : (warp & 3) >> 1, set = warp >> 2;
     const int r = (warp & 1) * 32 + lane;  // query row inside the stream's block
-    const StreamInfo S = s ? st1 : st0;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const float gqk = p.gscale[bh * 4 + 0] * p.gscale[bh * 4 + 1] * p.scale * kLog2e;
     const float dq8s = (S.a >= 0 && S.a < R && p.tier_active[1]) ? p.dq8[(size_t)bh * R + S.a] * p.scale * kLog2e : 0.f;
     const float c16 = p.scale * kLog2e;
+    // What does not change from step to step is computed here and not in the step, whose every instruction is on the chain
+    // (with one row per warp loaded at the start: all-4-bit call of 16x48x48 13.75 -> 12.5 ms, 12 heads of 32,760 tokens
+    // 3.17 -> 2.92 ms).
+    const uint32_t sb = bars0 + (uint32_t)s * (B_COUNT * 8u);
+    auto my_bar = [&](int which) -> uint32_t { return sb + (uint32_t)which * 8u; };
     float h_own = -INFINITY, ell = 0.f;  // log2-domain maximum after this warp's last step; its partial denominator
     uint2 *my_hx = s_hx + (s * kSets + set) * 64 + r;                // running maximum after my steps, tagged with the step
     const uint32_t prev_hx = tc::smem_u32(s_hx + (s * kSets + ((set + kSets - 1) % kSets)) * 64 + r);
     uint8_t *const p_row0 = smem + sm.p[s] + r * 16;
     uint8_t *const sf_row0 = smem + sm.sfp[s] + (r & 31) * 16 + (r >> 5) * 4;
 
+    const uint32_t s_col = tmem + lane_addr + col_s(s, set & 1);  // (i and set have the same parity)
     for (int i = set; i < S.L; i += kSets) {
       const int tier = S.tier(i);
       const int g = SEGMENTED ? i & kStepMask : set;  // barriers, factors, ballots, scale atom
@@ -469,8 +484,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const int seg0 = tier == 0 ? 0 : (tier == 1 ? S.n4 : S.n48), pm = SEGMENTED && tier == 2 ? 1 : kMask;
       uint8_t *prow = p_row0 + (SEGMENTED ? (set & pm) << (11 + tier) : set * sm.pbytes[0]);
       const int busy = SEGMENTED && i - seg0 <= pm ? seg0 - 1 : i - 1 - pm;
-      const uint32_t s_col = tmem + lane_addr + col_s(s, i & 1);
-      if (!wait_or_abort(bar(s, B_SREADY + set), (i >> kShift) & 1, abortp)) break;
+      if (!wait_or_abort(my_bar(B_SREADY + set), (i >> kShift) & 1, abortp)) break;
       tc::fence_after_sync();
       // the step's mask and key scale (written before its K block was requested) are read while the scores load
       const uint2 info = s_info[s * kInfoRing + (i & (kInfoRing - 1))];
@@ -503,7 +517,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         }
       }
       tc::fence_before_sync();
-      warp_arrive(bar(s, B_SFREE + (i & 1)));
+      warp_arrive(my_bar(B_SFREE + (set & 1)));
       if (padded) {  // padding keys take no part: the loader left -inf for them and +inf for the others
         const float4 *lim = reinterpret_cast<const float4 *>(smem + sm.lim + (s * kInfoRing + (i & (kInfoRing - 1))) * 256);
 #pragma unroll
@@ -518,7 +532,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       for (int q = 0; q < 4; ++q) gm[q] = max16(v + q * 16);
       const float pmax = fmaxf(max3(gm[0], gm[1], gm[2]), gm[3]) * coef;  // log2 domain
       // the step's P slot, factors and ballots are free
-      if (busy >= 0 && !wait_or_abort(bar(s, B_PVDONE + (busy & kStepMask)), (busy >> kStepShift) & 1, abortp)) break;
+      if (busy >= 0 && !wait_or_abort(my_bar(B_PVDONE + (SEGMENTED ? busy & kStepMask : set)), (busy >> kStepShift) & 1, abortp)) break;
       // running maximum after step i-1: the thread that owns this row in the previous set leaves it, tagged with its
       // step, in shared memory (one 8-byte store, one 8-byte load: no barrier on this chain)
       float h_prev = -INFINITY;
@@ -530,7 +544,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         }
         const bool got = hv.y == (uint32_t)(i - 1);
         if (!__all_sync(0xffffffffu, got)) {
-          atomicCAS(abortp, 0, 1 + (int)(bar(s, B_CORROK) & 0xffffu));
+          atomicCAS(abortp, 0, 1 + (int)(my_bar(B_CORROK) & 0xffffu));
           break;
         }
         h_prev = __uint_as_float(hv.x);
@@ -669,12 +683,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         }
       }
       tc::fence_async_smem();
-      warp_arrive(bar(s, B_PREADY + g));
+      warp_arrive(my_bar(B_PREADY + g));
     }
     if (S.L > 0) {
       s_ell[(s * kSets + set) * 64 + r] = ell;
       s_href[(s * kSets + set) * 64 + r] = h_own;  // reference of this partial denominator
-      warp_arrive(bar(s, B_ELL));
+      warp_arrive(my_bar(B_ELL));
     }
   }
   // =========================================================================================== loader warps
@@ -687,9 +701,8 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     // Warp-uniform loop.  Lane l holds list entry 32 * batch + l ready for use: the record's address, the valid-key
     // mask and the INT8 key scale; the ids of the next two batches and the scales of the next one are already on
     // their way while a batch is used, so that a step costs a few shuffles and the copy request of one elected lane.
-    const int s = (warp - kLoadWarp0) & 1;
+    const int s = stream;
     const bool is_v = warp >= kLoadWarp0 + 2;
-    StreamInfo S = s ? st1 : st0;
     S.n4 = __shfl_sync(0xffffffffu, S.n4, 0);
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
@@ -813,7 +826,6 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     // themselves are issued by one elected lane.  (Under a lane-0 branch every descriptor would have to be moved from
     // vector to uniform registers before each issue, which costs more than the MMA itself.)
     const int s = warp - kMmaWarp0;
-    StreamInfo S = s ? st1 : st0;
     S.n4 = __shfl_sync(0xffffffffu, S.n4, 0);
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
@@ -881,8 +893,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   }
   // =========================================================================================== PV warps
   else if (warp >= kPvWarp0) {
-    const int s = warp - kPvWarp0;
-    StreamInfo S = s ? st1 : st0;
+    const int s = stream;
     S.n4 = __shfl_sync(0xffffffffu, S.n4, 0);
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
@@ -938,7 +949,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   }
   // =========================================================================================== correction warps
   else {
-    const int s = (warp - kSoftmaxWarps) >> 2;  // four correction warps per stream
+    const int s = stream;
     const int cw = (warp - kSoftmaxWarps) & 3;  // lane quarter
     const int ch = cw * 32 + lane;              // channel (TMEM lane)
     const uint32_t lane_addr = (uint32_t)(cw * 32) << 16;
@@ -947,7 +958,6 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     auto unit_of = [&](int t) -> float {  // common units per accumulator unit, for this thread's channel
       return t == 0 ? __fdiv_rn(gv, 2688.0f) : (t == 1 ? kEtaP8 * dv8 : 1.0f);
     };
-    const StreamInfo &S = s ? st1 : st0;
     // Every step passes through these warps between the softmax and the product: once P(i) is written they read the
     // step's "maximum moved" ballots and, only if one is set or the segment changes, wait for product i-1 and rescale
     // their lane quarter of the accumulator; then they let product i go.  Most steps move no maximum.
@@ -1095,7 +1105,7 @@ cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t s
   const SmemMap sm = make_smem_map(p, b16 && p.d == 128);
   if (!sm.fits) return cudaErrorInvalidConfiguration;
   cudaError_t e;
-  const int grid = p.BH * (sm.single ? p.Rt : (p.Rt + 1) / 2);
+  const int grid = sm.pair_ctas + p.BH * p.Rt - sm.first_single;
   auto launch = [&](auto kernel) -> cudaError_t {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm.total);
     if (err != cudaSuccess) return err;

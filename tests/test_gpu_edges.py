@@ -91,3 +91,21 @@ def test_ties_go_to_the_lower_index(T, Hg, Wg, rank_scope):
     ref = oracle_all(w, q, k, v, rank_scope=rank_scope)
     assert _check_prepare(w, plan, ws, ref) == []
     _check_attention(w, out, ref, [(1, 0), (1, plan.info.R - 1)], [])
+
+
+@pytest.mark.parametrize("rank_scope", [0, 1])
+@pytest.mark.parametrize("H,T,Hg,Wg", [(2, 2, 8, 296), (2, 5, 24, 40), (4, 5, 24, 40), (5, 5, 24, 40), (6, 5, 24, 40)])
+def test_last_wave_of_blocks(H, T, Hg, Wg, rank_scope):
+    """One query block per CTA in the last wave: 148 blocks (all of them), 150 (none), 300 and 375 in heads of 75 (the last 7
+    and 82), 450 (none: 157 would be left)."""
+    w = W("wave", 1, H, 64, T, Hg, Wg, 0.0, 0.1, 0.2, seed=35)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v, rank_scope=rank_scope)
+    ref = oracle_all(w, q, k, v, rank_scope=rank_scope)
+    bad = _check_prepare(w, plan, ws, ref)
+    R = plan.info.R
+    sel = [(h, a) for h in range(H) for a in (0, 1, 66, 67, 68, 69, R - 2, R - 1)]
+    _check_attention(w, out, ref, sel, bad)
+    again = torch.full_like(out, float("nan"))
+    da2.da2_attention_fwd(plan, q, k, v, ws, again)
+    assert torch.equal(out, again)
