@@ -47,9 +47,9 @@
 // then sums and packing), which gives the single warp the instruction-level parallelism it lacks when the three are
 // interleaved per pair.  And the code is kept small: the hot code of all roles shares a 32 KB instruction cache, and the
 // all-4-bit call follows its hit rate (99.9 % 13.5 ms, 99.0 % 13.8, 97.6 % 14.4, 93.8 % 15.1).
-// Measured (kernel alone, ms; before the packed conversions, the smaller code, four sets for every plan and the shorter
-// start and end of a CTA -> now):  wan14b_720p 69.3 -> 64.4;  wan1p3b_480p 3.52 -> 3.08;  with a 400-token prefix, whose
-// blocks are bf16 (two softmax sets before), 4.85 -> 3.95;  a 1,024-token call 0.020 -> 0.014.
+// Measured (kernel alone, ms; before the packed conversions, the smaller code, four sets for every plan, the shorter start
+// and end of a CTA and the shorter step -> now):  wan14b_720p 69.3 -> 60.0;  wan1p3b_480p 3.52 -> 2.92;  with a 226-token
+// prefix, whose blocks are bf16 (two softmax sets before), 4.55 -> 3.90.
 // Every wait on an mbarrier is bounded; a wait that gives up records device status "timeout", all roles leave their
 // loops and the CTA exits normally after releasing TMEM.
 #include <type_traits>

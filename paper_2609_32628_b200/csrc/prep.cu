@@ -12,7 +12,7 @@
 // thread takes its 32 channels of a row (Q, K) or 16 slots of two channels (V) out of shared memory once and makes the
 // codes of all formats from those registers, in packed pairs where an instruction for pairs exists, and the block needs
 // three barriers in all.
-// Measured: 40 heads x 75,600 tokens (4.31 GB read and written) 1.41 -> 1.08 ms, 4.0 TB/s; 12 heads x 32,760 tokens 95 -> 75 us
+// Measured: 40 heads x 75,600 tokens (4.31 GB read and written) 1.41 -> 1.08 ms, 4.0 TB/s; 24 heads x 8,192 tokens 95 -> 75 us
 // (before: a thread per 16 channels and format, quotients and casts one by one, a barrier per format).
 #include <cuda_fp8.h>
 
