@@ -455,8 +455,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     // The warps w, w+4, w+8, ... share a scheduler and own the same 32 query rows; they take the steps of their sets
     // in turn, one thread per full 64-key row: while one exponentiates and packs its step (special-function bound),
     // the others fetch, mask and reduce later ones.  The only hand-off between them is the running maximum.
-    // (`stream` again, from the warp directly or not: the compiler's schedule of the step decides, as for FP4 above)
-    const int s = FP4 ? stream : (warp & 3) >> 1, set = warp >> 2;
+    const int s = stream, set = warp >> 2;
     const int r = (warp & 1) * 32 + lane;  // query row inside the stream's block
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const float gqk = p.gscale[bh * 4 + 0] * p.gscale[bh * 4 + 1] * p.scale * kLog2e;
