@@ -12,6 +12,9 @@
  *   - q, k, v, out: DEVICE pointers, contiguous bf16 [B, H, P + N, head_dim]: first the P = n_prefix prefix (text)
  *     tokens, if any, then the N = T*Hg*Wg video tokens in raster order u = (t*Hg + y)*Wg + x; 16-byte aligned.
  *     out must not alias the inputs.
+ *     A NaN takes no part in the maxima behind the quantiser scales (nor in the max-pooled descriptors); it spoils the
+ *     draft-map rows that its average descriptor enters: the row of its block for Q, every row of its head for K.  Such a
+ *     row ranks as one tie (the lower indices).
  *   - workspace: DEVICE pointer, 256-byte aligned, at least da2_plan_info().workspace_bytes long.  The caller owns
  *     all device memory; the library allocates none and keeps no device state between calls (one exception:
  *     da2_draft_map_noalloc, which owns a fixed scratch array, see there).

@@ -106,6 +106,18 @@ __host__ __device__ inline long long slot_token(const Params &p, int a, int j) {
 // operand records per head and tier: the 16-bit tier also holds the prefix blocks
 __host__ __device__ inline int rec_blocks(const Params &p, int tier) { return tier == 2 ? p.Rt : p.R; }
 
+#ifdef __CUDACC__
+// Largest magnitudes of bf16 pairs, half by half: max(|m|, |a|).  The signs of the result are left over (clear them with
+// magnitudes2); a NaN loses against every number, so that it stays out of the statistics that scales are derived from.
+__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a) {
+  uint32_t r;
+  asm("max.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(m), "r"(a));
+  return r;
+}
+__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a, uint32_t b) { return max_abs2(max_abs2(m, a), b); }
+__device__ __forceinline__ uint32_t magnitudes2(uint32_t m) { return m & 0x7fff7fffu; }  // of numbers: they order like integers
+#endif
+
 // Programmatic dependent launch: a kernel of the chain may be scheduled as soon as every block of the kernel before it has
 // called grid_trigger() (all of them do so at their start), so that launch latency and set-up overlap that kernel's last
 // blocks; grid_wait() then waits until the kernel before has completed and its writes are visible.  Every block of every

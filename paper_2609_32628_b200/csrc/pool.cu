@@ -28,10 +28,6 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
   return r;
 }
-// magnitudes of bf16 pairs order like 16-bit integers
-__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a, uint32_t b) {
-  return __vimax3_u16x2(m, a & 0x7fff7fffu, b & 0x7fff7fffu);
-}
 __device__ __forceinline__ float abs_max_of(uint32_t m) { return fmaxf(bf16lo(m), bf16hi(m)); }
 
 template <int W> struct Row { uint32_t w[W]; };  // one token's channels of a lane
@@ -101,10 +97,10 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
           sk[2 * c] += (double)bf16lo(xk[i].w[c]); sk[2 * c + 1] += (double)bf16hi(xk[i].w[c]);
           mq[c] = max_bf16x2(mq[c], xq[i].w[c]);
           mk[c] = max_bf16x2(mk[c], xk[i].w[c]);
-          av[c] = max_abs2(av[c], xv[i].w[c], 0u);
+          av[c] = max_abs2(av[c], xv[i].w[c]);
         }
-        aq = max_abs2(aq, xq[i].w[0], xq[i].w[W - 1]);
-        ak = max_abs2(ak, xk[i].w[0], xk[i].w[W - 1]);
+        aq = W == 2 ? max_abs2(aq, xq[i].w[0], xq[i].w[W - 1]) : max_abs2(aq, xq[i].w[0]);
+        ak = W == 2 ? max_abs2(ak, xk[i].w[0], xk[i].w[W - 1]) : max_abs2(ak, xk[i].w[0]);
       }
     }
   }
@@ -149,7 +145,9 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
   // statistics of the head: combined over the CTA first, then one atomic per channel (non-negative floats order like
   // their bit patterns)
 #pragma unroll
-  for (int c = 0; c < W; ++c) s_av[warp][lane * W + c] = av[c];
+  for (int c = 0; c < W; ++c) s_av[warp][lane * W + c] = magnitudes2(av[c]);
+  aq = magnitudes2(aq);
+  ak = magnitudes2(ak);
 #pragma unroll
   for (int off = 16; off >= 1; off >>= 1) {
     aq = __vmaxu2(aq, __shfl_xor_sync(0xffffffffu, aq, off));

@@ -76,10 +76,6 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
-// magnitudes of bf16 pairs order like 16-bit integers
-__device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a, uint32_t b) {
-  return __vimax3_u16x2(m, a & 0x7fff7fffu, b & 0x7fff7fffu);
-}
 __device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
@@ -198,6 +194,8 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       ak = max_abs2(max_abs2(ak, xk[i].x, xk[i].y), xk[i].z, xk[i].w);
     }
     if (t8) {
+      aq = magnitudes2(aq);
+      ak = magnitudes2(ak);
 #pragma unroll
       for (int o = 16; o >= 1; o >>= 1) {
         aq = __vmaxu2(aq, __shfl_xor_sync(0xffffffffu, aq, o));
@@ -274,7 +272,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         uint32_t m = max_abs2(max_abs2(0u, nw[h][0], nw[h][1]), nw[h][2], nw[h][3]);
-        m = max_abs2(max_abs2(m, nw[h][4], nw[h][5]), nw[h][6], nw[h][7]);
+        m = magnitudes2(max_abs2(max_abs2(m, nw[h][4], nw[h][5]), nw[h][6], nw[h][7]));
         sc[h] = nvfp4_group(nw[h], fmaxf(bf16lo(m), bf16hi(m)), g6, g, c[2 * h], c[2 * h + 1]);
       }
       uint8_t *dst = which ? p.kvrec[0] + blk * p.kvrec_bytes[0] : p.qrec[0] + blk * p.qrec_bytes[0];
@@ -303,6 +301,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
       nw[0][i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410) ^ 0x80008000u;
       nw[1][i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632) ^ 0x80008000u;
     }
+    m = magnitudes2(m);
     // Hands over the channel the other lane stores; mine[e]: this lane's 16 bytes of channel e.  Afterwards out[0] / out[1]
     // are the 16 bytes of slot groups gh*2 / gh*2 + 1 of channel 2 * pair + h.
     auto exchange = [&](const uint4 (&mine)[2], uint4 (&both)[2]) {
