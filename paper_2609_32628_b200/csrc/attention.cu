@@ -232,6 +232,11 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float r;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -517,12 +522,14 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       }
       tc::fence_before_sync();
       warp_arrive(my_bar(B_SFREE + (set & 1)));
-      if (padded) {  // padding keys take no part: the loader left -inf for them and +inf for the others
+      // Padding keys take no part: the loader left -inf for them and +inf for the others.  A score that is no number stays one
+      // (at a padding key only a query that is not finite makes it one, and then every score of the row is not finite).
+      if (padded) {
         const float4 *lim = reinterpret_cast<const float4 *>(smem + sm.lim + (s * kInfoRing + (i & (kInfoRing - 1))) * 256);
 #pragma unroll
         for (int c = 0; c < 64; c += 4) {
           const float4 x = lim[c >> 2];
-          v[c] = fminf(v[c], x.x); v[c + 1] = fminf(v[c + 1], x.y); v[c + 2] = fminf(v[c + 2], x.z); v[c + 3] = fminf(v[c + 3], x.w);
+          v[c] = min_nan(v[c], x.x); v[c + 1] = min_nan(v[c + 1], x.y); v[c + 2] = min_nan(v[c + 2], x.z); v[c + 3] = min_nan(v[c + 3], x.w);
         }
       }
       // maxima of the four 16-key groups (pairwise trees), then of the row

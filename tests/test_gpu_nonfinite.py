@@ -75,3 +75,21 @@ def test_nan_stays_out_of_the_scales(which, channels, d):
     g, dv = V.gscale(), V.dv8()
     da2.da2_prepare_cached_scales(plan, x["q"], x["k"], x["v"], ws, reselect=True)
     _check_operands(plan, ws, ref, dv=dv, g=g)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("slot_of", ["full", "edge"])
+def test_nan_key_reaches_every_query_that_attends_to_it(slot_of, d):
+    """bf16 products carry a NaN key into each output row that keeps its block, whether or not the block has padding slots
+    beside it; the other head is untouched."""
+    w = W("nan16", 1, 2, d, 3, 12, 20, 1.0, 0.0, 0.0, seed=42)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    pl = oracle.plan(w.T, w.Hg, w.Wg)
+    full = int((pl.slot_token >= 0).sum(1).argmax())
+    block = full if slot_of == "full" else pl.R - 1
+    assert ((pl.slot_token[block] < 0).any()) == (slot_of == "edge")
+    k[0, 0, int(pl.slot_token[block, 0]), 5] = float("nan")
+    plan, ws, out = run_gpu(w, q, k, v)
+    assert torch.isnan(out[0, 0]).all()
+    ref = oracle_all(w, q, k, v)
+    _check_attention(w, out, ref, [(1, a) for a in range(pl.R)], [])
