@@ -14,7 +14,8 @@
  *     out must not alias the inputs.
  *     A NaN takes no part in the maxima behind the quantiser scales (nor in the max-pooled descriptors); it spoils the
  *     draft-map rows that its average descriptor enters: the row of its block for Q, every row of its head for K.  Such a
- *     row ranks as one tie (the lower indices).
+ *     row ranks as one tie (the lower indices).  An infinity makes the scales it enters infinite.  Output rows whose
+ *     scores are not all finite are NaN or zero.
  *   - workspace: DEVICE pointer, 256-byte aligned, at least da2_plan_info().workspace_bytes long.  The caller owns
  *     all device memory; the library allocates none and keeps no device state between calls (one exception:
  *     da2_draft_map_noalloc, which owns a fixed scratch array, see there).

@@ -253,7 +253,9 @@ __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
   kmax = __reduce_max_sync(0xffffffffu, kmax);
   kmin = __reduce_min_sync(0xffffffffu, kmin);
   Cut cut[3];  // cumulative: 16-bit, 16 + 8, 16 + 8 + 4
-  int cum = 0, top = kmax + 1, above = 0;  // keys >= top: `above` of them, fewer than any boundary still to come
+  // Keys >= top: `above` of them, fewer than any boundary still to come.  A row of NaN scores (one in a row makes all of them
+  // NaN, 0x7fffffff) has no key above: its search is over at once, and the boundary's ties go to the lower indices.
+  int cum = 0, top = kmax < 0x7fffffff ? kmax + 1 : kmax, above = 0;
 #pragma unroll
   for (int t = 0; t < 3; ++t) {
     const int c = cum + (int)p.quota[2 - t];
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(NT) head_hist_kernel(Params p) {
   for (size_t i = lo + tid; i < hi; i += NT) {
     const uint32_t key = __ldg(&keys[i]);
     if (PASS == 0) {
-      atomicAdd(&h[key >> 20], 1u);
+      atomicAdd(&h[(key >> 20) & (kBins0 - 1)], 1u);  // (a score has no sign)
     } else {
 #pragma unroll
       for (int t = 0; t < 3; ++t)

@@ -93,3 +93,23 @@ def test_nan_key_reaches_every_query_that_attends_to_it(slot_of, d):
     assert torch.isnan(out[0, 0]).all()
     ref = oracle_all(w, q, k, v)
     _check_attention(w, out, ref, [(1, a) for a in range(pl.R)], [])
+
+
+@pytest.mark.parametrize("f16,f8,f4", [(0.1, 0.2, 0.3), (0.0, 0.3, 0.0), (0.5, 0.25, 0.25)])
+@pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (1, 24, 56), (13, 8, 40), (23, 24, 56), (61, 24, 56), (683, 8, 24)])
+def test_rows_of_nan_scores_keep_the_lower_indices(T, Hg, Wg, f16, f8, f4):
+    """A NaN in K makes every score of its head NaN: all rows of head 0 are one tie; head 1 has its ordinary lists."""
+    w = W("nanrows", 1, 2, 64, T, Hg, Wg, f16, f8, f4, seed=43)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    k[0, 0, w.N // 2, 7] = float("nan")
+    plan = da2.da2_plan(w.B, w.H, w.T, w.Hg, w.Wg, w.head_dim, f16, f8, f4)
+    ws = torch.empty(int(plan.info.workspace_bytes), dtype=torch.uint8, device="cuda")
+    da2.da2_prepare(plan, q, k, v, ws)
+    torch.cuda.synchronize()
+    ids, cnt = Workspace(plan, ws, [0]).lists()
+    k4, k8, k16 = (int(x) for x in plan.info.quota)
+    n = k4 + k8 + k16
+    assert (cnt == np.array([k4, k8, k16])).all()
+    assert (ids[0, :, :n] == np.r_[k16 + k8:n, k16:k16 + k8, 0:k16]).all()
+    ref = oracle_all(w, q, k, v, heads=[1])
+    compare_lists(ref["A"], ref["ids"], ref["counts"], *Workspace(plan, ws, [1]).lists())
