@@ -96,7 +96,7 @@ typedef struct {
   int64_t ids_per_head;              /* uint16 entries of the id array belonging to one head */
   float lambda, softmax_scale;
   uint64_t workspace_bytes;
-  uint64_t off_status;               /* int32[64]: [0] status code, [1..] diagnostics */
+  uint64_t off_status;               /* int32[64]: [0] status code, [1..] diagnostics and hand-over words of a call */
   uint64_t off_amax;                 /* uint32[BH][4]: fp32 bit patterns of max|Q|, max|K|, max|V| per head */
   uint64_t off_vmax;                 /* uint32[BH][d]: fp32 bit patterns of max_v |V_vc| */
   uint64_t off_gscale;               /* fp32[BH][4]: NVFP4 per-tensor scales g_Q, g_K, g_V */

@@ -17,6 +17,7 @@ constexpr int kSfAtomBytes = 512;  // one scale-factor atom: 128 rows x 4 groups
 constexpr int kDevOk = 0;
 constexpr int kDevTimeout = 1;
 constexpr int kDevBadList = 2;
+constexpr int kPooledWord = 16;  // status word that says, within a call, that the pooling kernel's results may be read
 
 // Plain-old-data parameter block handed to every kernel by value.
 struct Params {
@@ -138,6 +139,15 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, siz
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+// griddepcontrol.wait vouches for the kernel directly before only.  A kernel that runs beside that one, on results of the one
+// before it, needs them handed on: a thread of the kernel between has waited for them and then publishes the word (release),
+// and the reader takes it (acquire) before it reads them; a reader that does not find it set yet waits for the whole grid.
+__device__ __forceinline__ void publish(int *word) { asm volatile("st.release.gpu.global.u32 [%0], 1;" ::"l"(word) : "memory"); }
+__device__ __forceinline__ bool published(const int *word) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(word) : "memory");
+  return v != 0;
 }
 #endif
 

@@ -54,7 +54,8 @@ __global__ void __launch_bounds__(128) draft_logits_kernel(Params p) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) { acc[i][j][0] = 0.0; acc[i][j][1] = 0.0; }
   grid_wait();
-  grid_trigger();  // only now: what runs beside this kernel may rely on the kernels before it
+  if (p.status != nullptr && tid == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0) publish(p.status + kPooledWord);
+  grid_trigger();  // only now: what runs beside this kernel finds the kernels before it complete (and the word, as a rule, set)
   // 64 rows x 8 quarters of four channels per operand and group: 4 + 4 copies per thread
   const int lc = (tid & 7) * 4, lr = tid >> 3;
   for (int base = 0; base < d; base += kChunk) {

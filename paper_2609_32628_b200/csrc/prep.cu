@@ -141,7 +141,9 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
                                                   const __nv_bfloat16 *__restrict__ v, bool beside_draft) {
   extern __shared__ __align__(16) uint8_t smem[];
   // beside_draft: the kernel before is the draft-logits kernel, which this one does not depend on; its blocks have waited
-  // for the pooling kernel before they let this kernel start.  So the two overlap, and the wait comes at the end.
+  // for the pooling kernel before they let this kernel start.  So the two overlap, and the wait comes at the end.  What the
+  // kernels before it wrote (scales; caller-fixed ones too) is read only after the block has taken the word that the
+  // draft-logits kernel publishes.
   grid_trigger();
   if (!beside_draft) grid_wait();
   // Q, K: rows padded by 16 bytes, so that threads that read the same channels of consecutive slots fall on different
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
   constexpr int NATOM = D / 64;
   uint8_t *sf_v = sf_img + 2 * NATOM * kSfAtomBytes;
   __shared__ uint32_t s_red[2][NT / 32];
+  __shared__ bool s_pooled;
 
   const int a = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned long long mask = block_valid_mask(p, a);
@@ -183,6 +186,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
         xv[i] = __ldg(reinterpret_cast<const uint4 *>(v + off));
       }
     }
+    if (beside_draft && tid == 0) s_pooled = published(p.status + kPooledWord);
     uint32_t aq = 0, ak = 0;
 #pragma unroll
     for (int i = 0; i < PASSES; ++i) {
@@ -207,6 +211,7 @@ __global__ void __launch_bounds__(NT, 4) prep_kernel(Params p, const __nv_bfloat
     if (D == 64 && tid < kSfAtomBytes / 16) *reinterpret_cast<uint4 *>(sf_v + tid * 16) = make_uint4(0, 0, 0, 0);
   }
   __syncthreads();
+  if (beside_draft && !s_pooled) grid_wait();
 
   if (POOL && video) {
     // one thread per (tensor, channel): sum and maximum over the valid slots of the staged tile.  A sum of at most

@@ -109,3 +109,35 @@ def test_last_wave_of_blocks(H, T, Hg, Wg, rank_scope):
     again = torch.full_like(out, float("nan"))
     da2.da2_attention_fwd(plan, q, k, v, ws, again)
     assert torch.equal(out, again)
+
+
+@pytest.mark.parametrize("fixed", [False, True])
+@pytest.mark.parametrize("H,T,Hg,Wg", [(1, 1, 8, 8), (2, 4, 16, 16), (12, 8, 32, 32)])
+def test_operands_follow_their_own_call(H, T, Hg, Wg, fixed):
+    """The operand kernel runs beside the draft logits on scales that the kernels before those wrote: calls on inputs of very
+    different range, enqueued one after the other on one workspace, leave what each leaves when it runs alone."""
+    w = W("order", 1, H, 128, T, Hg, Wg, 0.1, 0.2, 0.3, seed=36)
+    x = da2_inputs.make_qkv(w, "cuda")
+    inputs = [x, [t * 512 for t in x], [t.flip(2) / 256 for t in x]]
+    g = [np.full(H, s, np.float32) for s in (0.002, 0.003, 0.004)] if fixed else (None, None, None)
+    plan = da2.da2_plan(1, H, T, Hg, Wg, 128, 0.1, 0.2, 0.3, g_q=g[0], g_k=g[1], g_v=g[2])
+    I = plan.info
+    kept = lambda ws: torch.cat([ws[I.off_gscale:I.off_gscale + H * 16],
+                                 *(ws[I.off_qrec[t]:I.off_qrec[t] + H * I.R * I.qrec_bytes[t]] for t in range(3)),
+                                 *(ws[I.off_kvrec[t]:I.off_kvrec[t] + H * I.R * I.kvrec_bytes[t]] for t in range(3)),
+                                 ws[I.off_dq8:I.off_dq8 + H * I.R * 4], ws[I.off_dv8:I.off_dv8 + H * 128 * 4]])
+    alone = []
+    for qkv in inputs:
+        ws = torch.zeros(int(I.workspace_bytes), dtype=torch.uint8, device="cuda")
+        da2.da2_prepare(plan, *qkv, ws)
+        torch.cuda.synchronize()
+        alone.append(kept(ws))
+    ws = torch.zeros(int(I.workspace_bytes), dtype=torch.uint8, device="cuda")
+    got = []
+    for i in range(60):
+        da2.da2_prepare(plan, *inputs[i % 3], ws)
+        if i % 4 == 3:
+            got.append((i % 3, kept(ws)))
+    torch.cuda.synchronize()
+    for i, g_ in got:
+        assert torch.equal(g_, alone[i])
