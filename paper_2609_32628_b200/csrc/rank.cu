@@ -205,8 +205,10 @@ struct Quotient {
 };
 
 // RANK: ranking and lists (ROW scope); otherwise the draft map rows only
+// (20 entries fit the 80 registers of six CTAs an SM; the compiler's own choice is 96, five CTAs: logits and ranking of 12 heads
+// at 588 entries 84.6 us instead of 82.5)
 template <int E, bool RANK>
-__global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
+__global__ void __launch_bounds__(kRowWarps * 32, E == 20 ? 6 : 0) rank_warp_kernel(Params p) {
   const int lane = threadIdx.x & 31, a = blockIdx.x * kRowWarps + (threadIdx.x >> 5), bh = blockIdx.y, R = p.R;
   grid_trigger();
   grid_wait();
@@ -312,26 +314,28 @@ __global__ void __launch_bounds__(kRowWarps * 32) rank_warp_kernel(Params p) {
     *reinterpret_cast<int4 *>(p.counts + ((size_t)bh * p.Rt + a) * 4) = make_int4(k4, k8, k16 + p.Rp, a * p.row_stride);
 }
 
-// registers per lane that hold a row of R entries, 0 where they would be too many
-template <bool RANK> bool launch_rank_warp(const Params &p, cudaStream_t st) {
+// Launches the kernel whose registers hold a row: entries per lane in steps of 2 up to 16, of 4 up to 32 and of 8 up to 64, so
+// that the entries a row pays for beyond its own stay few; false for rows above 2,048 entries.  (With seven sizes, 2 to 64,
+// da2_prepare of 12 heads took 261 us at 609 entries and 978 us at 1,400 instead of 236 and 765.)
+template <bool RANK, int E = 2> bool launch_rank_warp(const Params &p, cudaStream_t st, cudaError_t *err) {
+  if ((p.R + 31) / 32 > E) {
+    constexpr int next = E < 16 ? E + 2 : (E < 32 ? E + 4 : E + 8);
+    if constexpr (next <= 64) return launch_rank_warp<RANK, next>(p, st, err);
+    else return false;
+  }
   const dim3 grid((p.R + kRowWarps - 1) / kRowWarps, p.BH);
-  // Chained to the kernel before only where the rows are few: there it hides the launch (2 us of 33 for the smallest call);
-  // waiting blocks of a large grid hold registers the kernel before still wants (1.8 us of 27 for two heads of 588 rows).
+  // Chained to the kernel before only where the rows are few: there it hides the launch, while waiting blocks of a larger grid
+  // hold registers that the kernel before still wants.  da2_prepare chained / not, us: 32 rows of 16 19.2 / 22.0, 512 rows of
+  // 128 30.1 / 31.0; 960 rows of 480 55.8 / 51.5, 1,176 rows of 588 61.9 / 58.9 (and 1,280 rows of 160, 49.7 / 50.6, lose it
+  // again in the call: 264 / 262).
   const bool chained = (long long)p.R * p.BH <= 512;
-  auto go = [&](auto kernel) {
-    if (chained) launch_chained(kernel, grid, kRowWarps * 32, 0, st, p);
-    else kernel<<<grid, kRowWarps * 32, 0, st>>>(p);
-    return true;
-  };
-  const int e = (p.R + 31) / 32;
-  if (e <= 2) return go(rank_warp_kernel<2, RANK>);
-  if (e <= 5) return go(rank_warp_kernel<5, RANK>);
-  if (e <= 10) return go(rank_warp_kernel<10, RANK>);
-  if (e <= 19) return go(rank_warp_kernel<19, RANK>);
-  if (e <= 28) return go(rank_warp_kernel<28, RANK>);
-  if (e <= 40) return go(rank_warp_kernel<40, RANK>);
-  if (e <= 64) return go(rank_warp_kernel<64, RANK>);
-  return false;
+  if (chained) {
+    *err = launch_chained(rank_warp_kernel<E, RANK>, grid, kRowWarps * 32, 0, st, p);
+  } else {
+    rank_warp_kernel<E, RANK><<<grid, kRowWarps * 32, 0, st>>>(p);
+    *err = cudaGetLastError();
+  }
+  return true;
 }
 
 // ---------------------------------------------------------------------------------------------- ROW scope, long rows
@@ -648,14 +652,15 @@ __global__ void __launch_bounds__(kRowWarps * 32) head_emit_kernel(Params p) {
 // Draft map rows only (softmax of both logit branches and their mixture into p.map); used by callers that want
 // the map without the ranking.
 cudaError_t launch_map_rows(const Params &p, cudaStream_t st, int *launches) {
-  if (launch_rank_warp<false>(p, st)) {
+  cudaError_t e;
+  if (launch_rank_warp<false>(p, st, &e)) {
     *launches += 1;
-    return cudaGetLastError();
+    return e;
   }
   dim3 grid(p.R, p.BH);
   const size_t smem = (size_t)p.R * sizeof(uint32_t);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(head_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(head_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
   launch_chained(head_map_kernel, grid, NT, smem, st, p);
@@ -668,9 +673,9 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
   const size_t smem = (size_t)p.R * sizeof(uint32_t);
   cudaError_t e;
   if (p.rank_scope == DA2_RANK_ROW) {
-    if (launch_rank_warp<true>(p, st)) {
+    if (launch_rank_warp<true>(p, st, &e)) {
       *launches += 1;
-      return cudaGetLastError();
+      return e;
     }
     if (smem > 48 * 1024) {
       e = cudaFuncSetAttribute(rank_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
