@@ -1128,9 +1128,8 @@ cudaError_t launch_attention(const Params &p, __nv_bfloat16 *out, cudaStream_t s
   using I128 = std::integral_constant<int, 128>;
   if (p.d == 128) e = b16 ? pick(I128{}, std::true_type{}) : pick(I128{}, std::false_type{});
   else e = b16 ? pick(I64{}, std::true_type{}) : pick(I64{}, std::false_type{});
-  if (e != cudaSuccess) return e;
   *launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace da2

@@ -126,8 +126,9 @@ __device__ __forceinline__ uint32_t magnitudes2(uint32_t m) { return m & 0x7fff7
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A launch's own status, chained or not.  It is taken out of the runtime's record, so that the next call does not report it again.
 template <class... KArgs, class... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+cudaError_t launch(bool chained, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -137,8 +138,14 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, siz
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  cfg.numAttrs = chained ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+template <class... KArgs, class... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  return launch(true, kernel, grid, threads, smem, st, args...);
 }
 // griddepcontrol.wait vouches for the kernel directly before only.  A kernel that runs beside that one, on results of the one
 // before it, needs them handed on: a thread of the kernel between has waited for them and then publishes the word (release),

@@ -117,10 +117,8 @@ cudaError_t launch_draft(const Params &p, cudaStream_t st, int *launches) {
     const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  const cudaError_t e = launch_chained(draft_logits_kernel, grid, 128, smem, st, p);
-  if (e != cudaSuccess) return e;
   *launches += 1;
-  return cudaGetLastError();
+  return launch_chained(draft_logits_kernel, grid, 128, smem, st, p);
 }
 
 }  // namespace da2

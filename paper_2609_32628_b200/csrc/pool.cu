@@ -202,9 +202,8 @@ cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bflo
   cudaError_t e;
   if (p.d == 128) e = split == 1 ? launch(pool_kernel<128, 1>) : (split == 4 ? launch(pool_kernel<128, 4>) : launch(pool_kernel<128, 8>));
   else e = split == 1 ? launch(pool_kernel<64, 1>) : (split == 4 ? launch(pool_kernel<64, 4>) : launch(pool_kernel<64, 8>));
-  if (e != cudaSuccess) return e;
   *launches += 1;
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace da2

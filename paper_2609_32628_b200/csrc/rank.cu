@@ -329,12 +329,7 @@ template <bool RANK, int E = 2> bool launch_rank_warp(const Params &p, cudaStrea
   // 128 30.1 / 31.0; 960 rows of 480 55.8 / 51.5, 1,176 rows of 588 61.9 / 58.9 (and 1,280 rows of 160, 49.7 / 50.6, lose it
   // again in the call: 264 / 262).
   const bool chained = (long long)p.R * p.BH <= 512;
-  if (chained) {
-    *err = launch_chained(rank_warp_kernel<E, RANK>, grid, kRowWarps * 32, 0, st, p);
-  } else {
-    rank_warp_kernel<E, RANK><<<grid, kRowWarps * 32, 0, st>>>(p);
-    *err = cudaGetLastError();
-  }
+  *err = launch(chained, rank_warp_kernel<E, RANK>, grid, kRowWarps * 32, 0, st, p);
   return true;
 }
 
@@ -663,9 +658,8 @@ cudaError_t launch_map_rows(const Params &p, cudaStream_t st, int *launches) {
     e = cudaFuncSetAttribute(head_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  launch_chained(head_map_kernel, grid, NT, smem, st, p);
   *launches += 1;
-  return cudaGetLastError();
+  return launch_chained(head_map_kernel, grid, NT, smem, st, p);
 }
 
 cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
@@ -681,26 +675,27 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
       e = cudaFuncSetAttribute(rank_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
     }
-    launch_chained(rank_row_kernel, grid, NT, smem, st, p);
     *launches += 1;
-    return cudaGetLastError();
+    return launch_chained(rank_row_kernel, grid, NT, smem, st, p);
   }
   e = launch_map_rows(p, st, launches);
   if (e != cudaSuccess) return e;
   // about eight CTAs an SM share the scores of all heads; a share is at least one pass of the CTA's threads
   const long long M = (long long)p.R * p.R, most = (M + 4 * NT - 1) / (4 * NT), fair = (148 * 8 + p.BH - 1) / p.BH;
   const dim3 shares((unsigned)(most < fair ? most : fair), p.BH), rows((p.R + kRowWarps - 1) / kRowWarps, p.BH);
-  launch_chained(head_init_kernel, p.BH, NT, 0, st, p);
-  launch_chained(head_hist_kernel<0>, shares, NT, 0, st, p);
-  launch_chained(head_hist_kernel<1>, shares, NT, 0, st, p);
-  launch_chained(head_hist_kernel<2>, shares, NT, 0, st, p);
-  launch_chained(head_count_kernel, rows, kRowWarps * 32, 0, st, p);
-  launch_chained(head_offsets_kernel, p.BH, NT, 0, st, p);
-  launch_chained(head_emit_kernel, rows, kRowWarps * 32, 0, st, p);
+  auto next = [&](auto kernel, dim3 grid, int threads) {  // enqueued only if the one before was
+    if (e == cudaSuccess) e = launch_chained(kernel, grid, threads, 0, st, p);
+  };
+  next(head_init_kernel, p.BH, NT);
+  next(head_hist_kernel<0>, shares, NT);
+  next(head_hist_kernel<1>, shares, NT);
+  next(head_hist_kernel<2>, shares, NT);
+  next(head_count_kernel, rows, kRowWarps * 32);
+  next(head_offsets_kernel, p.BH, NT);
+  next(head_emit_kernel, rows, kRowWarps * 32);
   *launches += 7;
-  return cudaGetLastError();
+  return e;
 }
-
 
 // Scheduling order of the query blocks of a head for the attention kernel: by decreasing list length, ties by index.
 // O(R^2) comparisons per head on lengths staged in shared memory (R is a few thousand at most).
@@ -737,9 +732,8 @@ __global__ void __launch_bounds__(256) order_rows_kernel(Params p) {
 
 cudaError_t launch_prefix_rows(const Params &p, cudaStream_t st, int *launches) {
   if (p.Rp == 0) return cudaSuccess;
-  launch_chained(prefix_rows_kernel, dim3(p.Rp, p.BH), NT, 0, st, p);
   *launches += 1;
-  return cudaGetLastError();
+  return launch_chained(prefix_rows_kernel, dim3(p.Rp, p.BH), NT, 0, st, p);
 }
 
 cudaError_t launch_order(const Params &p, cudaStream_t st, int *launches) {
@@ -748,9 +742,8 @@ cudaError_t launch_order(const Params &p, cudaStream_t st, int *launches) {
     cudaError_t e = cudaFuncSetAttribute(order_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  launch_chained(order_rows_kernel, dim3((p.R + 31) / 32, p.BH), 256, smem, st, p);
   *launches += 1;
-  return cudaGetLastError();
+  return launch_chained(order_rows_kernel, dim3((p.R + 31) / 32, p.BH), 256, smem, st, p);
 }
 
 }  // namespace da2

@@ -1,6 +1,8 @@
 """Failure detection on the GPU, in forms that fault, trap or hang nothing: a bounded device-side wait that is made
 to run out reports through the status word and leaves the context usable; a list id that the host corrupts is
 clamped by the kernel and reported; both codes are cleared by the next da2_prepare."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -57,3 +59,30 @@ def test_list_id_out_of_range_is_clamped_and_reported():
     torch.cuda.synchronize()
     assert da2.da2_device_status(plan, ws) == 0
     assert torch.equal(bad.view(torch.int16), out.view(torch.int16))
+
+
+@pytest.mark.parametrize("rank_scope", [0, 1])
+def test_a_refused_launch_is_reported_once(rank_scope):
+    """Launches into a stream whose capture the host has spoiled are refused; the next call, on a sound stream, succeeds."""
+    w = W("refused", 1, 2, 64, 2, 16, 16, 0.1, 0.2, 0.3, seed=43)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v, rank_scope=rank_scope)
+    again = torch.full_like(out, float("nan"))
+    stream = torch.cuda.Stream()
+    handle = ctypes.c_void_p(stream.cuda_stream)
+    rt = ctypes.CDLL("libcudart.so.12")
+    graph = ctypes.c_void_p()
+    for fn in (lambda: da2.da2_attention_fwd(plan, q, k, v, ws, again, stream),
+               lambda: da2.da2_prepare(plan, q, k, v, ws, stream)):
+        torch.cuda.synchronize()
+        assert rt.cudaStreamBeginCapture(handle, 2) == 0          # relaxed mode: other streams stay usable
+        assert rt.cudaStreamSynchronize(handle) != 0              # not allowed in a capture: it is void from here on
+        with pytest.raises(da2.Da2Error) as e:
+            fn()
+        assert e.value.code == 4
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0
+        rt.cudaGetLastError()
+        da2.da2_attention_fwd(plan, q, k, v, ws, again)
+        da2.da2_prepare(plan, q, k, v, ws)
+        torch.cuda.synchronize()
+        assert torch.equal(again.view(torch.int16), out.view(torch.int16))
