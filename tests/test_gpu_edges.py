@@ -9,16 +9,17 @@ import pytest
 import torch
 
 import da2_inputs
+import oracle
 import paper_2609_32628_b200 as da2
-from helpers import oracle_all, run_gpu
+from helpers import Workspace, oracle_all, run_gpu
 from test_gpu_parity import _check_attention, _check_prepare
 
 pytestmark = pytest.mark.gpu
 W = da2_inputs.Workload
 
 
-# R = T * tiles on either side of 64, 160, 320, 608, 896, 1280 and 2048 entries per row (2, 5, 10, 19, 28, 40 and 64 per
-# lane; longer rows are ranked by a whole thread block), and the smallest rows there are
+# R = T * tiles from the smallest rows there are to beyond 2,048 entries (longer rows are ranked by a whole thread block), whole
+# calls; the edges of every register count of the ranking: test_rows_at_every_register_count
 @pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (1, 9, 8), (4, 32, 32), (13, 8, 40), (32, 8, 40), (23, 8, 56), (107, 8, 24),
                                      (29, 24, 56), (23, 24, 104), (61, 24, 56), (128, 32, 32), (683, 8, 24)])
 def test_row_lengths(T, Hg, Wg):
@@ -141,3 +142,45 @@ def test_operands_follow_their_own_call(H, T, Hg, Wg, fixed):
     torch.cuda.synchronize()
     for i, g_ in got:
         assert torch.equal(g_, alone[i])
+
+
+_HELD = (2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 56, 64)  # entries per lane a row may be held in
+
+
+@pytest.mark.parametrize("lam", [0.0, 1.0])
+@pytest.mark.parametrize("R", [1, 33] + [32 * e + x for e in _HELD for x in (0, 1)])
+def test_rows_at_every_register_count(R, lam):
+    """The last register of a row full and the first of the next size, three boundaries at once.  Scores: at lambda 0 and 1 the
+    map is the quotient of one branch, so its bits follow from the stored logits by correctly rounded steps: exponentials,
+    their sum in the order of 256 threads (whatever kernel takes the row), one division.  The logits are spread so that
+    exponentials from 1 to below 2^-100 occur.  Lists: exactly the oracle's ranking of the stored map."""
+    w = W("registers", 1, 1, 64, R, 8, 8, 0.1, 0.2, 0.3, seed=37)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, _ = run_gpu(w, q * 40, k, v, lam=lam)
+    I = plan.info
+    V = Workspace(plan, ws)
+    A = V.draft_map()
+    logits = ws[I.off_logits[int(lam)]:I.off_logits[int(lam)] + R * R * 4].view(torch.float32).view(R, R)
+    x = torch.exp(logits - logits.max(1, keepdim=True).values)
+    if R > 64:
+        assert ((x > 0) & (x < 2.0 ** -100)).any()
+    y = torch.zeros(R, -(-R // 256) * 256, device="cuda")
+    y[:, :R] = x
+    y = y.view(R, -1, 256)
+    z = torch.zeros(R, 256, device="cuda")
+    for i in range(y.shape[1]):
+        z = z + y[:, i]
+    z = z.view(R, 8, 32)
+    lane = torch.arange(32, device="cuda")
+    for o in (16, 8, 4, 2, 1):
+        z = z + z[:, :, lane ^ o]
+    total = torch.zeros(R, device="cuda")
+    for i in range(8):
+        total = total + z[:, i, 0]
+    exp = x.cpu().numpy() / total.cpu().numpy()[:, None]
+    assert np.array_equal(A[0].view(np.int32), exp.view(np.int32))
+    k4, k8, k16 = (int(n) for n in I.quota)
+    ids, cnt = V.lists()
+    ids_o, cnt_o = oracle.lists(oracle.rank_row(A, k16, k8, k4))
+    n = k4 + k8 + k16
+    assert np.array_equal(cnt, cnt_o) and np.array_equal(ids[:, :, :n], ids_o[:, :, :n])

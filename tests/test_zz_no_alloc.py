@@ -63,3 +63,16 @@ def test_noalloc_rejects_sizes_beyond_its_fixed_scratch():
     assert rc == 3  # DA2_ERR_WORKSPACE_TOO_SMALL, nothing launched
     rc = fn(*(int(t.data_ptr()) for t in desc), 40000, 5, d, 0.2, 0.125, int(x.data_ptr()), None)
     assert rc == 2  # DA2_ERR_UNSUPPORTED: more heads than a launch dimension holds, nothing launched
+
+
+@pytest.mark.parametrize("d", [16, 48, 144, 272])
+@pytest.mark.parametrize("BH,R", [(1, 1), (3, 65), (2, 130)])
+def test_noalloc_takes_every_multiple_of_16_channels(BH, R, d):
+    """Channels beyond one staged chunk of 128 and groups of 32 that are only partly filled, with blocks beyond one tile."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + R)
+    desc = [torch.randn(BH, R, d, generator=gen, device="cuda") for _ in range(4)]
+    out = torch.full((BH, R, R), float("nan"), device="cuda")
+    da2.da2_draft_map_noalloc(*desc, 0.2, d ** -0.5, out)
+    exp = oracle.draft(*(t.cpu().numpy() for t in desc), float(np.float32(0.2)), float(np.float32(d ** -0.5)))
+    assert np.allclose(out.cpu().numpy(), exp, rtol=2e-5, atol=1e-12)
