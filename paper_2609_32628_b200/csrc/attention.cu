@@ -70,7 +70,6 @@ constexpr int kMmaWarp0 = kSoftmaxWarps + kCorrWarps;     // Q K^T issue for str
 constexpr int kPvWarp0 = kMmaWarp0 + 2;                   // V^T P^T issue for stream 0, 1
 constexpr int kLoadWarp0 = kPvWarp0 + 2;                  // K loaders for stream 0, 1, then V loaders
 constexpr int NT = (kLoadWarp0 + 4) * 32;                 // 1024
-constexpr int kSms = 148;
 constexpr uint32_t kTmemCols = 512;
 // TMEM column map
 __host__ __device__ constexpr uint32_t col_s(int s, int buf) { return (uint32_t)(s * 2 + buf) * 64u; }
@@ -210,18 +209,8 @@ __device__ __forceinline__ float lg2(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// packed pairs of fp32 (two lanes per instruction on this architecture) and a three-input maximum
-__device__ __forceinline__ uint64_t f2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
+// the packed pairs of da2_internal.cuh taken apart and added; a three-input maximum, a minimum that keeps a NaN
 __device__ __forceinline__ void unf2(uint64_t x, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(x)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -235,11 +224,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 __device__ __forceinline__ float min_nan(float a, float b) {
   float r;
   asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 // eight accumulator columns of one channel times the columns' factors (and the channel's change of unit)
@@ -270,23 +254,6 @@ __device__ __forceinline__ uint32_t pack_e4m3x2(float lo, float hi) {
   uint16_t r;
   asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return (uint32_t)r;
-}
-// four floats -> four E4M3 codes, eight floats -> eight E2M1 codes (the first in the low bits): one assembly block each, so
-// that the narrow results are merged by the conversions themselves and not by separate shifts and permutes
-__device__ __forceinline__ uint32_t pack_e4m3x4(const float *x) {
-  uint32_t r;
-  asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
-      : "=r"(r)
-      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]));
-  return r;
-}
-__device__ __forceinline__ uint32_t pack_e2m1x8(const float *x) {
-  uint32_t r;
-  asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
-      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
-      : "=r"(r)
-      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]));
-  return r;
 }
 // two E4M3 codes -> two floats
 __device__ __forceinline__ void decode_e4m3x2(uint32_t codes, float &lo, float &hi) {

@@ -14,6 +14,8 @@ constexpr int kTile = 8;
 constexpr int kSfAtomBytes = 512;  // one scale-factor atom: 128 rows x 4 groups of E4M3 codes
 
 // device status word values (workspace off_status[0])
+constexpr int kSms = 148;  // streaming multiprocessors of a B200: splits and waves of blocks are counted in them
+
 constexpr int kDevOk = 0;
 constexpr int kDevTimeout = 1;
 constexpr int kDevBadList = 2;
@@ -108,6 +110,42 @@ __host__ __device__ inline long long slot_token(const Params &p, int a, int j) {
 __host__ __device__ inline int rec_blocks(const Params &p, int tier) { return tier == 2 ? p.Rt : p.R; }
 
 #ifdef __CUDACC__
+__device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+// packed pairs of fp32 (two lanes per instruction on this architecture)
+__device__ __forceinline__ uint64_t f2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// four floats -> four E4M3 codes, eight floats -> eight E2M1 codes (round to nearest even, saturating; the first in the low
+// bits): one assembly block each, so that the narrow results are merged by the conversions themselves and not by separate
+// shifts and permutes
+__device__ __forceinline__ uint32_t pack_e4m3x4(const float *x) {
+  uint32_t r;
+  asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
+      : "=r"(r)
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]));
+  return r;
+}
+__device__ __forceinline__ uint32_t pack_e2m1x8(const float *x) {
+  uint32_t r;
+  asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
+      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
+      : "=r"(r)
+      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]));
+  return r;
+}
 // Largest magnitudes of bf16 pairs, half by half: max(|m|, |a|).  The signs of the result are left over (clear them with
 // magnitudes2); a NaN loses against every number, so that it stays out of the statistics that scales are derived from.
 __device__ __forceinline__ uint32_t max_abs2(uint32_t m, uint32_t a) {

@@ -21,8 +21,6 @@ namespace {
 
 constexpr int kPoolWarps = 8;
 
-__device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   uint32_t r;
   asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
@@ -194,7 +192,7 @@ cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bflo
                         cudaStream_t st, int *launches) {
   // warps per block: one where the blocks alone give every SM about 16 warps, else up to all eight
   const long long blocks = (long long)p.R * p.BH;
-  const int split = blocks >= 148 * 16 ? 1 : (blocks >= 148 * 4 ? 4 : 8);
+  const int split = blocks >= kSms * 16 ? 1 : (blocks >= kSms * 4 ? 4 : 8);
   const dim3 grid((p.R * split + kPoolWarps - 1) / kPoolWarps, p.BH);
   const uint16_t *q16 = reinterpret_cast<const uint16_t *>(q), *k16 = reinterpret_cast<const uint16_t *>(k),
                  *v16 = reinterpret_cast<const uint16_t *>(v);

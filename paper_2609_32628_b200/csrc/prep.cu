@@ -36,8 +36,7 @@ __device__ __forceinline__ float decode_e4m3(uint32_t c) {
   const __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)c, __NV_E4M3);
   return __half2float(*reinterpret_cast<const __half *>(&h));
 }
-// four ints -> four int8 codes; four floats -> four E4M3 codes; eight floats -> eight E2M1 codes (round to nearest even,
-// saturating; the first in the low bits)
+// four ints -> four int8 codes (saturating; the first in the low bits)
 __device__ __forceinline__ uint32_t pack_s8x4(int c0, int c1, int c2, int c3) {
   uint32_t r;
   asm("{ .reg .b32 t; cvt.pack.sat.s8.s32.b32 t, %4, %3, 0; cvt.pack.sat.s8.s32.b32 %0, %2, %1, t; }"
@@ -45,39 +44,6 @@ __device__ __forceinline__ uint32_t pack_s8x4(int c0, int c1, int c2, int c3) {
       : "r"(c0), "r"(c1), "r"(c2), "r"(c3));
   return r;
 }
-__device__ __forceinline__ uint32_t pack_e4m3x4(const float *x) {
-  uint32_t r;
-  asm("{ .reg .b16 a, b; cvt.rn.satfinite.e4m3x2.f32 a, %2, %1; cvt.rn.satfinite.e4m3x2.f32 b, %4, %3; mov.b32 %0, {a, b}; }"
-      : "=r"(r)
-      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]));
-  return r;
-}
-__device__ __forceinline__ uint32_t pack_e2m1x8(const float *x) {
-  uint32_t r;
-  asm("{ .reg .b8 a, b, c, d; cvt.rn.satfinite.e2m1x2.f32 a, %2, %1; cvt.rn.satfinite.e2m1x2.f32 b, %4, %3; "
-      "cvt.rn.satfinite.e2m1x2.f32 c, %6, %5; cvt.rn.satfinite.e2m1x2.f32 d, %8, %7; mov.b32 %0, {a, b, c, d}; }"
-      : "=r"(r)
-      : "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]), "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7]));
-  return r;
-}
-// packed pairs of fp32
-__device__ __forceinline__ uint64_t f2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ float bf16lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 
 // Correctly rounded x / d for many x and one positive divisor d, without a division per element: with r = RN(1/d),
 // q0 = RN(x r), e = q0 d - x (exact in one fused multiply-add) and q = RN(q0 - e r) is the correctly rounded quotient
@@ -419,7 +385,7 @@ __global__ void selfcheck_round_kernel(unsigned long long *bad_out) {
 cudaError_t launch_quantiser_selfcheck(int mode, int n_divisors, uint32_t seed, unsigned long long *out, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(out, 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
-  if (mode == 2) selfcheck_round_kernel<<<148 * 8, 256, 0, st>>>(out);
+  if (mode == 2) selfcheck_round_kernel<<<kSms * 8, 256, 0, st>>>(out);
   else selfcheck_quotient_kernel<<<(n_divisors + 127) / 128, 128, 0, st>>>(n_divisors, mode == 1, seed, out);
   return cudaGetLastError();
 }

@@ -681,7 +681,7 @@ cudaError_t launch_rank(const Params &p, cudaStream_t st, int *launches) {
   e = launch_map_rows(p, st, launches);
   if (e != cudaSuccess) return e;
   // about eight CTAs an SM share the scores of all heads; a share is at least one pass of the CTA's threads
-  const long long M = (long long)p.R * p.R, most = (M + 4 * NT - 1) / (4 * NT), fair = (148 * 8 + p.BH - 1) / p.BH;
+  const long long M = (long long)p.R * p.R, most = (M + 4 * NT - 1) / (4 * NT), fair = (kSms * 8 + p.BH - 1) / p.BH;
   const dim3 shares((unsigned)(most < fair ? most : fair), p.BH), rows((p.R + kRowWarps - 1) / kRowWarps, p.BH);
   auto next = [&](auto kernel, dim3 grid, int threads) {  // enqueued only if the one before was
     if (e == cudaSuccess) e = launch_chained(kernel, grid, threads, 0, st, p);
