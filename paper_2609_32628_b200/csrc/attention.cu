@@ -7,8 +7,8 @@
 // the accumulator only changes units (Eq. "precision-state-conversion"), and the output is normalised once.
 //
 // Mapping onto sm_100a
-//   A CTA owns two neighbouring query blocks ("streams" 0 and 1; a call whose blocks are no more than the SMs gives each
-//   block its own CTA) and 1024 threads in six roles, with four softmax sets:
+//   A CTA owns two neighbouring query blocks ("streams" 0 and 1; in the last wave of CTAs, if its blocks are no more than the
+//   SMs, each block has its own) and 1024 threads in six roles, with four softmax sets:
 //     warps 0..15     softmax, set k = warp/4 takes the steps i = k (mod 4); inside a set stream = (warp%4)/2 and one
 //                     thread owns one full 64-key row.  A thread reads its S row from TMEM, takes the running maximum
 //                     of step i-1 from the thread of the previous set through a shared-memory word tagged with the
@@ -40,13 +40,14 @@
 //                   kind::mxf4nvf4 with E4M3 scales per 16 elements (NVFP4), scale factors moved by tcgen05.cp.
 // What bounds it: the chain of hand-offs of one stream's step (scores ready -> registers -> maximum -> weights -> barrier ->
 // correction -> product -> P slot free), not the tensor pipe and not the special-function unit: a step of a CTA takes about
-// 1,000 cycles with two streams and still about 900 with one.  So the work inside the chain is kept short: the row maximum
+// 900 cycles with two streams (40 heads of 1,260 blocks); of 144 lists of 144 entries in one wave, their start and end
+// included, 820 with two and 720 with one.  So the work inside the chain is kept short: the row maximum
 // is taken on raw accumulator values, the scale and the maximum are folded into one packed FMA feeding ex2, the NVFP4 group
 // scale is folded into the exponent so the scaled weight needs no extra multiply, narrow weights are packed by the
 // conversions themselves, and the exponentiate phase runs over the whole row in batches (all arguments, all exponentials,
 // then sums and packing), which gives the single warp the instruction-level parallelism it lacks when the three are
 // interleaved per pair.  And the code is kept small: the hot code of all roles shares a 32 KB instruction cache, and the
-// all-4-bit call follows its hit rate (99.9 % 13.5 ms, 99.0 % 13.8, 97.6 % 14.4, 93.8 % 15.1).
+// all-4-bit call followed its hit rate (99.9 % 13.5 ms, 99.0 % 13.8, 97.6 % 14.4, 93.8 % 15.1; it has come to 12.5 since).
 // Measured (kernel alone, ms; before the packed conversions, the smaller code, four sets for every plan, the shorter start
 // and end of a CTA and the shorter step -> now):  wan14b_720p 69.3 -> 60.0;  wan1p3b_480p 3.52 -> 2.92;  with a 226-token
 // prefix, whose blocks are bf16 (two softmax sets before), 4.55 -> 3.90.
@@ -265,7 +266,7 @@ __device__ __forceinline__ void decode_e4m3x2(uint32_t codes, float &lo, float &
 // bounded wait that also gives up as soon as another thread of the CTA has flagged a failure
 // (the flag then holds 1 + the shared-memory offset of the barrier that was never completed, for diagnosis)
 //
-// A plain mbarrier.try_wait blocks in hardware for a while (about 4 us here) before it reports failure, so the retry loop
+// A plain mbarrier.try_wait blocks in hardware for a while (7,760 cycles, about 4 us) before it reports failure, so the retry loop
 // issues next to nothing.  The bound is on elapsed clock cycles.  Barriers are named by their shared-memory address, and
 // the loop is kept short: every wait is a copy of it, and the hot code of all roles shares a 32 KB instruction cache.
 constexpr uint32_t kWaitLimitCycles = 400000000u;  // about 0.2 s
@@ -392,8 +393,8 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + sm.bars);
   const uint32_t bars0 = tc::smem_u32(bars);
   auto bar = [&](int s, int which) -> uint32_t { return bars0 + (uint32_t)(s * B_COUNT + which) * 8u; };
-  float *s_factor = reinterpret_cast<float *>(smem + sm.factor);      // [s][set][64]
-  uint32_t *s_chg = reinterpret_cast<uint32_t *>(smem + sm.chg);      // [s][set][2]
+  float *s_factor = reinterpret_cast<float *>(smem + sm.factor);      // [s][kStepBars][64]
+  uint32_t *s_chg = reinterpret_cast<uint32_t *>(smem + sm.chg);      // [s][kStepBars][2]
   uint2 *s_hx = reinterpret_cast<uint2 *>(smem + sm.hx);              // [s][set][64]
   float *s_href = reinterpret_cast<float *>(smem + sm.href);          // [s][set][64]
   float *s_ell = reinterpret_cast<float *>(smem + sm.ell);            // [s][set][64]
@@ -1067,9 +1068,7 @@ __global__ void bounded_wait_probe_kernel(int *status, uint32_t limit) {
 }  // namespace
 
 cudaError_t launch_bounded_wait_probe(int *status, long long limit_cycles, cudaStream_t st) {
-  // the wait counts on a 32-bit clock, which a limit close to its range might never be seen to pass
-  const long long limit = limit_cycles < 0 ? 0 : (limit_cycles > 4000000000LL ? 4000000000LL : limit_cycles);
-  bounded_wait_probe_kernel<<<1, 32, 0, st>>>(status, (uint32_t)limit);
+  bounded_wait_probe_kernel<<<1, 32, 0, st>>>(status, (uint32_t)limit_cycles);  // 1 .. 2e9: well inside the 32-bit clock's range
   return cudaGetLastError();
 }
 

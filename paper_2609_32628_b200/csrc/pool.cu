@@ -9,7 +9,7 @@
 // fill the GPU, up to 8 for the smallest calls, whose time is the latency of one block); only their results are combined.
 // HBM-bound: reads Q, K, V once (3*N*d*2 bytes per head), writes 4*R*d*4 bytes.
 // Measured: 40 heads x 75,600 tokens (2.42 GB) 0.94 -> 0.41 ms, 5.9 TB/s (before: a CTA per block, sums across threads through
-// shared memory, scales in a launch of their own); 24 heads x 8,192 tokens 72 -> 46 us.
+// shared memory, scales in a launch of their own); 24 heads x 8,192 tokens 72 -> 43 us.
 //
 // Sums are carried in fp64: a sum of at most 64 bf16 values is exact there, so the fp32 descriptor equals the
 // correctly rounded mean regardless of summation order.

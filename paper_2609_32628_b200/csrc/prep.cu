@@ -11,9 +11,10 @@
 // HBM would allow it in half the time it takes: what bounds it is the integer and conversion work per element.  So every
 // thread takes its 32 channels of a row (Q, K) or 16 slots of two channels (V) out of shared memory once and makes the
 // codes of all formats from those registers, in packed pairs where an instruction for pairs exists, and the block needs
-// three barriers in all.
-// Measured: 40 heads x 75,600 tokens (4.31 GB read and written) 1.41 -> 1.08 ms, 4.0 TB/s; 24 heads x 8,192 tokens 95 -> 75 us
-// (before: a thread per 16 channels and format, quotients and casts one by one, a barrier per format).
+// two barriers in all.
+// Measured: 40 heads x 75,600 tokens (4.31 GB read and written) 1.41 -> 1.08 ms, 4.0 TB/s; 24 heads x 8,192 tokens 95 -> 73 us
+// (before: a thread per 16 channels and format, quotients and casts one by one, a barrier per format); 12 heads x 32,760 tokens
+// 166 us (176 with the maxima taken on masked magnitudes as integers, which also let a NaN win).
 #include <cuda_fp8.h>
 
 #include "da2_internal.cuh"

@@ -166,7 +166,8 @@ __device__ __forceinline__ int tier_of(uint32_t key, const Boundary *bd, const i
 // hits the quota exactly ends the search (about log2(R) + 2 steps; only ties need all of them).  No barrier and no shared
 // memory: the CTA version spends 32 barriers a row, and its 12 histogram passes three times the instructions
 // (R = 1260, two boundaries).  Bound by instruction issue: the exponentials of both branches, the bisection, the prefix counts.
-// Measured: 40 heads, R = 1260 1.05 -> 0.51 ms; 12 heads, R = 588 115 -> 27 us; 24 heads, R = 128 38 -> 6 us.
+// Measured (kernel alone, cold cache): 40 heads, R = 1260 1.05 -> 0.84 ms; 12 heads, R = 588 115 -> 42 us; 24 heads, R = 128
+// 38 -> 7 us.
 struct Cut { int value, take; };  // admitted: keys above value, and the first `take` keys equal to it
 
 template <int E> __device__ __forceinline__ int count_at_least(const int (&key)[E], int t) {
