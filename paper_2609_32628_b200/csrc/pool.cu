@@ -5,14 +5,16 @@
 //
 // A block is an 8 x 8 tile of one frame (or a run of 64 tokens).  A warp walks tokens of one block and every lane owns
 // D / 32 channels of it, so a token row is one coalesced load and sums and maxima stay in registers from the first token
-// to the last: no shuffles and no shared memory per block.  SPLIT warps share a block (1 where there are enough blocks to
-// fill the GPU, up to 8 for the smallest calls, whose time is the latency of one block); only their results are combined.
+// to the last: no shuffles and no shared memory per block.  SPLIT warps share a block (1, 2, 4 or 8 by the waves that the
+// blocks make, see launch_pool); only their results are combined.
 // HBM-bound: reads Q, K, V once (3*N*d*2 bytes per head), writes 4*R*d*4 bytes.
 // Measured: 40 heads x 75,600 tokens (2.42 GB) 0.94 -> 0.41 ms, 5.9 TB/s (before: a CTA per block, sums across threads through
-// shared memory, scales in a launch of their own); 24 heads x 8,192 tokens 72 -> 43 us.
+// shared memory, scales in a launch of their own); 24 heads x 8,192 tokens 72 -> 38 us.
 //
 // Sums are carried in fp64: a sum of at most 64 bf16 values is exact there, so the fp32 descriptor equals the
 // correctly rounded mean regardless of summation order.
+#include <type_traits>
+
 #include "da2_internal.cuh"
 
 namespace da2 {
@@ -20,6 +22,7 @@ namespace da2 {
 namespace {
 
 constexpr int kPoolWarps = 8;
+constexpr int kBatch = 8;  // tokens whose loads are in flight together
 
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   uint32_t r;
@@ -46,7 +49,7 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
   constexpr int W = D / 64;                  // words (channel pairs) per lane
   constexpr int BLOCKS = kPoolWarps / SPLIT;  // blocks per CTA
   constexpr int TOK = kSlots / SPLIT;        // tokens per warp
-  constexpr int BATCH = 8;                   // tokens whose loads are in flight together
+  constexpr int BATCH = kBatch;
   const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int a = blockIdx.x * BLOCKS + warp / SPLIT, part = warp % SPLIT;
   const bool live = a < p.R;
@@ -190,16 +193,33 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
 
 cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                         cudaStream_t st, int *launches) {
-  // warps per block: one where the blocks alone give every SM about 16 warps, else up to all eight
+  // Warps per block.  A few blocks an SM: up to all eight, the call is the latency of one block.  Else the number with the
+  // shortest waves: an SM holds two CTAs at d = 128 and three at d = 64 (registers); a wave lasts the batches of loads that a
+  // warp walks one after the other, and start, combination and atomics cost about three more.  So a last wave that would be
+  // nearly empty is made shorter instead.  (da2_prepare, us, with the split by the number of blocks alone, 4 below 2,368, else
+  // 1 -> now; d = 128, 128 blocks a head: 8 heads 63.6 -> 59.7, 12 heads 86.4 -> 80.0, 17 heads 113.5 -> 102.5, 24 heads
+  // 143.3 -> 138.3; d = 64, 8 heads of 168 blocks 53.2 -> 51.0.  Below 6 blocks an SM the waves do not decide: 5 heads of 128
+  // blocks 48.6 with four warps, 54.2 with two, although those pool faster.)
   const long long blocks = (long long)p.R * p.BH;
-  const int split = blocks >= kSms * 16 ? 1 : (blocks >= kSms * 4 ? 4 : 8);
+  int split = blocks >= kSms * 4 ? 4 : 8;
+  if (blocks >= kSms * 6) {
+    const long long wave = (long long)kSms * (p.d == 128 ? 2 : 3);
+    long long best = 0;
+    for (int s = 1; s <= 4; s *= 2) {
+      const long long ctas = (long long)p.BH * ((p.R * s + kPoolWarps - 1) / kPoolWarps);
+      const long long cost = (ctas + wave - 1) / wave * (kSlots / kBatch / s + 3);
+      if (s == 1 || cost < best) { best = cost; split = s; }
+    }
+  }
   const dim3 grid((p.R * split + kPoolWarps - 1) / kPoolWarps, p.BH);
   const uint16_t *q16 = reinterpret_cast<const uint16_t *>(q), *k16 = reinterpret_cast<const uint16_t *>(k),
                  *v16 = reinterpret_cast<const uint16_t *>(v);
   auto launch = [&](auto kernel) { return launch_chained(kernel, grid, kPoolWarps * 32, 0, st, p, q16, k16, v16); };
-  cudaError_t e;
-  if (p.d == 128) e = split == 1 ? launch(pool_kernel<128, 1>) : (split == 4 ? launch(pool_kernel<128, 4>) : launch(pool_kernel<128, 8>));
-  else e = split == 1 ? launch(pool_kernel<64, 1>) : (split == 4 ? launch(pool_kernel<64, 4>) : launch(pool_kernel<64, 8>));
+  auto pick = [&](auto dtag) -> cudaError_t {
+    constexpr int D = decltype(dtag)::value;
+    return split == 1 ? launch(pool_kernel<D, 1>) : (split == 2 ? launch(pool_kernel<D, 2>) : (split == 4 ? launch(pool_kernel<D, 4>) : launch(pool_kernel<D, 8>)));
+  };
+  const cudaError_t e = p.d == 128 ? pick(std::integral_constant<int, 128>{}) : pick(std::integral_constant<int, 64>{});
   *launches += 1;
   return e;
 }

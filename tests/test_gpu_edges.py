@@ -65,6 +65,16 @@ def test_pooling_splits(H):
     _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
 
 
+# 80 blocks a head: 4, 2 and 1 warps per block at d = 128; 8, 4, 2 and 1 at d = 64
+@pytest.mark.parametrize("H,d", [(8, 128), (12, 128), (20, 128), (5, 64), (8, 64), (20, 64), (30, 64)])
+def test_pooling_by_waves(H, d):
+    w = W("pool", 1, H, d, 5, 27, 30, 0.1, 0.2, 0.2, seed=36)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, _ = run_gpu(w, q, k, v)
+    heads = sorted({0, H - 1})
+    _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
+
+
 @pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (3, 9, 20), (13, 8, 40), (23, 24, 56), (683, 8, 24)])
 @pytest.mark.parametrize("f16,f8,f4", [(0.1, 0.2, 0.3), (0.0, 0.1, 0.2)])
 def test_head_scope_sizes(T, Hg, Wg, f16, f8, f4):
