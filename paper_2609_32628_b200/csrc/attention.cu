@@ -28,8 +28,9 @@
 //                     issues), operand descriptors are built once and only offset inside the loop
 //     last 4 warps    loaders: per stream one warp for K (and the Q records) and one for V^T, 1-D bulk copies into
 //                     rings of their own (a K block is needed as soon as a score buffer is free, a V block only after
-//                     the step's weights are written, so the V ring is the deeper one); lane l holds list entry
-//                     32*batch + l (address, mask, key scale)
+//                     the step's weights are written, so the V ring is the deeper one); a ring entry takes two blocks of
+//                     the list under one barrier (one of the 16-bit tier); lane l holds list entry 32*batch + l
+//                     (address, mask, key scale)
 //   S   = Q K^T   : M = 128, N = 64 keys, K = d.  The block-scaled instruction only exists at M = 128, so stream 0's
 //                   queries sit in rows 0..63 and stream 1's in rows 64..127 (its operand descriptor starts 1 KB
 //                   early); the other 64 rows of each product are don't-care.  S is double buffered.
@@ -38,19 +39,23 @@
 //                   per-channel unit changes (eta*delta_c^V, g_V/2688) per-lane scalars.
 //   kinds         : kind::f16 (BF16); kind::i8 for QK^T + kind::f8f6f4 E4M3 x E4M3 for PV (App. C.1); and
 //                   kind::mxf4nvf4 with E4M3 scales per 16 elements (NVFP4), scale factors moved by tcgen05.cp.
-// What bounds it: the chain of hand-offs of one stream's step (scores ready -> registers -> maximum -> weights -> barrier ->
-// correction -> product -> P slot free), not the tensor pipe and not the special-function unit: a step of a CTA takes about
-// 900 cycles with two streams (40 heads of 1,260 blocks); of 144 lists of 144 entries in one wave, their start and end
-// included, 820 with two and 720 with one.  So the work inside the chain is kept short: the row maximum
+// What bounds it: the fetch of instructions.  Eight warps of a scheduler are at eight places of the code, so that nearly every
+// line comes from the SM's instruction cache (32 KB, shared by all roles), and its request rate was 94 % of the peak (all-4-bit
+// call of 16x48x48, 24 heads; special-function pipe 70 %, issue slots 69 %, tensor pipe 22 %): the time followed the requests in
+// every variant that was tried.  So the instructions of a step are what is saved, in the roles around the softmax above all, a
+// quarter of them: the loaders, the Q K^T warps and the PV warps take the blocks of a list in pairs, with one ring entry, one
+// wait and one round of the loop for two, and run along the rings by increments (requests 1.59 -> 1.29 G, 80 % of the peak rate;
+// 12.53 -> 11.9 ms).  Taking PV and correction in pairs as well makes the products late (13.3 ms), and softmax steps of two
+// blocks need fewer instructions still (7.3 instead of 8.6 G) but leave two warps a scheduler, too few (13.7 ms).
+// The softmax keeps the work inside the chain of hand-offs short: the row maximum
 // is taken on raw accumulator values, the scale and the maximum are folded into one packed FMA feeding ex2, the NVFP4 group
 // scale is folded into the exponent so the scaled weight needs no extra multiply, narrow weights are packed by the
 // conversions themselves, and the exponentiate phase runs over the whole row in batches (all arguments, all exponentials,
 // then sums and packing), which gives the single warp the instruction-level parallelism it lacks when the three are
-// interleaved per pair.  And the code is kept small: the hot code of all roles shares a 32 KB instruction cache, and the
-// all-4-bit call followed its hit rate (99.9 % 13.5 ms, 99.0 % 13.8, 97.6 % 14.4, 93.8 % 15.1; it has come to 12.5 since).
-// Measured (kernel alone, ms; before the packed conversions, the smaller code, four sets for every plan, the shorter start
-// and end of a CTA and the shorter step -> now):  wan14b_720p 69.3 -> 60.0;  wan1p3b_480p 3.52 -> 2.92;  with a 226-token
-// prefix, whose blocks are bf16 (two softmax sets before), 4.55 -> 3.90.
+// interleaved per pair.  And the code is kept small: beyond about 47 KB in all the hits fall (99.9 % 11.9 ms, 99.0 % 12.0 to
+// 12.1 with the same instructions; 97.6 % 14.4 and 93.8 % 15.1 in earlier states).
+// Measured (kernel alone, ms, before -> with pairs):  12 heads of 32,760 tokens 2.92 -> 2.77, one ranking per head 2.91 -> 2.79,
+// with a 226-token prefix, whose blocks are bf16, 3.91 -> 3.67;  24 heads of 36,864 tokens all in 8 bit at d = 64 11.79 -> 10.8.
 // Every wait on an mbarrier is bounded; a wait that gives up records device status "timeout", all roles leave their
 // loops and the CTA exits normally after releasing TMEM.
 #include <type_traits>
@@ -88,7 +93,7 @@ constexpr float kOffsetP8 = 8.807f;      // base-2 exponent offset (about log2 4
 // barrier indices inside one stream's group
 // (a parity wait can only tell the latest completion from the one before, so every barrier is laid out such that no
 // waiter can fall two completions behind: buffers indexed by step parity get one barrier per buffer)
-constexpr int kMaxK = 6, kMaxV = 8, kInfoRing = 16;  // (steps between a K request and its scores: at most nk + 2)
+constexpr int kMaxK = 3, kMaxV = 4, kInfoRing = 16;  // (steps between a K request and its scores: at most 2 nk + 3)
 // barriers, factors, ballots and scale atoms of the steps between softmax and product (kSets of them unless SEGMENTED, where a
 // softmax warp may wait for the last product of the segment before: twice as many keep that use the barrier's latest)
 constexpr int kStepBars = 8;
@@ -98,17 +103,18 @@ enum {
   B_ELL = B_PVDONE + kStepBars, B_Q = B_ELL + 1, B_COUNT = B_Q + 1
 };
 
-// Shared memory.  The operand rings and the P slots hold blocks of one size (the largest of the plan's tiers) and the Q
-// records of all tiers are resident, if that leaves rings of at least 2 K and 3 V blocks.  Otherwise (a 16-bit tier at
-// head_dim 128: 16 KB blocks, 8 KB P images) the layout is SEGMENTED: every segment cuts the same bytes into blocks of its
-// own tier, so that only the 16-bit segment has shallow rings, and a stream has one Q buffer, reloaded at the segment
-// boundary.  The price is a drain of the rings at each boundary (about 1.5 us a row).
+// Shared memory.  An entry of the operand rings holds two consecutive blocks of a list, or one of the 16-bit tier (which is
+// about as large as two of the others): one wait, one barrier and one round of a loader's loop for both.  The Q records of the
+// 4- and the 8-bit tier are resident; that of the 16-bit tier takes their place when its segment starts.
+// With a 16-bit tier at head_dim 128 (8 KB P images) the layout is SEGMENTED: every segment cuts the bytes of the P slots into
+// slots of its own tier, four, four and two.
 struct SmemMap {
-  uint32_t q[2][3];               // Q record per stream and tier (SEGMENTED: the same buffer for every tier)
+  uint32_t q[2][3];               // Q record per stream and tier
   uint32_t kring[2], vring[2];    // per stream: K blocks (K image + scale atoms), V blocks (V^T image + scale atom)
   uint32_t kbytes[3], vbytes[3];  // bytes to copy per block
-  uint32_t kstage[3], vstage[3];  // bytes per ring entry
-  int nk[3], nv[3];               // ring entries
+  uint32_t kstage, vstage;        // from the first block of a ring entry to the second
+  uint32_t kentry, ventry;        // bytes of a ring entry
+  int nk, nv;                     // ring entries
   uint32_t p[2];                  // P operand images per stream
   uint32_t pbytes[3];             // bytes of a P slot (there are four, or SEGMENTED 4, 4, 2)
   uint32_t sfp[2];    // P scale atoms (512 B), one per step barrier
@@ -140,20 +146,25 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   uint32_t cur = 0;
   auto r128 = [](uint32_t b) { return (b + 127u) / 128u * 128u; };
   auto take = [&](uint32_t bytes) { uint32_t o = cur; cur = r128(cur + bytes); return o; };
-  uint32_t qmax = 0, kmax = 0, vmax = 0, pmax = 0;
+  uint32_t qlow = 0, pmax = 0;
+  m.kstage = m.vstage = m.kentry = m.ventry = 0;
   for (int t = 0; t < 3; ++t) {
     m.kbytes[t] = p.qrec_bytes[t];                     // the K part of a record is laid out like a Q record
     m.vbytes[t] = p.kvrec_bytes[t] - p.qrec_bytes[t];
     if (!p.tier_active[t]) continue;
-    qmax = max(qmax, p.qrec_bytes[t]);
-    kmax = max(kmax, r128(m.kbytes[t]));
-    vmax = max(vmax, r128(m.vbytes[t]));
     pmax = 2048u << t;
+    if (t < 2) {
+      m.kstage = max(m.kstage, r128(m.kbytes[t]));
+      m.vstage = max(m.vstage, r128(m.vbytes[t]));
+      qlow += r128(p.qrec_bytes[t]);
+    }
+    m.kentry = max(2 * m.kstage, t < 2 ? 0u : r128(m.kbytes[t]));
+    m.ventry = max(2 * m.vstage, t < 2 ? 0u : r128(m.vbytes[t]));
   }
   // stream 1's Q descriptors start 1 KB before its images: stream 0's records precede them, so that is valid memory
   for (int s = 0; s < 2; ++s) {
-    const uint32_t one = segmented ? take(qmax) : 0;
-    for (int t = 0; t < 3; ++t) m.q[s][t] = segmented ? one : (p.tier_active[t] ? take(p.qrec_bytes[t]) : 0);
+    m.q[s][0] = m.q[s][2] = take(p.tier_active[2] ? max(qlow, p.qrec_bytes[2]) : qlow);
+    m.q[s][1] = m.q[s][0] + (p.tier_active[0] ? r128(p.qrec_bytes[0]) : 0u);
   }
   const uint32_t pregion = segmented ? 16384u : kSets * pmax;  // per stream
   const uint32_t fixed = 2 * (pregion + kStepBars * 512) + r128(2 * kStepBars * 64 * 4) + 2 * r128(2 * kSets * 64 * 4) +
@@ -163,27 +174,16 @@ __host__ SmemMap make_smem_map(const Params &p, bool segmented) {
   const uint32_t left = cur + fixed < kLimit ? (kLimit - cur - fixed) / 256u * 128u : 0u;  // ring bytes per stream
   // a K block is consumed as soon as a score buffer is free (two per stream), a V block only after the weights of
   // its step are written: the V ring is the deep one
-  uint32_t kring = 2 * kmax, vring = 2 * vmax;
-  m.fits = kring + vring <= left;
-  if (segmented) {
-    if (m.fits) vring = left - kring;
-  } else {
-    const int cand[5][2] = {{3, 6}, {3, 5}, {3, 4}, {2, 4}, {2, 3}};
-    m.fits = false;
-    for (int c = 0; c < 5 && !m.fits; ++c) {
-      kring = cand[c][0] * kmax; vring = cand[c][1] * vmax;
-      m.fits = kring + vring <= left;
-    }
+  const int cand[5][2] = {{3, 4}, {3, 3}, {2, 3}, {2, 2}, {1, 2}};
+  m.fits = false;
+  for (int c = 0; c < 5 && !m.fits; ++c) {
+    m.nk = cand[c][0];
+    m.nv = cand[c][1];
+    m.fits = m.nk * m.kentry + m.nv * m.ventry <= left;
   }
-  for (int t = 0; t < 3; ++t) {
-    m.kstage[t] = segmented ? r128(m.kbytes[t]) : kmax;
-    m.vstage[t] = segmented ? r128(m.vbytes[t]) : vmax;
-    m.pbytes[t] = segmented ? 2048u << t : pmax;
-    m.nk[t] = m.kstage[t] ? min(kMaxK, (int)(kring / m.kstage[t])) : 1;
-    m.nv[t] = m.vstage[t] ? min(kMaxV, (int)(vring / m.vstage[t])) : 1;
-  }
-  for (int s = 0; s < 2; ++s) m.kring[s] = take(kring);
-  for (int s = 0; s < 2; ++s) m.vring[s] = take(vring);
+  for (int t = 0; t < 3; ++t) m.pbytes[t] = segmented ? 2048u << t : pmax;
+  for (int s = 0; s < 2; ++s) m.kring[s] = take(m.nk * m.kentry);
+  for (int s = 0; s < 2; ++s) m.vring[s] = take(m.nv * m.ventry);
   for (int s = 0; s < 2; ++s) m.p[s] = take(pregion);
   for (int s = 0; s < 2; ++s) m.sfp[s] = take(kStepBars * 512);
   m.factor = take(2 * kStepBars * 64 * 4);
@@ -279,12 +279,11 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, int
                                               uint32_t limit = kWaitLimitCycles) {
   if (tc::mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = clock32();
-  for (;;) {
+#pragma unroll 1
+  do {
     if (tc::mbar_try_wait(bar, parity)) return true;
-    if (*(volatile int *)abort_flag) return false;
-    if (clock32() - t0 > limit) break;
-  }
-  atomicCAS(abort_flag, 0, 1 + (int)(bar & 0xffffu));
+  } while (!*(volatile int *)abort_flag && clock32() - t0 <= limit);
+  if (!*(volatile int *)abort_flag) *(volatile int *)abort_flag = 1 + (int)(bar & 0xffffu);
   return false;
 }
 
@@ -447,7 +446,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
 
     const uint32_t s_col = tmem + lane_addr + col_s(s, set & 1);  // (i and set have the same parity)
     for (int i = set; i < S.L; i += kSets) {
-      const int tier = S.tier(i);
+      const int tier = B16 ? S.tier(i) : (FP4 && i < S.n4 ? 0 : 1);
       const int g = SEGMENTED ? i & kStepMask : set;  // barriers, factors, ballots, scale atom
       // the step's P slot, and the product that last used it: step i - 4, or i - 2 in the 16-bit segment of a SEGMENTED plan,
       // where the first steps of every segment also wait for the last product of the segment before, whose slots were cut
@@ -612,20 +611,20 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         // A group whose scale code is 0 takes the smallest scale for u: its codes do not matter, the product multiplies
         // them by the stored scale 0, and the denominator gets w = u * sigma / 2688 either way.
         float bb[4], sl[4];
+        const uint64_t nm2 = f2(-m_new, -m_new);
         uint32_t sfw[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const float g0 = __fmul_rn(448.0f, ex2(fmaf(gm[2 * h], coef, -m_new)));
-          const float g1 = __fmul_rn(448.0f, ex2(fmaf(gm[2 * h + 1], coef, -m_new)));
-          sfw[h] = pack_e4m3x2(g0, g1);
-          float s0, s1;
+          float x0, x1, s0, s1;
+          unf2(fma2(f2(gm[2 * h], gm[2 * h + 1]), coef2, nm2), x0, x1);
+          unf2(mul2(f2(ex2(x0), ex2(x1)), f2(448.0f, 448.0f)), x0, x1);
+          sfw[h] = pack_e4m3x2(x0, x1);
           decode_e4m3x2(sfw[h], s0, s1);
           s0 = fmaxf(s0, 0.001953125f);
           s1 = fmaxf(s1, 0.001953125f);
-          bb[2 * h] = (11.392317422778762f - lg2(s0)) - m_new;  // log2(2688) = 11.3923...
-          bb[2 * h + 1] = (11.392317422778762f - lg2(s1)) - m_new;
-          sl[2 * h] = s0 * (1.0f / 2688.0f);
-          sl[2 * h + 1] = s1 * (1.0f / 2688.0f);
+          unf2(mul2(f2(s0, s1), f2(1.0f / 2688.0f, 1.0f / 2688.0f)), sl[2 * h], sl[2 * h + 1]);
+          // log2(2688) - log2(sigma) - m (log2(2688) = 11.3923...)
+          unf2(add2(fma2(f2(lg2(s0), lg2(s1)), f2(-1.0f, -1.0f), f2(11.392317422778762f, 11.392317422778762f)), nm2), bb[2 * h], bb[2 * h + 1]);
         }
         const uint32_t sfword = __byte_perm(sfw[0], sfw[1], 0x5410);
         *reinterpret_cast<uint32_t *>(sf_row0 + g * 512) = sfword;
@@ -681,19 +680,20 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
     if (S.L > 0) {
-      // Q records: of every segment at once, or (SEGMENTED) of the segment that starts, into the stream's one buffer
+      // Q records: of the 4- and the 8-bit segment at once, that of the 16-bit segment when it starts
       auto load_q = [&](int first, int last) {
         if (is_v || !tc::elect_one()) return;
         const int nn[3] = {S.n4, S.n48 - S.n4, S.L - S.n48};
         uint32_t bytes = 0;
         for (int t = first; t <= last; ++t) if (nn[t] > 0) bytes += p.qrec_bytes[t];
+        if (bytes == 0) return;
         tc::mbar_arrive_expect_tx(bar(s, B_Q), bytes);
         for (int t = first; t <= last; ++t)
           if (nn[t] > 0)
             tc::bulk_g2s(tc::smem_u32(smem + sm.q[s][t]), p.qrec[t] + ((size_t)bh * rec_blocks(p, t) + S.a) * p.qrec_bytes[t], p.qrec_bytes[t],
                          bar(s, B_Q));
       };
-      if (!SEGMENTED) load_q(0, 2);
+      load_q(0, 1);
       __syncwarp();
       const size_t head_blocks = (size_t)bh * R;
       auto checked = [&](int b) -> int {
@@ -704,90 +704,82 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       auto key_scale = [&](int idx, int b) -> float {
         return (!is_v && idx < S.L && S.tier(idx) == 1) ? p.dk8[head_blocks + b] : 0.f;
       };
-      auto record = [&](int idx, int b) -> unsigned long long {
-        const int t = S.tier(idx);
-        return reinterpret_cast<unsigned long long>(p.kvrec[t] + ((size_t)bh * rec_blocks(p, t) + b) * p.kvrec_bytes[t] +
-                                                    (is_v ? sm.kbytes[t] : 0u));
-      };
-      // batch -1 is empty: the loop's refill at "src == 31" then also serves the first batch
       int nxt_b = checked(pre0), nn_b = checked(pre1);
       float cur_dk = 0.f, nxt_dk = key_scale(lane, nxt_b);
-      unsigned long long cur_rec = 0, cur_mask = 0;
+      unsigned long long cur_mask = 0;
       uint32_t padded_lanes = 0;
       const uint32_t dst = tc::smem_u32(smem) + (is_v ? sm.vring[s] : sm.kring[s]);
       const int b_full = is_v ? B_FULLV : B_FULLK, b_free = is_v ? B_VFREE : B_KFREE;
-      const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1],
-                     nb2 = is_v ? sm.vbytes[2] : sm.kbytes[2];
-      uint32_t stage = is_v ? sm.vstage[0] : sm.kstage[0];  // bytes per ring entry
-      int depth = is_v ? sm.nv[0] : sm.nk[0];               // ring entries
-      int kk = 0;                                           // ring entry
-      uint32_t used = 0, par = 0;     // per ring entry: used so far, parity of its last use
-      uint32_t kpar = 1;              // (not SEGMENTED: parity of the consumption that frees the entry, ring gone round)
-      bool kwrapped = false, ok = true;
-      for (int i = -1; i < S.L; ++i) {
+      const uint32_t stage = is_v ? sm.vstage : sm.kstage, entry = is_v ? sm.ventry : sm.kentry;
+      const int depth = is_v ? sm.nv : sm.nk;  // ring entries
+      int kk = 0;                              // ring entry
+      uint32_t kpar = 1;                       // parity of the consumption that frees the entry
+      bool kwrapped = false, ok = true;        // ring gone round
+      // lane l holds the record's address, the mask and the key scale of list entry 32 * batch + l
+      auto record = [&](int idx, int b) -> unsigned long long {
+        const int t = S.tier(idx);
+        return reinterpret_cast<unsigned long long>(p.kvrec[t] + ((size_t)bh * rec_blocks(p, t) + b) * p.kvrec_bytes[t] + (is_v ? sm.kbytes[t] : 0u));
+      };
+      const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1], nb2 = is_v ? sm.vbytes[2] : sm.kbytes[2];
+      uint2 *const infos = s_info + s * kInfoRing;
+      unsigned long long cur_rec = 0;
+      uint32_t full = bar(s, b_full), to = dst;
+      const uint32_t to_free = (uint32_t)(b_free - b_full) * 8u;
+#pragma unroll 1
+      for (int i = 0; i < S.L;) {
         const int src = i & 31;
-        if (i >= 0) {
-        const uint32_t rlo = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src);
-        const uint32_t rhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src);
-        const uint8_t *rec = reinterpret_cast<const uint8_t *>(((unsigned long long)rhi << 32) | rlo);
-        const uint32_t nb = i < S.n4 ? nb0 : (i < S.n48 ? nb1 : nb2);
-        if (SEGMENTED) {
-          if (i == 0 || i == S.n4 || i == S.n48) {  // the ring is cut anew once every block of the segment before is consumed
-            const int t = S.tier(i);
-            for (int k = 0; ok && k < (is_v ? kMaxV : kMaxK); ++k)
-              if ((used >> k) & 1u) ok = wait_or_abort(bar(s, b_free + k), (par >> k) & 1u, abortp);
-            if (!ok) break;
-            stage = is_v ? sm.vstage[t] : sm.kstage[t];
-            depth = is_v ? sm.nv[t] : sm.nk[t];
-            kk = 0;
-            load_q(t, t);
-            __syncwarp();
-          }
-          if ((used >> kk) & 1u) {
-            if (!(ok = wait_or_abort(bar(s, b_free + kk), (par >> kk) & 1u, abortp))) break;
-            par ^= 1u << kk;
-          }
-          used |= 1u << kk;
-        } else if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) {
-          break;
-        }
-        if (!is_v) {
-          // the step's mask and key scale are written before the data the softmax waits for is requested
-          const int e = s * kInfoRing + (i & (kInfoRing - 1));
-          const bool padded = (padded_lanes >> src) & 1u;
-          if (padded) {
-            const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src);
-            const uint32_t mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src);
-            float *lim = reinterpret_cast<float *>(smem + sm.lim) + e * 64;
-            lim[lane] = (mlo >> lane) & 1u ? INFINITY : -INFINITY;
-            lim[32 + lane] = (mhi >> lane) & 1u ? INFINITY : -INFINITY;
-          }
-          if (lane == src) s_info[e] = make_uint2(__float_as_uint(cur_dk), padded);
-          __syncwarp();
-        }
-        if (tc::elect_one()) {
-          tc::mbar_arrive_expect_tx(bar(s, b_full + kk), nb);
-          tc::bulk_g2s(dst + (uint32_t)kk * stage, rec, nb, bar(s, b_full + kk));
-        }
-        __syncwarp();
-        if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
-        }
-        if (src == 31) {  // next batch: its ids and scales were requested one batch ago
+        const bool two = i + 1 < S.n48;
+        if (src == 0) {  // next batch: its ids and scales were requested one batch ago
           const int b = nxt_b;
           cur_dk = nxt_dk;
-          cur_rec = record(i + 1 + lane, b);
+          cur_rec = record(i + lane, b);
           cur_mask = is_v ? ~0ull : table_mask(p, b);
           padded_lanes = __ballot_sync(0xffffffffu, cur_mask != ~0ull);
           nxt_b = nn_b;
-          nxt_dk = key_scale(i + 33 + lane, nxt_b);
-          nn_b = list_id(i + 65 + lane);
+          nxt_dk = key_scale(i + 32 + lane, nxt_b);
+          nn_b = list_id(i + 64 + lane);
         }
+        const uint32_t lo0 = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src), hi0 = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src);
+        const uint32_t lo1 = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src + 1), hi1 = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src + 1);
+        const uint32_t n0 = B16 && i >= S.n48 ? nb2 : (FP4 && i < S.n4 ? nb0 : nb1), n1 = !two ? 0u : (FP4 && i + 1 < S.n4 ? nb0 : nb1);
+        if (B16 && i == S.n48 && !is_v) {
+          // the Q buffer is free once every product of the segments before is done: their last K blocks are consumed
+          if (i > 0 && !(ok = wait_or_abort(bar(s, B_KFREE) + (uint32_t)(kk == 0 ? depth - 1 : kk - 1) * 8u, kk == 0 ? kpar : kpar ^ 1u, abortp))) break;
+          load_q(2, 2);
+          __syncwarp();
+        }
+        if (kwrapped && !(ok = wait_or_abort(full + to_free, kpar, abortp))) break;
+        if (!is_v) {
+          // the steps' masks and key scales are written before the data the softmax waits for is requested
+          const int e = i & (kInfoRing - 1);
+          if ((padded_lanes >> src) & (two ? 3u : 1u)) {
+            float *lim = reinterpret_cast<float *>(smem + sm.lim) + (s * kInfoRing + e) * 64;
+#pragma unroll 1
+            for (int x = 0; x <= (int)two; ++x) {
+              const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src + x);
+              const uint32_t mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src + x);
+              lim[x * 64 + lane] = (mlo >> lane) & 1u ? INFINITY : -INFINITY;
+              lim[x * 64 + 32 + lane] = (mhi >> lane) & 1u ? INFINITY : -INFINITY;
+            }
+          }
+          if (lane == src || (two && lane == src + 1)) infos[lane & (kInfoRing - 1)] = make_uint2(__float_as_uint(cur_dk), cur_mask != ~0ull);
+          __syncwarp();
+        }
+        if (tc::elect_one()) {
+          tc::mbar_arrive_expect_tx(full, n0 + n1);
+          tc::bulk_g2s(to, reinterpret_cast<const uint8_t *>(((unsigned long long)hi0 << 32) | lo0), n0, full);
+          if (n1) tc::bulk_g2s(to + stage, reinterpret_cast<const uint8_t *>(((unsigned long long)hi1 << 32) | lo1), n1, full);
+        }
+        __syncwarp();
+        full += 8u;
+        to += entry;
+        i += two ? 2 : 1;
+        if (++kk == depth) { kk = 0; full = bar(s, b_full); to = dst; kpar ^= 1u; kwrapped = true; }
       }
       if (!ok || *(volatile int *)abortp) {  // after a give-up: this warp's own copies land before the block may exit (bounded)
-        if (!SEGMENTED) {  // entries before kk were used in this round of the ring, the others in the round before
-          used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
-          par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
-        }
+        // entries before kk were used in this round of the ring, the others in the round before
+        const uint32_t used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
+        const uint32_t par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
 #pragma unroll 1
         for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
           if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
@@ -803,7 +795,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     S.n4 = __shfl_sync(0xffffffffu, S.n4, 0);
     S.n48 = __shfl_sync(0xffffffffu, S.n48, 0);
     S.L = __shfl_sync(0xffffffffu, S.L, 0);
-    if (S.L > 0 && (SEGMENTED || wait_or_abort(bar(s, B_Q), 0, abortp))) {
+    if (S.L > 0 && wait_or_abort(bar(s, B_Q), 0, abortp)) {
       // operand descriptors, built once; inside the loop only the 16-byte-unit start address (low bits) moves
       const uint64_t qd0 = tc::smem_desc(tc::smem_u32(smem + sm.q[s][0]) - (s ? 1024u : 0u), 1024, 128);
       const uint64_t qd1 = tc::smem_desc(tc::smem_u32(smem + sm.q[s][1]) - (s ? 1024u : 0u), 1024, 128);
@@ -811,57 +803,70 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const uint64_t kd0 = tc::smem_desc(tc::smem_u32(smem + sm.kring[s]), 1024, 128);
       const uint64_t ksf0 = tc::smem_desc(tc::smem_u32(smem + sm.kring[s]) + kSlots * D / 2, 128, 128);
       const uint32_t t_sfq = tmem + col_sfq(s), t_sfk = tmem + col_sfk(s);
-      int kk = 0, nk = sm.nk[0];
-      uint32_t kpar = 0, kstep = sm.kstage[0] >> 4;  // parity of the next use (SEGMENTED: a bit per ring entry); ring stride
-      uint32_t qseg = 0;                             // segments so far
-      auto q_scales = [&]() {  // Q scale factors go to TMEM once; the record carries them for rows 0..63 and again for rows
-        if (tc::elect_one()) { // 64..127, so the same atom serves either stream
+      if (S.n4 > 0) {  // Q scale factors go to TMEM once; the record carries them for rows 0..63 and again for rows
+        if (tc::elect_one()) {  // 64..127, so the same atom serves either stream
 #pragma unroll
           for (int k = 0; k < D / 64; ++k)
             tc::tmem_cp_sf(t_sfq + 4 * k, tc::smem_desc(tc::smem_u32(smem + sm.q[s][0]) + kSlots * D / 2 + k * kSfAtomBytes,
                                                          128, 128));
         }
         __syncwarp();
-      };
-      if (!SEGMENTED && S.n4 > 0) q_scales();
+      }
       // the score tiles are double buffered, so Q K^T runs up to two steps ahead of the softmax
-      for (int j = 0; j < S.L; ++j) {
-        const int g = j & 1;
-        if (SEGMENTED && (j == 0 || j == S.n4 || j == S.n48)) {
-          const int t = S.tier(j);
-          kstep = sm.kstage[t] >> 4;
-          nk = sm.nk[t];
-          kk = 0;
-          if (!wait_or_abort(bar(s, B_Q), qseg & 1u, abortp)) break;
-          ++qseg;
-          if (j < S.n4) q_scales();
-        }
-        if (!wait_or_abort(bar(s, B_FULLK + kk), SEGMENTED ? (kpar >> kk) & 1u : kpar, abortp)) break;
-        if (SEGMENTED) kpar ^= 1u << kk;
-        if (!wait_or_abort(bar(s, B_SFREE + g), ((j >> 1) & 1) ^ 1, abortp)) break;
-        tc::fence_after_sync();
-        const uint64_t kd = kd0 + (uint64_t)(kk * kstep);
-        const uint32_t d_s = tmem + col_s(s, g);
-        if (tc::elect_one()) {
-          if (B16 && j >= S.n48) {
+      const uint32_t full0 = bar(s, B_FULLK), last = full0 + (uint32_t)sm.nk * 8u, kstep = sm.kstage >> 4, kentry = sm.kentry >> 4;
+      uint32_t full = full0, kpar = 0;  // ring entry, parity of its next use
+      uint64_t kd = kd0;
+      auto next_entry = [&]() {
+        full += 8u;
+        kd += kentry;
+        if (full == last) { full = full0; kd = kd0; kpar ^= 1u; }
+      };
+      bool ok = true;
+#pragma unroll 1
+      for (int j = 0; ok && j < S.n48; j += 2) {
+        if (!(ok = wait_or_abort(full, kpar, abortp))) break;
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) tc::mma_f16(d_s, qd2 + ks * 128, kd + ks * 128, tc::idesc_bf16(64), ks > 0);
-          } else if (!FP4 || j >= S.n4) {
+        for (int e = 0; e < 2; ++e) {
+          if (e == 1 && j + 1 >= S.n48) break;
+          if (!(ok = wait_or_abort(bar(s, B_SFREE + e), ((j >> 1) & 1) ^ 1, abortp))) break;
+          tc::fence_after_sync();
+          const uint32_t d_s = tmem + col_s(s, e);
+          const uint64_t kde = kd + (e ? kstep : 0u);
+          if (tc::elect_one()) {
+            if (!FP4 || j + e >= S.n4) {
 #pragma unroll
-            for (int ks = 0; ks < D / 32; ++ks) tc::mma_i8(d_s, qd1 + ks * 128, kd + ks * 128, tc::idesc_i8(64), ks > 0);
-          } else {
-            const uint64_t ksf = ksf0 + (uint64_t)(kk * kstep);
+              for (int ks = 0; ks < D / 32; ++ks) tc::mma_i8(d_s, qd1 + ks * 128, kde + ks * 128, tc::idesc_i8(64), ks > 0);
+            } else {
+              const uint64_t ksf = ksf0 + (kde - kd0);
 #pragma unroll
-            for (int k = 0; k < D / 64; ++k) tc::tmem_cp_sf(t_sfk + 4 * k, ksf + k * (kSfAtomBytes >> 4));
+              for (int k = 0; k < D / 64; ++k) tc::tmem_cp_sf(t_sfk + 4 * k, ksf + k * (kSfAtomBytes >> 4));
 #pragma unroll
-            for (int ks = 0; ks < D / 64; ++ks)
-              tc::mma_nvfp4(d_s, qd0 + ks * 128, kd + ks * 128, tc::idesc_nvfp4(64), ks > 0, t_sfq + 4 * ks, t_sfk + 4 * ks);
+              for (int ks = 0; ks < D / 64; ++ks)
+                tc::mma_nvfp4(d_s, qd0 + ks * 128, kde + ks * 128, tc::idesc_nvfp4(64), ks > 0, t_sfq + 4 * ks, t_sfk + 4 * ks);
+            }
+            tc::mma_commit(bar(s, B_SREADY + e) + (uint32_t)(j & 2) * 8u);
+            if (e == 1 || (B16 && j + 1 == S.n48)) tc::mma_commit(full + (B_KFREE - B_FULLK) * 8u);
           }
-          tc::mma_commit(bar(s, B_SREADY + (j & kMask)));
-          tc::mma_commit(bar(s, B_KFREE + kk));
+          __syncwarp();
         }
-        __syncwarp();
-        if (++kk == nk) { kk = 0; if (!SEGMENTED) kpar ^= 1u; }
+        next_entry();
+      }
+      if (B16 && ok && S.n48 < S.L && wait_or_abort(bar(s, B_Q), S.n48 > 0 ? 1u : 0u, abortp)) {
+#pragma unroll 1
+        for (int j = S.n48; j < S.L; ++j) {
+          const int g = j & 1;
+          if (!wait_or_abort(full, kpar, abortp)) break;
+          if (!wait_or_abort(bar(s, B_SFREE + g), ((j >> 1) & 1) ^ 1, abortp)) break;
+          tc::fence_after_sync();
+          if (tc::elect_one()) {
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) tc::mma_f16(tmem + col_s(s, g), qd2 + ks * 128, kd + ks * 128, tc::idesc_bf16(64), ks > 0);
+            tc::mma_commit(bar(s, B_SREADY + (j & kMask)));
+            tc::mma_commit(full + (B_KFREE - B_FULLK) * 8u);
+          }
+          __syncwarp();
+          next_entry();
+        }
       }
     }
   }
@@ -877,47 +882,65 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const uint64_t pd0 = tc::smem_desc(tc::smem_u32(smem + sm.p[s]), 1024, 128);
       const uint64_t sfpd0 = tc::smem_desc(tc::smem_u32(smem + sm.sfp[s]), 128, 128);
       const uint32_t t_sfv = tmem + col_sfv(s), t_sfp = tmem + col_sfp(s), t_o = tmem + col_o(s);
-      int vv = 0, nv = sm.nv[0], pm = kMask;  // V ring entry and depth; number of P slots - 1
-      uint32_t vpar = 0;                          // parity of the next use (SEGMENTED: a bit per ring entry)
-      uint32_t vstep = sm.vstage[0] >> 4, pstep = sm.pbytes[0] >> 4;
-      for (int j = 0; j < S.L; ++j) {
-        // ---- O^T += V(j)^T P(j)^T, once P(j) is written and the accumulator is rescaled for step j
-        const int g = j & kStepMask;
-        if (SEGMENTED && (j == 0 || j == S.n4 || j == S.n48)) {
-          const int t = S.tier(j);
-          vstep = sm.vstage[t] >> 4;
-          nv = sm.nv[t];
-          pstep = sm.pbytes[t] >> 4;
-          pm = t == 2 ? 1 : kMask;
-          vv = 0;
+      const uint32_t full0 = bar(s, B_FULLV), last = full0 + (uint32_t)sm.nv * 8u, vstep = sm.vstage >> 4, ventry = sm.ventry >> 4;
+      uint32_t full = full0, vpar = 0, vo = 0;  // ring entry, parity of its next use, its place in the ring
+      auto next_entry = [&]() {
+        full += 8u;
+        vo += ventry;
+        if (full == last) { full = full0; vo = 0; vpar ^= 1u; }
+      };
+      // O^T += V(j)^T P(j)^T, once P(j) is written and the stream's correction warps have rescaled the accumulator where step j
+      // asked for it
+      bool ok = true;
+#pragma unroll 1
+      for (int j = 0; ok && j < S.n48; j += 2) {
+        if (!(ok = wait_or_abort(full, vpar, abortp))) break;
+        const uint32_t g0 = (uint32_t)j & kStepMask, par = (uint32_t)(j >> kStepShift) & 1u;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          if (e == 1 && j + 1 >= S.n48) break;
+          if (!(ok = wait_or_abort(bar(s, B_CORROK + e) + g0 * 8u, par, abortp))) break;
+          tc::fence_after_sync();
+          const uint32_t ve = vo + (e ? vstep : 0u), acc = (e == 0) ? j > 0 : 1u;
+          const bool four = FP4 && j + e < S.n4;
+          const uint64_t vd = vd0 + ve;
+          const uint64_t pdg = pd0 + (uint64_t)(((g0 & 2u) + e) * (SEGMENTED ? (four ? 128u : 256u) : sm.pbytes[0] >> 4));
+          if (tc::elect_one()) {
+            if (!four) {
+#pragma unroll
+              for (int ks = 0; ks < 2; ++ks)
+                tc::mma_f8f6f4(t_o, vd + ks * (2 * D), pdg + ks * 128, tc::idesc_e4m3(64), acc | (ks > 0));
+            } else {
+              tc::tmem_cp_sf(t_sfv, vsf0 + ve);
+              tc::tmem_cp_sf(t_sfp, sfpd0 + (uint64_t)((g0 + e) * 32));
+              tc::mma_nvfp4(t_o, vd, pdg, tc::idesc_nvfp4(64), acc, t_sfv, t_sfp);
+            }
+            tc::mma_commit(bar(s, B_PVDONE + e) + g0 * 8u);
+            if (e == 1 || (B16 && j + 1 == S.n48)) tc::mma_commit(full + (B_VFREE - B_FULLV) * 8u);
+          }
+          __syncwarp();
         }
-        if (!wait_or_abort(bar(s, B_FULLV + vv), SEGMENTED ? (vpar >> vv) & 1u : vpar, abortp)) break;
-        if (SEGMENTED) vpar ^= 1u << vv;
-        // P(j) is written and the stream's correction warps have rescaled the accumulator where step j asked for it
-        if (!wait_or_abort(bar(s, B_CORROK + g), (j >> kStepShift) & 1, abortp)) break;
-        tc::fence_after_sync();
-        const uint64_t vd = vd0 + (uint64_t)(vv * vstep);
-        const uint64_t pdg = pd0 + (uint64_t)((g & pm) * pstep), sfpdg = sfpd0 + (uint64_t)(g * 32);
-        const uint32_t acc = j > 0;
-        if (tc::elect_one()) {
-          if (B16 && j >= S.n48) {
+        next_entry();
+      }
+      if (B16 && ok) {
+#pragma unroll 1
+        for (int j = S.n48; j < S.L; ++j) {
+          const uint32_t g = (uint32_t)j & kStepMask;
+          if (!wait_or_abort(full, vpar, abortp)) break;
+          if (!wait_or_abort(bar(s, B_CORROK) + g * 8u, (j >> kStepShift) & 1, abortp)) break;
+          tc::fence_after_sync();
+          const uint64_t vd = vd0 + vo, pdg = pd0 + (uint64_t)((g & (SEGMENTED ? 1u : 3u)) * (sm.pbytes[2] >> 4));
+          const uint32_t acc = j > 0;
+          if (tc::elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               tc::mma_f16(t_o, vd + ks * (2 * D), pdg + ks * 128, tc::idesc_bf16(64), acc | (ks > 0));
-          } else if (!FP4 || j >= S.n4) {
-#pragma unroll
-            for (int ks = 0; ks < 2; ++ks)
-              tc::mma_f8f6f4(t_o, vd + ks * (2 * D), pdg + ks * 128, tc::idesc_e4m3(64), acc | (ks > 0));
-          } else {
-            tc::tmem_cp_sf(t_sfv, vsf0 + (uint64_t)(vv * vstep));
-            tc::tmem_cp_sf(t_sfp, sfpdg);
-            tc::mma_nvfp4(t_o, vd, pdg, tc::idesc_nvfp4(64), acc, t_sfv, t_sfp);
+            tc::mma_commit(bar(s, B_PVDONE) + g * 8u);
+            tc::mma_commit(full + (B_VFREE - B_FULLV) * 8u);
           }
-          tc::mma_commit(bar(s, B_PVDONE + g));
-          tc::mma_commit(bar(s, B_VFREE + vv));
+          __syncwarp();
+          next_entry();
         }
-        __syncwarp();
-        if (++vv == nv) { vv = 0; if (!SEGMENTED) vpar ^= 1u; }
       }
     }
   }
@@ -1013,20 +1036,20 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         const float unit = ok ? unit_of(S.tier(S.L - 1)) : 0.f;
         uint32_t *out_ch = reinterpret_cast<uint32_t *>(out_head + (ch & ~1));
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          uint32_t o[16];
-          tc::tmem_ld16(tmem + lane_addr + col_o(s) + c * 16, o);
+        for (int c = 0; c < 8; ++c) {
+          uint32_t o[8];
+          tc::tmem_ld8(tmem + lane_addr + col_o(s) + c * 8, o);
           tc::wait_ld();
 #pragma unroll
-          for (int j = 0; j < 16; j += 2) {
+          for (int j = 0; j < 8; j += 2) {
             // lanes 2x and 2x+1 hold neighbouring channels: after one exchange the even lane writes both of query j, the odd
             // lane both of query j + 1 (64 contiguous bytes per query and warp, no staging tile, no barrier)
-            const float2 inv = *reinterpret_cast<const float2 *>(s_inv + c * 16 + j);
+            const float2 inv = *reinterpret_cast<const float2 *>(s_inv + c * 8 + j);
             const float x = inv.x > 0.f ? __uint_as_float(o[j]) * unit * inv.x : 0.f;
             const float y = inv.y > 0.f ? __uint_as_float(o[j + 1]) * unit * inv.y : 0.f;
             const float got = __shfl_xor_sync(0xffffffffu, (lane & 1) ? x : y, 1);
             const uint32_t word = (lane & 1) ? pack_bf16x2(got, y) : pack_bf16x2(x, got);
-            const int tok = s_tok[c * 16 + j + (lane & 1)];
+            const int tok = s_tok[c * 8 + j + (lane & 1)];
             if (tok >= 0) out_ch[(size_t)tok * (D / 2)] = word;
           }
         }

@@ -55,6 +55,21 @@ def test_segments_of_three_tiers(d, f16, f8, f4):
     _check_attention(w, out, ref, sel, bad, heads=heads)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("n16,n8,n4", [(0, 0, 1), (0, 1, 0), (0, 1, 1), (0, 2, 3), (0, 3, 2), (0, 33, 4), (0, 1, 34), (1, 0, 0),
+                                       (1, 1, 0), (1, 0, 1), (2, 1, 2), (3, 2, 1), (1, 32, 3), (5, 16, 17)])
+def test_lists_of_odd_and_even_segments(n16, n8, n4, d):
+    """Blocks of a list are fetched in pairs (those of the 16-bit tier one by one): segments that end in the middle of a pair, and
+    one below, at and above the 32 entries that a loader holds, on ragged tiles."""
+    w = W("pairs", 1, 2, d, 5, 12, 28, n16 / 40, n8 / 40, n4 / 40, seed=37)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v)
+    assert [int(x) for x in plan.info.quota] == [n4, n8, n16] and plan.info.R == 40
+    ref = oracle_all(w, q, k, v)
+    bad = _check_prepare(w, plan, ws, ref)
+    _check_attention(w, out, ref, [(h, a) for h in range(2) for a in (0, 3, 20, 39)], bad)
+
+
 @pytest.mark.parametrize("H", [1, 8, 30])
 def test_pooling_splits(H):
     """80 blocks a head: eight, four and one warp per block."""
