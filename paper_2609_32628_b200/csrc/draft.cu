@@ -112,9 +112,17 @@ __global__ void __launch_bounds__(128) draft_logits_kernel(Params p) {
 
 cudaError_t launch_draft(const Params &p, cudaStream_t st, int *launches) {
   const dim3 grid((p.R + TILE - 1) / TILE, (p.R + TILE - 1) / TILE, p.BH * 2);
-  const int smem = 2 * TILE * ((p.d < kChunk ? p.d : kChunk) + 4) * (int)sizeof(float);
+  // Three CTAs fit an SM, but the kernel starts while the pooling kernel still fills the SMs, and the few CTAs of a small map
+  // would be packed three to an SM wherever there is room, to share its fp64 pipe while others stay idle.  So a grid of up to
+  // one, or two, CTAs per SM asks for so much shared memory that no more than that fit.  (da2_prepare, us: 2 heads of 128
+  // blocks 36.8 -> 28.2, 8 heads 59.3 -> 52.5, 12 heads 80.0 -> 76.7, 24 heads 138.1 -> 134.6; d = 64, 8 heads of 168 blocks
+  // 50.7 -> 47.5; larger grids as before.)
+  const int tiles = 2 * TILE * ((p.d < kChunk ? p.d : kChunk) + 4) * (int)sizeof(float);
+  const long long ctas = (long long)grid.x * grid.y * grid.z;
+  constexpr int kOne = 116 * 1024, kTwo = 78 * 1024;  // one CTA to an SM's 228 KB, two
+  const int smem = ctas <= kSms ? kOne : (ctas <= 2 * kSms ? kTwo : tiles);
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOne);
     if (e != cudaSuccess) return e;
   }
   *launches += 1;
