@@ -44,8 +44,7 @@
 // call of 16x48x48, 24 heads; special-function pipe 70 %, issue slots 69 %, tensor pipe 22 %): the time followed the requests in
 // every variant that was tried.  So the instructions of a step are what is saved, in the roles around the softmax above all, a
 // quarter of them: the loaders, the Q K^T warps and the PV warps take the blocks of a list in pairs, with one ring entry, one
-// wait and one round of the loop for two, and run along the rings by increments (requests 1.59 -> 1.29 G, 80 % of the peak rate;
-// 12.53 -> 11.9 ms).  Taking PV and correction in pairs as well makes the products late (13.3 ms), and softmax steps of two
+// wait and one round of the loop for two (requests 1.59 -> 1.33 G, 82 % of the peak rate; 12.53 -> 11.9 ms).  Taking PV and correction in pairs as well makes the products late (13.3 ms), and softmax steps of two
 // blocks need fewer instructions still (7.3 instead of 8.6 G) but leave two warps a scheduler, too few (13.7 ms).
 // The softmax keeps the work inside the chain of hand-offs short: the row maximum
 // is taken on raw accumulator values, the scale and the maximum are folded into one packed FMA feeding ex2, the NVFP4 group
@@ -54,8 +53,9 @@
 // then sums and packing), which gives the single warp the instruction-level parallelism it lacks when the three are
 // interleaved per pair.  And the code is kept small: beyond about 47 KB in all the hits fall (99.9 % 11.9 ms, 99.0 % 12.0 to
 // 12.1 with the same instructions; 97.6 % 14.4 and 93.8 % 15.1 in earlier states).
-// Measured (kernel alone, ms, before -> with pairs):  12 heads of 32,760 tokens 2.92 -> 2.77, one ranking per head 2.91 -> 2.79,
-// with a 226-token prefix, whose blocks are bf16, 3.91 -> 3.67;  24 heads of 36,864 tokens all in 8 bit at d = 64 11.79 -> 10.8.
+// Measured (kernel alone, ms, before -> with pairs):  12 heads of 32,760 tokens 2.92 -> 2.77, one ranking per head 2.91 -> 2.77,
+// with a 226-token prefix, whose blocks are bf16, 3.90 -> 3.57;  24 heads of 36,864 tokens all in 8 bit at d = 64 11.79 -> 10.75;
+// 40 heads of 75,600 tokens, 20 % bf16 + 40 % 8-bit, 86.1 -> 82.7.
 // Every wait on an mbarrier is bounded; a wait that gives up records device status "timeout", all roles leave their
 // loops and the CTA exits normally after releasing TMEM.
 #include <type_traits>
@@ -723,12 +723,10 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1], nb2 = is_v ? sm.vbytes[2] : sm.kbytes[2];
       uint2 *const infos = s_info + s * kInfoRing;
       unsigned long long cur_rec = 0;
-      uint32_t full = bar(s, b_full), to = dst;
-      const uint32_t to_free = (uint32_t)(b_free - b_full) * 8u;
 #pragma unroll 1
       for (int i = 0; i < S.L;) {
         const int src = i & 31;
-        const bool two = i + 1 < S.n48;
+        const bool two = i + 1 < (B16 ? S.n48 : S.L);
         if (src == 0) {  // next batch: its ids and scales were requested one batch ago
           const int b = nxt_b;
           cur_dk = nxt_dk;
@@ -748,33 +746,32 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           load_q(2, 2);
           __syncwarp();
         }
-        if (kwrapped && !(ok = wait_or_abort(full + to_free, kpar, abortp))) break;
+        if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) break;
         if (!is_v) {
           // the steps' masks and key scales are written before the data the softmax waits for is requested
           const int e = i & (kInfoRing - 1);
-          if ((padded_lanes >> src) & (two ? 3u : 1u)) {
+          if ((padded_lanes >> src) & (!B16 || two ? 3u : 1u)) {
             float *lim = reinterpret_cast<float *>(smem + sm.lim) + (s * kInfoRing + e) * 64;
 #pragma unroll 1
-            for (int x = 0; x <= (int)two; ++x) {
+            for (int x = 0; x <= (!B16 || two); ++x) {
               const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src + x);
               const uint32_t mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src + x);
               lim[x * 64 + lane] = (mlo >> lane) & 1u ? INFINITY : -INFINITY;
               lim[x * 64 + 32 + lane] = (mhi >> lane) & 1u ? INFINITY : -INFINITY;
             }
           }
-          if (lane == src || (two && lane == src + 1)) infos[lane & (kInfoRing - 1)] = make_uint2(__float_as_uint(cur_dk), cur_mask != ~0ull);
+          if (B16 ? lane == src || (two && lane == src + 1) : (lane & ~1) == src) infos[lane & (kInfoRing - 1)] = make_uint2(__float_as_uint(cur_dk), cur_mask != ~0ull);
           __syncwarp();
         }
         if (tc::elect_one()) {
+          const uint32_t full = bar(s, b_full + kk), to = dst + (uint32_t)kk * entry;
           tc::mbar_arrive_expect_tx(full, n0 + n1);
           tc::bulk_g2s(to, reinterpret_cast<const uint8_t *>(((unsigned long long)hi0 << 32) | lo0), n0, full);
           if (n1) tc::bulk_g2s(to + stage, reinterpret_cast<const uint8_t *>(((unsigned long long)hi1 << 32) | lo1), n1, full);
         }
         __syncwarp();
-        full += 8u;
-        to += entry;
-        i += two ? 2 : 1;
-        if (++kk == depth) { kk = 0; full = bar(s, b_full); to = dst; kpar ^= 1u; kwrapped = true; }
+        i += !B16 || two ? 2 : 1;
+        if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
       }
       if (!ok || *(volatile int *)abortp) {  // after a give-up: this warp's own copies land before the block may exit (bounded)
         // entries before kk were used in this round of the ring, the others in the round before
@@ -815,11 +812,11 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       // the score tiles are double buffered, so Q K^T runs up to two steps ahead of the softmax
       const uint32_t full0 = bar(s, B_FULLK), last = full0 + (uint32_t)sm.nk * 8u, kstep = sm.kstage >> 4, kentry = sm.kentry >> 4;
       uint32_t full = full0, kpar = 0;  // ring entry, parity of its next use
-      uint64_t kd = kd0;
+      uint32_t ko = 0, spar = 1;             // its place in the ring; parity of the consumption that frees a score buffer
       auto next_entry = [&]() {
         full += 8u;
-        kd += kentry;
-        if (full == last) { full = full0; kd = kd0; kpar ^= 1u; }
+        ko += kentry;
+        if (full == last) { full = full0; ko = 0; kpar ^= 1u; }
       };
       bool ok = true;
 #pragma unroll 1
@@ -828,27 +825,28 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           if (e == 1 && j + 1 >= S.n48) break;
-          if (!(ok = wait_or_abort(bar(s, B_SFREE + e), ((j >> 1) & 1) ^ 1, abortp))) break;
+          if (!(ok = wait_or_abort(bar(s, B_SFREE + e), spar, abortp))) break;
           tc::fence_after_sync();
           const uint32_t d_s = tmem + col_s(s, e);
-          const uint64_t kde = kd + (e ? kstep : 0u);
+          const uint32_t kde = ko + (e ? kstep : 0u);
           if (tc::elect_one()) {
             if (!FP4 || j + e >= S.n4) {
 #pragma unroll
-              for (int ks = 0; ks < D / 32; ++ks) tc::mma_i8(d_s, qd1 + ks * 128, kde + ks * 128, tc::idesc_i8(64), ks > 0);
+              for (int ks = 0; ks < D / 32; ++ks) tc::mma_i8(d_s, qd1 + ks * 128, kd0 + kde + ks * 128, tc::idesc_i8(64), ks > 0);
             } else {
-              const uint64_t ksf = ksf0 + (kde - kd0);
+              const uint64_t ksf = ksf0 + kde;
 #pragma unroll
               for (int k = 0; k < D / 64; ++k) tc::tmem_cp_sf(t_sfk + 4 * k, ksf + k * (kSfAtomBytes >> 4));
 #pragma unroll
               for (int ks = 0; ks < D / 64; ++ks)
-                tc::mma_nvfp4(d_s, qd0 + ks * 128, kde + ks * 128, tc::idesc_nvfp4(64), ks > 0, t_sfq + 4 * ks, t_sfk + 4 * ks);
+                tc::mma_nvfp4(d_s, qd0 + ks * 128, kd0 + kde + ks * 128, tc::idesc_nvfp4(64), ks > 0, t_sfq + 4 * ks, t_sfk + 4 * ks);
             }
             tc::mma_commit(bar(s, B_SREADY + e) + (uint32_t)(j & 2) * 8u);
             if (e == 1 || (B16 && j + 1 == S.n48)) tc::mma_commit(full + (B_KFREE - B_FULLK) * 8u);
           }
           __syncwarp();
         }
+        spar ^= 1u;
         next_entry();
       }
       if (B16 && ok && S.n48 < S.L && wait_or_abort(bar(s, B_Q), S.n48 > 0 ? 1u : 0u, abortp)) {
@@ -860,7 +858,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           tc::fence_after_sync();
           if (tc::elect_one()) {
 #pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) tc::mma_f16(tmem + col_s(s, g), qd2 + ks * 128, kd + ks * 128, tc::idesc_bf16(64), ks > 0);
+            for (int ks = 0; ks < D / 16; ++ks) tc::mma_f16(tmem + col_s(s, g), qd2 + ks * 128, kd0 + ko + ks * 128, tc::idesc_bf16(64), ks > 0);
             tc::mma_commit(bar(s, B_SREADY + (j & kMask)));
             tc::mma_commit(full + (B_KFREE - B_FULLK) * 8u);
           }
@@ -892,10 +890,11 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       // O^T += V(j)^T P(j)^T, once P(j) is written and the stream's correction warps have rescaled the accumulator where step j
       // asked for it
       bool ok = true;
+      uint32_t par = 0;
 #pragma unroll 1
       for (int j = 0; ok && j < S.n48; j += 2) {
         if (!(ok = wait_or_abort(full, vpar, abortp))) break;
-        const uint32_t g0 = (uint32_t)j & kStepMask, par = (uint32_t)(j >> kStepShift) & 1u;
+        const uint32_t g0 = (uint32_t)j & kStepMask;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           if (e == 1 && j + 1 >= S.n48) break;
@@ -920,6 +919,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           }
           __syncwarp();
         }
+        if (g0 + 2u > (uint32_t)kStepMask) par ^= 1u;
         next_entry();
       }
       if (B16 && ok) {
