@@ -165,6 +165,22 @@ __global__ void set_gscale_kernel(float *gscale, int which, int first, int n, Sc
   if (i < n) gscale[(size_t)(first + i) * 4 + which] = c.v[i];
 }
 
+// Zeros in front of a call's kernels, as a kernel of their chain: a memset node starts when everything before it has ended, and
+// the first kernel after it when the memset has (smallest call 31.9 -> 29.3 us, 24 heads of 8,192 tokens 404.7 -> 402.5).  Workspace regions are
+// multiples of 256 bytes.
+constexpr int kClearThreads = 256;
+__global__ void clear_kernel(uint4 *words, uint32_t n) {
+  const uint32_t i = blockIdx.x * kClearThreads + threadIdx.x;
+  da2::grid_trigger();
+  da2::grid_wait();
+  if (i < n) words[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+cudaError_t clear(void *workspace, uint64_t offset, uint64_t bytes, cudaStream_t st) {
+  const uint32_t n = (uint32_t)(bytes / sizeof(uint4));
+  return da2::launch_chained(clear_kernel, dim3((n + kClearThreads - 1) / kClearThreads), kClearThreads, 0, st,
+                             reinterpret_cast<uint4 *>((uint8_t *)workspace + offset), n);
+}
+
 }  // namespace
 
 extern "C" {
@@ -310,8 +326,7 @@ da2_status_t prepare_impl(const da2_plan_t *plan, const void *q, const void *k, 
   int launches = 0;
   t_last_launches = 0;
   // status word, head maxima and per-channel maxima start at zero (they are contiguous)
-  if (cudaMemsetAsync((uint8_t *)workspace + I.off_status, 0, I.off_gscale - I.off_status, st) != cudaSuccess)
-    return DA2_ERR_CUDA;
+  if (clear(workspace, I.off_status, I.off_gscale - I.off_status, st) != cudaSuccess) return DA2_ERR_CUDA;
   const __nv_bfloat16 *qb = (const __nv_bfloat16 *)q, *kb = (const __nv_bfloat16 *)k, *vb = (const __nv_bfloat16 *)v;
   if (da2::launch_pool(p, qb, kb, vb, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   for (int i = 0; i < 3; ++i) {  // caller-fixed NVFP4 per-tensor scales replace the derived ones
@@ -361,8 +376,7 @@ da2_status_t da2_prepare_cached_scales(const da2_plan_t *plan, const void *q, co
   int launches = 0;
   t_last_launches = 0;
   // only the status word is cleared: the statistics and the scales derived from them stay as the earlier call left them
-  if (cudaMemsetAsync((uint8_t *)workspace + plan->info.off_status, 0, 64 * sizeof(int), st) != cudaSuccess)
-    return DA2_ERR_CUDA;
+  if (clear(workspace, plan->info.off_status, 64 * sizeof(int), st) != cudaSuccess) return DA2_ERR_CUDA;
   const __nv_bfloat16 *qb = (const __nv_bfloat16 *)q, *kb = (const __nv_bfloat16 *)k, *vb = (const __nv_bfloat16 *)v;
   if (da2::launch_prep(p, qb, kb, vb, st, &launches, /*pool=*/true) != cudaSuccess) return DA2_ERR_CUDA;
   if (reselect) {
