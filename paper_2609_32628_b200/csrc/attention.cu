@@ -40,22 +40,24 @@
 //   kinds         : kind::f16 (BF16); kind::i8 for QK^T + kind::f8f6f4 E4M3 x E4M3 for PV (App. C.1); and
 //                   kind::mxf4nvf4 with E4M3 scales per 16 elements (NVFP4), scale factors moved by tcgen05.cp.
 // What bounds it: the fetch of instructions.  Eight warps of a scheduler are at eight places of the code, so that nearly every
-// line comes from the SM's instruction cache (32 KB, shared by all roles), and its request rate was 94 % of the peak (all-4-bit
-// call of 16x48x48, 24 heads; special-function pipe 70 %, issue slots 69 %, tensor pipe 22 %): the time followed the requests in
-// every variant that was tried.  So the instructions of a step are what is saved, in the roles around the softmax above all, a
-// quarter of them: the loaders, the Q K^T warps and the PV warps take the blocks of a list in pairs, with one ring entry, one
-// wait and one round of the loop for two (requests 1.59 -> 1.33 G, 82 % of the peak rate; 12.53 -> 11.9 ms).  Taking PV and correction in pairs as well makes the products late (13.3 ms), and softmax steps of two
-// blocks need fewer instructions still (7.3 instead of 8.6 G) but leave two warps a scheduler, too few (13.7 ms).
-// The softmax keeps the work inside the chain of hand-offs short: the row maximum
-// is taken on raw accumulator values, the scale and the maximum are folded into one packed FMA feeding ex2, the NVFP4 group
-// scale is folded into the exponent so the scaled weight needs no extra multiply, narrow weights are packed by the
-// conversions themselves, and the exponentiate phase runs over the whole row in batches (all arguments, all exponentials,
-// then sums and packing), which gives the single warp the instruction-level parallelism it lacks when the three are
-// interleaved per pair.  And the code is kept small: beyond about 47 KB in all the hits fall (99.9 % 11.9 ms, 99.0 % 12.0 to
-// 12.1 with the same instructions; 97.6 % 14.4 and 93.8 % 15.1 in earlier states).
-// Measured (kernel alone, ms, before -> with pairs):  12 heads of 32,760 tokens 2.92 -> 2.77, one ranking per head 2.91 -> 2.77,
-// with a 226-token prefix, whose blocks are bf16, 3.90 -> 3.57;  24 heads of 36,864 tokens all in 8 bit at d = 64 11.79 -> 10.75;
-// 40 heads of 75,600 tokens, 20 % bf16 + 40 % 8-bit, 86.1 -> 82.7.
+// line comes from the SM's instruction cache (32 KB, shared by all roles), and its request rate was 94 % of the peak
+// (all-4-bit call of 16x48x48, 24 heads; special-function pipe 70 %, issue slots 69 %, tensor pipe 22 %): the time followed
+// the requests in every variant that was tried.  So the instructions of a step are what is saved, in the roles around the
+// softmax above all, a quarter of them: the loaders, the Q K^T warps and the PV warps take the blocks of a list in pairs, with
+// one ring entry, one wait and one round of the loop for two (requests 1.59 -> 1.33 G, 82 % of the peak rate; 12.53 -> 11.9
+// ms).  Taking PV and correction in pairs as well makes the products late (13.3 ms), and softmax steps of two blocks need
+// fewer instructions still (7.3 instead of 8.6 G) but leave two warps a scheduler, too few (13.7 ms).
+// The softmax keeps the work inside the chain of hand-offs short: the row maximum is taken on raw accumulator values, the
+// scale and the maximum are folded into one packed FMA feeding ex2, the NVFP4 group scale is folded into the exponent so the
+// scaled weight needs no extra multiply, narrow weights are packed by the conversions themselves, and the exponentiate phase
+// runs over the whole row in batches (all arguments, all exponentials, then sums and packing), which gives the single warp the
+// instruction-level parallelism it lacks when the three are interleaved per pair.  And the code is kept small: beyond about 47
+// KB in all the hits fall (99.9 % 11.9 ms, 99.0 % 12.0 to 12.1 with the same instructions; 97.6 % 14.4 and 93.8 % 15.1 in
+// earlier states).
+// Measured (kernel alone, ms, before -> with pairs):  12 heads of 32,760 tokens 2.92 -> 2.77, one ranking per head 2.91 ->
+// 2.77, with a 226-token prefix, whose blocks are bf16, 3.90 -> 3.57;  24 heads of 36,864 tokens all in 8 bit at d = 64 11.79
+// -> 10.75; 40 heads of 75,600 tokens, 20 % bf16 + 40 % 8-bit, 86.1 -> 82.7. And the first list entries' masks and key scales
+// are fetched while a block is set up (three tiers at d = 64, whole call, 395.0 -> 390.8 us).
 // Every wait on an mbarrier is bounded; a wait that gives up records device status "timeout", all roles leave their
 // loops and the CTA exits normally after releasing TMEM.
 #include <type_traits>
@@ -378,11 +380,19 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
     if (a < Rt) a = p.order[(size_t)bh * ((Rt + 1) / 2) * 2 + a];
   }
   StreamInfo S = load_stream<ORDERED>(p, bh, a);
-  // the loaders' first ids, and the correction warps' table of query tokens, are on their way while the block is set up
+  // the loaders' first ids (for K with their blocks' masks and key scales) and the correction warps' table of query tokens are
+  // on their way while the block is set up
   int pre0 = 0, pre1 = 0;
+  unsigned long long pre_mask = 0;
+  float pre_dk = 0.f;
   if (warp >= kLoadWarp0) {
     if (lane < S.L) pre0 = S.ids[lane];
     if (32 + lane < S.L) pre1 = S.ids[32 + lane];
+    if (warp < kLoadWarp0 + 2) {
+      const int b = pre0 < Rt ? pre0 : 0;  // (an id beyond the head's blocks is reported by the loader)
+      pre_mask = table_mask(p, b);
+      if (lane < S.n48 && lane >= S.n4) pre_dk = p.dk8[(size_t)bh * R + b];
+    }
   } else if (warp >= kSoftmaxWarps && warp < kMmaWarp0 && (warp & 3) < 2 && S.a >= 0) {
     const int j = (warp & 1) * 32 + lane;
     reinterpret_cast<int *>(smem + sm.tok)[stream * 64 + j] =
@@ -705,7 +715,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         return (!is_v && idx < S.L && S.tier(idx) == 1) ? p.dk8[head_blocks + b] : 0.f;
       };
       int nxt_b = checked(pre0), nn_b = checked(pre1);
-      float cur_dk = 0.f, nxt_dk = key_scale(lane, nxt_b);
+      float cur_dk = 0.f, nxt_dk = pre_dk;
       unsigned long long cur_mask = 0;
       uint32_t padded_lanes = 0;
       const uint32_t dst = tc::smem_u32(smem) + (is_v ? sm.vring[s] : sm.kring[s]);
@@ -731,7 +741,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
           const int b = nxt_b;
           cur_dk = nxt_dk;
           cur_rec = record(i + lane, b);
-          cur_mask = is_v ? ~0ull : table_mask(p, b);
+          cur_mask = is_v ? ~0ull : (i == 0 ? pre_mask : table_mask(p, b));
           padded_lanes = __ballot_sync(0xffffffffu, cur_mask != ~0ull);
           nxt_b = nn_b;
           nxt_dk = key_scale(i + 32 + lane, nxt_b);

@@ -166,8 +166,8 @@ __global__ void set_gscale_kernel(float *gscale, int which, int first, int n, Sc
 }
 
 // Zeros in front of a call's kernels, as a kernel of their chain: a memset node starts when everything before it has ended, and
-// the first kernel after it when the memset has (smallest call 31.9 -> 29.3 us, 24 heads of 8,192 tokens 404.7 -> 402.5).  Workspace regions are
-// multiples of 256 bytes.
+// the first kernel after it when the memset has (smallest call 31.9 -> 29.3 us, 24 heads of 8,192 tokens 404.7 -> 402.5).
+// Workspace regions are multiples of 256 bytes.
 constexpr int kClearThreads = 256;
 __global__ void clear_kernel(uint4 *words, uint32_t n) {
   const uint32_t i = blockIdx.x * kClearThreads + threadIdx.x;
