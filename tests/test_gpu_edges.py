@@ -72,7 +72,7 @@ def test_lists_of_odd_and_even_segments(n16, n8, n4, d):
 
 @pytest.mark.parametrize("H", [1, 8, 30])
 def test_pooling_splits(H):
-    """80 blocks a head: eight, four and one warp per block."""
+    """80 blocks a head: eight, four and two warps per block."""
     w = W("pool", 1, H, 128, 5, 27, 30, 0.1, 0.2, 0.2, seed=33)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
     plan, ws, _ = run_gpu(w, q, k, v)
