@@ -72,7 +72,7 @@ def test_lists_of_odd_and_even_segments(n16, n8, n4, d):
 
 @pytest.mark.parametrize("H", [1, 8, 30])
 def test_pooling_splits(H):
-    """80 blocks a head: eight, four and two warps per block."""
+    """80 blocks a head: eight and two warps per block."""
     w = W("pool", 1, H, 128, 5, 27, 30, 0.1, 0.2, 0.2, seed=33)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
     plan, ws, _ = run_gpu(w, q, k, v)
@@ -81,7 +81,7 @@ def test_pooling_splits(H):
 
 
 # 80 blocks a head: 4, 2 and 1 warps per block at d = 128; 8, 4, 2 and 1 at d = 64
-@pytest.mark.parametrize("H,d", [(8, 128), (12, 128), (20, 128), (5, 64), (8, 64), (20, 64), (30, 64)])
+@pytest.mark.parametrize("H,d", [(5, 128), (8, 128), (20, 128), (2, 64), (5, 64), (20, 64), (30, 64)])
 def test_pooling_by_waves(H, d):
     w = W("pool", 1, H, d, 5, 27, 30, 0.1, 0.2, 0.2, seed=36)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
