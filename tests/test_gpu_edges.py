@@ -4,6 +4,8 @@ head around the pooling splits, lists whose segments are shorter or longer than 
 Bars as in test_gpu_parity.py (its checks are used): descriptors, codes, scales and lists exact, outputs within the bf16
 tolerance of the oracle.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -167,6 +169,35 @@ def test_operands_follow_their_own_call(H, T, Hg, Wg, fixed):
     torch.cuda.synchronize()
     for i, g_ in got:
         assert torch.equal(g_, alone[i])
+
+
+@pytest.mark.parametrize("rank_scope", [0, 1])
+@pytest.mark.parametrize("call", ["prepare", "refresh", "cached", "cached_reselect"])
+def test_a_call_starts_behind_all_earlier_work(call, rank_scope):
+    """The first kernel of a preparation depends on the completion of what the caller enqueued before it; only the kernels behind
+    it may start early.  Read off the edges of a captured graph."""
+    w = W("edges", 1, 2, 64, 2, 16, 16, 0.1, 0.2, 0.3, seed=38)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, _ = run_gpu(w, q, k, v, rank_scope=rank_scope)
+    rt = ctypes.CDLL("libcudart.so.12")
+    stream = torch.cuda.Stream()
+    handle, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        assert rt.cudaStreamBeginCapture(handle, 2) == 0          # relaxed mode
+        q.mul_(1.0)                                               # a kernel of the caller's
+        {"prepare": lambda: da2.da2_prepare(plan, q, k, v, ws), "refresh": lambda: da2.da2_refresh_operands(plan, q, k, v, ws),
+         "cached": lambda: da2.da2_prepare_cached_scales(plan, q, k, v, ws, reselect=False),
+         "cached_reselect": lambda: da2.da2_prepare_cached_scales(plan, q, k, v, ws, reselect=True)}[call]()
+        assert rt.cudaStreamEndCapture(handle, ctypes.byref(graph)) == 0
+    assert rt.cudaGraphGetEdges_v2(graph, None, None, None, ctypes.byref(n)) == 0
+    src, dst = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)()
+    data = (ctypes.c_uint8 * (8 * n.value))()                     # 8 bytes an edge; the third says: 0 full, 1 programmatic
+    assert rt.cudaGraphGetEdges_v2(graph, src, dst, data, ctypes.byref(n)) == 0
+    kinds = {src[i]: data[8 * i + 2] for i in range(n.value)}     # a chain: one edge out of every node but the last
+    caller = set(src) - set(dst)
+    assert len(kinds) == n.value and len(caller) == 1 and kinds[caller.pop()] == 0 and 1 in kinds.values()
+    assert rt.cudaGraphDestroy(graph) == 0
 
 
 _HELD = (2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 56, 64)  # entries per lane a row may be held in
