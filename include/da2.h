@@ -207,8 +207,7 @@ da2_status_t da2_attention_host(const da2_config_t *cfg, const void *hq, const v
 da2_status_t da2_device_status(const da2_plan_t *plan, const void *workspace, void *stream);
 
 /* Number of kernels that the CALLING THREAD's last da2_prepare / da2_refresh_operands / da2_attention_fwd enqueued
- * (launch accounting; kept per thread, so the plan stays immutable; the kernel that only clears words is not counted).
- * plan must be non-NULL. */
+ * (launch accounting; kept per thread, so the plan stays immutable).  plan must be non-NULL. */
 int32_t da2_last_launch_count(const da2_plan_t *plan);
 
 /* Failure-path probe (the paper has no counterpart; it exists so that the bounded device-side waits can be tested

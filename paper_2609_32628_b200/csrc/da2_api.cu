@@ -168,10 +168,10 @@ __global__ void set_gscale_kernel(float *gscale, int which, int first, int n, Sc
 // Zeros in front of a call's kernels.  This kernel is the first of a call and the only one of it that is launched without
 // programmatic serialization: it starts when everything before it in the caller's stream has ended, whether or not the caller's
 // own kernels wait for each other, and the kernels behind it are chained to it.  (Chained to the caller's last kernel as well it
-// hides another 1.7 us of a small call, but vouches for that kernel only, and blocks that wait early cost more than that
+// hides another 1.9 us of a small call, but vouches for that kernel only, and blocks that wait early cost more than that
 // elsewhere: da2_prepare_cached_scales of 2 heads of 128 blocks 29.2 -> 34.8 us, da2_refresh_operands of 24 heads of 256 blocks
-// 209 -> 218.  A memset in its place, behind which the next kernel cannot be launched early: smallest call 32.4 us, with the
-// kernel 31.9 us; 24 heads of 8,192 tokens the same.)  Workspace regions are multiples of 256 bytes.
+// 209 -> 218.  With a memset in its place, behind which the next kernel cannot be launched early, 2 heads of 1,024 tokens take
+// 30.0 us instead of 29.2.)  Workspace regions are multiples of 256 bytes.
 constexpr int kClearThreads = 256;
 __global__ void clear_kernel(uint4 *words, uint32_t n) {
   const uint32_t i = blockIdx.x * kClearThreads + threadIdx.x;
@@ -179,8 +179,9 @@ __global__ void clear_kernel(uint4 *words, uint32_t n) {
   da2::grid_wait();
   if (i < n) words[i] = make_uint4(0u, 0u, 0u, 0u);
 }
-cudaError_t clear(void *workspace, uint64_t offset, uint64_t bytes, cudaStream_t st) {
+cudaError_t clear(void *workspace, uint64_t offset, uint64_t bytes, cudaStream_t st, int *launches) {
   const uint32_t n = (uint32_t)(bytes / sizeof(uint4));
+  *launches += 1;
   return da2::launch(false, clear_kernel, dim3((n + kClearThreads - 1) / kClearThreads), kClearThreads, 0, st,
                      reinterpret_cast<uint4 *>((uint8_t *)workspace + offset), n);
 }
@@ -330,7 +331,7 @@ da2_status_t prepare_impl(const da2_plan_t *plan, const void *q, const void *k, 
   int launches = 0;
   t_last_launches = 0;
   // status word, head maxima and per-channel maxima start at zero (they are contiguous)
-  if (clear(workspace, I.off_status, I.off_gscale - I.off_status, st) != cudaSuccess) return DA2_ERR_CUDA;
+  if (clear(workspace, I.off_status, I.off_gscale - I.off_status, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   const __nv_bfloat16 *qb = (const __nv_bfloat16 *)q, *kb = (const __nv_bfloat16 *)k, *vb = (const __nv_bfloat16 *)v;
   if (da2::launch_pool(p, qb, kb, vb, st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   for (int i = 0; i < 3; ++i) {  // caller-fixed NVFP4 per-tensor scales replace the derived ones
@@ -380,7 +381,7 @@ da2_status_t da2_prepare_cached_scales(const da2_plan_t *plan, const void *q, co
   int launches = 0;
   t_last_launches = 0;
   // only the status word is cleared: the statistics and the scales derived from them stay as the earlier call left them
-  if (clear(workspace, plan->info.off_status, 64 * sizeof(int), st) != cudaSuccess) return DA2_ERR_CUDA;
+  if (clear(workspace, plan->info.off_status, 64 * sizeof(int), st, &launches) != cudaSuccess) return DA2_ERR_CUDA;
   const __nv_bfloat16 *qb = (const __nv_bfloat16 *)q, *kb = (const __nv_bfloat16 *)k, *vb = (const __nv_bfloat16 *)v;
   if (da2::launch_prep(p, qb, kb, vb, st, &launches, /*pool=*/true) != cudaSuccess) return DA2_ERR_CUDA;
   if (reselect) {

@@ -175,7 +175,7 @@ def test_operands_follow_their_own_call(H, T, Hg, Wg, fixed):
 @pytest.mark.parametrize("call", ["prepare", "refresh", "cached", "cached_reselect"])
 def test_a_call_starts_behind_all_earlier_work(call, rank_scope):
     """The first kernel of a preparation depends on the completion of what the caller enqueued before it; only the kernels behind
-    it may start early.  Read off the edges of a captured graph."""
+    it may start early.  Read off the edges of a captured graph, whose nodes are as many as the launches reported."""
     w = W("edges", 1, 2, 64, 2, 16, 16, 0.1, 0.2, 0.3, seed=38)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
     plan, ws, _ = run_gpu(w, q, k, v, rank_scope=rank_scope)
@@ -197,6 +197,8 @@ def test_a_call_starts_behind_all_earlier_work(call, rank_scope):
     kinds = {src[i]: data[8 * i + 2] for i in range(n.value)}     # a chain: one edge out of every node but the last
     caller = set(src) - set(dst)
     assert len(kinds) == n.value and len(caller) == 1 and kinds[caller.pop()] == 0 and 1 in kinds.values()
+    assert rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    assert n.value == 1 + da2.da2_last_launch_count(plan)
     assert rt.cudaGraphDestroy(graph) == 0
 
 

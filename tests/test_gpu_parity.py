@@ -411,7 +411,7 @@ def test_prepare_cached_scales_is_one_pass_with_carried_over_scales(reselect):
     g_fixed = (g1[:, 0], g1[:, 1], g1[:, 2])
     out = torch.full_like(q2, float("nan"))
     da2.da2_prepare_cached_scales(plan, q2, k2, v2, ws, reselect=reselect)
-    assert da2.da2_last_launch_count(plan) == (3 if reselect else 1)   # one pass over Q, K, V (+ draft map, ranking)
+    assert da2.da2_last_launch_count(plan) == (4 if reselect else 2)   # words cleared, one pass over Q, K, V (+ draft map, ranking)
     da2.da2_attention_fwd(plan, q2, k2, v2, ws, out)
     torch.cuda.synchronize()
     assert da2.da2_device_status(plan, ws) == 0
@@ -427,7 +427,7 @@ def test_prepare_cached_scales_is_one_pass_with_carried_over_scales(reselect):
 
 
 def test_prepare_and_attention_replay_from_a_cuda_graph():
-    """The two calls only enqueue kernels and a memset on the caller's stream (no allocation, no synchronisation), so
+    """The two calls only enqueue kernels on the caller's stream (no allocation, no synchronisation), so
     a captured graph of them replays to the same bits as the eager calls."""
     w = SMALL["ragged64"]
     q, k, v = _inputs(w)
