@@ -193,23 +193,21 @@ __global__ void __launch_bounds__(kPoolWarps * 32) pool_kernel(Params p, const u
 
 cudaError_t launch_pool(const Params &p, const __nv_bfloat16 *q, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                         cudaStream_t st, int *launches) {
-  // Warps per block.  Up to two blocks an SM: all eight, the call is the latency of one block.  Else the number with the
-  // shortest waves: an SM holds two CTAs at d = 128 and three at d = 64 (registers); a wave lasts the batches of loads that a
-  // warp walks one after the other, and start, combination and atomics cost about three more.  So a last wave that would be
-  // nearly empty is made shorter instead.  (With the split by the number of blocks alone, 8 below 592, 4 below 2,368, else 1
+  // Warps per block: the number with the shortest waves.  An SM holds two CTAs at d = 128 and three at d = 64 (registers); a wave
+  // lasts the batches of loads that a warp walks one after the other, and start, combination and atomics cost about three more.
+  // So a call whose blocks fit one wave with eight warps each takes eight (it is the latency of one block), and a last wave that
+  // would be nearly empty is made shorter.  (With the split by the number of blocks alone, 8 below 592, 4 below 2,368, else 1
   // -> now, us; da2_prepare at d = 128, 128 blocks a head: 8 heads 63.6 -> 59.7, 12 heads 86.4 -> 80.0, 17 heads 113.5 -> 102.5,
   // 24 heads 143.3 -> 138.3; d = 64, 8 heads of 168 blocks 53.2 -> 51.0; whole calls, 4 heads of 128 blocks 97.8 -> 92.0, 5 heads
-  // 118.4 -> 115.7, one head of 588 blocks 220.8 -> 215.0.)
-  const long long blocks = (long long)p.R * p.BH;
-  int split = 8;
-  if (blocks >= kSms * 2) {
-    const long long wave = (long long)kSms * (p.d == 128 ? 2 : 3);
-    long long best = 0;
-    for (int s = 1; s <= 4; s *= 2) {
-      const long long ctas = (long long)p.BH * ((p.R * s + kPoolWarps - 1) / kPoolWarps);
-      const long long cost = (ctas + wave - 1) / wave * (kSlots / kBatch / s + 3);
-      if (s == 1 || cost < best) { best = cost; split = s; }
-    }
+  // 118.4 -> 115.7, one head of 588 blocks 220.8 -> 215.0.  Eight and four warps at d = 64, da2_refresh_operands: 20 heads of 16
+  // blocks 18.8 and 20.6, 24 heads 19.4 and 20.7, 5 heads of 64 blocks 19.1 and 20.6, of 80 blocks 20.5 and 20.7.)
+  const long long wave = (long long)kSms * (p.d == 128 ? 2 : 3);
+  int split = 1;
+  long long best = 0;
+  for (int s = 1; s <= kPoolWarps; s *= 2) {
+    const long long ctas = (long long)p.BH * ((p.R * s + kPoolWarps - 1) / kPoolWarps);
+    const long long cost = (ctas + wave - 1) / wave * (kSlots / kBatch / s + 3);
+    if (s == 1 || cost < best) { best = cost; split = s; }
   }
   const dim3 grid((p.R * split + kPoolWarps - 1) / kPoolWarps, p.BH);
   const uint16_t *q16 = reinterpret_cast<const uint16_t *>(q), *k16 = reinterpret_cast<const uint16_t *>(k),

@@ -82,8 +82,8 @@ def test_pooling_splits(H):
     _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
 
 
-# 80 blocks a head: 4, 2 and 1 warps per block at d = 128; 8, 4, 2 and 1 at d = 64
-@pytest.mark.parametrize("H,d", [(5, 128), (8, 128), (20, 128), (2, 64), (5, 64), (20, 64), (30, 64)])
+# 80 blocks a head: 4, 2 and 1 warps per block at d = 128; 8, 8, 4, 2 and 1 at d = 64
+@pytest.mark.parametrize("H,d", [(5, 128), (8, 128), (20, 128), (2, 64), (5, 64), (8, 64), (20, 64), (30, 64)])
 def test_pooling_by_waves(H, d):
     w = W("pool", 1, H, d, 5, 27, 30, 0.1, 0.2, 0.2, seed=36)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
