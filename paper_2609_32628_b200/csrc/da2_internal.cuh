@@ -165,21 +165,32 @@ __device__ __forceinline__ uint32_t magnitudes2(uint32_t m) { return m & 0x7fff7
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // A launch's own status, chained or not.  It is taken out of the runtime's record, so that the next call does not report it again.
+// all_shared: the SMs that the kernel comes to are set to their largest shared memory, not to what its own blocks need.
 template <class... KArgs, class... Args>
-cudaError_t launch(bool chained, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch(bool chained, bool all_shared, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                   Args... args) {
+  cudaLaunchAttribute attr[2] = {};
   cudaLaunchConfig_t cfg = {};
+  if (chained) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (all_shared) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[cfg.numAttrs++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  }
   cfg.gridDim = grid;
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = chained ? 1 : 0;
+  cfg.attrs = attr;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
   if (e != cudaSuccess) cudaGetLastError();
   return e;
+}
+template <class... KArgs, class... Args>
+cudaError_t launch(bool chained, void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+  return launch(chained, false, kernel, grid, threads, smem, st, args...);
 }
 template <class... KArgs, class... Args>
 cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {

@@ -114,19 +114,25 @@ cudaError_t launch_draft(const Params &p, cudaStream_t st, int *launches) {
   const dim3 grid((p.R + TILE - 1) / TILE, (p.R + TILE - 1) / TILE, p.BH * 2);
   // Three CTAs fit an SM, but the kernel starts while the pooling kernel still fills the SMs, and the few CTAs of a small map
   // would be packed three to an SM wherever there is room, to share its fp64 pipe while others stay idle.  So a grid of up to
-  // one, or two, CTAs per SM asks for so much shared memory that no more than that fit.  (da2_prepare, us: 2 heads of 128
-  // blocks 36.8 -> 28.2, 8 heads 59.3 -> 52.5, 12 heads 80.0 -> 76.7, 24 heads 138.1 -> 134.6; d = 64, 8 heads of 168 blocks
-  // 50.7 -> 47.5; larger grids as before.)
+  // one, or two, CTAs per SM asks for so much shared memory that no more than that fit.  Rows of up to half a tile give a CTA
+  // one working warp and the pipe nothing to share.  (da2_prepare, us: 2 heads of 128 blocks 36.8 -> 28.2, 8 heads 59.3 -> 52.5,
+  // 12 heads 80.0 -> 76.7, 24 heads 138.1 -> 134.6; d = 64, 8 heads of 168 blocks 50.7 -> 47.5; larger grids as before.)
+  // The operand kernel's blocks run beside these CTAs.  Where they are one wave (four an SM), the SMs keep all of their shared
+  // memory: set to what a CTA of this kernel needs they take no such block until it has ended, and the last blocks then start
+  // late (whole calls, d = 128: 4 heads of 128 blocks 117.8 -> 110.5, 6 heads of 80 95.8 -> 89.9; d = 64: 4 heads of 128 blocks
+  // 103.4 -> 98.7).  With more blocks there is a second wave anyway, and the logits are the sooner ready if they have the SM to
+  // themselves (6 heads of 128 blocks 154.4, with blocks beside them 156.8).
   const int tiles = 2 * TILE * ((p.d < kChunk ? p.d : kChunk) + 4) * (int)sizeof(float);
   const long long ctas = (long long)grid.x * grid.y * grid.z;
   constexpr int kOne = 116 * 1024, kTwo = 78 * 1024;  // one CTA to an SM's 228 KB, two
-  const int smem = ctas <= kSms ? kOne : (ctas <= 2 * kSms ? kTwo : tiles);
+  const bool spread = p.R > TILE / 2 && ctas <= 2 * kSms;
+  const int smem = !spread ? tiles : (ctas <= kSms ? kOne : kTwo);
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(draft_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOne);
     if (e != cudaSuccess) return e;
   }
   *launches += 1;
-  return launch_chained(draft_logits_kernel, grid, 128, smem, st, p);
+  return launch(true, spread && (long long)p.BH * p.Rt <= 4 * kSms, draft_logits_kernel, grid, 128, smem, st, p);
 }
 
 }  // namespace da2

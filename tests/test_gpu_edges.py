@@ -92,6 +92,26 @@ def test_pooling_by_waves(H, d):
     _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
 
 
+# rows of half a tile and one more, and the grids of one and of two CTAs per SM with the next larger ones
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("H,R", [(16, 32), (16, 33), (74, 33), (75, 33), (148, 33), (149, 33)])
+def test_draft_logits_by_grid(H, R, d):
+    """Logits against their definition in fp64 (one rounding to fp32; an fp64 sum of d terms errs by d half ulps of its largest
+    partial sum at most), and what runs beside them against the oracle."""
+    w = W("logits", 1, H, d, R, 8, 8, 0.0, 0.1, 0.3, seed=39)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, _ = run_gpu(w, q, k, v)
+    I = plan.info
+    desc = [ws[I.off_desc[i]:I.off_desc[i] + H * R * d * 4].view(torch.float32).view(H, R, d).double() for i in range(4)]
+    for i in range(2):
+        got = ws[I.off_logits[i]:I.off_logits[i] + H * R * R * 4].view(torch.float32).view(H, R, R).double()
+        exp = float(I.softmax_scale) * desc[i] @ desc[2 + i].transpose(1, 2)
+        mag = float(I.softmax_scale) * desc[i].abs() @ desc[2 + i].abs().transpose(1, 2)
+        assert ((got - exp).abs() <= exp.abs() * 2.0 ** -24 + mag * (2 * d * 2.0 ** -53 + 2.0 ** -52)).all()
+    heads = [0, H - 1]
+    _check_prepare(w, plan, ws, oracle_all(w, q, k, v, heads=heads), heads=heads)
+
+
 @pytest.mark.parametrize("T,Hg,Wg", [(1, 8, 8), (3, 9, 20), (13, 8, 40), (23, 24, 56), (683, 8, 24)])
 @pytest.mark.parametrize("f16,f8,f4", [(0.1, 0.2, 0.3), (0.0, 0.1, 0.2)])
 def test_head_scope_sizes(T, Hg, Wg, f16, f8, f4):
