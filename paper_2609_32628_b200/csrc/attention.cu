@@ -724,7 +724,8 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const int depth = is_v ? sm.nv : sm.nk;  // ring entries
       int kk = 0;                              // ring entry
       uint32_t kpar = 1;                       // parity of the consumption that frees the entry
-      bool kwrapped = false, ok = true;        // ring gone round
+      bool kwrapped = false;                   // ring gone round
+      int q_par = S.n48 > 0 ? 0 : -1;          // parity of the last request for Q records
       // lane l holds the record's address, the mask and the key scale of list entry 32 * batch + l
       auto record = [&](int idx, int b) -> unsigned long long {
         const int t = S.tier(idx);
@@ -752,11 +753,12 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         const uint32_t n0 = B16 && i >= S.n48 ? nb2 : (FP4 && i < S.n4 ? nb0 : nb1), n1 = !two ? 0u : (FP4 && i + 1 < S.n4 ? nb0 : nb1);
         if (B16 && i == S.n48 && !is_v) {
           // the Q buffer is free once every product of the segments before is done: their last K blocks are consumed
-          if (i > 0 && !(ok = wait_or_abort(bar(s, B_KFREE) + (uint32_t)(kk == 0 ? depth - 1 : kk - 1) * 8u, kk == 0 ? kpar : kpar ^ 1u, abortp))) break;
+          if (i > 0 && !wait_or_abort(bar(s, B_KFREE) + (uint32_t)(kk == 0 ? depth - 1 : kk - 1) * 8u, kk == 0 ? kpar : kpar ^ 1u, abortp)) break;
           load_q(2, 2);
           __syncwarp();
+          q_par = S.n48 > 0;
         }
-        if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) break;
+        if (kwrapped && !wait_or_abort(bar(s, b_free + kk), kpar, abortp)) break;
         if (!is_v) {
           // the steps' masks and key scales are written before the data the softmax waits for is requested
           const int e = i & (kInfoRing - 1);
@@ -783,14 +785,14 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         i += !B16 || two ? 2 : 1;
         if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
       }
-      if (!ok || *(volatile int *)abortp) {  // after a give-up: this warp's own copies land before the block may exit (bounded)
-        // entries before kk were used in this round of the ring, the others in the round before
-        const uint32_t used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
-        const uint32_t par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
+      // A block exits only when its copies have landed, also those that nobody waits for any more after a give-up (bounded).
+      // Entries before kk were used in this round of the ring, the others in the round before.
+      const uint32_t used = kwrapped ? (1u << depth) - 1u : (1u << kk) - 1u;
+      const uint32_t par = kpar ? (kwrapped ? ((1u << depth) - 1u) & ~((1u << kk) - 1u) : 0u) : (1u << kk) - 1u;
 #pragma unroll 1
-        for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
-          if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
-      }
+      for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
+        if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
+      if (!is_v && q_par >= 0) tc::mbar_wait(bar(s, B_Q), (uint32_t)q_par, 1u << 14);
     }
   }
   // =========================================================================================== MMA warps
