@@ -725,7 +725,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       int kk = 0;                              // ring entry
       uint32_t kpar = 1;                       // parity of the consumption that frees the entry
       bool kwrapped = false;                   // ring gone round
-      int q_par = S.n48 > 0 ? 0 : -1;          // parity of the last request for Q records
+      uint32_t q_par = 0;                      // parity of the last request for Q records (one comes before the first wait)
       // lane l holds the record's address, the mask and the key scale of list entry 32 * batch + l
       auto record = [&](int idx, int b) -> unsigned long long {
         const int t = S.tier(idx);
@@ -792,7 +792,7 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
 #pragma unroll 1
       for (int k = 0; k < (is_v ? kMaxV : kMaxK); ++k)
         if ((used >> k) & 1u) tc::mbar_wait(bar(s, b_full + k), (par >> k) & 1u, 1u << 14);
-      if (!is_v && q_par >= 0) tc::mbar_wait(bar(s, B_Q), (uint32_t)q_par, 1u << 14);
+      if (!is_v) tc::mbar_wait(bar(s, B_Q), q_par, 1u << 14);
     }
   }
   // =========================================================================================== MMA warps
