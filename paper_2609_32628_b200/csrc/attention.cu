@@ -734,8 +734,14 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
       const uint32_t nb0 = is_v ? sm.vbytes[0] : sm.kbytes[0], nb1 = is_v ? sm.vbytes[1] : sm.kbytes[1], nb2 = is_v ? sm.vbytes[2] : sm.kbytes[2];
       uint2 *const infos = s_info + s * kInfoRing;
       unsigned long long cur_rec = 0;
+      // The 16-bit segment has a loop of its own where the plan has no 4-bit tier: its blocks come one by one, and in the loop
+      // for pairs the second one's instructions cost plans of the 16-bit tier alone 2 % (24 heads of 8,192 tokens at d = 64, 30 %
+      // kept: 343 and 336 us).  Beside a 4-bit tier the one loop for both is the faster one, as the code is smaller.
+      constexpr bool kOwnLoop = B16 && !FP4;
+      bool ok = true;
+      int i = 0;
 #pragma unroll 1
-      for (int i = 0; i < S.L;) {
+      while (i < (kOwnLoop ? S.n48 : S.L)) {
         const int src = i & 31;
         const bool two = i + 1 < (B16 ? S.n48 : S.L);
         if (src == 0) {  // next batch: its ids and scales were requested one batch ago
@@ -751,14 +757,14 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         const uint32_t lo0 = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src), hi0 = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src);
         const uint32_t lo1 = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src + 1), hi1 = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src + 1);
         const uint32_t n0 = B16 && i >= S.n48 ? nb2 : (FP4 && i < S.n4 ? nb0 : nb1), n1 = !two ? 0u : (FP4 && i + 1 < S.n4 ? nb0 : nb1);
-        if (B16 && i == S.n48 && !is_v) {
+        if (B16 && !kOwnLoop && i == S.n48 && !is_v) {
           // the Q buffer is free once every product of the segments before is done: their last K blocks are consumed
           if (i > 0 && !wait_or_abort(bar(s, B_KFREE) + (uint32_t)(kk == 0 ? depth - 1 : kk - 1) * 8u, kk == 0 ? kpar : kpar ^ 1u, abortp)) break;
           load_q(2, 2);
           __syncwarp();
           q_par = S.n48 > 0;
         }
-        if (kwrapped && !wait_or_abort(bar(s, b_free + kk), kpar, abortp)) break;
+        if (kwrapped && !(ok = wait_or_abort(bar(s, b_free + kk), kpar, abortp))) break;
         if (!is_v) {
           // the steps' masks and key scales are written before the data the softmax waits for is requested
           const int e = i & (kInfoRing - 1);
@@ -784,6 +790,49 @@ __global__ void __launch_bounds__(NT, 1) attention_kernel(Params p, SmemMap sm, 
         __syncwarp();
         i += !B16 || two ? 2 : 1;
         if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
+      }
+      if (kOwnLoop && ok && i < S.L) {  // (the steps are those of the loop above, which compiles to slower code with any of them shared)
+        if (!is_v) {
+          ok = i == 0 || wait_or_abort(bar(s, B_KFREE) + (uint32_t)(kk == 0 ? depth - 1 : kk - 1) * 8u, kk == 0 ? kpar : kpar ^ 1u, abortp);
+          if (ok) {
+            load_q(2, 2);
+            q_par = S.n48 > 0;
+          }
+          __syncwarp();
+        }
+#pragma unroll 1
+        for (; ok && i < S.L; ++i) {
+          const int src = i & 31;
+          if (src == 0) {
+            const int b = nxt_b;
+            cur_rec = record(i + lane, b);
+            cur_mask = is_v ? ~0ull : (i == 0 ? pre_mask : table_mask(p, b));
+            padded_lanes = __ballot_sync(0xffffffffu, cur_mask != ~0ull);
+            nxt_b = nn_b;
+            nn_b = list_id(i + 64 + lane);
+          }
+          const uint32_t lo = __shfl_sync(0xffffffffu, (uint32_t)cur_rec, src), hi = __shfl_sync(0xffffffffu, (uint32_t)(cur_rec >> 32), src);
+          if (kwrapped && !wait_or_abort(bar(s, b_free + kk), kpar, abortp)) break;
+          if (!is_v) {
+            const int e = i & (kInfoRing - 1);
+            const bool padded = (padded_lanes >> src) & 1u;
+            if (padded) {
+              float *lim = reinterpret_cast<float *>(smem + sm.lim) + (s * kInfoRing + e) * 64;
+              const uint32_t mlo = __shfl_sync(0xffffffffu, (uint32_t)cur_mask, src), mhi = __shfl_sync(0xffffffffu, (uint32_t)(cur_mask >> 32), src);
+              lim[lane] = (mlo >> lane) & 1u ? INFINITY : -INFINITY;
+              lim[32 + lane] = (mhi >> lane) & 1u ? INFINITY : -INFINITY;
+            }
+            if (lane == 0) infos[e] = make_uint2(0u, padded);  // (no key scale in the 16-bit tier)
+            __syncwarp();
+          }
+          if (tc::elect_one()) {
+            const uint32_t full = bar(s, b_full + kk);
+            tc::mbar_arrive_expect_tx(full, nb2);
+            tc::bulk_g2s(dst + (uint32_t)kk * entry, reinterpret_cast<const uint8_t *>(((unsigned long long)hi << 32) | lo), nb2, full);
+          }
+          __syncwarp();
+          if (++kk == depth) { kk = 0; kpar ^= 1u; kwrapped = true; }
+        }
       }
       // A block exits only when its copies have landed, also those that nobody waits for any more after a give-up (bounded).
       // Entries before kk were used in this round of the ring, the others in the round before.
