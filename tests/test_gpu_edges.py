@@ -59,10 +59,12 @@ def test_segments_of_three_tiers(d, f16, f8, f4):
 
 @pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("n16,n8,n4", [(0, 0, 1), (0, 1, 0), (0, 1, 1), (0, 2, 3), (0, 3, 2), (0, 33, 4), (0, 1, 34), (1, 0, 0),
-                                       (1, 1, 0), (1, 0, 1), (2, 1, 2), (3, 2, 1), (1, 32, 3), (5, 16, 17)])
+                                       (1, 1, 0), (1, 0, 1), (2, 1, 2), (3, 2, 1), (1, 32, 3), (5, 16, 17), (0, 0, 31), (0, 0, 32),
+                                       (0, 1, 31), (0, 3, 31), (0, 3, 32), (4, 0, 31), (4, 0, 32), (3, 15, 16), (3, 14, 17),
+                                       (1, 15, 16), (31, 0, 0), (32, 0, 0), (33, 0, 0), (2, 31, 0), (1, 0, 30)])
 def test_lists_of_odd_and_even_segments(n16, n8, n4, d):
-    """Blocks of a list are fetched in pairs (those of the 16-bit tier one by one): segments that end in the middle of a pair, and
-    one below, at and above the 32 entries that a loader holds, on ragged tiles."""
+    """Blocks of a list are fetched in pairs (those of the 16-bit tier one by one): segments and lists that end in the middle of a
+    pair, and one below, at and above the 32 entries that a loader holds, on ragged tiles."""
     w = W("pairs", 1, 2, d, 5, 12, 28, n16 / 40, n8 / 40, n4 / 40, seed=37)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
     plan, ws, out = run_gpu(w, q, k, v)
@@ -72,9 +74,25 @@ def test_lists_of_odd_and_even_segments(n16, n8, n4, d):
     _check_attention(w, out, ref, [(h, a) for h in range(2) for a in (0, 3, 20, 39)], bad)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("f16,f8,f4", [(0.1, 0.2, 0.45), (0.0, 0.25, 0.5), (0.25, 0.5, 0.0)])
+def test_head_scope_lists_that_end_at_a_loaders_batch(f16, f8, f4, d):
+    """The same with one ranking per head: every row whose segments or list end one below, at or above 32 entries."""
+    w = W("batch", 1, 8, d, 5, 12, 28, f16, f8, f4, seed=40)
+    q, k, v = da2_inputs.make_qkv(w, "cuda")
+    plan, ws, out = run_gpu(w, q, k, v, rank_scope=1)
+    ref = oracle_all(w, q, k, v, rank_scope=1)
+    bad = _check_prepare(w, plan, ws, ref)
+    _, cnt = Workspace(plan, ws).lists()
+    ends = np.cumsum(cnt, 2)
+    sel = [(int(h), int(a)) for h, a in np.argwhere(((ends >= 31) & (ends <= 33)).any(2))]
+    assert all((ends == n).any() for n in (31, 32, 33))
+    _check_attention(w, out, ref, sel, bad)
+
+
 @pytest.mark.parametrize("H", [1, 8, 30])
 def test_pooling_splits(H):
-    """80 blocks a head: eight and two warps per block."""
+    """80 blocks a head: eight and two warps per block (two twice)."""
     w = W("pool", 1, H, 128, 5, 27, 30, 0.1, 0.2, 0.2, seed=33)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
     plan, ws, _ = run_gpu(w, q, k, v)
