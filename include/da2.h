@@ -20,7 +20,10 @@
  *     all device memory; the library allocates none and keeps no device state between calls (one exception:
  *     da2_draft_map_noalloc, which owns a fixed scratch array, see there).
  *   - stream: a cudaStream_t passed as void* (NULL = default stream).  da2_prepare and da2_attention_fwd only
- *     enqueue work and never synchronise.
+ *     enqueue work and never synchronise.  The preparation calls start when everything enqueued before them has ended.
+ *     da2_attention_fwd and da2_draft_map_noalloc wait for the end of the kernel directly before them in the stream; if
+ *     that is a kernel of the caller's launched with programmatic stream serialization, it has to wait for the kernels
+ *     before it itself (griddepcontrol.wait), as such kernels do.
  *   - Errors are return codes.  Argument errors are detected before any launch.  A device-side bounded wait that
  *     gives up records a code in the workspace status word; da2_device_status reports it.
  *   - The plan is host memory owned by the library until da2_plan_destroy; it is immutable (no call writes to it,
