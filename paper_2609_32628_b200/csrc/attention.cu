@@ -43,8 +43,8 @@
 // block by block, its request rate was 94 % of the peak (all-4-bit call of 16x48x48, 24 heads; special-function pipe 70 %, issue
 // slots 69 %, tensor pipe 22 %).  So the instructions of a step are what is saved, in the roles around the softmax above all: the
 // loaders, the Q K^T warps and the PV warps take the blocks of a list in pairs, with one ring entry, one wait and one round of
-// the loop for two.  Requests fell by a sixth (1.59 -> 1.33 G), instructions by 8 % (9.34 -> 8.60 G) and the time by 5.5 %
-// (12.59 -> 11.90 ms): at 82 % of the peak rate the fetch is no longer alone.  Taking PV and correction in pairs as well makes
+// the loop for two.  Requests fell by 18 % (1.59 -> 1.30 G), instructions by 8 % (9.34 -> 8.61 G) and the time by 5 %
+// (12.59 -> 11.99 ms): at 81 % of the peak rate the fetch is no longer alone.  Taking PV and correction in pairs as well makes
 // the products late (13.3 ms), and softmax steps of two blocks have 7.33 G instructions and 67 % of the request rate, but leave
 // two warps a scheduler, which do not cover the latencies (13.7 ms).
 // The softmax keeps the work inside the chain of hand-offs short: the row maximum is taken on raw accumulator values, the
