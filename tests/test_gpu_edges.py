@@ -210,13 +210,15 @@ def test_operands_follow_their_own_call(H, T, Hg, Wg, fixed):
 
 
 @pytest.mark.parametrize("rank_scope", [0, 1])
+@pytest.mark.parametrize("T,Hg,Wg", [(2, 16, 16), (5, 24, 40)])
 @pytest.mark.parametrize("call", ["prepare", "refresh", "cached", "cached_reselect"])
-def test_a_call_starts_behind_all_earlier_work(call, rank_scope):
+def test_a_call_starts_behind_all_earlier_work(call, T, Hg, Wg, rank_scope):
     """The first kernel of a preparation depends on the completion of what the caller enqueued before it; only the kernels behind
-    it may start early.  Read off the edges of a captured graph, whose nodes are as many as the launches reported."""
-    w = W("edges", 1, 2, 64, 2, 16, 16, 0.1, 0.2, 0.3, seed=38)
+    it may start early.  Read off the edges of a captured graph, whose nodes are as many as the launches reported; a replay
+    leaves the same bits in the workspace (8 and 75 blocks a head: logits in plain and in spread grids)."""
+    w = W("edges", 1, 2, 64, T, Hg, Wg, 0.1, 0.2, 0.3, seed=38)
     q, k, v = da2_inputs.make_qkv(w, "cuda")
-    plan, ws, _ = run_gpu(w, q, k, v, rank_scope=rank_scope)
+    plan, ws, _ = run_gpu(w, q, k, v, rank_scope=rank_scope, zero_ws=True)
     rt = ctypes.CDLL("libcudart.so.12")
     stream = torch.cuda.Stream()
     handle, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
@@ -237,7 +239,15 @@ def test_a_call_starts_behind_all_earlier_work(call, rank_scope):
     assert len(kinds) == n.value and len(caller) == 1 and kinds[caller.pop()] == 0 and 1 in kinds.values()
     assert rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)) == 0
     assert n.value == 1 + da2.da2_last_launch_count(plan)
-    assert rt.cudaGraphDestroy(graph) == 0
+    I, ref, run = plan.info, ws.clone(), ctypes.c_void_p()
+    ws[I.off_qrec[0]:I.off_dq8].zero_()
+    torch.cuda.synchronize()
+    assert rt.cudaGraphInstantiate(ctypes.byref(run), graph, ctypes.c_ulonglong(0)) == 0
+    assert rt.cudaGraphLaunch(run, handle) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(ws[I.off_vmax:I.off_select], ref[I.off_vmax:I.off_select])
+    assert torch.equal(ws[I.off_qrec[0]:], ref[I.off_qrec[0]:])
+    assert rt.cudaGraphExecDestroy(run) == 0 and rt.cudaGraphDestroy(graph) == 0
 
 
 _HELD = (2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40, 48, 56, 64)  # entries per lane a row may be held in
